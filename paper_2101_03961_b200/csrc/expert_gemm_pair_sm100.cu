@@ -13,7 +13,7 @@
 // orientation (dW_out = H^T dY_d, dW_in = X_d^T dH: M = weight rows, N = weight columns, contraction over tokens).
 //
 // A CTA pair shares the B operand: each CTA stages its own 128 A rows and half of B per 64-deep k-block, the leader
-// CTA's single MMA thread issues M=256 instructions that read both CTAs' shared memory, and tcgen05.commit with a
+// CTA's MMA warp issues M=256 instructions that read both CTAs' shared memory, and tcgen05.commit with a
 // cluster mask releases stages and publishes accumulators in both CTAs.  TMA loads carry no multicast.  Each CTA
 // drains its own 128 TMEM lanes with 8 epilogue warps while the next tile's MMAs run.
 //
@@ -210,8 +210,8 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
   int* kept_s = reinterpret_cast<int*>(bar_gen + 256);
   int4* tile_s = reinterpret_cast<int4*>(bar_gen + 256 + kPKeptCache * 4);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_ctarank();                   // 0 = leader (issues the MMAs)
+  const int warp = uniform_warp_id(), lane = threadIdx.x & 31;
+  const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);   // 0 = leader (issues the MMAs)
   const uint32_t n_stages = kTok ? (uint32_t)p.stages : (uint32_t)kPStages;
   const uint32_t stage_bytes = kTok ? (uint32_t)p.stage_bytes : (uint32_t)kPStageBytes;
 
@@ -245,34 +245,34 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
   // share the middle columns when n + n_next > 512.
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer (both CTAs)
-    if (lane == 0) {
-      uint32_t stage = 0, phase = 0;
-      bool ok = true;
-      for (int id = pair; id < n_tiles && ok; id += n_pairs) {
-        const PTile t = p_decode(p, id, kept_s, tile_s);
-        // coordinates of this CTA's boxes; only the contraction coordinate moves inside the tile
-        // gated GEMM1: 64 columns of W_0 and the same 64 columns of W_1 (a pair covers 128 hidden units)
-        const int a_m = kGated ? (t.m0 >> 1) + 64 * (int)rank : t.m0 + 128 * (int)rank;
-        const int a_m2 = kGated ? p.gate_f + a_m : a_m + 64;
-        const int e = t.e, kbs = t.k_blocks;
-        // token products: this CTA's half of each column segment's token rows, in boxes of exactly that height;
-        // weight gradients: this CTA's 128 of the 256 output columns
-        const int h1 = t.n1 >> 1, h2 = (t.n - t.n1) >> 1;
-        const int b_r = kTok ? t.row0 + (int)rank * h1 : t.n0 + 128 * (int)rank;
-        const int b_r2 = t.row0 + t.n1 + (int)rank * h2;
-        const CUtensorMap* tmB = kTok ? &bm.m[(h1 >> 3) - 1] : &bm.m[0];
-        const CUtensorMap* tmB2 = (kTok && h2 > 0) ? &bm.m[(h2 >> 3) - 1] : tmB;
-        // both CTAs' bytes land on the leader's barrier
-        const uint32_t tx_bytes = kTok ? 2u * (uint32_t)(kPHalfBytes + (t.n >> 1) * 128) : 2u * (uint32_t)kPStageBytes;
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int id = pair; id < n_tiles && ok; id += n_pairs) {
+      const PTile t = p_decode(p, id, kept_s, tile_s);
+      // coordinates of this CTA's boxes; only the contraction coordinate moves inside the tile
+      // gated GEMM1: 64 columns of W_0 and the same 64 columns of W_1 (a pair covers 128 hidden units)
+      const int a_m = kGated ? (t.m0 >> 1) + 64 * (int)rank : t.m0 + 128 * (int)rank;
+      const int a_m2 = kGated ? p.gate_f + a_m : a_m + 64;
+      const int e = t.e, kbs = t.k_blocks;
+      // token products: this CTA's half of each column segment's token rows, in boxes of exactly that height;
+      // weight gradients: this CTA's 128 of the 256 output columns
+      const int h1 = t.n1 >> 1, h2 = (t.n - t.n1) >> 1;
+      const int b_r = kTok ? t.row0 + (int)rank * h1 : t.n0 + 128 * (int)rank;
+      const int b_r2 = t.row0 + t.n1 + (int)rank * h2;
+      const CUtensorMap* tmB = kTok ? &bm.m[(h1 >> 3) - 1] : &bm.m[0];
+      const CUtensorMap* tmB2 = (kTok && h2 > 0) ? &bm.m[(h2 >> 3) - 1] : tmB;
+      // both CTAs' bytes land on the leader's barrier
+      const uint32_t tx_bytes = kTok ? 2u * (uint32_t)(kPHalfBytes + (t.n >> 1) * 128) : 2u * (uint32_t)kPStageBytes;
 #pragma unroll 1
-        for (int kb = 0; kb < kbs; ++kb) {
-          const uint32_t eb = empty0 + 8u * stage;
-          ok = mbar_wait(eb, phase ^ 1u, abort_flag, p.status, 21);
-          if (!ok) break;
-          const uint32_t a_dst = smem_base + stage * stage_bytes, b_dst = a_dst + kPHalfBytes;
-          const uint32_t fb = full0 + 8u * stage;
-          const uint32_t lead_full = fb & kPeerMask;
-          const int k0 = kb * kBK;
+      for (int kb = 0; kb < kbs; ++kb) {
+        const uint32_t eb = empty0 + 8u * stage;
+        ok = mbar_wait_warp(eb, phase ^ 1u, abort_flag, p.status, 21);
+        if (!ok) break;
+        const uint32_t a_dst = smem_base + stage * stage_bytes, b_dst = a_dst + kPHalfBytes;
+        const uint32_t fb = full0 + 8u * stage;
+        const uint32_t lead_full = fb & kPeerMask;
+        const int k0 = kb * kBK;
+        if (elect_one()) {
           if (rank == 0) mbar_arrive_expect_tx(fb, tx_bytes);
           if (kAMn) {
             tma_load_3d_pair(a_dst, &tmA, lead_full, a_m, k0, e);
@@ -287,17 +287,17 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
             tma_load_3d_pair(b_dst, tmB, lead_full, k0, b_r, e);
             if (h2 > 0) tma_load_3d_pair(b_dst + (uint32_t)h1 * 128u, tmB2, lead_full, k0, b_r2, e);
           }
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
+        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
-      if (*abort_flag != 0) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < 4000000ll) __nanosleep(1000);  // let copies in flight land (about 2 ms)
-      }
+    }
+    if (*abort_flag != 0) {
+      const long long t0 = clock64();
+      while (clock64() - t0 < 4000000ll) __nanosleep(1000);  // let copies in flight land (about 2 ms)
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------------------------------ MMA issuer (leader CTA)
-    if (lane == 0 && rank == 0) {
+    if (rank == 0) {
       constexpr uint32_t idesc_base = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)kAMn << 15) |
                                       ((uint32_t)kBMn << 16) | ((uint32_t)(256 >> 4) << 24);
       // descriptors differ between stages and k-steps only in the start-address field (units of 16 bytes)
@@ -317,11 +317,11 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
         const uint32_t b2_off = ((uint32_t)(t.n1 >> 1) * 128u) >> 4;    // second segment's rows in this CTA's half of B
         const int kbs = t.k_blocks, last_mmas = t.last_mmas;
         // the side's previous tile has been read out completely ...
-        ok = mbar_wait(tempty0 + 8u * side, (use & 1u) ^ 1u, abort_flag, p.status, 22);
+        ok = mbar_wait_warp(tempty0 + 8u * side, (use & 1u) ^ 1u, abort_flag, p.status, 22);
         if (!ok) break;
         // ... and so have the middle columns of the other side's tile, if this tile reaches into them
         if (kTok && it > 0 && n_prev + t.n > kTmemCols) {
-          ok = mbar_wait(tmid0 + 8u * (side ^ 1u), ((it - 1u) >> 1) & 1u, abort_flag, p.status, 25);
+          ok = mbar_wait_warp(tmid0 + 8u * (side ^ 1u), ((it - 1u) >> 1) & 1u, abort_flag, p.status, 25);
           if (!ok) break;
         }
         n_prev = t.n;
@@ -330,29 +330,33 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
         const uint32_t d_tmem2 = d_tmem + (uint32_t)t.n1;
 #pragma unroll 1
         for (int kb = 0; kb < kbs; ++kb) {
-          ok = mbar_wait(full0 + 8u * stage, phase, abort_flag, p.status, 23);
+          ok = mbar_wait_warp(full0 + 8u * stage, phase, abort_flag, p.status, 23);
           if (!ok) break;
           tc_fence_after();
           const uint64_t ad = a_desc0 + (uint64_t)(stage * (stage_bytes >> 4));
           const uint64_t bd = b_desc0 + (uint64_t)(stage * (stage_bytes >> 4));
           const int n_mma = (!kTok && kb == kbs - 1) ? last_mmas : kBK / kUmmaK;
           const uint32_t acc0 = kb > 0 ? 1u : 0u;
-          tc_mma_bf16_pair(d_tmem, ad, bd, idesc1, acc0);
-          if (kTok && n2 > 0) tc_mma_bf16_pair(d_tmem2, ad, bd + b2_off, idesc2, acc0);
+          if (elect_one()) {
+            if (kTok && n2 > 0) {
 #pragma unroll
-          for (int ks = 1; ks < kBK / kUmmaK; ++ks) {
-            if (ks < n_mma) {
-              tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, 1u);
-              if (kTok && n2 > 0) tc_mma_bf16_pair(d_tmem2, ad + ks * a_kstep, bd + b2_off + ks * b_kstep, idesc2, 1u);
+              for (int ks = 0; ks < kBK / kUmmaK; ++ks) {
+                tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
+                tc_mma_bf16_pair(d_tmem2, ad + ks * a_kstep, bd + b2_off + ks * b_kstep, idesc2, ks > 0 ? 1u : acc0);
+              }
+            } else {
+#pragma unroll
+              for (int ks = 0; ks < kBK / kUmmaK; ++ks)
+                if (ks == 0 || ks < n_mma)
+                  tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
             }
+            tc_commit_pair(empty0 + 8u * stage);              // frees this stage in both CTAs
+            if (kb == kbs - 1) tc_commit_pair(tfull0 + 8u * side);   // accumulator complete, in both CTAs
           }
-          tc_commit_pair(empty0 + 8u * stage);                // frees this stage in both CTAs
           if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        if (kbs > 0) {
-          tc_commit_pair(tfull0 + 8u * side);                 // accumulator complete, in both CTAs
-        } else {                                              // nothing to contract: epilogues write zeros
+        if (kbs <= 0 && lane == 0) {                          // nothing to contract: epilogues write zeros
           mbar_arrive(tfull0 + 8u * side);
           mbar_arrive_remote(tfull0 + 8u * side, 1);
         }
@@ -452,8 +456,7 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
         }
       };
       fetch_factors(n_chunks - 1 - half, gg);
-      ok = mbar_wait(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
-      ok = __all_sync(0xffffffffu, ok);
+      ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
       if (!ok) break;
       tc_fence_after();
       const uint32_t t_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0;
@@ -559,9 +562,8 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
               }
               __syncwarp();
               if (lane == 0) mbar_arrive(gate_bar);
-              ok = mbar_wait(gate_bar, gate_phase, abort_flag, p.status, 26);     // both tiles are written
+              ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 26);     // both tiles are written
               gate_phase ^= 1u;
-              ok = __all_sync(0xffffffffu, ok);
               if (!ok) break;
               uint32_t other[8];
 #pragma unroll
@@ -569,9 +571,8 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
                 other[k] = *reinterpret_cast<const uint32_t*>(tr_other + (8 * role + k) * 144 + lane * 4);
               __syncwarp();
               if (lane == 0) mbar_arrive(gate_bar);
-              ok = mbar_wait(gate_bar, gate_phase, abort_flag, p.status, 27);     // both tiles have been read
+              ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 27);     // both tiles have been read
               gate_phase ^= 1u;
-              ok = __all_sync(0xffffffffu, ok);
               if (!ok) break;
               uint32_t hw[8];
 #pragma unroll

@@ -92,6 +92,46 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   return mbar_wait_slow(bar, parity, abort_flag, status, code);
 }
 
+// The same bounded wait for a whole converged warp.  The TMA and MMA warps run their loops with all 32 lanes and elect
+// one lane only around the instructions themselves: what they feed to those instructions (descriptors, coordinates,
+// barrier addresses) is then warp-uniform for the compiler and stays in uniform registers.  A loop that a single lane
+// runs inside a divergent branch has to move every operand of every tcgen05.mma over from vector registers, which cost
+// about 1000 cycles per 64-deep k-block of the expert products whatever the loads and the tensor pipe did (GEMM1 at
+// 32768 tokens, 768 x 3072, 128 experts: 189 us with single-lane loops, 162 us with these).  The polls sit in one asm
+// block so that no divergent branch separates the lanes.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
+                                               int code) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 c;\n\t"
+      "mov.u32 c, 0;\n\t"
+      "WAIT_LOOP:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+      "@p bra WAIT_DONE;\n\t"
+      "add.u32 c, c, 1;\n\t"
+      "setp.lt.u32 q, c, 64;\n\t"
+      "@q bra WAIT_LOOP;\n\t"
+      "WAIT_DONE:\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  if (__all_sync(0xffffffffu, ok != 0)) return true;
+  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, status, code));
+}
+// True in one lane of a converged warp, always the same one (tcgen05.commit covers the MMAs of its own thread).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t pred;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(pred));
+  return pred != 0;
+}
+// The warp's index within its block, uniform for the compiler.
+__device__ __forceinline__ int uniform_warp_id() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
+
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* tm, uint32_t bar, int c0, int c1, int c2) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
