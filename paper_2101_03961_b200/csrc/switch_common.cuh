@@ -12,13 +12,12 @@
 namespace swmoe {
 
 constexpr int kMaxExperts = 256;        // router kernels keep ceil(E/32) <= 8 experts per lane
-constexpr int kRouterBlockTokens = 64;  // tokens per router-forward block (one partial P-sum row each)
 constexpr int kPlanBlockTokens = 256;   // tokens per dispatch-plan block (one histogram row each)
 constexpr int kTileM = 128;             // token rows per tensor-core tile; tails are zero-filled to this
 constexpr int kPairTileTokens = 320;    // widest token tile of the paired-CTA GEMM (tokens on the MMA's N side, two
                                         // column segments above 256): an expert within the capacity of the paper's
                                         // layers (capacity factor 1.25 at 256 tokens per expert) is one tile
-constexpr int kDwrChunkTokens = 512;    // tokens per split of the dW_r reduction
+constexpr int kDwrChunkTokens = 512;    // most tokens per split of the dW_r reduction (FP32-FMA router)
 constexpr int kMaxGroups = 64;          // routing groups per call
 
 struct Shape {
@@ -34,6 +33,7 @@ struct Shape {
   int router_tc;    // 1: router on the tensor cores (bf16 x, bf16 split of fp32 operands); 0: FP32 FMA
   int router_hist;  // 1: the router's forward kernel also writes the dispatch plan's block histograms
   int router_blocks, plan_blocks, max_mtiles, dwr_chunks;
+  int router_block_tokens, dwr_chunk_tokens;   // FP32-FMA router: tokens per forward block, per split of the dW_r sum
   int residual;     // 1: y = x + layer(x), dx = dy + d layer / dx (SWITCH_MOE_FLAG_RESIDUAL)
   int reroute;      // 1: overflowed tokens are offered to their second-choice expert (SWITCH_MOE_FLAG_REROUTE)
   int reroute_stages;   // stages after the first (0 without the flag): stage k + 1 offers the k-th next choice
@@ -130,6 +130,8 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
   s->router_hist = (s->router_tc && s->Epad64 <= 128 && !s->top2) ? 1 : 0;
   s->plan_blocks = (s->Tv + kPlanBlockTokens - 1) / kPlanBlockTokens;
   s->max_mtiles = cfg->E * ((s->C + kTileM - 1) / kTileM);
+  s->router_block_tokens = 2 * kTileM;
+  s->dwr_chunk_tokens = 0;
   if (s->router_tc) {
     // dW_r split so that tiles x splits fills the GPU
     s->router_blocks = (cfg->T + 255) / 256;                 // one partial P-sum row per block of 256 tokens
@@ -141,8 +143,17 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
     if (splits > k_blocks) splits = k_blocks;
     s->dwr_chunks = splits;
   } else {
-    s->router_blocks = (cfg->T + kRouterBlockTokens - 1) / kRouterBlockTokens;
-    s->dwr_chunks = (cfg->T + kDwrChunkTokens - 1) / kDwrChunkTokens;
+    // 64 tokens per forward block where that fills the chip, else 16: the kernel is bound by the latency of its k-chunks
+    s->router_block_tokens = cfg->T >= 64 * 148 ? 64 : 16;
+    s->router_blocks = (cfg->T + s->router_block_tokens - 1) / s->router_block_tokens;
+    // x^T dh: blocks of 64 rows of d x splits of the tokens, about four per SM, each with 64 to 512 tokens
+    const int k_blocks = (cfg->d_model + 63) / 64;
+    const int want = (4 * 148 + k_blocks - 1) / k_blocks;
+    int chunk = ((cfg->T + want - 1) / want + 31) / 32 * 32;
+    if (chunk < 64) chunk = 64;
+    if (chunk > kDwrChunkTokens) chunk = kDwrChunkTokens;
+    s->dwr_chunk_tokens = chunk;
+    s->dwr_chunks = (cfg->T + chunk - 1) / chunk;
   }
   return SWITCH_MOE_OK;
 }

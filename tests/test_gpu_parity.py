@@ -214,6 +214,16 @@ def test_tiny_fp32_layer_matches_oracle():
     _check_layer(TINY, sm.GEMM_DEFAULT, TOL_F32)
 
 
+@pytest.mark.parametrize("T,d,f,E", [
+    (33, 8, 8, 1),              # one small tile, one group of four outputs inside it
+    (700, 72, 136, 3),          # small tiles, ragged in every direction; x^T dh in splits of 64 tokens
+    (1111, 264, 520, 7),        # medium tiles with remainders
+    (2050, 136, 2056, 16),      # large tiles for d_ff outputs, medium ones for d_model outputs
+    (9600, 40, 72, 5)])         # 64 router tokens per block, the longest x^T dh splits
+def test_float32_layer_on_every_tile_size_matches_oracle(T, d, f, E):
+    _check_layer(si.SwitchConfig("f32_tiles", T, d, f, E, 1.25, dtype=si.DTYPE_F32), sm.GEMM_DEFAULT, TOL_F32)
+
+
 @pytest.mark.parametrize("cfg", [MID, RAGGED, MANY], ids=lambda c: c.name)
 def test_bf16_layer_on_fp32_fma_path_matches_oracle(cfg):
     _check_layer(cfg, sm.GEMM_SIMT, TOL_BF16)
