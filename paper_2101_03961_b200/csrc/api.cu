@@ -111,7 +111,7 @@ int switch_moe_router_fwd(const switch_moe_config* cfg, const void* x, const flo
   SWMOE_TRY(prepare(cfg, workspace, workspace_bytes, true, &c));
   if (x == nullptr || W_r == nullptr) return SWITCH_MOE_INVALID_ARGUMENT;
   if (!aligned16(x) || !aligned16(W_r)) return SWITCH_MOE_UNSUPPORTED_SHAPE;
-  return launch_router_fwd(c.s, c.p, x, W_r, router_bias, cfg->router_noise, workspace,
+  return launch_router_fwd(c.s, c.p, x, W_r, router_bias, cfg->router_noise, false, workspace,
                            static_cast<cudaStream_t>(stream));
 }
 
@@ -131,9 +131,8 @@ int switch_moe_fwd(const switch_moe_config* cfg, const void* x, const float* W_r
   if (!aligned16(x) || !aligned16(W_r) || !aligned16(W_in) || !aligned16(W_out) || !aligned16(y))
     return SWITCH_MOE_UNSUPPORTED_SHAPE;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(ws_ptr<char>(workspace, c.p.status), 0, 16 * 4, st) != cudaSuccess) return SWITCH_MOE_CUDA_ERROR;
   SWMOE_TRY(mark(cfg, 0, st));
-  SWMOE_TRY(launch_router_fwd(c.s, c.p, x, W_r, router_bias, cfg->router_noise, workspace, st));
+  SWMOE_TRY(launch_router_fwd(c.s, c.p, x, W_r, router_bias, cfg->router_noise, true, workspace, st));
   if (c.s.top2) SWMOE_TRY(launch_top2_choice(c.s, c.p, workspace, st));     // assignments T .. 2T - 1
   SWMOE_TRY(mark(cfg, 1, st));
   SWMOE_TRY(launch_dispatch_plan(c.s, c.p, nullptr, aux_loss, workspace, st));
@@ -323,10 +322,9 @@ int switch_moe_stage_launches(const switch_moe_config* cfg, int32_t* launches_ou
   SWMOE_TRY(resolve_shape(cfg, &s));
   int32_t* n = launches_out;
   for (int i = 0; i < SWITCH_MOE_STAGE_EVENTS - 1; ++i) n[i] = 0;
-  // forward.  Router: the kernel itself; on the tensor cores also the bf16 split of W_r and, with more than 128
-  // experts, the column sums of the probabilities (up to 128 experts the router kernel's epilogue leaves them, and
-  // the plan's block histograms too); input jitter adds the element-wise product, top-2 routing the second-choice kernel.
-  n[0] = (s.router_tc ? (s.Epad64 <= 128 ? 2 : 3) : 1) + (s.jitter ? 1 : 0) + (s.top2 ? 1 : 0);
+  // forward.  Router: the kernel itself and, on the tensor cores, the bf16 split of W_r; input jitter adds the
+  // element-wise product, top-2 routing the second-choice kernel.
+  n[0] = (s.router_tc ? 2 : 1) + (s.jitter ? 1 : 0) + (s.top2 ? 1 : 0);
   // plan: one fused kernel when the router left the histograms and there is one routing group; else (histogram,)
   // scan, assign; stage 2 of rerouting adds four
   n[1] = (s.router_hist ? (s.G == 1 ? 1 : 2) : 3) + 4 * s.reroute_stages;

@@ -248,7 +248,7 @@ plan_assign_kernel(const int* __restrict__ expert_index, const int* __restrict__
 }
 
 // The whole plan in one launch, for one routing group whose block histograms already exist (the tensor-core router's
-// forward kernel leaves hist[r][e] = tokens of the r-th block of 256 tokens routed to expert e).  Every block of 1024
+// forward kernel leaves hist[r][e] = tokens of its r-th block of `hist_tokens` tokens routed to expert e).  Every block of 1024
 // tokens adds up the histogram columns itself -- all rows for the totals (kept_i = min(count_i, C), Eq. 3), the rows
 // before its own tokens for its position base -- instead of waiting for a scan kernel: the table is small (64 KB at
 // 128 x 128) and stays in L2.  Then, as in plan_assign_kernel, pos_t = base + (tokens of earlier warps with the same
@@ -256,7 +256,7 @@ plan_assign_kernel(const int* __restrict__ expert_index, const int* __restrict__
 // counts, the P-sums, the auxiliary loss (Eq. 4-6) and the tile lists.
 constexpr int kFusedTokens = 1024;
 __global__ void __launch_bounds__(kFusedTokens)
-plan_fused_kernel(const int* __restrict__ expert_index, const int* __restrict__ hist, int hist_rows,
+plan_fused_kernel(const int* __restrict__ expert_index, const int* __restrict__ hist, int hist_rows, int hist_tokens,
                   const float* __restrict__ psum_partial, int router_blocks, int T, int E, int Ew, int C, float alpha,
                   int* __restrict__ slot, int* __restrict__ token_of_slot, int* __restrict__ count,
                   int* __restrict__ kept, float* __restrict__ psum, float* __restrict__ aux_loss,
@@ -273,7 +273,7 @@ plan_fused_kernel(const int* __restrict__ expert_index, const int* __restrict__ 
   const int n_token_blocks = (int)gridDim.x - 1;
   const bool summary = (int)blockIdx.x == n_token_blocks;
   const int Q = kFusedTokens / Ew, q = tid / Ew, e = tid % Ew;
-  const int row_end = summary ? hist_rows : min(hist_rows, (int)blockIdx.x * (kFusedTokens / kPlanBlockTokens));
+  const int row_end = summary ? hist_rows : min(hist_rows, (int)blockIdx.x * (kFusedTokens / hist_tokens));
   int pre = 0, tot = 0;
   if (e < E) {
     for (int r0 = q; r0 < hist_rows; r0 += 8 * Q) {
@@ -658,7 +658,7 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
     while (Ewf < s.E) Ewf *= 2;
     const int token_blocks = (s.T + kFusedTokens - 1) / kFusedTokens;
     launch_k(plan_fused_kernel, dim3(token_blocks + 1), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist),
-             s.plan_blocks, ws_ptr<float>(ws, p.psum_partial), s.router_blocks, s.T, s.E, Ewf, s.Cg, s.alpha,
+             s.router_blocks, s.router_block_tokens, ws_ptr<float>(ws, p.psum_partial), s.router_blocks, s.T, s.E, Ewf, s.Cg, s.alpha,
              ws_ptr<int>(ws, p.slot), ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.count),
              ws_ptr<int>(ws, p.kept), ws_ptr<float>(ws, p.psum), aux_loss, ws_ptr<int>(ws, p.tile_expert),
              ws_ptr<int>(ws, p.tile_row0), ws_ptr<int4>(ws, p.ntile), ws_ptr<int>(ws, p.count_g),

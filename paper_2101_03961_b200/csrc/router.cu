@@ -534,7 +534,7 @@ int router_bwd_t(const Shape& s, const Plan& p, const void* x, const float* W_r,
   }
 
 int launch_router_fwd(const Shape& s, const Plan& p, const void* x, const float* W_r, const float* bias,
-                      const float* noise, void* ws,
+                      const float* noise, bool clear_status, void* ws,
                       cudaStream_t st) {
   if (s.jitter) {
     if (s.jitter_u == nullptr || !aligned16(s.jitter_u)) return SWITCH_MOE_INVALID_ARGUMENT;
@@ -549,7 +549,10 @@ int launch_router_fwd(const Shape& s, const Plan& p, const void* x, const float*
                static_cast<const uint4*>(s.jitter_u), n_vec, xr);
     x = xr;
   }
-  if (s.router_tc && s.dtype == SWITCH_MOE_BF16) return launch_router_tc_fwd(s, p, x, W_r, bias, noise, ws, st);
+  if (s.router_tc && s.dtype == SWITCH_MOE_BF16)
+    return launch_router_tc_fwd(s, p, x, W_r, bias, noise, clear_status, ws, st);
+  if (clear_status && cudaMemsetAsync(ws_ptr<char>(ws, p.status), 0, kStatusWords * 4, st) != cudaSuccess)
+    return SWITCH_MOE_CUDA_ERROR;
   SWMOE_DISPATCH_NE(router_fwd_t, s, p, x, W_r, bias, noise, ws, st)
 }
 

@@ -19,6 +19,7 @@ constexpr int kPairTileTokens = 320;    // widest token tile of the paired-CTA G
                                         // layers (capacity factor 1.25 at 256 tokens per expert) is one tile
 constexpr int kDwrChunkTokens = 512;    // most tokens per split of the dW_r reduction (FP32-FMA router)
 constexpr int kMaxGroups = 64;          // routing groups per call
+constexpr int kStatusWords = 16;        // status words at the start of the workspace
 
 struct Shape {
   int T, d, f, E;
@@ -33,7 +34,8 @@ struct Shape {
   int router_tc;    // 1: router on the tensor cores (bf16 x, bf16 split of fp32 operands); 0: FP32 FMA
   int router_hist;  // 1: the router's forward kernel also writes the dispatch plan's block histograms
   int router_blocks, plan_blocks, max_mtiles, dwr_chunks;
-  int router_block_tokens, dwr_chunk_tokens;   // FP32-FMA router: tokens per forward block, per split of the dW_r sum
+  int router_block_tokens;   // tokens per block of the router's forward kernel: one row of P-sums (tensor cores: and histogram)
+  int dwr_chunk_tokens;      // FP32-FMA router: tokens per split of the dW_r sum
   int residual;     // 1: y = x + layer(x), dx = dy + d layer / dx (SWITCH_MOE_FLAG_RESIDUAL)
   int reroute;      // 1: overflowed tokens are offered to their second-choice expert (SWITCH_MOE_FLAG_REROUTE)
   int reroute_stages;   // stages after the first (0 without the flag): stage k + 1 offers the k-th next choice
@@ -127,14 +129,16 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
   s->Epad = 32 * ne_pow2;
   s->Epad64 = (cfg->E + 63) / 64 * 64;
   s->router_tc = s->gemm_path != 1 ? 1 : 0;
-  s->router_hist = (s->router_tc && s->Epad64 <= 128 && !s->top2) ? 1 : 0;
+  s->router_hist = (s->router_tc && !s->top2) ? 1 : 0;
   s->plan_blocks = (s->Tv + kPlanBlockTokens - 1) / kPlanBlockTokens;
   s->max_mtiles = cfg->E * ((s->C + kTileM - 1) / kTileM);
-  s->router_block_tokens = 2 * kTileM;
   s->dwr_chunk_tokens = 0;
   if (s->router_tc) {
+    // One 128-token tile per block while there are SMs for all of them, then two tiles that share the staged W_r.
+    // (Several routing groups: the plan's kernels count in blocks of 256 tokens.)
+    s->router_block_tokens = G == 1 && cfg->T <= 148 * kTileM ? kTileM : 2 * kTileM;
+    s->router_blocks = (cfg->T + s->router_block_tokens - 1) / s->router_block_tokens;
     // dW_r split so that tiles x splits fills the GPU
-    s->router_blocks = (cfg->T + 255) / 256;                 // one partial P-sum row per block of 256 tokens
     const int m_tiles = (cfg->d_model + kTileM - 1) / kTileM;
     const int k_blocks = (cfg->T + 63) / 64;
     int splits = 144 / m_tiles;
@@ -173,7 +177,7 @@ inline void make_plan(const Shape& s, Plan* p) {
   p->group_base = take((size_t)s.G * E * 4);               // per group: kept tokens of expert i in earlier groups
   p->psum = take(E * 4);
   p->psum_partial = take((size_t)s.router_blocks * E * 4);
-  p->hist = take((size_t)s.plan_blocks * E * 4);
+  p->hist = take((size_t)(s.plan_blocks > s.router_blocks ? s.plan_blocks : s.router_blocks) * E * 4);
   p->hist_base = take((size_t)s.plan_blocks * E * 4);
   p->tile_expert = take(((size_t)s.max_mtiles + 4) * 4);   // [0] = number of token tiles, then one entry per tile
   p->tile_row0 = take(((size_t)s.max_mtiles + 4) * 4);
@@ -245,7 +249,7 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 // ---- kernels' host launchers (each returns a switch_moe_status) ----------------------------------------
 int launch_router_fwd(const Shape& s, const Plan& p, const void* x, const float* W_r, const float* bias,
-                      const float* noise, void* ws, cudaStream_t st);
+                      const float* noise, bool clear_status, void* ws, cudaStream_t st);
 int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, float* aux_loss, void* ws,
                          cudaStream_t st);
 int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void* ws, cudaStream_t st);
@@ -261,7 +265,7 @@ int launch_router_bwd(const Shape& s, const Plan& p, const void* x, const float*
 
 // Tensor-core router (bf16 x): forward (logits, softmax, top-1, gate, P-sum partials) and the two backward products.
 int launch_router_tc_fwd(const Shape& s, const Plan& p, const void* x, const float* W_r, const float* bias,
-                         const float* noise, void* ws, cudaStream_t st);
+                         const float* noise, bool clear_status, void* ws, cudaStream_t st);
 int launch_router_tc_bwd(const Shape& s, const Plan& p, const void* x, const float* W_r, void* ws, void* dx,
                          bool accumulate_dx, cudaStream_t st);
 

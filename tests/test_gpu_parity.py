@@ -54,6 +54,27 @@ def test_router_forward_matches_oracle(cfg):
     np.testing.assert_allclose(gpu_gate, p[np.arange(cfg.T), gpu_e], rtol=TOL_ROUTER, atol=1e-7)
 
 
+@pytest.mark.parametrize("T,d,E,bias,noise", [
+    (1, 64, 1, 0.0, 0.0), (129, 128, 31, 0.5, 0.0), (300, 192, 130, 0.0, 0.3), (1000, 64, 192, 0.3, 0.2),
+    (148 * 128, 64, 65, 0.0, 0.0),              # the last size with one 128-token tile per block
+    (148 * 128 + 1, 64, 200, 0.3, 0.0),         # the first with two; 256 accumulator columns per tile, one set
+    (148 * 256 + 77, 64, 256, 0.0, 0.0), (148 * 256 + 300, 64, 96, 0.0, 0.1)])   # more blocks than SMs
+def test_router_forward_and_its_plan_at_the_edges_of_its_blocks(T, d, E, bias, noise):
+    cfg = si.SwitchConfig("router_edges", T, d, 64, E, max(1.25, 1.01 * E / T), bias_std=bias)
+    data = si.gen_layer(cfg, seed=6)
+    if noise:
+        data["router_noise"] = si.gen_router_noise(cfg, noise, 6)
+    g = GpuLayer(cfg, data)
+    g.fwd()
+    fwd = oracle_following(cfg, data, g.expert_index(), experts=[])
+    assert rel_err(to_np(g.view(sm.WS_PROBS)).reshape(T, E), fwd["p"]) <= TOL_ROUTER
+    np.testing.assert_array_equal(g.view(sm.WS_SLOT).cpu().numpy(), fwd["slot"])
+    np.testing.assert_array_equal(g.view(sm.WS_COUNT).cpu().numpy(), fwd["count"])
+    np.testing.assert_array_equal(g.view(sm.WS_TOKEN_OF_SLOT).cpu().numpy(), fwd["token_of_slot"])
+    np.testing.assert_allclose(to_np(g.view(sm.WS_PSUM)), fwd["p"].sum(0), rtol=TOL_ROUTER)
+    assert abs(float(g.aux.item()) - fwd["aux"]) <= TOL_ROUTER * abs(fwd["aux"])
+
+
 def test_router_ties_go_to_lowest_expert():
     cfg = si.SwitchConfig("ties", 256, 64, 64, 16, 1.0)
     data = si.gen_layer(cfg, seed=1)
