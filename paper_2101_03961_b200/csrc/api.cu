@@ -325,9 +325,9 @@ int switch_moe_stage_launches(const switch_moe_config* cfg, int32_t* launches_ou
   // forward.  Router: the kernel itself and, on the tensor cores, the bf16 split of W_r; input jitter adds the
   // element-wise product, top-2 routing the second-choice kernel.
   n[0] = (s.router_tc ? 2 : 1) + (s.jitter ? 1 : 0) + (s.top2 ? 1 : 0);
-  // plan: one fused kernel when the router left the histograms and there is one routing group; else (histogram,)
-  // scan, assign; stage 2 of rerouting adds four
-  n[1] = (s.router_hist ? (s.G == 1 ? 1 : 2) : 3) + 4 * s.reroute_stages;
+  // plan: slots and, beside them, the summary when the router left the histograms and there is one routing group; else
+  // (histogram,) scan, assign; a stage of rerouting adds four
+  n[1] = (s.router_hist ? 2 : 3) + 4 * s.reroute_stages;
   n[2] = 1;                                           // gather
   const int slow = s.gemm_path != 0 ? 1 : 0;   // gating and dropout are element-wise kernels off the CTA-pair path
   n[3] = 1 + (s.geglu ? slow : 0) + (s.dropout ? slow : 0);   // GEMM1 (+ GEGLU gating kernel, + expert dropout kernel)
@@ -338,7 +338,8 @@ int switch_moe_stage_launches(const switch_moe_config* cfg, int32_t* launches_ou
   n[8] = 1;
   n[9] = 1;
   n[10] = (s.gemm_path == 0 ? 0 : 1) + (s.top2 ? 1 : 0);
-  n[11] = 4;                                          // logit gradients, x^T dh partials, their reduction, dx += dh W_r^T
+  // logit gradients, x^T dh partials, dx += dh W_r^T (on the tensor cores one kernel with the partials), their reduction
+  n[11] = s.router_tc ? 3 : 4;
   return SWITCH_MOE_OK;
 }
 

@@ -26,58 +26,62 @@ plan_hist_kernel(const int* __restrict__ expert_index, int T, int E, int* __rest
   for (int e = threadIdx.x; e < E; e += blockDim.x) hist[(size_t)blockIdx.x * E + e] = h[e];
 }
 
-// Tile lists, shared by both scan kernels: 128-row token tiles (single-CTA GEMM) and, for the paired-CTA GEMM, each
-// expert's kept rows cut into the fewest pieces of at most kPairTileTokens rows, equal up to rounding each piece to a
-// multiple of 16 (the MMA's N granularity).  Thread 0 adds the loss terms and scans the per-expert tile counts; the first E
-// threads write their expert's entries.  `term` and `kept_s` are shared-memory arrays filled before the call.
+// Tile lists, shared by the scan kernels: 128-row token tiles (single-CTA GEMM; skipped where `tile_expert` is null) and,
+// for the paired-CTA GEMM, each expert's kept rows cut into the fewest pieces of at most kPairTileTokens rows, equal up to
+// rounding each piece to a multiple of 16 (the MMA's N granularity).  Thread e < 256 owns expert e: the tiles of earlier
+// experts and the loss terms come from warp scans and the eight warps' totals, in a fixed order (the loss is the same
+// number on every run).  `term` and `kept_s` are shared-memory arrays filled before the call, at the cost of one barrier;
+// log2 steps over the whole block cost sixteen, in a kernel of one block that others wait for.
 __device__ __forceinline__ void write_tile_lists(const float* term, const int* kept_s, int E, float loss_scale,
                                                  float* __restrict__ aux_loss, int* __restrict__ tile_expert,
                                                  int* __restrict__ tile_row0, int4* __restrict__ ntile) {
-  // Everything here is a sum or a running sum over the experts, done by the first kMaxExperts threads in log2 steps
-  // (a fixed tree, so the loss is the same number on every run): the loss terms, and the number of tiles before
-  // each expert in the two lists.
-  __shared__ int start128[kMaxExperts], startn[kMaxExperts];
-  __shared__ float lsum[kMaxExperts];
-  const int e = threadIdx.x;
+  constexpr int kWarps = kMaxExperts / 32;
+  __shared__ int tot128[kWarps], totn[kWarps];
+  __shared__ float totl[kWarps];
+  const int e = threadIdx.x, lane = e & 31, w = e >> 5;
   __syncthreads();
-  int n128 = 0, npair = 0;
+  int k = 0, n128 = 0, npair = 0, start128 = 0, startn = 0;
   if (e < kMaxExperts) {
-    const int k = e < E ? kept_s[e] : 0;
+    k = e < E ? kept_s[e] : 0;
     n128 = (k + kTileM - 1) / kTileM;
     npair = (k + kPairTileTokens - 1) / kPairTileTokens;
-    start128[e] = n128; startn[e] = npair;
-    lsum[e] = e < E ? term[e] : 0.f;
+    float l = e < E ? term[e] : 0.f;
+    int a = n128, b = npair;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {                   // inclusive scans within the warp
+      const int ua = __shfl_up_sync(0xffffffffu, a, off), ub = __shfl_up_sync(0xffffffffu, b, off);
+      if (lane >= off) { a += ua; b += ub; }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+    if (lane == 31) { tot128[w] = a; totn[w] = b; totl[w] = l; }
+    start128 = a - n128;
+    startn = b - npair;
   }
   __syncthreads();
-  for (int off = 1; off < kMaxExperts; off <<= 1) {            // inclusive scans (counts), pairwise tree (loss)
-    int a = 0, b = 0;
-    float c = 0.f;
-    const bool scan = e < kMaxExperts && e >= off;
-    const bool tree = e < kMaxExperts && (e & (2 * off - 1)) == 0 && e + off < kMaxExperts;
-    if (scan) { a = start128[e - off]; b = startn[e - off]; }
-    if (tree) c = lsum[e + off];
-    __syncthreads();
-    if (scan) { start128[e] += a; startn[e] += b; }
-    if (tree) lsum[e] += c;
-    __syncthreads();
+  if (e >= kMaxExperts) return;
+  int n_all = 0, m_all = 0;
+  float loss = 0.f;
+#pragma unroll
+  for (int i = 0; i < kWarps; ++i) {
+    if (i < w) { start128 += tot128[i]; startn += totn[i]; }
+    n_all += tot128[i];
+    m_all += totn[i];
+    loss += totl[i];
   }
   if (e == 0) {
-    if (aux_loss != nullptr) *aux_loss = loss_scale * lsum[0];                        // Eq. 4
-    const int n = start128[kMaxExperts - 1], m = startn[kMaxExperts - 1];
-    tile_expert[0] = n;
-    tile_row0[0] = n;
-    ntile[0] = make_int4(m, 0, 0, 0);
+    if (aux_loss != nullptr) *aux_loss = loss_scale * loss;                           // Eq. 4
+    ntile[0] = make_int4(m_all, 0, 0, 0);
+    if (tile_expert != nullptr) { tile_expert[0] = n_all; tile_row0[0] = n_all; }
   }
-  if (e < E) {
-    const int k = kept_s[e];
-    int n = start128[e] - n128;                                // tiles of earlier experts
-    for (int r = 0; r < k; r += kTileM, ++n) { tile_expert[1 + n] = e; tile_row0[1 + n] = r; }
-    if (k > 0) {
-      const int pieces = npair;
-      const int rows = ((k + pieces - 1) / pieces + 15) / 16 * 16;
-      int m = startn[e] - npair;
-      for (int r = 0; r < k; r += rows, ++m) ntile[1 + m] = make_int4(e, r, min(rows, (k - r + 15) / 16 * 16), 0);
+  if (k > 0) {
+    if (tile_expert != nullptr) {
+      int n = start128;
+      for (int r = 0; r < k; r += kTileM, ++n) { tile_expert[1 + n] = e; tile_row0[1 + n] = r; }
     }
+    const int rows = ((k + npair - 1) / npair + 15) / 16 * 16;
+    int m = startn;
+    for (int r = 0; r < k; r += rows, ++m) ntile[1 + m] = make_int4(e, r, min(rows, (k - r + 15) / 16 * 16), 0);
   }
 }
 
@@ -247,86 +251,64 @@ plan_assign_kernel(const int* __restrict__ expert_index, const int* __restrict__
   }
 }
 
-// The whole plan in one launch, for one routing group whose block histograms already exist (the tensor-core router's
-// forward kernel leaves hist[r][e] = tokens of its r-th block of `hist_tokens` tokens routed to expert e).  Every block of 1024
-// tokens adds up the histogram columns itself -- all rows for the totals (kept_i = min(count_i, C), Eq. 3), the rows
-// before its own tokens for its position base -- instead of waiting for a scan kernel: the table is small (64 KB at
-// 128 x 128) and stays in L2.  Then, as in plan_assign_kernel, pos_t = base + (tokens of earlier warps with the same
-// expert) + (earlier lanes with it), in token order, with no atomics deciding a position.  One extra block writes the
-// counts, the P-sums, the auxiliary loss (Eq. 4-6) and the tile lists.
+// The plan of one routing group whose block histograms already exist (the tensor-core router's forward kernel leaves
+// hist[r][e] = tokens of its r-th block of `hist_tokens` tokens routed to expert e), in two kernels that both start from
+// that table.
+//
+// Slots: every block of 1024 tokens adds up the histogram columns itself -- all rows for the totals (kept_i =
+// min(count_i, C), Eq. 3), the rows before its own tokens for its position base -- instead of waiting for a scan kernel:
+// the table is small (64 KB at 128 x 128) and stays in L2.  Then, as in plan_assign_kernel, pos_t = base + (tokens of
+// earlier warps with the same expert) + (earlier lanes with it), in token order, with no atomics deciding a position.
+//
+// Summary (one block): counts, P-sums, the auxiliary loss (Eq. 4-6) and the tile lists.  It runs beside the slots kernel:
+// that kernel lets its successor start only once its own wait on the router is over, hence the summary may read what the
+// router wrote without waiting for anything else.  (As one more block of the slots kernel it did the same work in code and
+// registers that every block had to carry: 96 tokens, d 256, E 8, whole forward pass 29.1 us against 28.4.  Launched
+// after the gather instead, to run beside that, it was no faster and delayed GEMM1 where the gather is short.)
 constexpr int kFusedTokens = 1024;
+
+// Column sums of the histogram table by the whole block: tot over all rows, pre over rows below row_end, as partial sums
+// per thread (column e = tid % Ew, slice q = tid / Ew of the rows, every Q-th one).
+__device__ __forceinline__ void hist_column_sums(const int* __restrict__ hist, int hist_rows, int row_end, int E, int e,
+                                                 int q, int Q, int* pre_out, int* tot_out) {
+  int pre = 0, tot = 0;
+  if (e < E) {
+    for (int r0 = q; r0 < hist_rows; r0 += 16 * Q) {           // 16 rows in flight
+      int v[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = r0 + j * Q < hist_rows ? hist[(size_t)(r0 + j * Q) * E + e] : 0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) { tot += v[j]; if (r0 + j * Q < row_end) pre += v[j]; }
+    }
+  }
+  *pre_out = pre;
+  *tot_out = tot;
+}
+
 __global__ void __launch_bounds__(kFusedTokens)
-plan_fused_kernel(const int* __restrict__ expert_index, const int* __restrict__ hist, int hist_rows, int hist_tokens,
-                  const float* __restrict__ psum_partial, int router_blocks, int T, int E, int Ew, int C, float alpha,
-                  int* __restrict__ slot, int* __restrict__ token_of_slot, int* __restrict__ count,
-                  int* __restrict__ kept, float* __restrict__ psum, float* __restrict__ aux_loss,
-                  int* __restrict__ tile_expert, int* __restrict__ tile_row0, int4* __restrict__ ntile,
-                  int* __restrict__ count_g, int* __restrict__ group_base) {
-  pdl_launch_dependents();
+plan_slots_kernel(const int* __restrict__ expert_index, const int* __restrict__ hist, int hist_rows, int hist_tokens, int T,
+                  int E, int Ew, int C, int* __restrict__ slot, int* __restrict__ token_of_slot, int* __restrict__ kept) {
   pdl_wait();
-  __shared__ int part_pre[kFusedTokens], part_tot[kFusedTokens];    // [slice][column]; the extra block keeps floats here
+  pdl_launch_dependents();                                      // (in this order: see above)
+  __shared__ int part_pre[kFusedTokens], part_tot[kFusedTokens];    // [slice][column]
   __shared__ int base_s[kMaxExperts], kept_s[kMaxExperts];
-  __shared__ float term[kMaxExperts];
   constexpr int kWarps = kFusedTokens / 32;
   __shared__ int warp_cnt[kMaxExperts][kWarps];                // [expert][warp of the block]
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int n_token_blocks = (int)gridDim.x - 1;
-  const bool summary = (int)blockIdx.x == n_token_blocks;
-  const int Q = kFusedTokens / Ew, q = tid / Ew, e = tid % Ew;
-  const int row_end = summary ? hist_rows : min(hist_rows, (int)blockIdx.x * (kFusedTokens / hist_tokens));
-  int pre = 0, tot = 0;
-  if (e < E) {
-    for (int r0 = q; r0 < hist_rows; r0 += 8 * Q) {
-      int v[8];
-#pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = r0 + j * Q < hist_rows ? hist[(size_t)(r0 + j * Q) * E + e] : 0;
-#pragma unroll
-      for (int j = 0; j < 8; ++j) { tot += v[j]; if (r0 + j * Q < row_end) pre += v[j]; }
-    }
-  }
-  part_pre[tid] = pre;
-  part_tot[tid] = tot;
-  for (int i = tid; i < kWarps * kMaxExperts; i += kFusedTokens) (&warp_cnt[0][0])[i] = 0;
+  const int Q = kFusedTokens / Ew;
+  const int t = (int)blockIdx.x * kFusedTokens + tid;
+  int et = t < T ? expert_index[t] : -1;                      // negative: no expert (takes no slot)
+  hist_column_sums(hist, hist_rows, min(hist_rows, (int)blockIdx.x * (kFusedTokens / hist_tokens)), E, tid % Ew, tid / Ew, Q,
+                   &part_pre[tid], &part_tot[tid]);
+  for (int i = tid; i < kWarps * E; i += kFusedTokens) (&warp_cnt[0][0])[i] = 0;
   __syncthreads();
-  int total = 0;
   if (tid < E) {
-    int b = 0;
+    int b = 0, total = 0;
     for (int k = 0; k < Q; ++k) { b += part_pre[k * Ew + tid]; total += part_tot[k * Ew + tid]; }
     base_s[tid] = b;
     kept_s[tid] = min(total, C);
+    if (blockIdx.x == 0) kept[tid] = min(total, C);
   }
-  __syncthreads();
-  if (summary) {
-    // P-sums in a fixed order (slice by slice, rows ascending inside a slice), then the loss and the tile lists
-    float* part_ps = reinterpret_cast<float*>(part_pre);
-    float ps = 0.f;
-    if (e < E) {
-      for (int r0 = q; r0 < router_blocks; r0 += 16 * Q) {      // 16 rows in flight, added in row order
-        float v[16];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = r0 + j * Q < router_blocks ? psum_partial[(size_t)(r0 + j * Q) * E + e] : 0.f;
-#pragma unroll
-        for (int j = 0; j < 16; ++j) ps += v[j];
-      }
-    }
-    __syncthreads();
-    part_ps[tid] = ps;
-    __syncthreads();
-    if (tid < E) {
-      float sum = 0.f;
-      for (int k = 0; k < Q; ++k) sum += part_ps[k * Ew + tid];
-      count[tid] = total;                                                              // f counts the argmax (Eq. 5)
-      count_g[tid] = total;
-      group_base[tid] = 0;
-      kept[tid] = kept_s[tid];
-      psum[tid] = sum;
-      term[tid] = ((float)total / (float)T) * (sum / (float)T);                        // f_i . P_i  (Eq. 5, 6)
-    }
-    write_tile_lists(term, kept_s, E, alpha * (float)E, aux_loss, tile_expert, tile_row0, ntile);
-    return;
-  }
-  const int t = (int)blockIdx.x * kFusedTokens + tid;
-  int et = t < T ? expert_index[t] : -1;                      // negative: no expert (takes no slot)
   if (et >= E) et = -1;
   const unsigned same = __match_any_sync(0xffffffffu, et >= 0 ? et : -1 - lane);   // distinct dummies for those lanes
   const int rank = __popc(same & ((1u << lane) - 1u));
@@ -353,10 +335,55 @@ plan_fused_kernel(const int* __restrict__ expert_index, const int* __restrict__ 
   }
   // empty slots of every expert: -1 (disjoint from the kept slots written above)
   const int total_slots = E * C;
-  for (int sidx = (int)blockIdx.x * kFusedTokens + tid; sidx < total_slots; sidx += n_token_blocks * kFusedTokens) {
+  for (int sidx = (int)blockIdx.x * kFusedTokens + tid; sidx < total_slots; sidx += (int)gridDim.x * kFusedTokens) {
     const int ex = sidx / C, pos = sidx - ex * C;
     if (pos >= kept_s[ex]) token_of_slot[sidx] = -1;
   }
+}
+
+// Launched after plan_slots_kernel.  Reads only what the router wrote, which is complete when it starts; its own wait comes
+// last, so that the next kernel's wait covers everything before this one.
+__global__ void __launch_bounds__(kFusedTokens)
+plan_summary_kernel(const int* __restrict__ hist, int hist_rows, const float* __restrict__ psum_partial, int T, int E, int Ew,
+                    int C, float alpha, int* __restrict__ count, float* __restrict__ psum, float* __restrict__ aux_loss,
+                    int* __restrict__ tile_expert, int* __restrict__ tile_row0, int4* __restrict__ ntile,
+                    int* __restrict__ count_g, int* __restrict__ group_base) {
+  pdl_launch_dependents();
+  __shared__ int part_tot[kFusedTokens];
+  __shared__ float part_ps[kFusedTokens], term[kMaxExperts];
+  __shared__ int kept_s[kMaxExperts];
+  const int tid = threadIdx.x, Q = kFusedTokens / Ew, q = tid / Ew, e = tid % Ew;
+  // column sums of the histograms and of p, the latter in a fixed order (slice by slice, rows ascending inside a slice)
+  int tot = 0;
+  float ps = 0.f;
+  if (e < E) {
+    for (int r0 = q; r0 < hist_rows; r0 += 16 * Q) {            // 16 rows of each table in flight, added in row order
+      int v[16];
+      float f[16];
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = r0 + j * Q < hist_rows ? hist[(size_t)(r0 + j * Q) * E + e] : 0;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) f[j] = r0 + j * Q < hist_rows ? psum_partial[(size_t)(r0 + j * Q) * E + e] : 0.f;
+#pragma unroll
+      for (int j = 0; j < 16; ++j) { tot += v[j]; ps += f[j]; }
+    }
+  }
+  part_tot[tid] = tot;
+  part_ps[tid] = ps;
+  __syncthreads();
+  if (tid < E) {
+    int total = 0;
+    float sum = 0.f;
+    for (int k = 0; k < Q; ++k) { total += part_tot[k * Ew + tid]; sum += part_ps[k * Ew + tid]; }
+    count[tid] = total;                                                                // f counts the argmax (Eq. 5)
+    count_g[tid] = total;
+    group_base[tid] = 0;
+    kept_s[tid] = min(total, C);
+    psum[tid] = sum;
+    term[tid] = ((float)total / (float)T) * (sum / (float)T);                          // f_i . P_i  (Eq. 5, 6)
+  }
+  write_tile_lists(term, kept_s, E, alpha * (float)E, aux_loss, tile_expert, tile_row0, ntile);
+  pdl_wait();
 }
 
 // ---- further stages of No-Token-Left-Behind routing (Appendix B) ---------------------------------------------
@@ -537,39 +564,66 @@ top2_sum_kernel(const uint4* __restrict__ rows, const uint4* __restrict__ skip, 
   }
 }
 
-// Forward gather.  Part 1 (blockIdx.x < slot_blocks): one warp per slot row; kept slots copy the token's row
-// with 128-bit loads and stores, slots in [kept_i, roundup(kept_i, kTileM)) are zero-filled so that tensor-core
-// tiles never read stale rows.  Part 2: one warp per token; dropped tokens get a zero output row (their
-// representation reaches the next layer only through the residual connection, Section 2.2), or, when the layer
-// itself adds the skip path (`residual`), their input row.
-__global__ void __launch_bounds__(256)
+// ---- gathers --------------------------------------------------------------------------------------------------
+// Bound by HBM; a warp per slot row at a time, and no more blocks than are resident at once: a grid of one row per warp
+// spends its time on launching blocks.  The forward gather takes four rows at a time, their loads in flight together
+// (65536 tokens, d_model 256, 128 experts: 27 -> 18 us; 32768 x 768: 24 -> 21); the backward gather, whose rows end in a
+// reduction, is faster with twice the warps and one row each (32768 x 768: 31 us; two rows on half the warps 35).
+constexpr int kGatherBlocksPerSm = 4, kGatherDyBlocksPerSm = 8;   // x 256 threads
+
+// Slot row s of the buffers: the token it holds (>= 0), -1: a row to zero-fill (up to a multiple of `pad` rows past the
+// expert's last token, so that tensor-core tiles never read stale rows), -2: leave alone.
+__device__ __forceinline__ int slot_source(int s, int slots, int C, int pad, const int* __restrict__ token_of_slot,
+                                           const int* __restrict__ kept) {
+  if (s >= slots) return -2;
+  const int ex = s / C, pos = s - ex * C, k = kept[ex];
+  if (pos < k) return token_of_slot[s];
+  return pos < (k + pad - 1) / pad * pad ? -1 : -2;
+}
+
+// Rows of dropped tokens: dst[t] = src[t], or zero where src is null.  A warp looks at 32 tokens.
+__device__ __forceinline__ void dropped_rows(const int* __restrict__ slot, int T, int row_vec, const uint4* __restrict__ src,
+                                             uint4* __restrict__ dst, int gw, int n_warps, int lane) {
+  for (int t0 = gw * 32; t0 < T; t0 += n_warps * 32) {
+    unsigned dropped = __ballot_sync(0xffffffffu, t0 + lane < T && slot[t0 + lane] < 0);
+    while (dropped != 0) {
+      const size_t at = (size_t)(t0 + __ffs(dropped) - 1) * row_vec;
+      dropped &= dropped - 1;
+      for (int v = lane; v < row_vec; v += 32) dst[at + v] = src != nullptr ? src[at + v] : make_uint4(0, 0, 0, 0);
+    }
+  }
+}
+
+// Forward: kept slots copy the token's row.  Dropped tokens get a zero output row (their representation reaches the next
+// layer only through the residual connection, Section 2.2), or, when the layer itself adds the skip path (`residual`),
+// their input row; `y` is null for top-2 routing, whose outputs are formed per assignment.  Top-2: slot s may hold
+// assignment T + t (the second choice of token t): its source row is still x[t].
+__global__ void __launch_bounds__(256, kGatherBlocksPerSm)
 gather_x_kernel(const uint4* __restrict__ x, const int* __restrict__ token_of_slot, const int* __restrict__ kept,
-                const int* __restrict__ slot, int T, int E, int C, int row_vec, int slot_blocks, int residual,
+                const int* __restrict__ slot, int T, int slots, int C, int row_vec, int pad, int residual,
                 uint4* __restrict__ xd, uint4* __restrict__ y) {
-  // top-2 routing: slot s may hold assignment T + t (the second choice of token t): its source row is still x[t]
   pdl_launch_dependents();
   pdl_wait();
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  if ((int)blockIdx.x < slot_blocks) {
-    const int s = blockIdx.x * 8 + wib;
-    if (s >= E * C) return;
-    const int ex = s / C, pos = s - ex * C, k = kept[ex];
-    uint4* dst = xd + (size_t)s * row_vec;
-    if (pos < k) {
-      int tok = token_of_slot[s];
-      if (tok >= T) tok -= T;
-      const uint4* src = x + (size_t)tok * row_vec;
-      for (int v = lane; v < row_vec; v += 32) dst[v] = src[v];
-    } else if (pos < (k + kTileM - 1) / kTileM * kTileM) {
-      for (int v = lane; v < row_vec; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+  constexpr int kRows = 4;
+  const int lane = threadIdx.x & 31, gw = blockIdx.x * 8 + (threadIdx.x >> 5), n_warps = gridDim.x * 8;
+  for (int s0 = gw * kRows; s0 < slots; s0 += n_warps * kRows) {
+    const uint4* src[kRows];
+    int tok[kRows];
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) tok[j] = slot_source(s0 + j, slots, C, pad, token_of_slot, kept);
+#pragma unroll
+    for (int j = 0; j < kRows; ++j) src[j] = x + (size_t)max(tok[j] >= T ? tok[j] - T : tok[j], 0) * row_vec;
+    uint4* dst = xd + (size_t)s0 * row_vec;
+    for (int v = lane; v < row_vec; v += 32) {
+      uint4 r[kRows];
+#pragma unroll
+      for (int j = 0; j < kRows; ++j) r[j] = tok[j] >= 0 ? src[j][v] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+      for (int j = 0; j < kRows; ++j)
+        if (tok[j] != -2) dst[(size_t)j * row_vec + v] = r[j];
     }
-  } else {
-    const int t = (blockIdx.x - slot_blocks) * 8 + wib;
-    if (t >= T || slot[t] >= 0) return;
-    uint4* dst = y + (size_t)t * row_vec;
-    const uint4* src = x + (size_t)t * row_vec;
-    for (int v = lane; v < row_vec; v += 32) dst[v] = residual ? src[v] : make_uint4(0, 0, 0, 0);
   }
+  if (y != nullptr) dropped_rows(slot, T, row_vec, residual ? x : nullptr, y, gw, n_warps, lane);
 }
 
 __device__ __forceinline__ float dot_scale8(const uint4& a, const uint4& b, float g, uint4* out) {
@@ -596,36 +650,29 @@ __device__ __forceinline__ float dot_scale4(const uint4& a, const uint4& b, floa
   return s;
 }
 
-// Backward gather: dY_d[slot] = g . dy[token] (derivative of Eq. 2 w.r.t. the expert output) and
-// dgate[token] = <dy, o> with o = y / g (derivative w.r.t. the gate).  Tail rows are zero-filled as in forward.
-// With the skip path inside the layer, blocks past `slot_blocks` (one warp per token) start the dropped tokens'
-// dx rows at dy: the router's gradient is added to them later, and no expert ever writes them.
+// Backward: dY_d[slot] = g . dy[token] (derivative of Eq. 2 w.r.t. the expert output) and dgate[token] = <dy, o> with
+// o = y / g (derivative w.r.t. the gate).  With the skip path inside the layer (`dx` not null) the dropped tokens' dx rows
+// start at dy: the router's gradient is added to them later, and no expert ever writes them.
 template <bool kBf16>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, kGatherDyBlocksPerSm)
 gather_dy_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ y, const float* __restrict__ gate,
                  const int* __restrict__ token_of_slot, const int* __restrict__ kept, const int* __restrict__ slot,
-                 int T, int E, int C, int row_vec, int slot_blocks, uint4* __restrict__ dyd,
+                 int T, int slots, int C, int row_vec, int pad, uint4* __restrict__ dyd,
                  float* __restrict__ dgate, uint4* __restrict__ dx) {
   pdl_launch_dependents();
   pdl_wait();
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  if ((int)blockIdx.x >= slot_blocks) {
-    const int t = (blockIdx.x - slot_blocks) * 8 + wib;
-    if (t >= T || slot[t] >= 0) return;
-    const uint4* src = dy + (size_t)t * row_vec;
-    uint4* dst = dx + (size_t)t * row_vec;
-    for (int v = lane; v < row_vec; v += 32) dst[v] = src[v];
-    return;
-  }
-  const int s = blockIdx.x * 8 + wib;
-  if (s >= E * C) return;
-  const int ex = s / C, pos = s - ex * C, k = kept[ex];
-  uint4* dst = dyd + (size_t)s * row_vec;
-  if (pos < k) {
-    const int t = token_of_slot[s];                           // top-2 routing: assignment t or T + t of token t mod T
-    const float g = gate[t];
-    const uint4* src = dy + (size_t)(t >= T ? t - T : t) * row_vec;
-    const uint4* ysrc = y + (size_t)t * row_vec;
+  const int lane = threadIdx.x & 31, gw = blockIdx.x * 8 + (threadIdx.x >> 5), n_warps = gridDim.x * 8;
+  for (int s = gw; s < slots; s += n_warps) {
+    const int tok = slot_source(s, slots, C, pad, token_of_slot, kept);
+    if (tok == -2) continue;
+    uint4* dst = dyd + (size_t)s * row_vec;
+    if (tok < 0) {
+      for (int v = lane; v < row_vec; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+      continue;
+    }
+    const float g = gate[tok];                                 // top-2 routing: assignment t or T + t of token t mod T
+    const uint4* src = dy + (size_t)(tok >= T ? tok - T : tok) * row_vec;
+    const uint4* ysrc = y + (size_t)tok * row_vec;
     float dot = 0.f;
     for (int v = lane; v < row_vec; v += 32) {
       uint4 o;
@@ -634,15 +681,27 @@ gather_dy_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ y, cons
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    if (lane == 0) dgate[t] = dot / g;
-  } else if (pos < (k + kTileM - 1) / kTileM * kTileM) {
-    for (int v = lane; v < row_vec; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+    if (lane == 0) dgate[tok] = dot / g;
   }
+  if (dx != nullptr) dropped_rows(slot, T, row_vec, dy, dx, gw, n_warps, lane);
 }
 
 }  // namespace
 
 int launch_reroute(const Shape& s, const Plan& p, void* ws, cudaStream_t st);
+
+namespace {
+// Columns of a plan block's [slice][expert] layout: E rounded up to a power of two, at least 32.
+int column_width(int E) {
+  int w = 32;
+  while (w < E) w *= 2;
+  return w;
+}
+// The 128-row tile list, for the path that reads it.
+int* list128(const Shape& s, const Plan& p, void* ws) {
+  return s.gemm_path == SWITCH_MOE_GEMM_TC_1CTA ? ws_ptr<int>(ws, p.tile_expert) : nullptr;
+}
+}  // namespace
 
 int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, float* aux_loss, void* ws,
                          cudaStream_t st) {
@@ -654,21 +713,19 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
   // the tensor-core router's forward kernel leaves the histograms of its own expert choices in the workspace
   const bool have_hist = expert_index == nullptr && s.router_hist;
   if (have_hist && s.G == 1) {
-    int Ewf = 32;
-    while (Ewf < s.E) Ewf *= 2;
     const int token_blocks = (s.T + kFusedTokens - 1) / kFusedTokens;
-    launch_k(plan_fused_kernel, dim3(token_blocks + 1), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist),
-             s.router_blocks, s.router_block_tokens, ws_ptr<float>(ws, p.psum_partial), s.router_blocks, s.T, s.E, Ewf, s.Cg, s.alpha,
-             ws_ptr<int>(ws, p.slot), ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.count),
-             ws_ptr<int>(ws, p.kept), ws_ptr<float>(ws, p.psum), aux_loss, ws_ptr<int>(ws, p.tile_expert),
-             ws_ptr<int>(ws, p.tile_row0), ws_ptr<int4>(ws, p.ntile), ws_ptr<int>(ws, p.count_g),
-             ws_ptr<int>(ws, p.group_base));
+    launch_k(plan_slots_kernel, dim3(token_blocks), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist), s.router_blocks,
+             s.router_block_tokens, s.T, s.E, column_width(s.E), s.Cg, ws_ptr<int>(ws, p.slot),
+             ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.kept));
+    launch_k(plan_summary_kernel, dim3(1), dim3(kFusedTokens), 0, st, ws_ptr<int>(ws, p.hist), s.router_blocks,
+             ws_ptr<float>(ws, p.psum_partial), s.T, s.E, column_width(s.E), s.Cg, s.alpha, ws_ptr<int>(ws, p.count),
+             ws_ptr<float>(ws, p.psum), aux_loss, list128(s, p, ws), ws_ptr<int>(ws, p.tile_row0),
+             ws_ptr<int4>(ws, p.ntile), ws_ptr<int>(ws, p.count_g), ws_ptr<int>(ws, p.group_base));
     return launch_reroute(s, p, ws, st);
   }
   if (!have_hist)
     launch_k(plan_hist_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, ei, s.Tv, s.E, ws_ptr<int>(ws, p.hist));
-  int Ew = 32;
-  while (Ew < s.E) Ew *= 2;
+  const int Ew = column_width(s.E);
   const int blocks_per_group = s.plan_blocks / s.G;
   int* count_g = ws_ptr<int>(ws, p.count_g);
   int* group_base = ws_ptr<int>(ws, p.group_base);
@@ -677,14 +734,14 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
              s.top2 ? s.plan_blocks / 2 : s.plan_blocks, ws_ptr<float>(ws, p.psum_partial), s.router_blocks, s.T, s.E, Ew,
              s.Cg, s.alpha,
              ws_ptr<int>(ws, p.hist_base), ws_ptr<int>(ws, p.count), ws_ptr<int>(ws, p.kept),
-             ws_ptr<float>(ws, p.psum), aux_loss, ws_ptr<int>(ws, p.tile_expert), ws_ptr<int>(ws, p.tile_row0),
+             ws_ptr<float>(ws, p.psum), aux_loss, list128(s, p, ws), ws_ptr<int>(ws, p.tile_row0),
              ws_ptr<int4>(ws, p.ntile), count_g, group_base);
   } else {
     if (s.G * Ew > kScanGroupCells || s.router_blocks % s.G != 0) return SWITCH_MOE_UNSUPPORTED_SHAPE;
     launch_k(plan_scan_groups_kernel, dim3(1), dim3(kScanThreads), 0, st, ws_ptr<int>(ws, p.hist), blocks_per_group,
              ws_ptr<float>(ws, p.psum_partial), s.router_blocks / s.G, s.G, s.Tg, s.E, Ew, s.Cg, s.alpha,
              ws_ptr<int>(ws, p.hist_base), ws_ptr<int>(ws, p.count), ws_ptr<int>(ws, p.kept),
-             ws_ptr<float>(ws, p.psum), aux_loss, ws_ptr<int>(ws, p.tile_expert), ws_ptr<int>(ws, p.tile_row0),
+             ws_ptr<float>(ws, p.psum), aux_loss, list128(s, p, ws), ws_ptr<int>(ws, p.tile_row0),
              ws_ptr<int4>(ws, p.ntile), count_g, group_base);
   }
   launch_k(plan_assign_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, ei, ws_ptr<int>(ws, p.hist_base),
@@ -706,7 +763,7 @@ int launch_reroute(const Shape& s, const Plan& p, void* ws, cudaStream_t st) {
     launch_k(plan_hist_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, alt, s.T, s.E,
              ws_ptr<int>(ws, p.hist));
     launch_k(reroute_scan_kernel, dim3(1), dim3(kMaxExperts), 0, st, ws_ptr<int>(ws, p.hist), s.plan_blocks, s.E, s.C,
-             ws_ptr<int>(ws, p.hist_base), ws_ptr<int>(ws, p.kept), ws_ptr<int>(ws, p.tile_expert),
+             ws_ptr<int>(ws, p.hist_base), ws_ptr<int>(ws, p.kept), list128(s, p, ws),
              ws_ptr<int>(ws, p.tile_row0), ws_ptr<int4>(ws, p.ntile));
     launch_k(reroute_assign_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, alt, ei,
              ws_ptr<int>(ws, p.hist_base), ws_ptr<float>(ws, p.probs), s.T, s.E, s.C, ws_ptr<int>(ws, p.slot),
@@ -716,35 +773,37 @@ int launch_reroute(const Shape& s, const Plan& p, void* ws, cudaStream_t st) {
   return launch_status();
 }
 
+namespace {
+dim3 gather_grid(long long warps, int per_sm) {
+  const long long blocks = (warps + 7) / 8, most = (long long)sm_count_or_default() * per_sm;
+  return dim3((unsigned)(blocks < most ? blocks : most));
+}
+// Rows past an expert's last token that the GEMMs' tiles may read: the CTA-pair path's tiles end at a multiple of 16.
+int pad_rows(const Shape& s) { return s.gemm_path == 0 ? 16 : kTileM; }
+}  // namespace
+
 int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void* ws, cudaStream_t st) {
   const int row_vec = (int)((size_t)s.d * s.elt / 16);
   // top-2 routing: the output rows of dropped assignments are skipped by the kernel that sums the two choices
-  const int slot_blocks = (s.E * s.C + 7) / 8, tok_blocks = s.top2 ? 0 : (s.T + 7) / 8;
-  launch_k(gather_x_kernel, dim3(slot_blocks + tok_blocks), dim3(256), 0, st, 
+  launch_k(gather_x_kernel, gather_grid(((long long)s.E * s.C + 3) / 4, kGatherBlocksPerSm), dim3(256), 0, st,
       static_cast<const uint4*>(x), ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.kept),
-      ws_ptr<int>(ws, p.slot), s.T, s.E, s.C, row_vec, slot_blocks, s.residual, ws_ptr<uint4>(ws, p.xd),
-      static_cast<uint4*>(y));
+      ws_ptr<int>(ws, p.slot), s.T, s.E * s.C, s.C, row_vec, pad_rows(s), s.residual, ws_ptr<uint4>(ws, p.xd),
+      s.top2 ? nullptr : static_cast<uint4*>(y));
   return launch_status();
 }
 
 int launch_gather_dy(const Shape& s, const Plan& p, const void* dy, const void* y, void* dx, void* ws, cudaStream_t st) {
   const int row_vec = (int)((size_t)s.d * s.elt / 16);
-  const int slot_blocks = (s.E * s.C + 7) / 8;
   // (top-2 routing: dx rows are formed by the kernel that sums the two assignments, and `y` is the per-assignment
   // output buffer already)
-  const int blocks = slot_blocks + ((s.residual && !s.top2) ? (s.T + 7) / 8 : 0);
+  const bool skip = s.residual && !s.top2;
   // with the skip path inside the layer, y holds x + g . E(x): the gate's gradient needs the copy without x
-  const void* ysrc = (s.residual && !s.top2) ? ws_ptr<char>(ws, p.layer_y) : y;
-  if (s.dtype == SWITCH_MOE_BF16)
-    launch_k(gather_dy_kernel<true>, dim3(blocks), dim3(256), 0, st, static_cast<const uint4*>(dy),
-             static_cast<const uint4*>(ysrc), ws_ptr<float>(ws, p.gate), ws_ptr<int>(ws, p.token_of_slot),
-             ws_ptr<int>(ws, p.kept), ws_ptr<int>(ws, p.slot), s.T, s.E, s.C, row_vec, slot_blocks,
-             ws_ptr<uint4>(ws, p.dyd), ws_ptr<float>(ws, p.dgate), static_cast<uint4*>(dx));
-  else
-    launch_k(gather_dy_kernel<false>, dim3(blocks), dim3(256), 0, st, static_cast<const uint4*>(dy),
-             static_cast<const uint4*>(ysrc), ws_ptr<float>(ws, p.gate), ws_ptr<int>(ws, p.token_of_slot),
-             ws_ptr<int>(ws, p.kept), ws_ptr<int>(ws, p.slot), s.T, s.E, s.C, row_vec, slot_blocks,
-             ws_ptr<uint4>(ws, p.dyd), ws_ptr<float>(ws, p.dgate), static_cast<uint4*>(dx));
+  const void* ysrc = skip ? ws_ptr<char>(ws, p.layer_y) : y;
+  auto kernel = s.dtype == SWITCH_MOE_BF16 ? gather_dy_kernel<true> : gather_dy_kernel<false>;
+  launch_k(kernel, gather_grid((long long)s.E * s.C, kGatherDyBlocksPerSm), dim3(256), 0, st, static_cast<const uint4*>(dy),
+           static_cast<const uint4*>(ysrc), ws_ptr<float>(ws, p.gate), ws_ptr<int>(ws, p.token_of_slot),
+           ws_ptr<int>(ws, p.kept), ws_ptr<int>(ws, p.slot), s.T, s.E * s.C, s.C, row_vec, pad_rows(s),
+           ws_ptr<uint4>(ws, p.dyd), ws_ptr<float>(ws, p.dgate), skip ? static_cast<uint4*>(dx) : nullptr);
   return launch_status();
 }
 

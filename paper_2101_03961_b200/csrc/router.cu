@@ -370,21 +370,32 @@ router_dwr_partial_kernel(const XT* __restrict__ x, const float* __restrict__ dl
   }
 }
 
-__global__ void router_dwr_reduce_kernel(const float* __restrict__ partial, int chunks, size_t n,
-                                         float* __restrict__ dW_r) {
+// dW_r = sum of the partials, in a fixed order: a block's eight warps take every eighth partial of 32 consecutive elements
+// (four loads in flight each), then the eight sums are added in warp order.
+__global__ void __launch_bounds__(256)
+router_dwr_reduce_kernel(const float* __restrict__ partial, int chunks, size_t n, float* __restrict__ dW_r) {
   pdl_launch_dependents();
   pdl_wait();
-  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
+  __shared__ float part[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const size_t i = (size_t)blockIdx.x * 32 + lane;
   float s = 0.f;
-  for (int c0 = 0; c0 < chunks; c0 += 8) {                     // eight rows in flight, added in a fixed order
-    float v[8];
+  if (i < n) {
+    for (int c0 = w; c0 < chunks; c0 += 32) {
+      float v[4];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = c0 + j < chunks ? partial[(size_t)(c0 + j) * n + i] : 0.f;
+      for (int j = 0; j < 4; ++j) v[j] = c0 + 8 * j < chunks ? partial[(size_t)(c0 + 8 * j) * n + i] : 0.f;
 #pragma unroll
-    for (int j = 0; j < 8; ++j) s += v[j];
+      for (int j = 0; j < 4; ++j) s += v[j];
+    }
   }
-  dW_r[i] = s;
+  part[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && i < n) {
+#pragma unroll
+    for (int k = 1; k < 8; ++k) s += part[k][lane];
+    dW_r[i] = s;
+  }
 }
 
 // dx[t,k] = (accumulate and t kept ? dx[t,k] : 0) + sum_i dh[t,i] W_r[k,i]; block = 64 tokens x 64 k per step.
@@ -496,14 +507,14 @@ int router_bwd_t(const Shape& s, const Plan& p, const void* x, const float* W_r,
       // tensor-core products (bf16-split operands), then the same fixed-order reduction of the token splits
       int rc = launch_router_tc_bwd(s, p, x, W_r, ws, dx, accumulate_dx, st);
       if (rc != SWITCH_MOE_OK) return rc;
-      launch_k(router_dwr_reduce_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, partial, s.dwr_chunks, n, dW_r);
+      launch_k(router_dwr_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, partial, s.dwr_chunks, n, dW_r);
       return launch_status();
     }
   }
   dim3 grid((s.d + kDwrK - 1) / kDwrK, s.dwr_chunks);
   launch_k(router_dwr_partial_kernel<XT, NE>, dim3(grid), dim3(256), 0, st, static_cast<const XT*>(x), dlogits, s.T, s.d, s.E,
            s.dwr_chunk_tokens, partial);
-  launch_k(router_dwr_reduce_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, partial, s.dwr_chunks, n, dW_r);
+  launch_k(router_dwr_reduce_kernel, dim3((unsigned)((n + 31) / 32)), dim3(256), 0, st, partial, s.dwr_chunks, n, dW_r);
   constexpr int ES = 32 * NE + 4;
   const size_t smem = 2 * 64 * ES * sizeof(float);
   if (cudaFuncSetAttribute(router_dx_kernel<XT, NE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=

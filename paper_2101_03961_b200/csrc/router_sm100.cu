@@ -19,380 +19,6 @@ namespace swmoe {
 using namespace tc;
 namespace {
 
-constexpr int kRTcThreads = 320;                     // generic kernel: TMA warp, MMA warp, 8 epilogue warps
-constexpr int kRTcOutStageBytes = 8 * 32 * 128;
-constexpr int kRTcSmemBytes = 1024 + kStages * kStageBytes + kRTcOutStageBytes + 128;
-
-// kRDxRes: dx with the two parts of one 256-row block of W_r resident in shared memory for the CTA's whole life
-// (up to 128 experts): only the logit gradients stream, and every staged block of them meets the W_r parts it pairs
-// with in the three cross terms without a reload.
-enum RouterOp { kRDwr = 1, kRDx = 2, kRDxRes = 3 };
-
-struct RouterTcParams {
-  int T, d, E, Epad64;
-  int mma_n;                 // MMA N: Epad64 (dwr) or 256 (dx)
-  int n_mtiles, n_ntiles;
-  int splits, chunk_kblocks, total_kblocks;   // dwr: split of the token contraction
-  int wrap;                  // k-blocks per part: Epad64/64 (dx); dwr derives it per tile
-  int both_parts;            // dwr: 1 = a stage holds the x block and both parts of dh (2 x mma_n columns <= 256)
-  float* partial;                                                                         // dwr
-  __nv_bfloat16* dx; const int* slot; int accumulate; const __nv_bfloat16* jitter_u;      // dx
-  int* status;
-};
-
-struct RTile {
-  int m0, n0, split, k_base, wrap, k_blocks;
-};
-
-template <int OP>
-__device__ __forceinline__ int r_total_tiles(const RouterTcParams& p) {
-  if (OP == kRDwr) return p.n_mtiles * p.splits;
-  if (OP == kRDxRes) return p.n_mtiles;
-  return p.n_mtiles * p.n_ntiles;
-}
-
-template <int OP>
-__device__ __forceinline__ RTile r_decode(const RouterTcParams& p, int id) {
-  RTile t;
-  t.split = 0; t.k_base = 0; t.n0 = 0;
-  if (OP == kRDwr) {
-    const int mt = id / p.splits;
-    t.split = id - mt * p.splits;
-    t.m0 = mt * kTileM;
-    t.k_base = t.split * p.chunk_kblocks;
-    t.wrap = max(0, min(p.chunk_kblocks, p.total_kblocks - t.k_base));
-  } else if (OP == kRDxRes) {                         // id = token tile; the CTA's block of W_r rows is fixed
-    t.m0 = id * kTileM;
-    t.n0 = (int)(blockIdx.x % (unsigned)p.n_ntiles) * kBN;
-    t.wrap = p.wrap;
-  } else {
-    const int mt = id / p.n_ntiles;
-    t.m0 = mt * kTileM;
-    t.n0 = (id - mt * p.n_ntiles) * kBN;
-    t.wrap = p.wrap;
-  }
-  // dW_r: dh = hi + mid, both parts staged with the x block they
-  // multiply when they fit (up to 128 experts), else one after the other; dx: three cross terms
-  t.k_blocks = (OP == kRDx ? 3 : (OP == kRDwr && p.both_parts) ? 1 : 2) * t.wrap;   // kRDxRes: hi and mid of dh
-  return t;
-}
-
-template <int OP, bool kJitter>                        // kJitter: dx under input jitter
-__global__ void __launch_bounds__(kRTcThreads, 1)
-router_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                 const RouterTcParams p) {
-  constexpr bool kAMn = (OP == kRDwr);                 // x^T: token rows are the contraction, d contiguous
-  constexpr bool kDx = (OP == kRDx || OP == kRDxRes);
-  constexpr bool kBMn = !kDx;                          // dwr: dh [T][E]; dx: W as [d rows][E contiguous]
-  pdl_launch_dependents();
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
-  uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
-  const uint32_t bar_base = smem_base + kStages * kStageBytes + kRTcOutStageBytes;
-  uint8_t* bar_gen = smem_gen + kStages * kStageBytes + kRTcOutStageBytes;
-  auto full_bar = [&](int s) { return bar_base + 8u * s; };
-  auto empty_bar = [&](int s) { return bar_base + 8u * (kStages + s); };
-  auto tfull_bar = [&](int a) { return bar_base + 8u * (2 * kStages + a); };
-  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 * kStages + 2 + a); };
-  volatile uint32_t* tmem_ptr_s = reinterpret_cast<volatile uint32_t*>(bar_gen + 8 * (2 * kStages + 4));
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 8 * (2 * kStages + 4) + 4);
-  const uint32_t wfull_bar = bar_base + 8u * (2 * kStages + 5);     // kRDxRes: the resident W_r parts have landed
-  const int warp = uniform_warp_id(), lane = threadIdx.x & 31;
-  // kRDxRes: the operand ring's first 64 KB are four 16 KB stages of logit-gradient blocks, the rest holds the
-  // resident W_r parts: [part][k-block] blocks of 256 rows x 64 experts (32 KB each)
-  const uint32_t w_res = smem_base + kStages * kABytes;
-  // tiles of this CTA: kRDxRes deals token tiles out among the CTAs that share a block of W_r rows
-  const int tile_first = OP == kRDxRes ? (int)(blockIdx.x / (unsigned)p.n_ntiles) : (int)blockIdx.x;
-  const int tile_step = OP == kRDxRes ? (int)(gridDim.x / (unsigned)p.n_ntiles) : (int)gridDim.x;
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-    for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), 8); }
-    mbar_init(wfull_bar, 1);
-    *abort_flag = 0;
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  }
-  if (warp == 2) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                     smem_u32(const_cast<uint32_t*>(tmem_ptr_s))), "r"(kTmemCols) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_ptr_s;
-  pdl_wait();                                                 // the previous kernel's results are needed from here on
-  const int n_tiles = r_total_tiles<OP>(p);
-  const int b_atoms = (p.mma_n + 63) / 64;
-  const bool both = OP == kRDwr && p.both_parts;
-  const uint32_t stage_tx = kABytes + (kBMn ? (uint32_t)(both ? 2 : 1) * b_atoms * kAtomBytes : (uint32_t)kBBytes);
-
-  if (warp == 0) {
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    if (OP == kRDxRes && elect_one()) {                       // W_r parts hi, mid of this CTA's 256 rows, once
-      const int n0 = (int)(blockIdx.x % (unsigned)p.n_ntiles) * kBN;
-      mbar_arrive_expect_tx(wfull_bar, 2u * (uint32_t)p.wrap * kBBytes);
-      for (int part = 0; part < 2; ++part)
-        for (int kk = 0; kk < p.wrap; ++kk)
-          tma_load_3d(w_res + (uint32_t)(part * p.wrap + kk) * kBBytes, &tmB, wfull_bar, kk * kBK, n0, part);
-    }
-    __syncwarp();
-    for (int id = tile_first; id < n_tiles && ok; id += tile_step) {
-      const RTile t = r_decode<OP>(p, id);
-#pragma unroll 1
-      for (int kb = 0; kb < t.k_blocks; ++kb) {
-        const int part = kb / t.wrap, kblk = t.k_base + (kb - part * t.wrap);
-        ok = mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status, 11);
-        if (!ok) break;
-        if (elect_one()) {
-          const uint32_t fb = full_bar(stage);
-          if (OP == kRDxRes) {                                // dh part [128 tok][64 e] only
-            mbar_arrive_expect_tx(fb, kABytes);
-            tma_load_3d(smem_base + stage * kABytes, &tmA, fb, kblk * kBK, t.m0, part);
-          } else {
-            const uint32_t a_dst = smem_base + stage * kStageBytes, b_dst = a_dst + kABytes;
-            mbar_arrive_expect_tx(fb, stage_tx);
-            if (OP == kRDwr) {
-              tma_load_3d(a_dst, &tmA, fb, t.m0, kblk * kBK, 0);                            // x^T: [64 tok][64 k-of-d]
-              tma_load_3d(a_dst + kAtomBytes, &tmA, fb, t.m0 + 64, kblk * kBK, 0);
-              for (int j = 0; j < b_atoms; ++j)                                              // dh part [64 tok][64 e]
-                tma_load_3d(b_dst + j * kAtomBytes, &tmB, fb, 64 * j, kblk * kBK, part);
-              if (both)                                                                      // the other part, behind it
-                for (int j = 0; j < b_atoms; ++j)
-                  tma_load_3d(b_dst + (b_atoms + j) * kAtomBytes, &tmB, fb, 64 * j, kblk * kBK, 1);
-            } else {
-              const int a_part = part == 2 ? 1 : 0, b_part = part == 1 ? 1 : 0;             // (hi,hi) (hi,mid) (mid,hi)
-              tma_load_3d(a_dst, &tmA, fb, kblk * kBK, t.m0, a_part);                       // dh part [128 tok][64 e]
-              tma_load_3d(b_dst, &tmB, fb, kblk * kBK, t.n0, b_part);                       // W part [256 k-of-d][64 e]
-            }
-          }
-        }
-        if (++stage == kStages) { stage = 0; phase ^= 1u; }
-      }
-    }
-    if (*abort_flag != 0) {
-      const unsigned long long t0 = global_ns();
-      while (global_ns() - t0 < 2000000ull) __nanosleep(1000);
-    }
-  } else if (warp == 1) {
-    const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)kAMn << 15) | ((uint32_t)kBMn << 16) |
-                           ((uint32_t)(p.mma_n >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
-    constexpr uint32_t a_lbo = kAMn ? kAtomBytes : 16u, b_lbo = kBMn ? kAtomBytes : 16u;
-    constexpr uint32_t a_kstep = (kAMn ? kUmmaK * 128u : kUmmaK * 2u) >> 4;       // descriptor units of 16 bytes
-    constexpr uint32_t b_kstep = (kBMn ? kUmmaK * 128u : kUmmaK * 2u) >> 4;
-    int stage = 0, acc = 0;
-    uint32_t phase = 0, acc_phase = 0;
-    bool ok = true;
-    if (OP == kRDxRes) ok = mbar_wait_warp(wfull_bar, 0u, abort_flag, p.status, 15);
-    for (int id = tile_first; id < n_tiles && ok; id += tile_step) {
-      const RTile t = r_decode<OP>(p, id);
-      ok = mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status, 12);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t d_tmem = tmem_base + (uint32_t)acc * kBN;
-#pragma unroll 1
-      for (int kb = 0; kb < t.k_blocks; ++kb) {
-        ok = mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status, 13);
-        if (!ok) break;
-        tc_fence_after();
-        if (elect_one()) {
-          if (OP == kRDxRes) {
-            // staged block: part `dpart` of dh, experts 64 kk .. 64 kk + 63.  dh_hi meets W_hi and W_mid, dh_mid meets W_hi.
-            const int dpart = kb / t.wrap, kk = kb - dpart * t.wrap;
-            const uint64_t ad = make_smem_desc(smem_base + stage * kABytes, a_lbo, 1024u);
-            const int n_w = dpart == 0 ? 2 : 1;
-#pragma unroll 1
-            for (int wp = 0; wp < n_w; ++wp) {
-              const uint64_t bd = make_smem_desc(w_res + (uint32_t)(wp * t.wrap + kk) * kBBytes, b_lbo, 1024u);
-#pragma unroll
-              for (int ks = 0; ks < kBK / kUmmaK; ++ks)
-                tc_mma_bf16(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc, (kb > 0 || wp > 0 || ks > 0) ? 1u : 0u);
-            }
-          } else {
-            const uint32_t a_src = smem_base + stage * kStageBytes;
-            const uint64_t ad = make_smem_desc(a_src, a_lbo, 1024u);
-            uint64_t bd = make_smem_desc(a_src + kABytes, b_lbo, 1024u);
-#pragma unroll
-            for (int ks = 0; ks < kBK / kUmmaK; ++ks)
-              tc_mma_bf16(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc, (kb > 0 || ks > 0) ? 1u : 0u);
-            if (both) {
-              bd += (uint64_t)((uint32_t)(b_atoms * kAtomBytes) >> 4);
-#pragma unroll
-              for (int ks = 0; ks < kBK / kUmmaK; ++ks) tc_mma_bf16(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc, 1u);
-            }
-          }
-          tc_commit(empty_bar(stage));
-          if (kb == t.k_blocks - 1) tc_commit(tfull_bar(acc));
-        }
-        if (++stage == kStages) { stage = 0; phase ^= 1u; }
-      }
-      if (!ok) break;
-      if (t.k_blocks <= 0 && lane == 0) mbar_arrive(tfull_bar(acc));
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-    }
-  } else {
-    const int lg = warp & 3;
-    const int half = (warp - 2) >> 2;                         // second warp of the lane group: other half of the columns
-    uint8_t* my_stage_gen = smem_gen + kStages * kStageBytes + (warp - 2) * 4096;
-    int acc = 0;
-    uint32_t acc_phase = 0;
-    bool ok = true;
-    for (int id = tile_first; id < n_tiles && ok; id += tile_step) {
-      const RTile t = r_decode<OP>(p, id);
-      const int r = lg * 32 + lane;
-      // dx: previous contents of the rows this thread will write (prefetched before the accumulator is ready)
-      long long offs[8];
-      unsigned add_mask = 0;
-      if (kDx) {
-        const int tok = t.m0 + r;
-        const long long row_off = tok < p.T ? (long long)tok * p.d : -1;
-        const int add = (p.accumulate && tok < p.T && (p.accumulate == 2 || p.slot[tok] >= 0)) ? 1 : 0;
-#pragma unroll
-        for (int it = 0; it < 8; ++it) {
-          offs[it] = __shfl_sync(0xffffffffu, row_off, it * 4 + (lane >> 3));
-          add_mask |= (unsigned)__shfl_sync(0xffffffffu, add, it * 4 + (lane >> 3)) << it;
-        }
-      }
-      ok = mbar_wait_warp(tfull_bar(acc), acc_phase, abort_flag, p.status, 14);
-      if (!ok) break;
-      tc_fence_after();
-      const uint32_t t_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)acc * kBN;
-      const bool have_acc = t.k_blocks > 0;
-
-      if (OP == kRDwr) {
-        // ---- float32 partial of x^T dh for this token split: row = m0 + r (an index into d_model)
-        const int row = t.m0 + r;
-        const int nch = p.mma_n / 32;
-        bool released = false;
-        for (int c = half; c < nch; c += 2) {
-          uint32_t v[32];
-          if (have_acc) {
-            tc_ld32(t_addr + c * 32, v);
-            tc_wait_ld();
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = 0u;
-          }
-          if (c + 2 >= nch) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(acc));
-            released = true;
-          }
-          if (row < p.d) {
-            float* dst = p.partial + ((size_t)t.split * p.d + row) * p.E + c * 32;
-            if ((p.E & 3) == 0) {
-#pragma unroll
-              for (int i = 0; i < 32; i += 4)
-                if (c * 32 + i < p.E)
-                  *reinterpret_cast<float4*>(dst + i) = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
-                                                                    __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
-            } else {
-#pragma unroll
-              for (int i = 0; i < 32; ++i)
-                if (c * 32 + i < p.E) dst[i] = __uint_as_float(v[i]);
-            }
-          }
-        }
-        if (!released) {
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(tempty_bar(acc));
-        }
-      } else {
-        // ---- dx[token] = (accumulate and kept ? dx[token] : 0) + dh W_r^T, 64 columns at a time
-#pragma unroll 1
-        for (int c = 2 * half; c < 2 * half + 2; ++c) {
-          const int col = t.n0 + c * 64 + (lane & 7) * 8;
-          uint4 prev[8];
-#pragma unroll
-          for (int it = 0; it < 8; ++it)
-            prev[it] = (((add_mask >> it) & 1u) && col < p.d) ? *reinterpret_cast<const uint4*>(p.dx + offs[it] + col)
-                                                             : make_uint4(0, 0, 0, 0);
-          uint4 uu[kJitter ? 8 : 1];                                        // jitter factors of the same elements, fetched early too
-          if (kJitter) {
-#pragma unroll
-            for (int it = 0; it < 8; ++it)
-              uu[kJitter ? it : 0] = (offs[it] >= 0 && col < p.d) ? *reinterpret_cast<const uint4*>(p.jitter_u + offs[it] + col)
-                                                    : make_uint4(0, 0, 0, 0);
-          }
-          uint32_t v[64];
-          tc_ld32(t_addr + c * 64, v);
-          tc_ld32(t_addr + c * 64 + 32, v + 32);
-          tc_wait_ld();
-          if (c == 2 * half + 1) {
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(tempty_bar(acc));
-          }
-          // stage the float32 values as two bf16-pair planes?  No: keep float32 accuracy of the sum by staging
-          // bf16(acc) only when nothing is added; otherwise add in float32 after the transpose (values are bf16
-          // on both sides, so staging bf16(acc) costs one extra rounding of the small router term only).
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            uint32_t w[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[j * 8 + 2 * q]),
-                                                        __uint_as_float(v[j * 8 + 2 * q + 1]));
-              w[q] = *reinterpret_cast<uint32_t*>(&h2);
-            }
-            *reinterpret_cast<uint4*>(my_stage_gen + lane * 128 + ((j ^ (lane & 7)) << 4)) =
-                make_uint4(w[0], w[1], w[2], w[3]);
-          }
-          __syncwarp();
-          if (col < p.d) {
-#pragma unroll
-            for (int it = 0; it < 8; ++it) {
-              const int rr = it * 4 + (lane >> 3);
-              uint4 val = *reinterpret_cast<const uint4*>(my_stage_gen + rr * 128 + (((lane & 7) ^ (rr & 7)) << 4));
-              if (kJitter && offs[it] >= 0) {      // d(x . u)/dx = u
-                __nv_bfloat162* vp = reinterpret_cast<__nv_bfloat162*>(&val);
-                const __nv_bfloat162* up = reinterpret_cast<const __nv_bfloat162*>(&uu[kJitter ? it : 0]);
-                if ((add_mask >> it) & 1u) {                     // one rounding for (router term . u) + dx
-                  const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&prev[it]);
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const float2 a = __bfloat1622float2(vp[q]), b = __bfloat1622float2(pp[q]), c2 = __bfloat1622float2(up[q]);
-                    vp[q] = __floats2bfloat162_rn(fmaf(a.x, c2.x, b.x), fmaf(a.y, c2.y, b.y));
-                  }
-                } else {
-#pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const float2 a = __bfloat1622float2(vp[q]), c2 = __bfloat1622float2(up[q]);
-                    vp[q] = __floats2bfloat162_rn(a.x * c2.x, a.y * c2.y);
-                  }
-                }
-              } else if ((add_mask >> it) & 1u) {
-                __nv_bfloat162* vp = reinterpret_cast<__nv_bfloat162*>(&val);
-                const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&prev[it]);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                  const float2 a = __bfloat1622float2(vp[q]), b = __bfloat1622float2(pp[q]);
-                  vp[q] = __floats2bfloat162_rn(a.x + b.x, a.y + b.y);
-                }
-              }
-              if (offs[it] >= 0) *reinterpret_cast<uint4*>(p.dx + offs[it] + col) = val;
-            }
-          }
-          __syncwarp();
-        }
-      }
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
-    }
-  }
-
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 2) {
-    tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
-  }
-}
-
 // ------------------------------------------------------------------------------------------------------------------
 // Forward router.  A CTA works on one or two 128-token tiles at a time that share every staged k-block of W_r; these
 // tokens are one row of the dispatch plan's histogram table and of the P-sum partials, which the epilogue leaves: the
@@ -712,6 +338,292 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
   }
 }
 
+// ------------------------------------------------------------------------------------------------------------------
+// Backward router: dW_r = x^T dh and dx += dh W_r^T in one pass over the tokens.
+//
+// A CTA owns a block of 128 columns of d_model and walks its share of the 128-token tiles.  Per tile it stages the x
+// block [128 tokens][128 columns] and, one 16 KB block of 64 experts at a time, both bfloat16 parts of the logit
+// gradients; the parts of W_r for its columns stay in shared memory for the CTA's life.  A staged block of dh serves both
+// products (as the K-major A operand of dh W_r^T and the N-major B operand of x^T dh: the same bytes).  dW_r accumulates
+// in tensor memory over all the CTA's tiles and leaves once, as one partial per CTA; dx has two accumulators, so the
+// epilogue of a tile (read dx, add, round, store) overlaps the next tile's products.
+//
+// What bounds it: x is read once and dx read and written once from HBM, and every column block reads dh from L2; the
+// operands of both products cross shared memory at about its rate.  Measured with its neighbours (logit gradients before,
+// reduction of the partials after) against one kernel per product: 32768 tokens, d 768, E 128 82 -> 67 us; 65536 tokens,
+// d 256, E 128 (jitter) 83 -> 63; 16384 tokens, d 768, E 64 45 -> 34; 20011 tokens, d 512, E 200 61 -> 63.
+struct RouterBwdParams {
+  int T, d, E, ka;           // ka: blocks of 64 experts (1..4)
+  int n_mtiles, n_cols, splits, x_stages, ring;
+  float* partial; __nv_bfloat16* dx; const int* slot; int accumulate; const __nv_bfloat16* jitter_u;
+  int* status;
+};
+constexpr int kRBThreads = 320;                                // TMA warp, MMA warp, 8 epilogue warps
+constexpr int kRBBlock = kTileM * 128;                         // 128 rows of 128 bytes: a block of dh, of W_r, half of x
+constexpr int kRBStageOut = 8 * 16 * 128;                      // epilogue transposition, 16 rows of 128 bytes per warp
+constexpr int kRBOperandBytes = 208 * 1024;                    // W_r parts, x stages, ring of dh blocks
+constexpr int kRBMaxRing = 6;
+constexpr int kRBSmemBytes = 1024 + kRBOperandBytes + kRBStageOut + 256;
+constexpr int kRBDwrCol = 256;                                 // first TMEM column of the dW_r accumulator
+
+template <bool kJitter>
+__global__ void __launch_bounds__(kRBThreads, 1)
+router_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmH,
+                     const __grid_constant__ CUtensorMap tmW, const RouterBwdParams p) {
+  pdl_launch_dependents();
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
+  uint8_t* smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
+  const uint32_t bar_base = smem_base + kRBOperandBytes + kRBStageOut;
+  uint8_t* bar_gen = smem_gen + kRBOperandBytes + kRBStageOut;
+  // barriers: ring full[6] | ring empty[6] | x full[2] | x empty[2] | dx full[2] | dx empty[2] | W_r full | dW_r full
+  const uint32_t rfull0 = bar_base, rempty0 = rfull0 + 8u * kRBMaxRing, xfull0 = rempty0 + 8u * kRBMaxRing;
+  const uint32_t xempty0 = xfull0 + 16u, tfull0 = xfull0 + 32u, tempty0 = xfull0 + 48u, wfull = xfull0 + 64u, dfull = xfull0 + 72u;
+  volatile uint32_t* tmem_ptr_s = reinterpret_cast<volatile uint32_t*>(bar_gen + 16 * kRBMaxRing + 80);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 16 * kRBMaxRing + 84);
+  const int warp = uniform_warp_id(), lane = threadIdx.x & 31;
+  const int col_block = (int)(blockIdx.x % (unsigned)p.n_cols), split = (int)(blockIdx.x / (unsigned)p.n_cols);
+  const int n0 = col_block * 128, ka = p.ka;
+  const uint32_t w_s = smem_base, x_s = w_s + 2u * ka * kRBBlock, ring_s = x_s + 2u * p.x_stages * kRBBlock;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kRBMaxRing; ++s) { mbar_init(rfull0 + 8u * s, 1); mbar_init(rempty0 + 8u * s, 1); }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(xfull0 + 8u * s, 1); mbar_init(xempty0 + 8u * s, 1);
+      mbar_init(tfull0 + 8u * s, 1); mbar_init(tempty0 + 8u * s, 8);
+    }
+    mbar_init(wfull, 1);
+    mbar_init(dfull, 1);
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                     smem_u32(const_cast<uint32_t*>(tmem_ptr_s))), "r"(kTmemCols) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_ptr_s;
+  pdl_wait();                                                 // the previous kernel's results are needed from here on
+
+  if (warp == 0) {
+    // ------------------------------------------------------------------------------------------ TMA producer
+    if (elect_one()) {
+      mbar_arrive_expect_tx(wfull, 2u * (uint32_t)ka * kRBBlock);
+      for (int part = 0; part < 2; ++part)
+        for (int kk = 0; kk < ka; ++kk) tma_load_3d(w_s + (uint32_t)(part * ka + kk) * kRBBlock, &tmW, wfull, kk * 64, n0, part);
+    }
+    __syncwarp();
+    uint32_t slot_i = 0, slot_phase = 0, xs = 0, x_phase = 0;
+    bool ok = true;
+    for (int tile = split; tile < p.n_mtiles && ok; tile += p.splits) {
+      const int m0 = tile * kTileM;
+      ok = mbar_wait_warp(xempty0 + 8u * xs, x_phase ^ 1u, abort_flag, p.status, 11);
+      if (!ok) break;
+      if (elect_one()) {
+        mbar_arrive_expect_tx(xfull0 + 8u * xs, 2u * kRBBlock);
+        tma_load_3d(x_s + 2u * xs * kRBBlock, &tmX, xfull0 + 8u * xs, n0, m0, 0);              // x [128 tok][64 columns]
+        tma_load_3d(x_s + (2u * xs + 1u) * kRBBlock, &tmX, xfull0 + 8u * xs, n0 + 64, m0, 0);
+      }
+      if (++xs == (uint32_t)p.x_stages) { xs = 0; x_phase ^= 1u; }
+#pragma unroll 1
+      for (int b = 0; b < 2 * ka; ++b) {
+        ok = mbar_wait_warp(rempty0 + 8u * slot_i, slot_phase ^ 1u, abort_flag, p.status, 12);
+        if (!ok) break;
+        const int part = b >= ka ? 1 : 0;
+        if (elect_one()) {
+          mbar_arrive_expect_tx(rfull0 + 8u * slot_i, kRBBlock);
+          tma_load_3d(ring_s + slot_i * kRBBlock, &tmH, rfull0 + 8u * slot_i, (b - part * ka) * 64, m0, part);
+        }
+        if (++slot_i == (uint32_t)p.ring) { slot_i = 0; slot_phase ^= 1u; }
+      }
+    }
+    if (*abort_flag != 0) {
+      const unsigned long long t0 = global_ns();
+      while (global_ns() - t0 < 2000000ull) __nanosleep(1000);
+    }
+  } else if (warp == 1) {
+    // ------------------------------------------------------------------------------------------ MMA issuer
+    constexpr uint32_t idesc_dx = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+    constexpr uint32_t idesc_dw = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) | ((64u >> 3) << 17) |
+                                  ((uint32_t)(kTileM >> 4) << 24);
+    uint32_t slot_i = 0, slot_phase = 0, xs = 0, x_phase = 0, acc = 0, acc_phase = 0;
+    bool first = true;
+    bool ok = mbar_wait_warp(wfull, 0u, abort_flag, p.status, 15);
+    for (int tile = split; tile < p.n_mtiles && ok; tile += p.splits) {
+      ok = mbar_wait_warp(tempty0 + 8u * acc, acc_phase ^ 1u, abort_flag, p.status, 13) &&
+           mbar_wait_warp(xfull0 + 8u * xs, x_phase, abort_flag, p.status, 16);
+      if (!ok) break;
+      tc_fence_after();
+      const uint64_t xd = make_smem_desc(x_s + 2u * xs * kRBBlock, kRBBlock, 1024u);           // x^T: two 64-column atoms
+#pragma unroll 1
+      for (int b = 0; b < 2 * ka; ++b) {
+        ok = mbar_wait_warp(rfull0 + 8u * slot_i, slot_phase, abort_flag, p.status, 17);
+        if (!ok) break;
+        tc_fence_after();
+        const int part = b >= ka ? 1 : 0, kk = b - part * ka;
+        const uint32_t blk = ring_s + slot_i * kRBBlock;
+        if (elect_one()) {
+          // dx: dh_hi meets W_hi and W_mid, dh_mid meets W_hi (the output is bfloat16: 2^-16 suffices)
+          const uint64_t ad = make_smem_desc(blk, 16u, 1024u);
+#pragma unroll 1
+          for (int wp = 0; wp < 2 - part; ++wp) {
+            const uint64_t bd = make_smem_desc(w_s + (uint32_t)(wp * ka + kk) * kRBBlock, 16u, 1024u);
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks)
+              tc_mma_bf16(tmem_base + acc * 128u, ad + ks * 2, bd + ks * 2, idesc_dx, (b > 0 || wp > 0 || ks > 0) ? 1u : 0u);
+          }
+          // dW_r, columns 64 kk ..: contraction over the tile's 128 tokens, 16 at a time
+          const uint64_t hd = make_smem_desc(blk, kRBBlock, 1024u);
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)
+            tc_mma_bf16(tmem_base + kRBDwrCol + 64u * kk, xd + ks * 128, hd + ks * 128, idesc_dw,
+                        (!first || part > 0 || ks > 0) ? 1u : 0u);
+          tc_commit(rempty0 + 8u * slot_i);
+          if (b == 2 * ka - 1) {
+            tc_commit(xempty0 + 8u * xs);
+            tc_commit(tfull0 + 8u * acc);
+          }
+        }
+        if (++slot_i == (uint32_t)p.ring) { slot_i = 0; slot_phase ^= 1u; }
+      }
+      if (!ok) break;
+      first = false;
+      if (++xs == (uint32_t)p.x_stages) { xs = 0; x_phase ^= 1u; }
+      acc ^= 1u;
+      if (acc == 0) acc_phase ^= 1u;
+    }
+    if (ok && elect_one()) tc_commit(dfull);
+    __syncwarp();
+  } else {
+    // ------------------------------------------------------------------------------------------ epilogue warps
+    const int lg = warp & 3, half = (warp - 2) >> 2;          // TMEM lane group (32 tokens); which 64 columns
+    uint8_t* stage_gen = smem_gen + kRBOperandBytes + (warp - 2) * 2048;
+    const int col = n0 + half * 64 + (lane & 7) * 8;          // this lane's 8 columns in every store
+    const bool col_ok = col < p.d;
+    const uint32_t t_lane = tmem_base + ((uint32_t)(lg * 32) << 16);
+    uint32_t acc = 0, acc_phase = 0;
+    bool ok = true;
+    // Store `it` of this lane writes token tok0 + 4 it + lane / 8.  What those rows hold so far is requested a tile ahead:
+    // the loads of the next tile are in flight while this one's sums are formed and its accumulator is awaited.  (Under
+    // jitter the factors take those registers: requested at the tile's start.)
+    unsigned add_rows = 0;
+    uint4 prev[8], uu[kJitter ? 8 : 1];
+    auto fetch_rows = [&](int tile) {
+      const int tok0 = tile * kTileM + lg * 32, mine = tok0 + lane;
+      add_rows = __ballot_sync(0xffffffffu, p.accumulate != 0 && mine < p.T && (p.accumulate == 2 || p.slot[mine] >= 0));
+#pragma unroll
+      for (int it = 0; it < 8; ++it) {
+        const int row = it * 4 + (lane >> 3);
+        const size_t off = (size_t)(tok0 + row) * p.d + col;
+        prev[it] = ((add_rows >> row) & 1u) && col_ok ? *reinterpret_cast<const uint4*>(p.dx + off) : make_uint4(0, 0, 0, 0);
+        if (kJitter)
+          uu[kJitter ? it : 0] = tok0 + row < p.T && col_ok ? *reinterpret_cast<const uint4*>(p.jitter_u + off)
+                                                            : make_uint4(0, 0, 0, 0);
+      }
+    };
+    if (!kJitter) fetch_rows(split);
+    for (int tile = split; tile < p.n_mtiles && ok; tile += p.splits) {
+      if (kJitter) fetch_rows(tile);
+      const int tok0 = tile * kTileM + lg * 32;
+      ok = mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.status, 14);
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t v[64];
+      tc_ld32(t_lane + acc * 128u + (uint32_t)half * 64u, v);
+      tc_ld32(t_lane + acc * 128u + (uint32_t)half * 64u + 32u, v + 32);
+      tc_wait_ld();
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty0 + 8u * acc);
+      // transposed through shared memory as bfloat16 (one extra rounding of the small router term); the sum is formed
+      // in float32 afterwards, with coalesced rows
+      uint32_t pk[32];
+#pragma unroll
+      for (int j = 0; j < 32; ++j) {
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1]));
+        pk[j] = *reinterpret_cast<const uint32_t*>(&h2);
+      }
+      uint4 old[8];
+      const unsigned add_now = add_rows;
+#pragma unroll
+      for (int it = 0; it < 8; ++it) old[it] = prev[it];
+      if (!kJitter && tile + p.splits < p.n_mtiles) fetch_rows(tile + p.splits);
+#pragma unroll
+      for (int it = 0; it < 8; ++it) {
+        if ((it & 3) == 0) {                                   // 16 rows at a time
+          if (it > 0) __syncwarp();
+          if ((lane >> 4) == (it >> 2)) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              *reinterpret_cast<uint4*>(stage_gen + (lane & 15) * 128 + ((j ^ (lane & 7)) << 4)) =
+                  make_uint4(pk[4 * j], pk[4 * j + 1], pk[4 * j + 2], pk[4 * j + 3]);
+          }
+          __syncwarp();
+        }
+        const int row = it * 4 + (lane >> 3);
+        uint4 val = *reinterpret_cast<const uint4*>(stage_gen + (row & 15) * 128 + (((lane & 7) ^ (row & 7)) << 4));
+        const bool add = (add_now >> row) & 1u;
+        if (kJitter || add) {                                  // d(x . u)/dx = u; one rounding for (router term . u) + dx
+          __nv_bfloat162* vp = reinterpret_cast<__nv_bfloat162*>(&val);
+          const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&old[it]);
+          const __nv_bfloat162* up = reinterpret_cast<const __nv_bfloat162*>(&uu[kJitter ? it : 0]);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float2 a = __bfloat1622float2(vp[q]), b = __bfloat1622float2(pp[q]);
+            float2 s = make_float2(a.x + b.x, a.y + b.y);
+            if (kJitter) {
+              const float2 u = __bfloat1622float2(up[q]);
+              s = add ? make_float2(fmaf(a.x, u.x, b.x), fmaf(a.y, u.y, b.y)) : make_float2(a.x * u.x, a.y * u.y);
+            }
+            vp[q] = __floats2bfloat162_rn(s.x, s.y);
+          }
+        }
+        if (tok0 + row < p.T && col_ok) *reinterpret_cast<uint4*>(p.dx + (size_t)(tok0 + row) * p.d + col) = val;
+      }
+      __syncwarp();
+      acc ^= 1u;
+      if (acc == 0) acc_phase ^= 1u;
+    }
+    // float32 partial of x^T dh over this CTA's tokens: row = an index into d_model
+    if (ok) ok = mbar_wait_warp(dfull, 0u, abort_flag, p.status, 18);
+    if (ok) {
+      tc_fence_after();
+      const int row = n0 + lg * 32 + lane, nch = (p.E + 31) >> 5;
+#pragma unroll 1
+      for (int c = half; c < nch; c += 2) {
+        uint32_t v[32];
+        tc_ld32(t_lane + kRBDwrCol + (uint32_t)c * 32u, v);
+        tc_wait_ld();
+        if (row < p.d) {
+          float* dst = p.partial + ((size_t)split * p.d + row) * p.E + c * 32;
+          if ((p.E & 3) == 0) {
+#pragma unroll
+            for (int i = 0; i < 32; i += 4)
+              if (c * 32 + i < p.E)
+                *reinterpret_cast<float4*>(dst + i) = make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]),
+                                                                  __uint_as_float(v[i + 2]), __uint_as_float(v[i + 3]));
+          } else {
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+              if (c * 32 + i < p.E) dst[i] = __uint_as_float(v[i]);
+          }
+        }
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 2) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(kTmemCols) : "memory");
+  }
+}
+
 // wsplit[part][k][e] for e < Epad64 (zero beyond E): W_r = hi + mid + (a remainder below 2^-18 relative that no
 // product uses: the forward logits and the backward dx both stop at hi + mid).  The layer's first kernel: it also clears
 // the status words (`status` may be null).
@@ -727,22 +639,6 @@ __global__ void split_w_kernel(const float* __restrict__ W_r, int d, int E, int 
   __nv_bfloat16 h, m, l;
   split3(e < E ? W_r[(size_t)k * E + e] : 0.f, &h, &m, &l);
   wsplit[i] = h; wsplit[n + i] = m;
-}
-
-int sm_count_or_default() {
-  int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
-  return n;
-}
-
-template <int OP, bool kJitter = false>
-int launch_op(const CUtensorMap& tmA, const CUtensorMap& tmB, const RouterTcParams& q, cudaStream_t st, int grid) {
-  if (cudaFuncSetAttribute(router_tc_kernel<OP, kJitter>, cudaFuncAttributeMaxDynamicSharedMemorySize, kRTcSmemBytes) !=
-      cudaSuccess)
-    return SWITCH_MOE_CUDA_ERROR;
-  launch_k(router_tc_kernel<OP, kJitter>, dim3(grid), dim3(kRTcThreads), kRTcSmemBytes, st, tmA, tmB, q);
-  return launch_status();
 }
 
 }  // namespace
@@ -791,38 +687,29 @@ int launch_router_tc_bwd(const Shape& s, const Plan& p, const void* x, const flo
     launch_k(split_w_kernel, dim3((unsigned)((nw + 255) / 256)), dim3(256), 0, st, W_r, s.d, s.E, s.Epad64, wsplit,
              static_cast<int*>(nullptr));
   }
-  RouterTcParams q{};
-  q.T = s.T; q.d = s.d; q.E = s.E; q.Epad64 = s.Epad64;
-  q.status = ws_ptr<int>(ws, p.status);
-  CUtensorMap tmA, tmB;
-  // dW_r partials: A = x^T (MN-major view of x [T][d]), B = dh parts [3][T][Epad64] (MN-major)
-  if (make_map(&tmA, x, 1, s.T, s.d, 64) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
-  if (make_map(&tmB, dhsplit, 3, s.T, s.Epad64, 64) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
-  q.mma_n = s.Epad64;
-  q.both_parts = s.Epad64 <= 128 ? 1 : 0;
-  q.n_mtiles = (s.d + kTileM - 1) / kTileM; q.n_ntiles = 1;
-  q.splits = s.dwr_chunks;
-  q.total_kblocks = (s.T + kBK - 1) / kBK;
-  q.chunk_kblocks = (q.total_kblocks + q.splits - 1) / q.splits;
+  RouterBwdParams q{};
+  q.T = s.T; q.d = s.d; q.E = s.E; q.ka = s.Epad64 / 64;
+  q.n_mtiles = (s.T + kTileM - 1) / kTileM; q.n_cols = (s.d + 127) / 128; q.splits = s.dwr_chunks;
+  // 208 KB of operands: W_r parts (32 KB per block of 64 experts), then two x stages if they leave at least four blocks
+  // of the dh ring (up to 128 experts), else one
+  const int left = kRBOperandBytes / kRBBlock - 2 * q.ka;
+  q.x_stages = left - 4 >= 4 ? 2 : 1;
+  q.ring = left - 2 * q.x_stages < kRBMaxRing ? left - 2 * q.x_stages : kRBMaxRing;
   q.partial = ws_ptr<float>(ws, p.dwr_partial);
-  const int sms = sm_count_or_default();
-  int rc = launch_op<kRDwr>(tmA, tmB, q, st, sms);
-  if (rc != SWITCH_MOE_OK) return rc;
-  // dx: A = dh parts (K-major), B = W parts [3][d][Epad64] (K-major: rows are d_model indices)
-  if (make_map(&tmA, dhsplit, 3, s.T, s.Epad64, kTileM) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
-  if (make_map(&tmB, wsplit, 3, s.d, s.Epad64, kBN) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
-  q.mma_n = kBN;
-  q.n_mtiles = (s.T + kTileM - 1) / kTileM; q.n_ntiles = (s.d + kBN - 1) / kBN;
-  q.wrap = s.Epad64 / kBK;
-  q.dx = static_cast<__nv_bfloat16*>(dx); q.slot = ws_ptr<int>(ws, p.slot); q.accumulate = accumulate_dx ? ((s.residual || s.top2) ? 2 : 1) : 0;   // 2: every row already holds a value
+  q.dx = static_cast<__nv_bfloat16*>(dx); q.slot = ws_ptr<int>(ws, p.slot);
+  q.accumulate = accumulate_dx ? ((s.residual || s.top2) ? 2 : 1) : 0;   // 2: every row already holds a value
   q.jitter_u = static_cast<const __nv_bfloat16*>(s.jitter_u);
-  // up to 128 experts the two parts of a 256-row block of W_r (at most 128 KB) stay in shared memory: the CTAs are
-  // dealt out evenly over the row blocks and each walks its share of the token tiles
-  if (s.Epad64 <= 128 && sms >= q.n_ntiles) {
-    const int grid = sms / q.n_ntiles * q.n_ntiles;
-    return s.jitter ? launch_op<kRDxRes, true>(tmA, tmB, q, st, grid) : launch_op<kRDxRes>(tmA, tmB, q, st, grid);
-  }
-  return s.jitter ? launch_op<kRDx, true>(tmA, tmB, q, st, sms) : launch_op<kRDx>(tmA, tmB, q, st, sms);
+  q.status = ws_ptr<int>(ws, p.status);
+  CUtensorMap tmX, tmH, tmW;
+  if (make_map(&tmX, x, 1, s.T, s.d, kTileM) != SWITCH_MOE_OK ||
+      make_map(&tmH, dhsplit, 3, s.T, s.Epad64, kTileM) != SWITCH_MOE_OK ||
+      make_map(&tmW, wsplit, 3, s.d, s.Epad64, kTileM) != SWITCH_MOE_OK)
+    return SWITCH_MOE_CUDA_ERROR;
+  auto kernel = s.jitter ? router_bwd_tc_kernel<true> : router_bwd_tc_kernel<false>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRBSmemBytes) != cudaSuccess)
+    return SWITCH_MOE_CUDA_ERROR;
+  launch_k(kernel, dim3(q.n_cols * q.splits), dim3(kRBThreads), kRBSmemBytes, st, tmX, tmH, tmW, q);
+  return launch_status();
 }
 
 }  // namespace swmoe

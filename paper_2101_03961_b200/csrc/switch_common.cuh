@@ -138,13 +138,10 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
     // (Several routing groups: the plan's kernels count in blocks of 256 tokens.)
     s->router_block_tokens = G == 1 && cfg->T <= 148 * kTileM ? kTileM : 2 * kTileM;
     s->router_blocks = (cfg->T + s->router_block_tokens - 1) / s->router_block_tokens;
-    // dW_r split so that tiles x splits fills the GPU
-    const int m_tiles = (cfg->d_model + kTileM - 1) / kTileM;
-    const int k_blocks = (cfg->T + 63) / 64;
-    int splits = 144 / m_tiles;
-    if (splits < 1) splits = 1;
-    if (splits > 64) splits = 64;
-    if (splits > k_blocks) splits = k_blocks;
+    // backward: blocks of 128 columns of d_model x splits of the token tiles, one CTA per SM
+    const int n_cols = (cfg->d_model + 127) / 128, m_tiles = (cfg->T + kTileM - 1) / kTileM;
+    int splits = n_cols < 148 ? 148 / n_cols : 1;
+    if (splits > m_tiles) splits = m_tiles;
     s->dwr_chunks = splits;
   } else {
     // 64 tokens per forward block where that fills the chip, else 16: the kernel is bound by the latency of its k-chunks
@@ -243,6 +240,13 @@ inline int launch_status() {
   const bool failed = launch_failed_flag();
   launch_failed_flag() = false;
   return (cudaGetLastError() == cudaSuccess && !failed) ? SWITCH_MOE_OK : SWITCH_MOE_CUDA_ERROR;
+}
+
+inline int sm_count_or_default() {
+  int dev = 0, n = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+  return n;
 }
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

@@ -448,6 +448,35 @@ def test_router_backward_given_identical_gate_gradient(cfg, path):
 
 
 # ---------------------------------------------------------------------------------------------- error paths
+@pytest.mark.parametrize("T,d,E", [
+    (1, 64, 1), (127, 192, 33), (300, 320, 65),      # less than a tile; column blocks of 128 with a half empty one
+    (148 * 128 + 5, 64, 128),                        # one column block: as many token splits as SMs, two tiles in some
+    (2000, 640, 192), (700, 128, 256)])              # three and four blocks of 64 experts: one x stage, a short dh ring
+@pytest.mark.parametrize("jitter", [0.0, 0.1])
+def test_router_backward_kernel_at_the_edges_of_its_blocks(T, d, E, jitter):
+    cfg = si.SwitchConfig("router_bwd_edges", T, d, 64, E, max(1.25, 1.01 * E / T))
+    data = si.gen_layer(cfg, seed=9)
+    if jitter:
+        data["router_jitter"] = si.gen_router_jitter(cfg, jitter, 9)
+    g = GpuLayer(cfg, data)
+    g.fwd()
+    gpu_e = g.expert_index()
+    fwd = oracle_following(cfg, data, gpu_e, experts=[])
+    dgate = np.random.default_rng(9).standard_normal(cfg.T).astype(np.float32)
+    dxr = torch.full_like(g.x, float("nan"))
+    sm.switch_moe_router_bwd(g.cfg, g.x, g.W_r, torch.from_numpy(dgate).cuda(), 0.7, g.ws, dxr, g.dW_r)
+    sm.switch_moe_check_device_status(g.cfg, g.ws)
+    xr = np.asarray(data["x"], dtype=np.float64)
+    if jitter:
+        xr = si.storage_round(cfg)(xr * data["router_jitter"])
+    ref = so.router_backward_given_dgate(to_np(g.view(sm.WS_PROBS)).reshape(T, E), gpu_e, fwd["keep"], fwd["count"], dgate,
+                                         xr, data["W_r"], cfg.alpha, d_aux=0.7)
+    assert rel_err(to_np(g.dW_r), ref["dW_r"]) <= TOL_ROUTER
+    want = ref["dx_router"] * data["router_jitter"] if jitter else ref["dx_router"]
+    # one bfloat16 rounding of the result, under jitter one more of the router term (each at most 2^-9 relative)
+    assert rel_err(to_np(dxr), want) <= 4e-3
+
+
 def test_undersized_workspace_and_misaligned_pointers_are_rejected():
     import ctypes
     cfg = sm.make_config(512, 64, 256, 8, 1.0)
