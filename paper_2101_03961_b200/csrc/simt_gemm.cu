@@ -8,9 +8,9 @@
 // per multiply-add and leaves none for the operand loads; the packed form (fma.rn.f32x2, two independent IEEE
 // multiply-adds) halves the slots.  In the large tile a thread keeps 8 x 8 outputs (two groups of 4 rows x two groups of
 // 4 columns), so four 16-byte shared-memory loads feed 64 multiply-adds, and the next k-chunk travels from global memory
-// to registers while the current one is multiplied.  Warps whose rows lie past an expert's last token multiply nothing.
-// Measured at 4096 tokens, 512 x 2048, 16 experts: weight gradients 186 us each (46 TFLOP/s, FMA pipes busy 71% of the
-// time) where 64 x 64 tiles with plain FFMA and no prefetch took 330; GEMM1 215 (377), dgrad2 232 (385).
+// to registers while the current one is multiplied; three blocks of four warps per SM leave it 168 registers.  Warps whose rows lie past an expert's last token multiply nothing.
+// Measured at 4096 tokens, 512 x 2048, 16 experts: weight gradients 168 us each (51 TFLOP/s) where 64 x 64 tiles with plain
+// FFMA and no prefetch took 330; GEMM1 187 (377), dgrad2 214 (385).
 #include "switch_common.cuh"
 
 namespace swmoe {
@@ -66,9 +66,19 @@ struct Tile {
   static constexpr int kMinBlocks = kMinBlocks_;
   static constexpr int RG = BM / WM / 16, CG = BN / WN / 32;
 };
-using BigTile = Tile<128, 128, 16, 4, 2, 2>;
+using BigTile = Tile<64, 128, 16, 2, 2, 3>;
 using MidTile = Tile<64, 64, 32, 2, 2, 4>;
 using SmallTile = Tile<32, 32, 64, 2, 1, 6>;
+
+// A k-contiguous operand is transposed on its way into shared memory: eight lanes write the same rows of eight different
+// steps, rows of R + 4 floats that start in only two banks.  Exchanging groups of four rows by the step spreads them over
+// all banks and keeps 16-byte reads whole.
+// (4096 tokens, 512 x 2048, 16 experts: dgrad1 254 -> 242 us, GEMM2 240 -> 233 with rounds of 32 steps; with rounds of 16,
+// four steps to a row, the extra address arithmetic costs what the conflicts did.)
+template <bool kKFast, int BK>
+__device__ __forceinline__ int swizzle(int k) {
+  return kKFast && BK > 16 ? ((k >> 2) & 7) << 2 : 0;
+}
 
 // One operand tile of R rows (m or n) x BK contraction steps: global -> registers -> shared memory [k][row].
 template <typename ET, int R, int BK, int kThreads, bool kKFast>
@@ -97,7 +107,7 @@ struct Stager {
   __device__ __forceinline__ void put(float (*s)[R + 4]) const {
 #pragma unroll
     for (int i = 0; i < kVecs; ++i) {
-      const int r = row_of(i), k = k_of(i);
+      const int k = k_of(i), r = row_of(i) ^ swizzle<kKFast, BK>(k);
       if (kKFast) {
         s[k][r] = v[i].x; s[k + 1][r] = v[i].y; s[k + 2][r] = v[i].z; s[k + 3][r] = v[i].w;
       } else {
@@ -155,10 +165,10 @@ __global__ void __launch_bounds__(TL::kThreads, TL::kMinBlocks) simt_grouped_gem
         float4 a[RG];
         unsigned long long b[CG * 2];
 #pragma unroll
-        for (int g = 0; g < RG; ++g) a[g] = *reinterpret_cast<const float4*>(&As[buf][kk][row + 16 * g]);
+        for (int g = 0; g < RG; ++g) a[g] = *reinterpret_cast<const float4*>(&As[buf][kk][(row + 16 * g) ^ swizzle<kAKFast, BK>(kk)]);
 #pragma unroll
         for (int g = 0; g < CG; ++g) {
-          const float4 t = *reinterpret_cast<const float4*>(&Bs[buf][kk][col + 32 * g]);
+          const float4 t = *reinterpret_cast<const float4*>(&Bs[buf][kk][(col + 32 * g) ^ swizzle<kBKFast, BK>(kk)]);
           b[2 * g] = pack2(t.x, t.y);
           b[2 * g + 1] = pack2(t.z, t.w);
         }
@@ -228,15 +238,16 @@ void launch_tile(const SimtProblem& pr, int max_m, int E, cudaStream_t st) {
 
 template <typename ET, int OP>
 void launch_op(const SimtProblem& pr, int max_m, int E, cudaStream_t st) {
-  // The largest tile that still occupies the chip: below about 1.5 blocks per SM a launch waits for the few blocks
-  // there are, each walking its whole contraction, and smaller tiles spread the outputs over more SMs.  GEMM2 of 4096
-  // tokens, 512 x 2048, 16 experts (192 large blocks): 371 us with 128 x 128 tiles, 240 with 64 x 64; GEMM1 of the same
-  // layer (768 large blocks): 215 and 229; GEMM2 of 512 tokens, 64 x 256, 8 experts: 27 with 64 x 64 tiles (16 steps per
-  // round), 13 with 32 x 32 (64 steps).
-  constexpr long long kEnough = 222;
-  auto blocks = [&](int b) { return (long long)((pr.N + b - 1) / b) * ((max_m + b - 1) / b) * E; };
-  if (blocks(128) >= kEnough) launch_tile<ET, OP, BigTile>(pr, max_m, E, st);
-  else if (blocks(64) >= kEnough) launch_tile<ET, OP, MidTile>(pr, max_m, E, st);
+  // The largest tile that still occupies the chip: below that a launch waits for the few blocks there are, each walking
+  // its whole contraction, and smaller tiles spread the outputs over more SMs.  64 x 128 tiles (three blocks per SM) want
+  // as many blocks as are resident: at 4096 tokens, 512 x 2048, 16 experts GEMM2's 320 blocks took 299 us, 64 x 64 tiles
+  // 240, while GEMM1 (1280 blocks) takes 187 and 221.  128 x 128 tiles: 371 and 215 (a third of their rows lie past the
+  // experts' last tokens).  GEMM2 of 512 tokens, 64 x 256, 8 experts: 27 us with 64 x 64 tiles and 16 steps per round, 13
+  // with 32 x 32 and 64 steps.
+  constexpr long long kEnoughBig = 444, kEnough = 222;
+  auto blocks = [&](int bm, int bn) { return (long long)((pr.N + bn - 1) / bn) * ((max_m + bm - 1) / bm) * E; };
+  if (blocks(BigTile::BM, BigTile::BN) >= kEnoughBig) launch_tile<ET, OP, BigTile>(pr, max_m, E, st);
+  else if (blocks(MidTile::BM, MidTile::BN) >= kEnough) launch_tile<ET, OP, MidTile>(pr, max_m, E, st);
   else launch_tile<ET, OP, SmallTile>(pr, max_m, E, st);
 }
 
