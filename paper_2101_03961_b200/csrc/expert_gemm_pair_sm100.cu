@@ -26,6 +26,13 @@
 // the middle columns and tells the MMA thread (barrier `tmid`) once the columns the next tile also uses have been
 // read; the next tile's MMAs then start while the rest of the tile is still being drained.
 //
+// Epilogue of the token products.  It has to turn lanes (weight rows) x columns (tokens) into token rows; with few k-blocks
+// per tile (small d_model) it is what a tile waits for, so it is kept to few instructions: the accumulator is read as matrix
+// fragments, scaled, rounded and masked in that order, transposed by stmatrix, and what dgrad2 needs from GEMM1 (ReLU bits,
+// GEGLU factors) is saved in fragment order and never transposed at all.  Against packing token pairs through 32-bit
+// shared-memory words: 65536 tokens, 256 x 512, 128 experts GEMM1 45 -> 35 us, dgrad2 42 -> 38; GEGLU 32768 tokens, 768 x
+// 2048, 128 experts GEMM1 260 -> 232, dgrad2 197 -> 170; 32768 x 768 x 3072 (ReLU) unchanged, HBM bounds it there.
+//
 // Every mbarrier wait is bounded in time (status word + abort flag); both CTAs always reach the final cluster
 // barrier, so tensor memory is freed and no CTA exits while its peer can still address its shared memory.
 #include "tc_common.cuh"
@@ -39,8 +46,7 @@ constexpr int kPMaxStages = 8;                         // token products: as man
 constexpr int kPHalfBytes = 16384;                     // A tile (128 x 64) and B half tile (<= 128 x 64)
 constexpr int kPStageBytes = 2 * kPHalfBytes;
 constexpr int kPRingBytes = kPStages * kPStageBytes;   // 192 KB of operand stages
-constexpr int kPTransWarp = 16 * 144;                  // per epilogue warp: 16 token pairs x (32 weight rows x 4 B, padded
-                                                       // to 144 B so that 16-byte reads of 8 rows do not collide)
+constexpr int kPTransWarp = 32 * 64;                   // per epilogue warp: 32 tokens x 32 weight rows of bfloat16
 constexpr int kPTransBytes = 8 * kPTransWarp;
 constexpr int kPAuxBytes = 8 * 128;                    // 8 epilogue warps x 32 gates
 constexpr int kPKeptCache = kMaxExperts;                 // kept[e] for every expert
@@ -71,18 +77,17 @@ struct PairParams {
   const int* token_of_slot;
   const float* gate;
   __nv_bfloat16* out;
-  uint32_t* hmask;          // [d_ff/32][E*C]: bit i of word [w][row]: H[row][32w + i] > 0 (written by GEMM1, read by
-                            // dgrad2); rows are contiguous so that 32 token rows are one 128-byte store / load
-  long long hmask_rows;     // E*C
+  uint16_t* hmask;          // [block][lane]: [H > 0] of a thread's 16 elements of a block of 16 tokens x 32 hidden units, in
+                            // fragment order (bits 0-7 the even tokens, 8-15 the odd ones); written by GEMM1, read by
+                            // dgrad2; block = (expert * cb + row / 16) * (hid / 32) + unit / 32
+  int cb, hid;              // 16-row blocks per expert, d_ff
   long long ld_out;
   int* status;
   const __nv_bfloat16* res;   // combine / scatter with the skip path inside the layer: rows added to the output (x or dy)
   __nv_bfloat16* out2;        // combine with the skip path: second copy of the output without it
-  int plain;                  // GEMM1 / dgrad2 without ReLU and without the ReLU mask (GEGLU experts)
-  int gate_f;                 // gated products: d_ff.  Gated GEMM1: W_in has 2 d_ff columns [W_0 | W_1]; out = the saved
-                              // factors, one 32-bit word {GELU(a), b GELU'(a)} per hidden unit and slot row; out2 = hidden.
-                              // Gated dgrad2: out = d[a | b] (2 d_ff columns), gate_in = those words.
-  const uint32_t* gate_in;
+  int gate_f;                 // gated products: d_ff.  Gated GEMM1: W_in has 2 d_ff columns [W_0 | W_1], out = hidden.
+                              // Gated dgrad2: out = d[a | b] (2 d_ff columns).
+  uint4* gate_buf;            // what the gated GEMM1 saves: [block][4][lane] of 4 words {GELU(a), b GELU'(a)}, in fragment order
   // expert dropout (Section 2.4) in the epilogues: GEMM1 multiplies the hidden activations by keep / (1 - rate) before
   // it rounds them and takes the mask bits (the gated GEMM1: the hidden activations and both saved factors); dgrad2
   // multiplies by 1 / (1 - rate), its mask bits already say "kept and positive".
@@ -162,6 +167,45 @@ __device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap
       " [%0], [%1, {%3, %4, %5}], [%2];"
       ::"r"(dst), "l"(reinterpret_cast<uint64_t>(tm)), "r"(leader_bar), "r"(c0), "r"(c1), "r"(c2)
       : "memory");
+}
+// 16 lanes x 32 columns of the accumulator as matrix fragments: registers 4 j .. 4 j + 3 of a thread are columns
+// 8 j + 2 (lane % 4), + 1 of TMEM lane lane / 4, then of lane lane / 4 + 8.
+__device__ __forceinline__ void tc_ld_16x256b_x4(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// Waits for this thread's loads; the registers pass through so that no use of them can move ahead of the wait.
+__device__ __forceinline__ void tc_wait_ld_regs(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23]),
+                 "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]), "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+}
+// Four 8 x 8 matrices of bfloat16, transposed: lane l's address is row l % 8 of matrix l / 8.
+__device__ __forceinline__ void stmatrix_trans(uint32_t addr, const uint32_t* w) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]),
+               "r"(w[2]), "r"(w[3])
+               : "memory");
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&h2);
+}
+__device__ __forceinline__ uint32_t relu_bf16x2(uint32_t w) {
+  const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
+  const __nv_bfloat162 r = __hmax2(*reinterpret_cast<const __nv_bfloat162*>(&w), z);
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+// 0xFFFF in each half that is positive.
+__device__ __forceinline__ uint32_t positive_bf16x2(uint32_t w) {
+  return __hgt2_mask(*reinterpret_cast<const __nv_bfloat162*>(&w), __floats2bfloat162_rn(0.f, 0.f));
 }
 __device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
   asm volatile(
@@ -375,96 +419,26 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
     const uint8_t* tr_other = trans_gen + (half * 4 + lg) * kPTransWarp;   // the transpose tile of the warp two lane groups away
     const uint32_t gate_bar = gate0 + 8u * (uint32_t)(half * 2 + (lg & 1));
     uint32_t gate_phase = 0;
+    // Token products.  A chunk of 32 accumulator columns (tokens) x the warp's 32 lanes (weight rows) is read as matrix
+    // fragments: word [4 g + i] of a thread = weight row 8 i + lane / 4 of tokens 8 g + 2 (lane % 4), + 1.  stmatrix with
+    // transposition turns that into token rows of 64 bytes in this warp's tile; a store then writes 16 bytes per lane,
+    // eight tokens at a time.  16-byte pieces are exchanged within a row by the row so that neither side conflicts.
+    const uint32_t st_addr = smem_u32(tr) + (uint32_t)((lane & 7) * 64 + (((lane >> 3) ^ ((lane >> 1) & 3)) << 4));
+    const uint8_t* ld_addr = tr + (lane >> 2) * 64 + (((lane & 3) ^ ((lane >> 3) & 3)) << 4);
     for (int id = pair; id < n_tiles && ok; id += n_pairs, ++it) {
       const PTile t = p_decode(p, id, kept_s, tile_s);
       const uint32_t side = it & 1u, use = it >> 1;
       const int unit0 = (t.m0 >> 1) + 64 * (int)rank + 32 * (lg & 1);        // gated GEMM1: first hidden unit of this warp
       // first M row (weight row = output column) this warp holds
       const int m_warp = kGated ? role * p.gate_f + unit0 : t.m0 + 128 * (int)rank + 32 * lg;
-      const int n_chunks = kTok ? (t.n + 31) >> 5 : 8;
-      const bool have_acc = t.k_blocks > 0;
       const int c0 = side ? kTmemCols - t.n : 0;              // first accumulator column of the tile
-      // Token products.  Chunks of 32 accumulator columns are numbered so that chunk j of an even tile holds the
-      // tile's tokens [32 j, 32 j + 32) and chunk j of an odd tile its tokens [n - 32 (j + 1), n - 32 j): a chunk is
-      // then always inside the 512 columns, and counting j down from the last chunk starts in the middle columns, the
-      // ones the next tile may also use.  Lane i describes token column (chunk's first token) + i: the element offset
-      // of its output row (or -1) and its gate.  This warp's chunks are j = n_chunks - 1 - half, then every second
-      // one down to 0; their descriptions (and ReLU masks) are fetched before the accumulator is awaited.
-      constexpr bool kSlotRows = (OP == kGemm1Relu || kGated || OP == kDgrad2Mask || kDGated);
-      constexpr int kQueue = 5;                                // (320 / 32) chunks over two warps
-      int row_limit = 0;
-      long long q_off[kQueue] = {-1, -1, -1, -1, -1};           // head = next chunk to process
-      float q_gate[kQueue] = {1.f, 1.f, 1.f, 1.f, 1.f};
-      uint32_t q_mw[kQueue] = {0u, 0u, 0u, 0u, 0u};             // dgrad2: ReLU mask bits of weight rows m_warp..+31 per token
-      const int mcol = m_warp + (lane & 3) * 8;               // store `it` writes weight rows mcol .. mcol + 7
-      const bool col_ok = kGated ? unit0 + (lane & 3) * 8 < p.gate_f : mcol < p.Mw;
-      auto chunk_tok0 = [&](int j) { return side ? t.n - 32 * (j + 1) : 32 * j; };
-      auto describe = [&](int j, long long* off, float* g) {
-        const int col = chunk_tok0(j) + lane, slot_row = t.row0 + col;
-        *off = -1;
-        *g = 1.f;
-        if (j >= 0 && col >= 0 && col < t.n && slot_row < row_limit) {
-          if (kSlotRows) {
-            *off = ((long long)t.e * p.C + slot_row) * p.ld_out;
-          } else {
-            const int tok = p.token_of_slot[(long long)t.e * p.C + slot_row];
-            *off = (long long)tok * p.ld_out;
-            if (OP == kGemm2Combine) *g = p.gate[tok];        // Eq. 2: y = p_i(x) E_i(x)
-          }
-        }
-      };
-      int j_mid = 0;                                            // chunks j >= j_mid hold columns the next tile uses too
-      if (kTok) {
-        const int kept_e = kept_s[t.e];
-        row_limit = kSlotRows ? min(p.C, (kept_e + 15) / 16 * 16) : kept_e;
-        const int id_next = id + n_pairs;
-        const int n_next = id_next < n_tiles ? p_decode(p, id_next, kept_s, tile_s).n : 0;
-        j_mid = (t.n - max(0, t.n + n_next - kTmemCols)) >> 5;
-        // everything the epilogue needs from global memory is requested here, before the accumulator is awaited
-#pragma unroll
-        for (int k = 0; k < kQueue; ++k) describe(n_chunks - 1 - half - 2 * k, &q_off[k], &q_gate[k]);
-        if (DROP && (OP == kGemm1Relu || kGated) && (kGated ? unit0 < p.gate_f : m_warp < p.Mw)) {
-          const int unit_word = (kGated ? unit0 : m_warp) >> 5;   // this warp's 32 hidden units are one word per row
-#pragma unroll
-          for (int k = 0; k < kQueue; ++k)
-            if (q_off[k] >= 0)
-              q_mw[k] = p.keep_bits[((long long)t.e * p.C + t.row0 + chunk_tok0(n_chunks - 1 - half - 2 * k) + lane) *
-                                        p.keep_words + unit_word];
-        }
-        if (OP == kDgrad2Mask && !p.plain && m_warp < p.Mw) {
-#pragma unroll
-          for (int k = 0; k < kQueue; ++k)
-            if (q_off[k] >= 0)
-              q_mw[k] = p.hmask[(long long)(m_warp >> 5) * p.hmask_rows + (long long)t.e * p.C + t.row0 +
-                                chunk_tok0(n_chunks - 1 - half - 2 * k) + lane];
-        }
-      }
-      // gated dgrad2: the saved factors of this lane's hidden unit for the 32 tokens of a chunk, one word per token
-      // ({GELU(a), b GELU'(a)} as two bfloat16), fetched one chunk ahead; 0 for columns that hold no token
-      uint32_t gg[kDGated ? 32 : 1];
-      auto fetch_factors = [&](int j, uint32_t* dst) {
-        if constexpr (kDGated) {
-          const int tok_first = chunk_tok0(j);
-          const bool unit_ok = m_warp < p.Mw;
-          const uint32_t* src = p.gate_in + ((long long)t.e * p.C + t.row0 + tok_first) * p.gate_f + m_warp + lane;
-#pragma unroll
-          for (int i = 0; i < 32; ++i) {
-            const int col = tok_first + i;
-            const bool valid = unit_ok && j >= 0 && col >= 0 && col < t.n && t.row0 + col < row_limit;
-            dst[i] = valid ? src[(long long)i * p.gate_f] : 0u;
-          }
-        }
-      };
-      fetch_factors(n_chunks - 1 - half, gg);
-      ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
-      if (!ok) break;
-      tc_fence_after();
       const uint32_t t_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0;
       if constexpr (!kTok) {
-        // Weight gradients (row = weight row): 64 output columns at a time, so that a row is a whole 128-byte line.
-        // The warp's 2 KB of shared memory hold 16 rows x 128 bytes: rows 0-15 and 16-31 of the warp take turns, and
-        // every store instruction then writes 4 complete lines (the store path's cost grows with the number of lines
-        // an instruction touches).
+        // ---- weight gradient: rows of the output are this warp's lanes
+        const bool have_acc = t.k_blocks > 0;
+        ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
+        if (!ok) break;
+        tc_fence_after();
 #pragma unroll 1
         for (int c = half; c < 4; c += 2) {
           uint32_t v[64];
@@ -514,20 +488,95 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
             __syncwarp();
           }
         }
-        continue;
       } else {
-        bool released = false, mid_sent = false;
-#pragma unroll 1
-        for (int j = n_chunks - 1 - half; j >= 0; j -= 2) {
-          const int tok0 = chunk_tok0(j);                       // token column of lane 0 (-16 in an odd tile's last chunk)
-          uint32_t v[32];
-          if (have_acc) {
-            tc_ld32(t_addr + (uint32_t)(tok0 + 0), v);
-            tc_wait_ld();
-          } else {
+        // Chunks are numbered so that chunk j of an even tile holds the tile's tokens [32 j, 32 j + 32) and chunk j of an
+        // odd tile its tokens [n - 32 (j + 1), n - 32 j): a chunk is then always inside the 512 columns, and counting j
+        // down from the last chunk starts in the middle columns, the ones the next tile may also use.  This warp's chunks
+        // are j = n_chunks - 1 - half, then every second one down to 0.
+        constexpr bool kSlotRows = (OP == kGemm1Relu || kGated || OP == kDgrad2Mask || kDGated);
+        constexpr int kQueue = 5;                              // (320 / 32) chunks over two warps
+        const int n_chunks = (t.n + 31) >> 5;
+        const bool m_ok = kGated ? unit0 < p.gate_f : m_warp < p.Mw;   // (weight rows come in multiples of 64)
+        const int kept_e = kept_s[t.e];
+        const int row_limit = kSlotRows ? min(p.C, (kept_e + 15) / 16 * 16) : kept_e;
+        const int id_next = id + n_pairs;
+        const int n_next = id_next < n_tiles ? p_decode(p, id_next, kept_s, tile_s).n : 0;
+        const int j_mid = (t.n - max(0, t.n + n_next - kTmemCols)) >> 5;   // chunks j >= j_mid: columns the next tile uses too
+        __nv_bfloat16* out_rows = p.out + ((long long)t.e * p.C + t.row0) * p.ld_out;   // slot-row products: the tile's first row
+        auto chunk_tok0 = [&](int j) { return side ? t.n - 32 * (j + 1) : 32 * j; };
+        auto row_ok = [&](int col) { return col >= 0 && col < t.n && t.row0 + col < row_limit; };
+        // 16-token blocks of 32 hidden units: what GEMM1 saves for dgrad2 is kept per block in fragment order.  block0 is the
+        // block of the tile's first token; 16 tokens further is hid / 32 blocks further.
+        const int words = p.hid >> 5;
+        const long long block0 = ((long long)t.e * p.cb + (t.row0 >> 4)) * words + ((kGated ? unit0 : m_warp) >> 5);
+        auto block_ok = [&](int col) { return m_ok && col >= 0 && col < t.n; };
+        // Everything the epilogue needs from global memory is requested here, before the accumulator is awaited; head of a
+        // queue = next chunk to process.  Lane i of a chunk describes its token column i: the token (scatter products), its
+        // gate, its dropout word.  dgrad2: ReLU mask bits of this thread's fragment, two blocks of 16 tokens.
+        int q_tok[kQueue] = {-1, -1, -1, -1, -1};
+        float q_gate[kQueue] = {1.f, 1.f, 1.f, 1.f, 1.f};
+        uint32_t q_mw[kQueue] = {0u, 0u, 0u, 0u, 0u};
+        if constexpr (!kSlotRows) {
+          const int* tos = p.token_of_slot + (long long)t.e * p.C + t.row0;
 #pragma unroll
-            for (int i = 0; i < 32; ++i) v[i] = 0u;
+          for (int k = 0; k < kQueue; ++k) {
+            const int j = n_chunks - 1 - half - 2 * k, col = chunk_tok0(j) + lane;
+            q_tok[k] = j >= 0 && row_ok(col) ? tos[col] : -1;
           }
+          if (OP == kGemm2Combine) {                            // Eq. 2: y = p_i(x) E_i(x)
+#pragma unroll
+            for (int k = 0; k < kQueue; ++k) q_gate[k] = p.gate[max(q_tok[k], 0)];
+          }
+        }
+        if constexpr (DROP && (OP == kGemm1Relu || kGated)) {   // 32 hidden units are one word per row
+          const uint32_t* keep = p.keep_bits + ((long long)t.e * p.C + t.row0) * p.keep_words + ((kGated ? unit0 : m_warp) >> 5);
+#pragma unroll
+          for (int k = 0; k < kQueue; ++k) {
+            const int j = n_chunks - 1 - half - 2 * k, col = chunk_tok0(j) + lane;
+            q_mw[k] = j >= 0 && m_ok && row_ok(col) ? keep[(long long)col * p.keep_words] : 0u;
+          }
+        }
+        if constexpr (OP == kDgrad2Mask) {
+          const uint16_t* hm = p.hmask + block0 * 32 + lane;
+#pragma unroll
+          for (int k = 0; k < kQueue; ++k) {
+            const int j = n_chunks - 1 - half - 2 * k, tok0 = chunk_tok0(j);
+            const uint32_t b0 = j >= 0 && block_ok(tok0) ? hm[(long long)(tok0 >> 4) * p.hid] : 0u;
+            const uint32_t b1 = j >= 0 && block_ok(tok0 + 16) ? hm[(long long)((tok0 >> 4) + 1) * p.hid] : 0u;
+            q_mw[k] = b0 | (b1 << 16);
+          }
+        }
+        // gated dgrad2: the saved factors of this thread's fragment ({GELU(a), b GELU'(a)} as two bfloat16 per element)
+        uint4 gg[kDGated ? 8 : 1];
+        auto fetch_factors = [&](int j) {
+          if constexpr (kDGated) {
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+              const int col = chunk_tok0(j) + 16 * b;
+              const bool valid = j >= 0 && block_ok(col);
+              const uint4* src = p.gate_buf + (valid ? (block0 + (long long)(col >> 4) * words) * 128 + lane : 0);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) gg[4 * b + q] = valid ? src[32 * q] : make_uint4(0, 0, 0, 0);
+            }
+          }
+        };
+        fetch_factors(n_chunks - 1 - half);
+        ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
+        if (!ok) break;
+        tc_fence_after();
+        bool released = false, mid_sent = false;
+        uint32_t v[32];                                         // [16 h + 4 g + ..]: weight rows 16 h .., tokens 8 g ..
+        auto load_acc = [&](int j) {
+          const uint32_t at = t_addr + (uint32_t)chunk_tok0(j);  // (-16 in an odd tile's last chunk: the columns before it)
+          tc_ld_16x256b_x4(at, v);
+          tc_ld_16x256b_x4(at + (16u << 16), v + 16);
+        };
+        auto value = [&](int g, int i, int b) { return __uint_as_float(v[16 * (i >> 1) + 4 * g + 2 * (i & 1) + b]); };
+        if (m_ok && n_chunks - 1 - half >= 0) load_acc(n_chunks - 1 - half);
+#pragma unroll 1
+        for (int j = n_chunks - 1 - half; j >= 0 && m_ok; j -= 2) {
+          const int tok0 = chunk_tok0(j);
+          tc_wait_ld_regs(v);
           if (!mid_sent && j - 2 < j_mid) {                     // this warp's share of the middle columns is read out
             tc_fence_before();
             __syncwarp();
@@ -540,203 +589,164 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
             if (lane == 0) mbar_arrive_remote(tempty0 + 8u * side, 0);
             released = true;
           }
-          uint32_t gn[kDGated ? 32 : 1];                        // gated dgrad2: the next chunk's factors, in flight meanwhile
-          fetch_factors(j - 2, gn);
-          {
-            // Store `st` of this lane writes weight rows mcol .. mcol + 7 of token column tcol(st) of the chunk:
-            // eight lanes' token pairs x four row groups per instruction.
-            auto tcol = [&](int st) { return 16 * (st >> 1) + 2 * (lane >> 2) + (st & 1); };
-            uint32_t mword[4] = {0u, 0u, 0u, 0u};
-            if constexpr (kGated) {
-              // GEGLU gating.  Both warps of a pair round their values (a or b of 32 hidden units x 32 tokens) into
-              // their transpose tiles; between two handshakes the a warp takes b of the chunk's tokens 0-15 from the
-              // other tile and the b warp a of tokens 16-31.  Each then has a and b of one hidden unit per lane for 16
-              // tokens and forms GELU(a), b GELU'(a) (saved for the backward pass as one word per unit and row) and the
-              // hidden activation GELU(a) b, and transposes both through its own tile.
-              uint32_t pk[16];
+          if constexpr (kGated) {
+            // GEGLU gating.  Both warps of a pair round their values (a or b of 32 hidden units x 32 tokens); the a warp
+            // gates the chunk's first 16 tokens, the b warp the others: each hands the other its half through its tile,
+            // between two handshakes.
+            uint32_t mine[8];
 #pragma unroll
-              for (int k = 0; k < 16; ++k) {
-                const __nv_bfloat162 t2 = __floats2bfloat162_rn(__uint_as_float(v[2 * k]), __uint_as_float(v[2 * k + 1]));
-                pk[k] = *reinterpret_cast<const uint32_t*>(&t2);
-                *reinterpret_cast<uint32_t*>(tr + k * 144 + lane * 4) = pk[k];
-              }
-              __syncwarp();
-              if (lane == 0) mbar_arrive(gate_bar);
-              ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 26);     // both tiles are written
-              gate_phase ^= 1u;
-              if (!ok) break;
-              uint32_t other[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k)
-                other[k] = *reinterpret_cast<const uint32_t*>(tr_other + (8 * role + k) * 144 + lane * 4);
-              __syncwarp();
-              if (lane == 0) mbar_arrive(gate_bar);
-              ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 27);     // both tiles have been read
-              gate_phase ^= 1u;
-              if (!ok) break;
-              uint32_t hw[8];
-#pragma unroll
-              for (int k = 0; k < 8; ++k) {                     // this warp's token pair k: tokens 16 role + 2 k, + 1
-                const uint32_t mine = role ? pk[8 + k] : pk[k];
-                const uint32_t aw = role ? other[k] : mine, bw = role ? mine : other[k];
-                const float2 af = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw));
-                const float2 bf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw));
-                float cdf0, pdf0, cdf1, pdf1;
-                gelu_cdf_pdf(af.x, &cdf0, &pdf0);
-                gelu_cdf_pdf(af.y, &cdf1, &pdf1);
-                float ga0 = af.x * cdf0, ga1 = af.y * cdf1;
-                float gp0 = bf.x * fmaf(af.x, pdf0, cdf0), gp1 = bf.y * fmaf(af.y, pdf1, cdf1);
-                if (DROP) {                                     // expert dropout: the hidden unit's factor on all three
-                  const uint32_t kw0 = __shfl_sync(0xffffffffu, q_mw[0], 16 * role + 2 * k);
-                  const uint32_t kw1 = __shfl_sync(0xffffffffu, q_mw[0], 16 * role + 2 * k + 1);
-                  const float f0 = (kw0 >> lane) & 1u ? p.keep_scale : 0.f, f1 = (kw1 >> lane) & 1u ? p.keep_scale : 0.f;
-                  ga0 *= f0; gp0 *= f0; ga1 *= f1; gp1 *= f1;
-                }
-                const __nv_bfloat162 s0 = __floats2bfloat162_rn(ga0, gp0);
-                const __nv_bfloat162 s1 = __floats2bfloat162_rn(ga1, gp1);
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(ga0 * bf.x, ga1 * bf.y);
-                hw[k] = *reinterpret_cast<const uint32_t*>(&h2);
-                // saved factors: tile row = token of this warp (0..15), one word per lane
-                *reinterpret_cast<uint32_t*>(tr + (2 * k) * 144 + lane * 4) = *reinterpret_cast<const uint32_t*>(&s0);
-                *reinterpret_cast<uint32_t*>(tr + (2 * k + 1) * 144 + lane * 4) = *reinterpret_cast<const uint32_t*>(&s1);
-              }
-              __syncwarp();
-              const bool warp_ok = unit0 < p.gate_f;
-#pragma unroll
-              for (int pass = 0; pass < 4; ++pass) {            // a store writes 4 tokens x 32 hidden units x 4 bytes
-                const int trow = 4 * pass + (lane >> 3);
-                const uint4 val = *reinterpret_cast<const uint4*>(tr + trow * 144 + (lane & 7) * 16);
-                const long long off = __shfl_sync(0xffffffffu, q_off[0], 16 * role + trow);
-                // the saved row has one word (two bfloat16) per hidden unit: d_ff words = the 2 d_ff elements of q_off's row
-                if (off >= 0 && warp_ok)
-                  *reinterpret_cast<uint4*>(p.out + off + 2 * (unit0 + (lane & 7) * 4)) = val;
-              }
-              __syncwarp();
-#pragma unroll
-              for (int k = 0; k < 8; ++k) *reinterpret_cast<uint32_t*>(tr + k * 144 + lane * 4) = hw[k];
-              __syncwarp();
-              const uint8_t* src = tr + (lane >> 2) * 144 + (lane & 3) * 32;
-              const uint4 lo = *reinterpret_cast<const uint4*>(src);
-              const uint4 hi = *reinterpret_cast<const uint4*>(src + 16);
-#pragma unroll
-              for (int tb = 0; tb < 2; ++tb) {
-                const uint32_t sel = tb ? 0x7632u : 0x5410u;
-                const uint4 val = make_uint4(__byte_perm(lo.x, lo.y, sel), __byte_perm(lo.z, lo.w, sel),
-                                             __byte_perm(hi.x, hi.y, sel), __byte_perm(hi.z, hi.w, sel));
-                const long long off = __shfl_sync(0xffffffffu, q_off[0], 16 * role + 2 * (lane >> 2) + tb);
-                // the saved row has 2 d_ff elements, the hidden row d_ff: half the element offset
-                if (off >= 0 && col_ok) *reinterpret_cast<uint4*>(p.out2 + (off >> 1) + unit0 + (lane & 3) * 8) = val;
-              }
-            } else {
-            long long offs[4];
-#pragma unroll
-            for (int st = 0; st < 4; ++st) offs[st] = __shfl_sync(0xffffffffu, q_off[0], tcol(st));
-            if (OP == kGemm2Combine) gate_s[lane] = q_gate[0];
-            __syncwarp();
-            // gated dgrad2 writes two sets of columns from one accumulator: d a = dH . (b GELU'(a)) at column j, then
-            // d b = dH . GELU(a) at column d_ff + j
-#pragma unroll
-            for (int rnd = 0; rnd < (kDGated ? 2 : 1); ++rnd) {
-            if (rnd > 0) __syncwarp();                          // the tile's readers of the first set are done
-            const int mcol_r = mcol + rnd * p.gate_f;
-            // transpose: this lane holds weight row m_warp + lane for 32 tokens.  Two tokens are packed into one
-            // 32-bit word, tr[token pair][lane]: half the shared-memory stores of a 16-bit layout, each a full
-            // 128-byte wavefront; a reader takes the words of eight rows (32 bytes) and separates the two tokens.
-#pragma unroll
-            for (int i4 = 0; i4 < 32; i4 += 4) {
-              float g[4] = {1.f, 1.f, 1.f, 1.f};
-              if (OP == kGemm2Combine) {
-                const float4 g4 = *reinterpret_cast<const float4*>(gate_s + i4);
-                g[0] = g4.x; g[1] = g4.y; g[2] = g4.z; g[3] = g4.w;
-              }
-              float a[4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {
-                a[u] = __uint_as_float(v[i4 + u]);
-                if (OP == kGemm2Combine) a[u] *= g[u];
-                if (OP == kGemm1Relu && !p.plain) a[u] = fmaxf(a[u], 0.f);
-                if (DROP && OP == kGemm1Relu) {                 // expert dropout before the rounding and the mask bits
-                  const uint32_t kw = __shfl_sync(0xffffffffu, q_mw[0], i4 + u);
-                  a[u] = (kw >> lane) & 1u ? a[u] * p.keep_scale : 0.f;
-                }
-                if (DROP && OP == kDgrad2Mask) a[u] *= p.keep_scale;
-                if (kDGated)                                    // high half: b GELU'(a); low half: GELU(a)
-                  a[u] *= __uint_as_float(rnd == 0 ? (gg[kDGated ? i4 + u : 0] & 0xFFFF0000u) : (gg[kDGated ? i4 + u : 0] << 16));
-              }
-              *reinterpret_cast<__nv_bfloat162*>(tr + (i4 >> 1) * 144 + lane * 4) = __floats2bfloat162_rn(a[0], a[1]);
-              *reinterpret_cast<__nv_bfloat162*>(tr + ((i4 >> 1) + 1) * 144 + lane * 4) = __floats2bfloat162_rn(a[2], a[3]);
+            for (int k = 0; k < 8; ++k) {                       // word 4 g + i of this warp's block, and of the other's
+              const int g = k >> 2, i = k & 3;
+              const uint32_t w0 = pack_bf16(value(g, i, 0), value(g, i, 1)), w1 = pack_bf16(value(g + 2, i, 0), value(g + 2, i, 1));
+              mine[k] = role ? w1 : w0;
+              *reinterpret_cast<uint32_t*>(tr + k * 128 + lane * 4) = role ? w0 : w1;
             }
+            if (j - 2 >= 0) load_acc(j - 2);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(gate_bar);
+            ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 26);     // both tiles are written
+            gate_phase ^= 1u;
+            if (!ok) break;
+            uint32_t other[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) other[k] = *reinterpret_cast<const uint32_t*>(tr_other + k * 128 + lane * 4);
+            __syncwarp();
+            if (lane == 0) mbar_arrive(gate_bar);
+            ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 27);     // both tiles have been read
+            gate_phase ^= 1u;
+            if (!ok) break;
+            const int col0 = tok0 + 16 * role;                  // this warp's block of 16 tokens
+            uint32_t fac[16], hw[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const int g = k >> 2, i = k & 3;
+              const uint32_t aw = role ? other[k] : mine[k], bw = role ? mine[k] : other[k];
+              const float2 af = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw));
+              const float2 bf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw));
+              float cdf0, pdf0, cdf1, pdf1;
+              gelu_cdf_pdf(af.x, &cdf0, &pdf0);
+              gelu_cdf_pdf(af.y, &cdf1, &pdf1);
+              float ga0 = af.x * cdf0, ga1 = af.y * cdf1;
+              float gp0 = bf.x * fmaf(af.x, pdf0, cdf0), gp1 = bf.y * fmaf(af.y, pdf1, cdf1);
+              if (DROP) {                                       // expert dropout: the hidden unit's factor on all three
+                const int tk = 16 * role + 8 * g + 2 * (lane & 3), unit = 8 * i + (lane >> 2);
+                const uint32_t kw0 = __shfl_sync(0xffffffffu, q_mw[0], tk), kw1 = __shfl_sync(0xffffffffu, q_mw[0], tk + 1);
+                const float f0 = (kw0 >> unit) & 1u ? p.keep_scale : 0.f, f1 = (kw1 >> unit) & 1u ? p.keep_scale : 0.f;
+                ga0 *= f0; gp0 *= f0; ga1 *= f1; gp1 *= f1;
+              }
+              fac[2 * k] = pack_bf16(ga0, gp0);
+              fac[2 * k + 1] = pack_bf16(ga1, gp1);
+              hw[k] = pack_bf16(ga0 * bf.x, ga1 * bf.y);
+            }
+            if (block_ok(col0)) {
+              uint4* dst = p.gate_buf + (block0 + (long long)(col0 >> 4) * words) * 128 + lane;
+#pragma unroll
+              for (int q = 0; q < 4; ++q) dst[32 * q] = make_uint4(fac[4 * q], fac[4 * q + 1], fac[4 * q + 2], fac[4 * q + 3]);
+            }
+#pragma unroll
+            for (int g = 0; g < 2; ++g) stmatrix_trans(st_addr + 512u * g, hw + 4 * g);
             __syncwarp();
 #pragma unroll
-            for (int pass = 0; pass < 2; ++pass) {
-              const uint8_t* src = tr + (8 * pass + (lane >> 2)) * 144 + (lane & 3) * 32;
-              const uint4 lo = *reinterpret_cast<const uint4*>(src);           // rows 8 g .. 8 g + 3, both tokens
-              const uint4 hi = *reinterpret_cast<const uint4*>(src + 16);      // rows 8 g + 4 .. 8 g + 7
+            for (int g = 0; g < 2; ++g) {
+              const uint4 val = *reinterpret_cast<const uint4*>(ld_addr + 512 * g);
+              const int col = col0 + 8 * g + (lane >> 2);
+              if (row_ok(col)) *reinterpret_cast<uint4*>(out_rows + (long long)col * p.ld_out + unit0 + (lane & 3) * 8) = val;
+            }
+          } else {
+            constexpr int kSets = kDGated ? 2 : 1;              // gated dgrad2 writes d a and d b from one accumulator
+            uint32_t pk[kSets][16];
+            // dgrad2: a block's bits with the even tokens' in the low half, the odd ones' in the high half
+            const uint32_t mask[2] = {__byte_perm(q_mw[0], 0, 0x4140), __byte_perm(q_mw[0], 0, 0x4342)};
+            if (OP == kGemm2Combine) { gate_s[lane] = q_gate[0]; __syncwarp(); }
 #pragma unroll
-              for (int tb = 0; tb < 2; ++tb) {
-                const int st = 2 * pass + tb;
-                const uint32_t sel = tb ? 0x7632u : 0x5410u;                   // high halves: the pair's second token
-                uint4 val = make_uint4(__byte_perm(lo.x, lo.y, sel), __byte_perm(lo.z, lo.w, sel),
-                                       __byte_perm(hi.x, hi.y, sel), __byte_perm(hi.z, hi.w, sel));
-                if (OP == kDgrad2Mask && !p.plain) {            // ReLU'(u) = [u > 0]: bits saved by the forward GEMM
-                  const uint32_t bits = __shfl_sync(0xffffffffu, q_mw[0], tcol(st)) >> ((lane & 3) * 8);
-                  uint32_t* w = reinterpret_cast<uint32_t*>(&val);
+            for (int g = 0; g < 4; ++g) {
+              float2 ga = make_float2(1.f, 1.f);
+              if (OP == kGemm2Combine) ga = *reinterpret_cast<const float2*>(gate_s + 8 * g + 2 * (lane & 3));
+              uint32_t kw0 = 0u, kw1 = 0u;
+              if (DROP && OP == kGemm1Relu) {                   // expert dropout before the rounding and the mask bits
+                kw0 = __shfl_sync(0xffffffffu, q_mw[0], 8 * g + 2 * (lane & 3));
+                kw1 = __shfl_sync(0xffffffffu, q_mw[0], 8 * g + 2 * (lane & 3) + 1);
+              }
 #pragma unroll
-                  for (int q = 0; q < 4; ++q)
-                    w[q] &= ((bits >> (2 * q)) & 1u ? 0x0000FFFFu : 0u) | ((bits >> (2 * q + 1)) & 1u ? 0xFFFF0000u : 0u);
+              for (int i = 0; i < 4; ++i) {
+                float x = value(g, i, 0), y = value(g, i, 1);
+                if (OP == kGemm2Combine) { x *= ga.x; y *= ga.y; }
+                if (DROP && OP == kGemm1Relu) {
+                  const int unit = 8 * i + (lane >> 2);
+                  x = (kw0 >> unit) & 1u ? x * p.keep_scale : 0.f;
+                  y = (kw1 >> unit) & 1u ? y * p.keep_scale : 0.f;
                 }
-                if (OP == kGemm1Relu && !p.plain) {             // save [H > 0] as one bit per element for the backward pass
-                  const uint32_t* w = reinterpret_cast<const uint32_t*>(&val);
-                  uint32_t m8 = 0;
-#pragma unroll
-                  for (int q = 0; q < 4; ++q)
-                    m8 |= ((w[q] & 0x00007FFFu) ? 1u << (2 * q) : 0u) | ((w[q] & 0x7FFF0000u) ? 1u << (2 * q + 1) : 0u);
-                  uint32_t word = m8 << ((lane & 3) * 8);
-                  word |= __shfl_xor_sync(0xffffffffu, word, 1);
-                  word |= __shfl_xor_sync(0xffffffffu, word, 2);
-                  mword[st] = word;                             // the word of token tcol(st), in all four lanes of its group
+                if (DROP && OP == kDgrad2Mask) { x *= p.keep_scale; y *= p.keep_scale; }
+                if constexpr (kDGated) {                        // high half: b GELU'(a); low half: GELU(a)
+                  const uint4 f4 = gg[4 * (g >> 1) + 2 * (g & 1) + (i >> 1)];
+                  const uint32_t f0 = i & 1 ? f4.z : f4.x, f1 = i & 1 ? f4.w : f4.y;
+                  pk[0][4 * g + i] = pack_bf16(x * __uint_as_float(f0 & 0xFFFF0000u), y * __uint_as_float(f1 & 0xFFFF0000u));
+                  pk[kSets - 1][4 * g + i] = pack_bf16(x * __uint_as_float(f0 << 16), y * __uint_as_float(f1 << 16));
+                } else {
+                  uint32_t w = pack_bf16(x, y);
+                  if (OP == kGemm1Relu) w = relu_bf16x2(w);
+                  if (OP == kDgrad2Mask)                        // ReLU'(u) = [u > 0]: bits saved by the forward GEMM
+                    w &= ((mask[g >> 1] >> (4 * (g & 1) + i)) & 0x00010001u) * 0xFFFFu;
+                  pk[0][4 * g + i] = w;
                 }
-                if ((OP == kGemm2Combine || OP == kDgrad1Scatter) && p.res != nullptr && offs[st] >= 0 && col_ok) {
-                  // skip path inside the layer: y = x + g E(x), dx = dy + dH W_in^T (the expert term is already bf16)
-                  if (OP == kGemm2Combine) *reinterpret_cast<uint4*>(p.out2 + offs[st] + mcol) = val;
-                  const uint4 r = *reinterpret_cast<const uint4*>(p.res + offs[st] + mcol);
-                  const __nv_bfloat162* rv = reinterpret_cast<const __nv_bfloat162*>(&r);
-                  __nv_bfloat162* vv = reinterpret_cast<__nv_bfloat162*>(&val);
+              }
+            }
+            if (j - 2 >= 0) load_acc(j - 2);                    // in flight while this chunk is stored
+            fetch_factors(j - 2);
+            if (OP == kGemm1Relu) {                             // save [H > 0], one bit per element, in fragment order
 #pragma unroll
-                  for (int q = 0; q < 4; ++q) {
-                    const float2 a2 = __bfloat1622float2(vv[q]), b2 = __bfloat1622float2(rv[q]);
-                    vv[q] = __floats2bfloat162_rn(a2.x + b2.x, a2.y + b2.y);
+              for (int b = 0; b < 2; ++b) {
+                uint32_t bits = 0;
+#pragma unroll
+                for (int k = 0; k < 8; ++k) bits |= positive_bf16x2(pk[0][8 * b + k]) & (0x00010001u << k);
+                if (block_ok(tok0 + 16 * b))
+                  p.hmask[block0 * 32 + (long long)((tok0 >> 4) + b) * p.hid + lane] = (uint16_t)((bits & 0xFFu) | (bits >> 8));
+              }
+            }
+#pragma unroll
+            for (int set = 0; set < kSets; ++set) {
+              if (set > 0) __syncwarp();                        // the tile's readers of the first set are done
+#pragma unroll
+              for (int g = 0; g < 4; ++g) stmatrix_trans(st_addr + 512u * g, pk[set] + 4 * g);
+              __syncwarp();
+              const int mcol = m_warp + (lane & 3) * 8 + set * p.gate_f;
+#pragma unroll
+              for (int g = 0; g < 4; ++g) {
+                uint4 val = *reinterpret_cast<const uint4*>(ld_addr + 512 * g);
+                if (kSlotRows) {
+                  const int col = tok0 + 8 * g + (lane >> 2);
+                  if (row_ok(col)) *reinterpret_cast<uint4*>(out_rows + (long long)col * p.ld_out + mcol) = val;
+                } else {
+                  const int tok = __shfl_sync(0xffffffffu, q_tok[0], 8 * g + (lane >> 2));
+                  if (tok >= 0) {
+                    const long long off = (long long)tok * p.ld_out + mcol;
+                    if (p.res != nullptr) {
+                      // skip path inside the layer: y = x + g E(x), dx = dy + dH W_in^T (the expert term is already bf16)
+                      if (OP == kGemm2Combine) *reinterpret_cast<uint4*>(p.out2 + off) = val;
+                      const uint4 r = *reinterpret_cast<const uint4*>(p.res + off);
+                      const __nv_bfloat162* rv = reinterpret_cast<const __nv_bfloat162*>(&r);
+                      __nv_bfloat162* vv = reinterpret_cast<__nv_bfloat162*>(&val);
+#pragma unroll
+                      for (int q = 0; q < 4; ++q) {
+                        const float2 a2 = __bfloat1622float2(vv[q]), b2 = __bfloat1622float2(rv[q]);
+                        vv[q] = __floats2bfloat162_rn(a2.x + b2.x, a2.y + b2.y);
+                      }
+                    }
+                    *reinterpret_cast<uint4*>(p.out + off) = val;
                   }
                 }
-                if (offs[st] >= 0 && col_ok) *reinterpret_cast<uint4*>(p.out + offs[st] + mcol_r) = val;
               }
             }
-            }
-            }
-            if constexpr (kDGated) {
-#pragma unroll
-              for (int i = 0; i < 32; ++i) gg[i] = gn[i];
-            }
-            if (OP == kGemm1Relu && !p.plain) {                 // lane i stores the mask word of token row i: one 128-byte line
-              // token `lane` was handled as st = 2 (lane / 16) + (lane & 1) by the four lanes 4 ((lane / 2) & 7) ..
-              uint32_t mine = 0;
-#pragma unroll
-              for (int st = 0; st < 4; ++st) {
-                const uint32_t w = __shfl_sync(0xffffffffu, mword[st], 4 * ((lane >> 1) & 7));
-                if (2 * (lane >> 4) + (lane & 1) == st) mine = w;
-              }
-              if (q_off[0] >= 0 && m_warp < p.Mw)
-                p.hmask[(long long)(m_warp >> 5) * p.hmask_rows + (long long)t.e * p.C + t.row0 + tok0 + lane] = mine;
-            }
-#pragma unroll
-            for (int k = 0; k < kQueue - 1; ++k) {              // advance the queue
-              q_off[k] = q_off[k + 1];
-              q_gate[k] = q_gate[k + 1];
-              q_mw[k] = q_mw[k + 1];
-            }
-            __syncwarp();
           }
+#pragma unroll
+          for (int k = 0; k < kQueue - 1; ++k) {                // advance the queue
+            q_tok[k] = q_tok[k + 1];
+            q_gate[k] = q_gate[k + 1];
+            q_mw[k] = q_mw[k + 1];
+          }
+          __syncwarp();
         }
+        if (!ok) break;
         if (!mid_sent) {                                        // this warp had no chunk in this tile
           tc_fence_before();
           __syncwarp();
@@ -845,8 +855,8 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
   q.token_of_slot = ws_ptr<int>(ws, p.token_of_slot);
   q.gate = ws_ptr<float>(ws, p.gate);
   q.status = ws_ptr<int>(ws, p.status);
-  q.hmask = ws_ptr<uint32_t>(ws, p.hmask);
-  q.hmask_rows = (long long)s.E * s.C;
+  q.hmask = ws_ptr<uint16_t>(ws, p.hmask);
+  q.cb = (s.C + 15) / 16; q.hid = s.f;
   q.keep_scale = 1.f;
   CUtensorMap& tmA = *tmA_out;
   BMapSet& bm = *tmB_out;
@@ -857,9 +867,8 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
     case kGemm1Relu:       // A = W_in [E][d (k)][f (m)]: m contiguous -> MN-major; B = X_d [E][C][d] K-major
       q.token_op = 1; q.a_mn_major = 1; q.Mw = fin; K = s.d;   // GEGLU: 2 f weight columns [W_0 | W_1], no ReLU
       rc = make_map(&tmA, a.W_in, s.E, s.d, fin, 64); rc2 = make_token_maps(&bm, xd, s.E, s.C, s.d);
-      q.out = s.geglu ? ws_ptr<__nv_bfloat16>(ws, p.ab) : ws_ptr<__nv_bfloat16>(ws, p.h); q.ld_out = fin;
-      q.plain = s.geglu;
-      if (s.geglu) { q.gate_f = s.f; q.out2 = ws_ptr<__nv_bfloat16>(ws, p.h); }   // gating in the epilogue
+      q.out = ws_ptr<__nv_bfloat16>(ws, p.h); q.ld_out = s.f;
+      if (s.geglu) { q.gate_f = s.f; q.gate_buf = ws_ptr<uint4>(ws, p.ab); }   // gating in the epilogue
       if (s.dropout) {
         if (s.keep_bits == nullptr || (reinterpret_cast<uintptr_t>(s.keep_bits) & 3u) != 0) return SWITCH_MOE_INVALID_ARGUMENT;
         q.keep_bits = s.keep_bits; q.keep_words = s.f / 32; q.keep_scale = s.keep_scale;
@@ -876,11 +885,11 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
     case kDgrad2Mask:      // A = W_out [E][f (m)][d (k)] K-major; B = dY_d [E][C][d] K-major
       q.token_op = 1; q.a_mn_major = 0; q.Mw = s.f; K = s.d;
       rc = make_map(&tmA, a.W_out, s.E, s.f, s.d, 128); rc2 = make_token_maps(&bm, dyd, s.E, s.C, s.d);
-      q.out = ws_ptr<__nv_bfloat16>(ws, p.dh); q.ld_out = s.f; q.plain = s.geglu;
+      q.out = ws_ptr<__nv_bfloat16>(ws, p.dh); q.ld_out = s.f;
       if (s.dropout && !s.geglu) q.keep_scale = s.keep_scale;   // (GEGLU: the saved factors carry the dropout factor)
       if (s.geglu) {   // the derivative of the gating in the epilogue: d[a | b] is written, dH never is
         q.out = ws_ptr<__nv_bfloat16>(ws, p.dab); q.ld_out = fin; q.gate_f = s.f;
-        q.gate_in = ws_ptr<uint32_t>(ws, p.ab);
+        q.gate_buf = ws_ptr<uint4>(ws, p.ab);
       }
       break;
     case kDgrad1Scatter:   // A = W_in [E][d (m)][f (k)] K-major; B = dH [E][C][f] K-major  (GEGLU: d[a | b], K = 2 f)

@@ -189,12 +189,13 @@ inline void make_plan(const Shape& s, Plan* p) {
   p->dwr_partial = take((size_t)s.dwr_chunks * d * E * 4);
   p->wsplit = take(3 * d * (size_t)s.Epad64 * 2);
   p->dhsplit = take(3 * T * (size_t)s.Epad64 * 2);
-  p->hmask = take(E * C * ((f + 31) / 32) * 4);            // one bit per element of H: [H > 0]
+  const size_t rows16 = (C + 15) / 16 * 16;                // the tensor-core epilogues save for backward in blocks of 16 rows
+  p->hmask = take(E * rows16 * ((f + 31) / 32) * 4);       // one bit per element of H: [H > 0]
   p->layer_y = s.residual ? take(T * d * s.elt) : 0;       // g . E(x) without the skip path (for the gate's gradient)
   p->alt = s.reroute ? take(T * 4 * (size_t)s.reroute_stages) : 0;   // per stage: next choice of the tokens without a slot, -1 for the others
   p->expert_proc = s.reroute ? take(T * 4) : p->expert_index;   // the expert that processes each token
   p->xr = s.jitter ? take(T * d * s.elt) : 0;               // the router's input x . u, rounded to the activation dtype
-  p->ab = s.geglu ? take(E * C * 2 * f * s.elt) : 0;        // GEGLU: [a | b] = X_d [W_0 | W_1] per slot
+  p->ab = s.geglu ? take(E * rows16 * 2 * f * s.elt) : 0;   // GEGLU: [a | b] = X_d [W_0 | W_1] per slot, or the saved factors
   p->dab = s.geglu ? take(E * C * 2 * f * s.elt) : 0;       // GEGLU: gradient of [a | b] per slot
   p->yv = s.top2 ? take(Tv * d * s.elt) : 0;                // top-2: weighted expert output per assignment
   p->dxv = s.top2 ? take(Tv * d * s.elt) : 0;               // top-2: input gradient per assignment

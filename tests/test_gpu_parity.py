@@ -417,6 +417,16 @@ def test_tensor_core_layer_single_expert_is_dense_ffn():
     np.testing.assert_allclose(to_np(g.view(sm.WS_GATE)), 1.0)
 
 
+@pytest.mark.parametrize("T,E,cf", [
+    (400, 5, 1.0),               # 80 rows: two and a half chunks of 32 tokens, three tiles of 256 hidden rows per pair
+    (330, 7, 1.0),               # 47 rows: the last block of 16 ends past the capacity
+    (2600, 8, 1.03), (2700, 8, 1.0)])   # 334 and 337 rows: two pieces, the second with an odd number of 16-token blocks
+@pytest.mark.parametrize("kw", [dict(), dict(geglu=True), dict(dropout=0.3), dict(geglu=True, dropout=0.3, residual=True)],
+                         ids=["relu", "geglu", "dropout", "geglu_dropout_residual"])
+def test_layer_at_the_edges_of_the_epilogue_blocks(T, E, cf, kw):
+    _check_layer(si.SwitchConfig("epilogue_edges", T, 192, 320, E, cf), sm.GEMM_DEFAULT, TOL_BF16, seed=8, **kw)
+
+
 def test_capacity_override_is_honoured():
     _check_layer(MID, sm.GEMM_DEFAULT, TOL_BF16, capacity_override=200)
 
