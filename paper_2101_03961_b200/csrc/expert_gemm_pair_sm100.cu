@@ -966,9 +966,12 @@ int launch_pair_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a
   }
 }
 
-// dgrad1 and wgrad1 in one launch (see expert_gemm_pair_dual_kernel).  The two products have the same flops; the
-// weight gradient's tiles are the slower ones, so it gets the larger share of the CTA pairs (39 of 74 measured best
-// on B200 at the bench shape: 1.3% of the step against two launches).
+// dgrad1 and wgrad1 in one launch (see expert_gemm_pair_dual_kernel).  The two products have the same flops, but a weight
+// gradient's tile contracts over the expert's tokens only, so with few of them its epilogue (256 x 256 outputs for a few
+// k-blocks) weighs more and it gets the larger share of the CTA pairs.  Measured on 74 pairs, pairs for dgrad1: 32 to 256
+// tokens per expert 33 is best (768 x 3072, 128 experts: 256 tokens 322 us against 329 with 35 and 347 with 37; 32 tokens
+// 211 / 214 / 225; 1792 x 4864, 113 tokens 154 / 162 / 169), 512 tokens and more an even split (512 x 1536, 2048 tokens 77 us
+// against 85 with 33; 256 x 512, 512 tokens 46 / 50).
 int launch_pair_dgrad1_wgrad1(const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st) {
   int dev = 0, sm_count = 0;
   if (device_and_sms(&dev, &sm_count) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
@@ -989,7 +992,8 @@ int launch_pair_dgrad1_wgrad1(const Shape& s, const Plan& p, const GemmArgs& a, 
     rc = launch_pair_op<kDgrad1Scatter>(tmA0, tmB0, q0, dev, sm_count, st);
     return rc != SWITCH_MOE_OK ? rc : launch_pair_op<kWgrad1>(tmA1, tmB1, q1, dev, sm_count, st);
   }
-  int split = (n_pairs * 35 + 37) / 74;
+  const bool few_tokens = s.Tv < 384 * s.E;                   // per expert, before the capacity cut
+  int split = few_tokens ? (n_pairs * 33 + 37) / 74 : n_pairs / 2;
   if (split < 1) split = 1;
   if (split > n_pairs - 1) split = n_pairs - 1;
   launch_k(kernel, dim3(grid), dim3(kPThreads), kPSmemBytes, st, tmA0, tmB0, q0, tmA1, tmB1, q1, split);
