@@ -224,10 +224,34 @@ router_jitter_kernel(const uint4* __restrict__ x, const uint4* __restrict__ u, s
   }
 }
 
+// N consecutive floats of a row from e0 on, zero past E.
+template <int N, bool kVec>
+__device__ __forceinline__ void load_lane(const float* __restrict__ row, int e0, int E, float* v) {
+  if constexpr (kVec && N >= 4) {
+#pragma unroll
+    for (int n = 0; n < N; n += 4) {
+      const float4 t = e0 + n < E ? *reinterpret_cast<const float4*>(row + e0 + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[n] = t.x; v[n + 1] = t.y; v[n + 2] = t.z; v[n + 3] = t.w;
+    }
+  } else if constexpr (kVec && N == 2) {
+    const float2 t = e0 < E ? *reinterpret_cast<const float2*>(row + e0) : make_float2(0.f, 0.f);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+#pragma unroll
+    for (int n = 0; n < N; ++n) v[n] = e0 + n < E ? row[e0 + n] : 0.f;
+  }
+}
+
 // dh[t,i] = p[t,i] (G[t,i] - sum_j p[t,j] G[t,j]),  G[t,i] = cG.count_gi + [i = e_t and t kept].dgate_t,
 // count_gi counted inside the token's own routing group g = t / Tg.  Top-2 routing (second > 0): the token's second
 // assignment T + t adds its own gate gradient at its own expert.
-template <int NE>
+//
+// A warp works on kTok tokens at a time; lane l holds experts NE l .. NE l + NE - 1 of each.  What bounds it is the number
+// of instructions (three quarters of the issue slots with one token per warp, scalar loads and a bound check per expert):
+// rows are loaded as vectors where E allows, experts past E carry p = 0 and need no checks, the loss term stays in
+// registers while the routing group does not change, and the bfloat16 parts are formed in pairs.  32768 tokens, 128 experts
+// 14.2 -> 12.0 us; router backward stage of 65536 tokens, 128 experts 63 -> 59, of top-2 with 64 experts 36 -> 32.
+template <int NE, bool kVec>                                   // kVec: E is a multiple of 4
 __global__ void __launch_bounds__(256)
 router_dlogits_kernel(const float* __restrict__ probs, const int* __restrict__ expert_index,
                       const int* __restrict__ slot, const int* __restrict__ count, const float* __restrict__ dgate,
@@ -235,46 +259,86 @@ router_dlogits_kernel(const float* __restrict__ probs, const int* __restrict__ e
                       __nv_bfloat16* __restrict__ dhsplit, int Epad64) {
   pdl_launch_dependents();
   pdl_wait();
-  const int lane = threadIdx.x & 31;
-  const int t = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (t >= T) return;
-  const int et = expert_index[t];
-  const float dg = slot[t] >= 0 ? dgate[t] : 0.f;
-  const int et2 = second ? expert_index[T + t] : -1;
-  const float dg2 = (second && slot[T + t] >= 0) ? dgate[T + t] : 0.f;
-  count += (size_t)(t / Tg) * E;
-  float p[NE], G[NE], s = 0.f;
+  constexpr int kTok = NE >= 8 ? 2 : 4;
+  const int lane = threadIdx.x & 31, e0 = lane * NE;
+  const int gw = blockIdx.x * 8 + (threadIdx.x >> 5), n_warps = gridDim.x * 8;
+  const size_t plane = (size_t)T * Epad64;
+  int group = -1;
+  float cg[NE];
+  for (int t0 = gw * kTok; t0 < T; t0 += n_warps * kTok) {
+    float p[kTok][NE], dg[kTok], s[kTok];
+    int et[kTok];
 #pragma unroll
-  for (int n = 0; n < NE; ++n) {
-    const int e = lane * NE + n;
-    p[n] = e < E ? probs[(size_t)t * E + e] : 0.f;
-    G[n] = e < E ? cG * (float)count[e] + (e == et ? dg : 0.f) + (e == et2 ? dg2 : 0.f) : 0.f;
-    s = fmaf(p[n], G[n], s);
-  }
+    for (int j = 0; j < kTok; ++j) {
+      const int t = min(t0 + j, T - 1);
+      load_lane<NE, kVec>(probs + (size_t)t * E, e0, E, p[j]);
+      et[j] = expert_index[t] - e0;                             // this lane's n if it holds the token's expert
+      dg[j] = slot[t] >= 0 ? dgate[t] : 0.f;
+    }
+    float G[kTok][NE];
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    for (int j = 0; j < kTok; ++j) {
+      const int g = Tg == T ? 0 : min(t0 + j, T - 1) / Tg;
+      if (g != group) {
+        group = g;
 #pragma unroll
-  for (int n = 0; n < NE; ++n) {
-    const int e = lane * NE + n;
-    const float dh = p[n] * (G[n] - s);
-    if (dlogits != nullptr && e < E) dlogits[(size_t)t * E + e] = dh;
-    G[n] = e < E ? dh : 0.f;
-  }
-  if (dhsplit != nullptr && lane * NE < Epad64) {             // bf16 hi / mid parts for the tensor-core products
-    __align__(16) __nv_bfloat16 hi[NE], mid[NE], lo[NE];
+        for (int n = 0; n < NE; ++n) cg[n] = e0 + n < E ? cG * (float)count[(size_t)g * E + e0 + n] : 0.f;
+      }
 #pragma unroll
-    for (int n = 0; n < NE; ++n) split3(G[n], &hi[n], &mid[n], &lo[n]);
-    const size_t plane = (size_t)T * Epad64, at = (size_t)t * Epad64 + lane * NE;    // NE consecutive experts per lane
-    using Vec = typename BfVec<NE>::type;
-    *reinterpret_cast<Vec*>(dhsplit + at) = *reinterpret_cast<const Vec*>(hi);
-    *reinterpret_cast<Vec*>(dhsplit + plane + at) = *reinterpret_cast<const Vec*>(mid);
-  }
-  if (dhsplit != nullptr) {                                   // padding columns beyond the lanes' experts
-    const __nv_bfloat16 z = __float2bfloat16(0.f);
-    const size_t plane = (size_t)T * Epad64;
-    for (int e = 32 * NE + lane; e < Epad64; e += 32) {
-      const size_t at = (size_t)t * Epad64 + e;
-      dhsplit[at] = z; dhsplit[plane + at] = z;
+      for (int n = 0; n < NE; ++n) G[j][n] = cg[n] + (n == et[j] ? dg[j] : 0.f);
+    }
+    if (second) {
+#pragma unroll
+      for (int j = 0; j < kTok; ++j) {
+        const int t = min(t0 + j, T - 1), et2 = expert_index[T + t] - e0;
+        const float dg2 = slot[T + t] >= 0 ? dgate[T + t] : 0.f;
+#pragma unroll
+        for (int n = 0; n < NE; ++n) G[j][n] += n == et2 ? dg2 : 0.f;
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < kTok; ++j) {
+      s[j] = 0.f;
+#pragma unroll
+      for (int n = 0; n < NE; ++n) s[j] = fmaf(p[j][n], G[j][n], s[j]);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+      for (int j = 0; j < kTok; ++j) s[j] += __shfl_xor_sync(0xffffffffu, s[j], off);
+#pragma unroll
+    for (int j = 0; j < kTok; ++j) {
+      const int t = t0 + j;
+      if (t >= T) break;
+#pragma unroll
+      for (int n = 0; n < NE; ++n) {
+        G[j][n] = p[j][n] * (G[j][n] - s[j]);
+        if (dlogits != nullptr && e0 + n < E) dlogits[(size_t)t * E + e0 + n] = G[j][n];
+      }
+      if (dhsplit == nullptr) continue;
+      if (e0 < Epad64) {                                        // bf16 hi / mid parts for the tensor-core products
+        __align__(16) __nv_bfloat16 hi[NE], mid[NE];
+        if constexpr (NE >= 2) {
+#pragma unroll
+          for (int n = 0; n < NE; n += 2) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(G[j][n], G[j][n + 1]);
+            const float2 f = __bfloat1622float2(h);
+            *reinterpret_cast<__nv_bfloat162*>(hi + n) = h;
+            *reinterpret_cast<__nv_bfloat162*>(mid + n) = __floats2bfloat162_rn(G[j][n] - f.x, G[j][n + 1] - f.y);
+          }
+        } else {
+          hi[0] = __float2bfloat16(G[j][0]);
+          mid[0] = __float2bfloat16(G[j][0] - __bfloat162float(hi[0]));
+        }
+        const size_t at = (size_t)t * Epad64 + e0;              // NE consecutive experts per lane
+        using Vec = typename BfVec<NE>::type;
+        *reinterpret_cast<Vec*>(dhsplit + at) = *reinterpret_cast<const Vec*>(hi);
+        *reinterpret_cast<Vec*>(dhsplit + plane + at) = *reinterpret_cast<const Vec*>(mid);
+      }
+      for (int e = 32 * NE + lane; e < Epad64; e += 32) {       // padding columns beyond the lanes' experts
+        const size_t at = (size_t)t * Epad64 + e;
+        dhsplit[at] = dhsplit[plane + at] = __float2bfloat16(0.f);
+      }
     }
   }
 }
@@ -489,13 +553,11 @@ int router_bwd_t(const Shape& s, const Plan& p, const void* x, const float* W_r,
   // The float32 logit gradients are an output of the staged call (and the operand of the FP32-FMA products); the
   // whole-layer backward pass on the tensor cores only needs their bfloat16 parts.
   const bool tc_products = s.router_tc && sizeof(XT) == 2;
-  launch_k(router_dlogits_kernel<NE>, dim3((s.T + 7) / 8), dim3(256), 0, st, ws_ptr<float>(ws, p.probs),
-                                                            ws_ptr<int>(ws, p.expert_proc), ws_ptr<int>(ws, p.slot),
-                                                            ws_ptr<int>(ws, p.count_g), dgate, cG, s.T, s.Tg, s.E, s.top2,
-                                                            (tc_products && accumulate_dx) ? nullptr : dlogits,
-                                                            (s.router_tc && sizeof(XT) == 2)
-                                                                ? ws_ptr<__nv_bfloat16>(ws, p.dhsplit) : nullptr,
-                                                            s.Epad64);
+  const int dl_blocks = (s.T + 31) / 32;                      // four tokens per warp, eight warps
+  launch_k(s.E % 4 == 0 ? router_dlogits_kernel<NE, true> : router_dlogits_kernel<NE, false>, dim3(dl_blocks), dim3(256), 0, st,
+           ws_ptr<float>(ws, p.probs), ws_ptr<int>(ws, p.expert_proc), ws_ptr<int>(ws, p.slot), ws_ptr<int>(ws, p.count_g),
+           dgate, cG, s.T, s.Tg, s.E, s.top2, (tc_products && accumulate_dx) ? nullptr : dlogits,
+           (s.router_tc && sizeof(XT) == 2) ? ws_ptr<__nv_bfloat16>(ws, p.dhsplit) : nullptr, s.Epad64);
   float* partial = ws_ptr<float>(ws, p.dwr_partial);
   const size_t n = (size_t)s.d * s.E;
   if (s.jitter) {                                             // the router's input was x . u (left by the forward pass)

@@ -348,8 +348,9 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 // in tensor memory over all the CTA's tiles and leaves once, as one partial per CTA; dx has two accumulators, so the
 // epilogue of a tile (read dx, add, round, store) overlaps the next tile's products.
 //
-// What bounds it: x is read once and dx read and written once from HBM, and every column block reads dh from L2; the
-// operands of both products cross shared memory at about its rate.  Measured with its neighbours (logit gradients before,
+// What bounds it: every column block reads all of dh from L2 (211 MB into the SMs at 32768 tokens, d 768, E 128; with the
+// stores, the dx reads and most MMAs taken out the kernel still took 24 of its 37 us, i.e. 9 TB/s).  More x stages, a longer
+// ring or x requested into L2 ahead changed nothing (one x stage: 47 us).  Measured with its neighbours (logit gradients before,
 // reduction of the partials after) against one kernel per product: 32768 tokens, d 768, E 128 82 -> 67 us; 65536 tokens,
 // d 256, E 128 (jitter) 83 -> 63; 16384 tokens, d 768, E 64 45 -> 34; 20011 tokens, d 512, E 200 61 -> 63.
 struct RouterBwdParams {
@@ -567,20 +568,15 @@ router_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
         const int row = it * 4 + (lane >> 3);
         uint4 val = *reinterpret_cast<const uint4*>(stage_gen + (row & 15) * 128 + (((lane & 7) ^ (row & 7)) << 4));
         const bool add = (add_now >> row) & 1u;
-        if (kJitter || add) {                                  // d(x . u)/dx = u; one rounding for (router term . u) + dx
-          __nv_bfloat162* vp = reinterpret_cast<__nv_bfloat162*>(&val);
-          const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&old[it]);
+        __nv_bfloat162* vp = reinterpret_cast<__nv_bfloat162*>(&val);
+        const __nv_bfloat162* pp = reinterpret_cast<const __nv_bfloat162*>(&old[it]);
+        if (kJitter) {                                         // d(x . u)/dx = u; one rounding for (router term . u) + dx
           const __nv_bfloat162* up = reinterpret_cast<const __nv_bfloat162*>(&uu[kJitter ? it : 0]);
 #pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const float2 a = __bfloat1622float2(vp[q]), b = __bfloat1622float2(pp[q]);
-            float2 s = make_float2(a.x + b.x, a.y + b.y);
-            if (kJitter) {
-              const float2 u = __bfloat1622float2(up[q]);
-              s = add ? make_float2(fmaf(a.x, u.x, b.x), fmaf(a.y, u.y, b.y)) : make_float2(a.x * u.x, a.y * u.y);
-            }
-            vp[q] = __floats2bfloat162_rn(s.x, s.y);
-          }
+          for (int q = 0; q < 4; ++q) vp[q] = add ? __hfma2(vp[q], up[q], pp[q]) : __hmul2(vp[q], up[q]);
+        } else if (add) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q) vp[q] = __hadd2(vp[q], pp[q]);
         }
         if (tok0 + row < p.T && col_ok) *reinterpret_cast<uint4*>(p.dx + (size_t)(tok0 + row) * p.d + col) = val;
       }
