@@ -422,30 +422,45 @@ reroute_choice_kernel(const float* __restrict__ probs, const int* __restrict__ p
 }
 
 // Position bases of a further stage: the rerouted tokens of expert e queue up behind the kept[e] tokens it has so far.
-// One thread per expert; also rewrites kept[] and the tile lists for the grown experts.
-__global__ void __launch_bounds__(kMaxExperts)
-reroute_scan_kernel(const int* __restrict__ hist, int plan_blocks, int E, int C, int* __restrict__ hist_base,
+// Also rewrites kept[] and the tile lists for the grown experts.  Thread (g, e) of the one block owns slice g of the rows of
+// column e, as in plan_scan_kernel (a thread per expert walking all rows waited for one batch of loads after another: 13.6
+// us from the previous kernel's end to its own at 32768 tokens and 64 experts; with slices 6.7).
+__global__ void __launch_bounds__(kScanThreads)
+reroute_scan_kernel(const int* __restrict__ hist, int plan_blocks, int E, int Ew, int C, int* __restrict__ hist_base,
                     int* __restrict__ kept, int* __restrict__ tile_expert, int* __restrict__ tile_row0,
                     int4* __restrict__ ntile) {
   pdl_launch_dependents();
   pdl_wait();
+  __shared__ int qsum[kScanThreads];                         // [g][e], Ew columns per row
   __shared__ float term[kMaxExperts];
   __shared__ int kept_s[kMaxExperts];
-  const int e = threadIdx.x;
+  const int G = kScanThreads / Ew;
+  const int e = threadIdx.x % Ew, g = threadIdx.x / Ew;
+  const int hq = (plan_blocks + G - 1) / G, h0 = g * hq, h1 = min(plan_blocks, h0 + hq);
+  int hv[kScanRows], run = 0;
   if (e < E) {
-    int run = kept[e];
-    for (int b0 = 0; b0 < plan_blocks; b0 += 8) {
-      int v[8];
+    run = kept[e];
 #pragma unroll
-      for (int j = 0; j < 8; ++j) v[j] = b0 + j < plan_blocks ? hist[(size_t)(b0 + j) * E + e] : 0;
+    for (int j = 0; j < kScanRows; ++j) hv[j] = h0 + j < h1 ? hist[(size_t)(h0 + j) * E + e] : 0;
+    int sum = 0;
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (b0 + j < plan_blocks) { hist_base[(size_t)(b0 + j) * E + e] = run; run += v[j]; }
+    for (int j = 0; j < kScanRows; ++j) sum += hv[j];
+    for (int b = h0 + kScanRows; b < h1; ++b) sum += hist[(size_t)b * E + e];
+    qsum[g * Ew + e] = sum;
+  }
+  __syncthreads();                                             // (also: kept[] has been read by every slice)
+  if (e < E) {
+    for (int q = 0; q < g; ++q) run += qsum[q * Ew + e];
+#pragma unroll
+    for (int j = 0; j < kScanRows; ++j)
+      if (h0 + j < h1) { hist_base[(size_t)(h0 + j) * E + e] = run; run += hv[j]; }
+    for (int b = h0 + kScanRows; b < h1; ++b) { hist_base[(size_t)b * E + e] = run; run += hist[(size_t)b * E + e]; }
+    if (g == G - 1) {
+      const int k = min(run, C);
+      kept[e] = k;
+      kept_s[e] = k;
+      term[e] = 0.f;
     }
-    const int k = min(run, C);
-    kept[e] = k;
-    kept_s[e] = k;
-    term[e] = 0.f;
   }
   write_tile_lists(term, kept_s, E, 0.f, nullptr, tile_expert, tile_row0, ntile);
 }
@@ -762,8 +777,8 @@ int launch_reroute(const Shape& s, const Plan& p, void* ws, cudaStream_t st) {
              ws_ptr<int>(ws, p.slot), s.T, s.E, alt);
     launch_k(plan_hist_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, alt, s.T, s.E,
              ws_ptr<int>(ws, p.hist));
-    launch_k(reroute_scan_kernel, dim3(1), dim3(kMaxExperts), 0, st, ws_ptr<int>(ws, p.hist), s.plan_blocks, s.E, s.C,
-             ws_ptr<int>(ws, p.hist_base), ws_ptr<int>(ws, p.kept), list128(s, p, ws),
+    launch_k(reroute_scan_kernel, dim3(1), dim3(kScanThreads), 0, st, ws_ptr<int>(ws, p.hist), s.plan_blocks, s.E,
+             column_width(s.E), s.C, ws_ptr<int>(ws, p.hist_base), ws_ptr<int>(ws, p.kept), list128(s, p, ws),
              ws_ptr<int>(ws, p.tile_row0), ws_ptr<int4>(ws, p.ntile));
     launch_k(reroute_assign_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, alt, ei,
              ws_ptr<int>(ws, p.hist_base), ws_ptr<float>(ws, p.probs), s.T, s.E, s.C, ws_ptr<int>(ws, p.slot),

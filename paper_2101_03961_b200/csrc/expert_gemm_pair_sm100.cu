@@ -830,14 +830,18 @@ int launch_pair_op(const CUtensorMap& tmA, const BMapSet& tmB, const PairParams&
   return launch_status();
 }
 
-// Operands, output and tile counts of one product.
-// The token operand's maps: one per box height (8 j rows, j = 1..16).
-int make_token_maps(BMapSet* bm, const void* base, long long E, long long rows, long long cols) {
-  for (int j = 1; j <= kBMaps; ++j)
-    if (make_map(&bm->m[j - 1], base, E, rows, cols, 8 * j) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
+// Widest token tile: what the capacity allows, rounded up to the MMA's granularity.
+int widest_tile(const Shape& s) { return s.C < kPairTileTokens ? (s.C + 15) / 16 * 16 : kPairTileTokens; }
+
+// The token operand's maps: one per box height (8 j rows) up to half of the widest tile or segment.
+int make_token_maps(BMapSet* bm, const Shape& s, const void* base, long long cols) {
+  const int most = widest_tile(s) / 16 < kBMaps ? widest_tile(s) / 16 : kBMaps;
+  for (int j = 1; j <= most; ++j)
+    if (make_map(&bm->m[j - 1], base, s.E, s.C, cols, 8 * j) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
   return SWITCH_MOE_OK;
 }
 
+// Operands, output and tile counts of one product.
 int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, PairParams* out,
                  CUtensorMap* tmA_out, BMapSet* tmB_out) {
   const void* xd = ws_ptr<char>(ws, p.xd);
@@ -866,7 +870,7 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
   switch (op) {
     case kGemm1Relu:       // A = W_in [E][d (k)][f (m)]: m contiguous -> MN-major; B = X_d [E][C][d] K-major
       q.token_op = 1; q.a_mn_major = 1; q.Mw = fin; K = s.d;   // GEGLU: 2 f weight columns [W_0 | W_1], no ReLU
-      rc = make_map(&tmA, a.W_in, s.E, s.d, fin, 64); rc2 = make_token_maps(&bm, xd, s.E, s.C, s.d);
+      rc = make_map(&tmA, a.W_in, s.E, s.d, fin, 64); rc2 = make_token_maps(&bm, s, xd, s.d);
       q.out = ws_ptr<__nv_bfloat16>(ws, p.h); q.ld_out = s.f;
       if (s.geglu) { q.gate_f = s.f; q.gate_buf = ws_ptr<uint4>(ws, p.ab); }   // gating in the epilogue
       if (s.dropout) {
@@ -876,7 +880,7 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
       break;
     case kGemm2Combine:    // A = W_out [E][f (k)][d (m)] MN-major; B = H [E][C][f] K-major
       q.token_op = 1; q.a_mn_major = 1; q.Mw = s.d; K = s.f;
-      rc = make_map(&tmA, a.W_out, s.E, s.f, s.d, 64); rc2 = make_token_maps(&bm, h, s.E, s.C, s.f);
+      rc = make_map(&tmA, a.W_out, s.E, s.f, s.d, 64); rc2 = make_token_maps(&bm, s, h, s.f);
       q.out = static_cast<__nv_bfloat16*>(a.y); q.ld_out = s.d;
       if (s.residual && !s.top2) {   // (top-2 routing adds the skip path where the two assignments' rows are summed)
         q.res = static_cast<const __nv_bfloat16*>(a.x); q.out2 = ws_ptr<__nv_bfloat16>(ws, p.layer_y);
@@ -884,7 +888,7 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
       break;
     case kDgrad2Mask:      // A = W_out [E][f (m)][d (k)] K-major; B = dY_d [E][C][d] K-major
       q.token_op = 1; q.a_mn_major = 0; q.Mw = s.f; K = s.d;
-      rc = make_map(&tmA, a.W_out, s.E, s.f, s.d, 128); rc2 = make_token_maps(&bm, dyd, s.E, s.C, s.d);
+      rc = make_map(&tmA, a.W_out, s.E, s.f, s.d, 128); rc2 = make_token_maps(&bm, s, dyd, s.d);
       q.out = ws_ptr<__nv_bfloat16>(ws, p.dh); q.ld_out = s.f;
       if (s.dropout && !s.geglu) q.keep_scale = s.keep_scale;   // (GEGLU: the saved factors carry the dropout factor)
       if (s.geglu) {   // the derivative of the gating in the epilogue: d[a | b] is written, dH never is
@@ -894,7 +898,7 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
       break;
     case kDgrad1Scatter:   // A = W_in [E][d (m)][f (k)] K-major; B = dH [E][C][f] K-major  (GEGLU: d[a | b], K = 2 f)
       q.token_op = 1; q.a_mn_major = 0; q.Mw = s.d; K = fin;
-      rc = make_map(&tmA, a.W_in, s.E, s.d, fin, 128); rc2 = make_token_maps(&bm, du, s.E, s.C, fin);
+      rc = make_map(&tmA, a.W_in, s.E, s.d, fin, 128); rc2 = make_token_maps(&bm, s, du, fin);
       q.out = static_cast<__nv_bfloat16*>(a.dx); q.ld_out = s.d;
       if (s.residual && !s.top2) q.res = static_cast<const __nv_bfloat16*>(a.dy);
       break;
@@ -912,7 +916,7 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
   q.n_mpairs = (q.Mw + 255) / 256;
   // operand ring of the token products: a stage holds A (16 KB) and this CTA's half of the widest token tile the
   // capacity allows (at most kPairTileTokens / 2 rows of 128 bytes, rounded up to whole 1 KB swizzle atoms)
-  const int widest = s.C < kPairTileTokens ? (s.C + 15) / 16 * 16 : kPairTileTokens;
+  const int widest = widest_tile(s);
   q.stage_bytes = kPHalfBytes + ((widest / 2) * 128 + 1023) / 1024 * 1024;
   q.stages = kPRingBytes / q.stage_bytes < kPMaxStages ? kPRingBytes / q.stage_bytes : kPMaxStages;
   q.n_ntiles_fixed = q.token_op ? 0 : (q.Nfix + 255) / 256;
