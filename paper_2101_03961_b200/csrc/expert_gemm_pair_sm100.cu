@@ -41,11 +41,12 @@ namespace swmoe {
 using namespace tc;
 namespace {
 
-constexpr int kPStages = 6;                            // weight gradients: six stages of A (16 KB) + half of B (16 KB)
+constexpr int kPStages = 6;                            // weight gradients: six blocks of A and six of half of B
 constexpr int kPMaxStages = 8;                         // token products: as many stages as fit, at most this
 constexpr int kPHalfBytes = 16384;                     // A tile (128 x 64) and B half tile (<= 128 x 64)
 constexpr int kPStageBytes = 2 * kPHalfBytes;
 constexpr int kPRingBytes = kPStages * kPStageBytes;   // 192 KB of operand stages
+constexpr int kPWgradA = kPStages, kPWgradB = kPStages;   // weight gradients: A and B blocks of 16 KB in rings of their own
 constexpr int kPTransWarp = 32 * 64;                   // per epilogue warp: 32 tokens x 32 weight rows of bfloat16
 constexpr int kPTransBytes = 8 * kPTransWarp;
 constexpr int kPAuxBytes = 8 * 128;                    // 8 epilogue warps x 32 gates
@@ -71,6 +72,8 @@ struct PairParams {
   int Nfix;                // weight gradients: output columns
   int k_blocks_fixed;      // token ops: K / 64
   int n_mpairs, n_ntiles_fixed;
+  int tokens_per_expert;   // average, at most the capacity
+  int strips;              // weight gradients: strips that a row of column tiles (256 output rows) is cut into
   int C, E;
   const int4* ntile;       // [0].x = number of token tiles; then {expert, first slot row, rows (multiple of 16)}
   const int* kept;
@@ -97,7 +100,7 @@ struct PairParams {
   int stages, stage_bytes;    // operand ring: token products size a stage for the widest tile the capacity allows
   // ceil(2^32 / divisor) for the three divisions of the tile decode (n_mpairs; n_mpairs * n_ntiles_fixed;
   // n_ntiles_fixed): id / d = umulhi(id, magic) as long as id * d < 2^32
-  uint32_t magic_mpairs, magic_per_e, magic_nt;
+  uint32_t magic_mpairs, magic_per_e, magic_strips;
 };
 
 __device__ __forceinline__ int fast_div(int id, uint32_t magic, int divisor) {
@@ -113,6 +116,7 @@ struct BMapSet {
 
 struct PTile {
   int e, m0, n0, row0, n, n1, k_blocks, last_mmas;   // n1: columns of the first segment (n if n <= 256)
+  int tiles;                                         // weight gradients: column tiles of the strip that starts at n0
 };
 
 // Tile decode reads the plan through shared-memory copies made at kernel start: a dependent global load per tile
@@ -125,15 +129,22 @@ __device__ __forceinline__ PTile p_decode(const PairParams& p, int id, const int
     t.e = q.x; t.row0 = q.y; t.n = q.z; t.n0 = 0;
     t.n1 = t.n <= 256 ? t.n : ((t.n >> 1) + 15) & ~15;         // two segments: both multiples of 16, both <= 256
     t.m0 = (id - nt * p.n_mpairs) * 256;
-    t.k_blocks = p.k_blocks_fixed;
+    t.k_blocks = p.k_blocks_fixed; t.tiles = 1;
     t.last_mmas = kBK / kUmmaK;
   } else {
-    const int per_e = p.n_mpairs * p.n_ntiles_fixed;
+    const int per_e = p.n_mpairs * p.strips;
     t.e = fast_div(id, p.magic_per_e, per_e);
     const int rem = id - t.e * per_e;
-    const int mp = fast_div(rem, p.magic_nt, p.n_ntiles_fixed);
+    const int mp = fast_div(rem, p.magic_strips, p.strips);
+    const int strip = rem - mp * p.strips;                      // strips of a row differ by at most one tile
+    int first = strip, last = strip + 1;
+    if (p.strips < p.n_ntiles_fixed) {
+      first = (int)((unsigned)strip * (unsigned)p.n_ntiles_fixed / (unsigned)p.strips);
+      last = (int)((unsigned)(strip + 1) * (unsigned)p.n_ntiles_fixed / (unsigned)p.strips);
+    }
     t.m0 = mp * 256;
-    t.n0 = (rem - mp * p.n_ntiles_fixed) * 256;
+    t.n0 = first * 256;
+    t.tiles = last - first;
     t.row0 = 0; t.n = 256; t.n1 = 256;
     const int k = kept_s[t.e];
     t.k_blocks = (k + kBK - 1) / kBK;
@@ -194,6 +205,11 @@ __device__ __forceinline__ void stmatrix_trans(uint32_t addr, const uint32_t* w)
                "r"(w[2]), "r"(w[3])
                : "memory");
 }
+__device__ __forceinline__ void stmatrix_x4(uint32_t addr, const uint32_t* w) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(w[0]), "r"(w[1]),
+               "r"(w[2]), "r"(w[3])
+               : "memory");
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   const __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&h2);
@@ -245,10 +261,10 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
   const uint32_t bar_base = smem_base + kPRingBytes + kPTransBytes + kPAuxBytes;
   // barrier block: full[S] | empty[S] | tmem_full[2] | tmem_empty[2] | tmem_mid[2] | tmem_ptr | abort | gate[4]
   // (S = kPMaxStages; gate[i] at byte 192 + 8 i: the handshake of the two epilogue warps that hold a and b of the
-  // same hidden units, gated GEMM1 only)
+  // same hidden units, gated GEMM1 only; there a weight gradient has aempty[kPWgradA], the release of its A blocks)
   const uint32_t full0 = bar_base, empty0 = bar_base + 8u * kPMaxStages;
   const uint32_t tfull0 = bar_base + 16u * kPMaxStages, tempty0 = tfull0 + 16u, tmid0 = tfull0 + 32u;
-  const uint32_t gate0 = bar_base + 192u;
+  const uint32_t gate0 = bar_base + 192u, aempty0 = gate0;
   volatile uint32_t* tmem_ptr_s = reinterpret_cast<volatile uint32_t*>(bar_gen + 8 * (2 * kPMaxStages + 6));
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 8 * (2 * kPMaxStages + 6) + 4);
   int* kept_s = reinterpret_cast<int*>(bar_gen + 256);
@@ -256,8 +272,8 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
 
   const int warp = uniform_warp_id(), lane = threadIdx.x & 31;
   const uint32_t rank = __shfl_sync(0xffffffffu, cluster_ctarank(), 0);   // 0 = leader (issues the MMAs)
-  const uint32_t n_stages = kTok ? (uint32_t)p.stages : (uint32_t)kPStages;
-  const uint32_t stage_bytes = kTok ? (uint32_t)p.stage_bytes : (uint32_t)kPStageBytes;
+  const uint32_t n_stages = kTok ? (uint32_t)p.stages : (uint32_t)kPWgradB;
+  const uint32_t stage_bytes = kTok ? (uint32_t)p.stage_bytes : (uint32_t)kPHalfBytes;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kPMaxStages; ++s) { mbar_init(full0 + 8u * s, 1); mbar_init(empty0 + 8u * s, 1); }
@@ -266,6 +282,8 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
     }
     if (kGated)
       for (int a = 0; a < 4; ++a) mbar_init(gate0 + 8u * a, 2);
+    if (!kTok)
+      for (int a = 0; a < kPWgradA; ++a) mbar_init(aempty0 + 8u * a, 1);
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -283,13 +301,13 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
   cluster_sync_all();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_s;
-  const int n_tiles = kTok ? n_ntiles_listed * p.n_mpairs : p.E * p.n_mpairs * p.n_ntiles_fixed;
+  const int n_tiles = kTok ? n_ntiles_listed * p.n_mpairs : p.E * p.n_mpairs * p.strips;
 
   // Accumulator columns of this pair's `it`-th tile: even tiles [0, n), odd tiles [512 - n, 512).  Consecutive tiles
   // share the middle columns when n + n_next > 512.
   if (warp == 0) {
     // ------------------------------------------------------------------------------------------ TMA producer (both CTAs)
-    uint32_t stage = 0, phase = 0;
+    uint32_t stage = 0, phase = 0, a_slot = 0, a_phase = 0;
     bool ok = true;
     for (int id = pair; id < n_tiles && ok; id += n_pairs) {
       const PTile t = p_decode(p, id, kept_s, tile_s);
@@ -306,33 +324,49 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
       const CUtensorMap* tmB = kTok ? &bm.m[(h1 >> 3) - 1] : &bm.m[0];
       const CUtensorMap* tmB2 = (kTok && h2 > 0) ? &bm.m[(h2 >> 3) - 1] : tmB;
       // both CTAs' bytes land on the leader's barrier
-      const uint32_t tx_bytes = kTok ? 2u * (uint32_t)(kPHalfBytes + (t.n >> 1) * 128) : 2u * (uint32_t)kPStageBytes;
+      const uint32_t tx_bytes = kTok ? 2u * (uint32_t)(kPHalfBytes + (t.n >> 1) * 128) : 2u * (uint32_t)kPHalfBytes;
+      // weight gradients: the tiles of a strip multiply the same A; it is loaded with the first of them and kept to the
+      // last if its k-blocks fit the A ring.  A block's full barrier counts the A bytes that come with it.
+      const bool resident = !kTok && kbs <= kPWgradA;
 #pragma unroll 1
-      for (int kb = 0; kb < kbs; ++kb) {
-        const uint32_t eb = empty0 + 8u * stage;
-        ok = mbar_wait_warp(eb, phase ^ 1u, abort_flag, p.status, 21);
-        if (!ok) break;
-        const uint32_t a_dst = smem_base + stage * stage_bytes, b_dst = a_dst + kPHalfBytes;
-        const uint32_t fb = full0 + 8u * stage;
-        const uint32_t lead_full = fb & kPeerMask;
-        const int k0 = kb * kBK;
-        if (elect_one()) {
-          if (rank == 0) mbar_arrive_expect_tx(fb, tx_bytes);
-          if (kAMn) {
-            tma_load_3d_pair(a_dst, &tmA, lead_full, a_m, k0, e);
-            tma_load_3d_pair(a_dst + kAtomBytes, &tmA, lead_full, a_m2, k0, e);
-          } else {
-            tma_load_3d_pair(a_dst, &tmA, lead_full, k0, a_m, e);
+      for (int j = 0; j < (kTok ? 1 : t.tiles) && ok; ++j) {
+        const bool load_a = kTok || j == 0 || !resident;
+#pragma unroll 1
+        for (int kb = 0; kb < kbs; ++kb) {
+          if (!kTok && load_a) {
+            ok = mbar_wait_warp(aempty0 + 8u * a_slot, a_phase ^ 1u, abort_flag, p.status, 28);
+            if (!ok) break;
           }
-          if (kBMn) {
-            tma_load_3d_pair(b_dst, tmB, lead_full, b_r, k0, e);
-            tma_load_3d_pair(b_dst + kAtomBytes, tmB, lead_full, b_r + 64, k0, e);
-          } else {
-            tma_load_3d_pair(b_dst, tmB, lead_full, k0, b_r, e);
-            if (h2 > 0) tma_load_3d_pair(b_dst + (uint32_t)h1 * 128u, tmB2, lead_full, k0, b_r2, e);
+          const uint32_t eb = empty0 + 8u * stage;
+          ok = mbar_wait_warp(eb, phase ^ 1u, abort_flag, p.status, 21);
+          if (!ok) break;
+          const uint32_t a_dst = smem_base + (kTok ? stage * stage_bytes : a_slot * (uint32_t)kPHalfBytes);
+          const uint32_t b_dst = kTok ? a_dst + kPHalfBytes : smem_base + (kPWgradA + stage) * (uint32_t)kPHalfBytes;
+          const uint32_t fb = full0 + 8u * stage;
+          const uint32_t lead_full = fb & kPeerMask;
+          const int k0 = kb * kBK;
+          if (elect_one()) {
+            if (rank == 0) mbar_arrive_expect_tx(fb, !kTok && load_a ? 2u * tx_bytes : tx_bytes);
+            if (kAMn) {
+              if (load_a) {
+                tma_load_3d_pair(a_dst, &tmA, lead_full, a_m, k0, e);
+                tma_load_3d_pair(a_dst + kAtomBytes, &tmA, lead_full, a_m2, k0, e);
+              }
+            } else {
+              tma_load_3d_pair(a_dst, &tmA, lead_full, k0, a_m, e);
+            }
+            if (kBMn) {
+              const int col = b_r + 256 * j;
+              tma_load_3d_pair(b_dst, tmB, lead_full, col, k0, e);
+              tma_load_3d_pair(b_dst + kAtomBytes, tmB, lead_full, col + 64, k0, e);
+            } else {
+              tma_load_3d_pair(b_dst, tmB, lead_full, k0, b_r, e);
+              if (h2 > 0) tma_load_3d_pair(b_dst + (uint32_t)h1 * 128u, tmB2, lead_full, k0, b_r2, e);
+            }
           }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+          if (!kTok && load_a && ++a_slot == (uint32_t)kPWgradA) { a_slot = 0; a_phase ^= 1u; }
         }
-        if (++stage == n_stages) { stage = 0; phase ^= 1u; }
       }
     }
     if (*abort_flag != 0) {
@@ -348,66 +382,140 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
       constexpr uint32_t a_kstep = (kAMn ? kUmmaK * 128u : kUmmaK * 2u) >> 4;
       constexpr uint32_t b_kstep = (kBMn ? kUmmaK * 128u : kUmmaK * 2u) >> 4;
       const uint64_t a_desc0 = make_smem_desc(smem_base, kAMn ? kAtomBytes : 16u, 1024u);
-      const uint64_t b_desc0 = make_smem_desc(smem_base + kPHalfBytes, kBMn ? kAtomBytes : 16u, 1024u);
-      uint32_t stage = 0, phase = 0, it = 0;
+      const uint64_t b_desc0 = make_smem_desc(smem_base + (kTok ? 1 : kPWgradA) * kPHalfBytes, kBMn ? kAtomBytes : 16u, 1024u);
+      uint32_t stage = 0, phase = 0, it = 0, a_first = 0;
       int n_prev = 0;
       bool ok = true;
-      for (int id = pair; id < n_tiles && ok; id += n_pairs, ++it) {
+      for (int id = pair; id < n_tiles && ok; id += n_pairs) {
         const PTile t = p_decode(p, id, kept_s, tile_s);
-        const uint32_t side = it & 1u, use = it >> 1;          // this side's `use`-th tile
-        const uint32_t idesc1 = idesc_base | ((uint32_t)(t.n1 >> 3) << 17);
-        const int n2 = t.n - t.n1;
-        const uint32_t idesc2 = idesc_base | ((uint32_t)(n2 >> 3) << 17);
-        const uint32_t b2_off = ((uint32_t)(t.n1 >> 1) * 128u) >> 4;    // second segment's rows in this CTA's half of B
-        const int kbs = t.k_blocks, last_mmas = t.last_mmas;
-        // the side's previous tile has been read out completely ...
-        ok = mbar_wait_warp(tempty0 + 8u * side, (use & 1u) ^ 1u, abort_flag, p.status, 22);
-        if (!ok) break;
-        // ... and so have the middle columns of the other side's tile, if this tile reaches into them
-        if (kTok && it > 0 && n_prev + t.n > kTmemCols) {
-          ok = mbar_wait_warp(tmid0 + 8u * (side ^ 1u), ((it - 1u) >> 1) & 1u, abort_flag, p.status, 25);
-          if (!ok) break;
-        }
-        n_prev = t.n;
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (side ? (uint32_t)(kTmemCols - t.n) : 0u);
-        const uint32_t d_tmem2 = d_tmem + (uint32_t)t.n1;
+        const bool resident = !kTok && t.k_blocks <= kPWgradA;
 #pragma unroll 1
-        for (int kb = 0; kb < kbs; ++kb) {
-          ok = mbar_wait_warp(full0 + 8u * stage, phase, abort_flag, p.status, 23);
+        for (int j = 0; j < (kTok ? 1 : t.tiles) && ok; ++j, ++it) {
+          const bool free_a = !kTok && (j == t.tiles - 1 || !resident);
+          uint32_t a_slot = a_first;
+          const uint32_t side = it & 1u, use = it >> 1;          // this side's `use`-th tile
+          const uint32_t idesc1 = idesc_base | ((uint32_t)(t.n1 >> 3) << 17);
+          const int n2 = t.n - t.n1;
+          const uint32_t idesc2 = idesc_base | ((uint32_t)(n2 >> 3) << 17);
+          const uint32_t b2_off = ((uint32_t)(t.n1 >> 1) * 128u) >> 4;    // second segment's rows in this CTA's half of B
+          const int kbs = t.k_blocks, last_mmas = t.last_mmas;
+          // the side's previous tile has been read out completely ...
+          ok = mbar_wait_warp(tempty0 + 8u * side, (use & 1u) ^ 1u, abort_flag, p.status, 22);
           if (!ok) break;
-          tc_fence_after();
-          const uint64_t ad = a_desc0 + (uint64_t)(stage * (stage_bytes >> 4));
-          const uint64_t bd = b_desc0 + (uint64_t)(stage * (stage_bytes >> 4));
-          const int n_mma = (!kTok && kb == kbs - 1) ? last_mmas : kBK / kUmmaK;
-          const uint32_t acc0 = kb > 0 ? 1u : 0u;
-          if (elect_one()) {
-            if (kTok && n2 > 0) {
-#pragma unroll
-              for (int ks = 0; ks < kBK / kUmmaK; ++ks) {
-                tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
-                tc_mma_bf16_pair(d_tmem2, ad + ks * a_kstep, bd + b2_off + ks * b_kstep, idesc2, ks > 0 ? 1u : acc0);
-              }
-            } else {
-#pragma unroll
-              for (int ks = 0; ks < kBK / kUmmaK; ++ks)
-                if (ks == 0 || ks < n_mma)
-                  tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
-            }
-            tc_commit_pair(empty0 + 8u * stage);              // frees this stage in both CTAs
-            if (kb == kbs - 1) tc_commit_pair(tfull0 + 8u * side);   // accumulator complete, in both CTAs
+          // ... and so have the middle columns of the other side's tile, if this tile reaches into them
+          if (kTok && it > 0 && n_prev + t.n > kTmemCols) {
+            ok = mbar_wait_warp(tmid0 + 8u * (side ^ 1u), ((it - 1u) >> 1) & 1u, abort_flag, p.status, 25);
+            if (!ok) break;
           }
-          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+          n_prev = t.n;
+          tc_fence_after();
+          const uint32_t d_tmem = tmem_base + (side ? (uint32_t)(kTmemCols - t.n) : 0u);
+          const uint32_t d_tmem2 = d_tmem + (uint32_t)t.n1;
+#pragma unroll 1
+          for (int kb = 0; kb < kbs; ++kb) {
+            ok = mbar_wait_warp(full0 + 8u * stage, phase, abort_flag, p.status, 23);
+            if (!ok) break;
+            tc_fence_after();
+            const uint64_t ad = a_desc0 + (uint64_t)((kTok ? stage : a_slot) * (stage_bytes >> 4));
+            const uint64_t bd = b_desc0 + (uint64_t)(stage * (stage_bytes >> 4));
+            const int n_mma = (!kTok && kb == kbs - 1) ? last_mmas : kBK / kUmmaK;
+            const uint32_t acc0 = kb > 0 ? 1u : 0u;
+            if (elect_one()) {
+              if (kTok && n2 > 0) {
+#pragma unroll
+                for (int ks = 0; ks < kBK / kUmmaK; ++ks) {
+                  tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
+                  tc_mma_bf16_pair(d_tmem2, ad + ks * a_kstep, bd + b2_off + ks * b_kstep, idesc2, ks > 0 ? 1u : acc0);
+                }
+              } else {
+#pragma unroll
+                for (int ks = 0; ks < kBK / kUmmaK; ++ks)
+                  if (ks == 0 || ks < n_mma)
+                    tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
+              }
+              tc_commit_pair(empty0 + 8u * stage);              // frees this stage in both CTAs
+              if (free_a) tc_commit_pair(aempty0 + 8u * a_slot);
+              if (kb == kbs - 1) tc_commit_pair(tfull0 + 8u * side);   // accumulator complete, in both CTAs
+            }
+            if (++stage == n_stages) { stage = 0; phase ^= 1u; }
+            if (!kTok && ++a_slot == (uint32_t)kPWgradA) a_slot = 0;
+          }
+          if (!ok) break;
+          if (free_a) a_first = a_slot;
+          if (kbs <= 0 && lane == 0) {                          // nothing to contract: epilogues write zeros
+            mbar_arrive(tfull0 + 8u * side);
+            mbar_arrive_remote(tfull0 + 8u * side, 1);
+          }
         }
+      }
+    }
+  } else if constexpr (!kTok) {
+    // --------------------------------------------------------------- epilogue warps (both CTAs), weight gradients
+    // Rows of the output are lanes of the accumulator.  A warp drains its 32 rows x 2 chunks of 64 columns in four units
+    // of 16 rows: read as matrix fragments, rounded, stored as 8 x 8 matrices into 128-byte rows (16-byte pieces
+    // exchanged by the row), written to memory as whole lines; the next unit's accumulator is in flight meanwhile.  The
+    // stores bound it: without them a 768 x 3072 x 128 launch takes 130 us, with them 172 (with 32-lane row reads and half
+    // warps storing in turn 154 and 172); 604 MB of output alone are 82 us of pure writes.
+    const int lg = warp & 3, half = (warp - 2) >> 2;
+    uint8_t* tr = trans_gen + (warp - 2) * kPTransWarp;
+    const uint32_t sa = smem_u32(tr) + (uint32_t)((lane & 15) * 128), sx = lane & 7, sq = lane >> 4;
+    const int rr0 = lane >> 3, chunk = lane & 7;
+    uint32_t it = 0;
+    bool ok = true;
+    for (int id = pair; id < n_tiles && ok; id += n_pairs) {
+      const PTile t = p_decode(p, id, kept_s, tile_s);
+      const int m_warp = t.m0 + 128 * (int)rank + 32 * lg;
+      const bool have_acc = t.k_blocks > 0, m_ok = m_warp < p.Mw;
+#pragma unroll 1
+      for (int j = 0; j < t.tiles; ++j, ++it) {
+        const uint32_t side = it & 1u, use = it >> 1;
+        const uint32_t t_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + (side ? 256u : 0u);
+        uint32_t v[32];
+        auto load_unit = [&](int u) {
+          const uint32_t at = t_addr + ((uint32_t)(16 * (u & 1)) << 16) + (uint32_t)((half + (u & 2)) * 64);
+          tc_ld_16x256b_x4(at, v);
+          tc_ld_16x256b_x4(at + 32u, v + 16);
+        };
+        ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
         if (!ok) break;
-        if (kbs <= 0 && lane == 0) {                          // nothing to contract: epilogues write zeros
-          mbar_arrive(tfull0 + 8u * side);
-          mbar_arrive_remote(tfull0 + 8u * side, 1);
+        tc_fence_after();
+        if (have_acc) load_unit(0);
+        else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) v[i] = 0u;
+        }
+        const int n0 = t.n0 + 256 * j + half * 64;              // (rows and columns come in multiples of 64)
+        __nv_bfloat16* o = p.out + ((long long)t.e * p.Mw + m_warp + rr0) * p.ld_out + n0 + chunk * 8;
+#pragma unroll 2
+        for (int u = 0; u < 4; ++u) {
+          if (have_acc) tc_wait_ld_regs(v);
+          if (u == 3) {                                         // accumulator read out
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_remote(tempty0 + 8u * side, 0);
+          }
+          uint32_t pk[16];
+#pragma unroll
+          for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+          if (have_acc && u < 3) load_unit(u + 1);
+          __syncwarp();
+#pragma unroll
+          for (int g = 0; g < 4; ++g)                           // 16-byte pieces 2 g and 2 g + 1 of rows 0-7 and 8-15
+            stmatrix_x4(sa + (((2u * g + sq) ^ sx) << 4), pk + 4 * g);
+          __syncwarp();
+          const bool inside = m_ok && n0 + (u & 2) * 64 < p.Nfix;
+          __nv_bfloat16* ou = o + (long long)(16 * (u & 1)) * p.ld_out + (u & 2) * 64;
+#pragma unroll
+          for (int st = 0; st < 4; ++st) {
+            const int rr = st * 4 + rr0;
+            const uint4 val = *reinterpret_cast<const uint4*>(tr + rr * 128 + ((chunk ^ (rr & 7)) << 4));
+            if (inside) *reinterpret_cast<uint4*>(ou + (long long)(4 * st) * p.ld_out) = val;
+          }
         }
       }
     }
   } else {
-    // ------------------------------------------------------------------------------------------ epilogue warps (both CTAs)
+    // --------------------------------------------------------------- epilogue warps (both CTAs), token products
     const int lg = warp & 3;
     const int half = (warp - 2) >> 2;
     uint8_t* tr = trans_gen + (warp - 2) * kPTransWarp;       // this warp's transpose tile
@@ -433,330 +541,273 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
       const int m_warp = kGated ? role * p.gate_f + unit0 : t.m0 + 128 * (int)rank + 32 * lg;
       const int c0 = side ? kTmemCols - t.n : 0;              // first accumulator column of the tile
       const uint32_t t_addr = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)c0;
-      if constexpr (!kTok) {
-        // ---- weight gradient: rows of the output are this warp's lanes
-        const bool have_acc = t.k_blocks > 0;
-        ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
-        if (!ok) break;
-        tc_fence_after();
+      // Chunks are numbered so that chunk j of an even tile holds the tile's tokens [32 j, 32 j + 32) and chunk j of an
+      // odd tile its tokens [n - 32 (j + 1), n - 32 j): a chunk is then always inside the 512 columns, and counting j
+      // down from the last chunk starts in the middle columns, the ones the next tile may also use.  This warp's chunks
+      // are j = n_chunks - 1 - half, then every second one down to 0.
+      constexpr bool kSlotRows = (OP == kGemm1Relu || kGated || OP == kDgrad2Mask || kDGated);
+      constexpr int kQueue = 5;                              // (320 / 32) chunks over two warps
+      const int n_chunks = (t.n + 31) >> 5;
+      const bool m_ok = kGated ? unit0 < p.gate_f : m_warp < p.Mw;   // (weight rows come in multiples of 64)
+      const int kept_e = kept_s[t.e];
+      const int row_limit = kSlotRows ? min(p.C, (kept_e + 15) / 16 * 16) : kept_e;
+      const int id_next = id + n_pairs;
+      const int n_next = id_next < n_tiles ? p_decode(p, id_next, kept_s, tile_s).n : 0;
+      const int j_mid = (t.n - max(0, t.n + n_next - kTmemCols)) >> 5;   // chunks j >= j_mid: columns the next tile uses too
+      __nv_bfloat16* out_rows = p.out + ((long long)t.e * p.C + t.row0) * p.ld_out;   // slot-row products: the tile's first row
+      auto chunk_tok0 = [&](int j) { return side ? t.n - 32 * (j + 1) : 32 * j; };
+      auto row_ok = [&](int col) { return col >= 0 && col < t.n && t.row0 + col < row_limit; };
+      // 16-token blocks of 32 hidden units: what GEMM1 saves for dgrad2 is kept per block in fragment order.  block0 is the
+      // block of the tile's first token; 16 tokens further is hid / 32 blocks further.
+      const int words = p.hid >> 5;
+      const long long block0 = ((long long)t.e * p.cb + (t.row0 >> 4)) * words + ((kGated ? unit0 : m_warp) >> 5);
+      auto block_ok = [&](int col) { return m_ok && col >= 0 && col < t.n; };
+      // Everything the epilogue needs from global memory is requested here, before the accumulator is awaited; head of a
+      // queue = next chunk to process.  Lane i of a chunk describes its token column i: the token (scatter products), its
+      // gate, its dropout word.  dgrad2: ReLU mask bits of this thread's fragment, two blocks of 16 tokens.
+      int q_tok[kQueue] = {-1, -1, -1, -1, -1};
+      float q_gate[kQueue] = {1.f, 1.f, 1.f, 1.f, 1.f};
+      uint32_t q_mw[kQueue] = {0u, 0u, 0u, 0u, 0u};
+      if constexpr (!kSlotRows) {
+        const int* tos = p.token_of_slot + (long long)t.e * p.C + t.row0;
+#pragma unroll
+        for (int k = 0; k < kQueue; ++k) {
+          const int j = n_chunks - 1 - half - 2 * k, col = chunk_tok0(j) + lane;
+          q_tok[k] = j >= 0 && row_ok(col) ? tos[col] : -1;
+        }
+        if (OP == kGemm2Combine) {                            // Eq. 2: y = p_i(x) E_i(x)
+#pragma unroll
+          for (int k = 0; k < kQueue; ++k) q_gate[k] = p.gate[max(q_tok[k], 0)];
+        }
+      }
+      if constexpr (DROP && (OP == kGemm1Relu || kGated)) {   // 32 hidden units are one word per row
+        const uint32_t* keep = p.keep_bits + ((long long)t.e * p.C + t.row0) * p.keep_words + ((kGated ? unit0 : m_warp) >> 5);
+#pragma unroll
+        for (int k = 0; k < kQueue; ++k) {
+          const int j = n_chunks - 1 - half - 2 * k, col = chunk_tok0(j) + lane;
+          q_mw[k] = j >= 0 && m_ok && row_ok(col) ? keep[(long long)col * p.keep_words] : 0u;
+        }
+      }
+      if constexpr (OP == kDgrad2Mask) {
+        const uint16_t* hm = p.hmask + block0 * 32 + lane;
+#pragma unroll
+        for (int k = 0; k < kQueue; ++k) {
+          const int j = n_chunks - 1 - half - 2 * k, tok0 = chunk_tok0(j);
+          const uint32_t b0 = j >= 0 && block_ok(tok0) ? hm[(long long)(tok0 >> 4) * p.hid] : 0u;
+          const uint32_t b1 = j >= 0 && block_ok(tok0 + 16) ? hm[(long long)((tok0 >> 4) + 1) * p.hid] : 0u;
+          q_mw[k] = b0 | (b1 << 16);
+        }
+      }
+      // gated dgrad2: the saved factors of this thread's fragment ({GELU(a), b GELU'(a)} as two bfloat16 per element)
+      uint4 gg[kDGated ? 8 : 1];
+      auto fetch_factors = [&](int j) {
+        if constexpr (kDGated) {
+#pragma unroll
+          for (int b = 0; b < 2; ++b) {
+            const int col = chunk_tok0(j) + 16 * b;
+            const bool valid = j >= 0 && block_ok(col);
+            const uint4* src = p.gate_buf + (valid ? (block0 + (long long)(col >> 4) * words) * 128 + lane : 0);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) gg[4 * b + q] = valid ? src[32 * q] : make_uint4(0, 0, 0, 0);
+          }
+        }
+      };
+      fetch_factors(n_chunks - 1 - half);
+      ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
+      if (!ok) break;
+      tc_fence_after();
+      bool released = false, mid_sent = false;
+      uint32_t v[32];                                         // [16 h + 4 g + ..]: weight rows 16 h .., tokens 8 g ..
+      auto load_acc = [&](int j) {
+        const uint32_t at = t_addr + (uint32_t)chunk_tok0(j);  // (-16 in an odd tile's last chunk: the columns before it)
+        tc_ld_16x256b_x4(at, v);
+        tc_ld_16x256b_x4(at + (16u << 16), v + 16);
+      };
+      auto value = [&](int g, int i, int b) { return __uint_as_float(v[16 * (i >> 1) + 4 * g + 2 * (i & 1) + b]); };
+      if (m_ok && n_chunks - 1 - half >= 0) load_acc(n_chunks - 1 - half);
 #pragma unroll 1
-        for (int c = half; c < 4; c += 2) {
-          uint32_t v[64];
-          if (have_acc) {
-            tc_ld32(t_addr + c * 64, v);
-            tc_ld32(t_addr + c * 64 + 32, v + 32);
-            tc_wait_ld();
-          } else {
-#pragma unroll
-            for (int i = 0; i < 64; ++i) v[i] = 0u;
-          }
-          if (c + 2 >= 4) {                                   // last chunk of this warp: accumulator read out
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote(tempty0 + 8u * side, 0);
-          }
-          uint4 ch[8];
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            uint32_t w[4];
-#pragma unroll
-            for (int h = 0; h < 4; ++h) {
-              __nv_bfloat162 h2 = __floats2bfloat162_rn(__uint_as_float(v[q * 8 + 2 * h]),
-                                                        __uint_as_float(v[q * 8 + 2 * h + 1]));
-              w[h] = *reinterpret_cast<uint32_t*>(&h2);
-            }
-            ch[q] = make_uint4(w[0], w[1], w[2], w[3]);
-          }
-          const int chunk = lane & 7;
-          const int col = t.n0 + c * 64 + chunk * 8;
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-            if ((lane >> 4) == hf) {
-#pragma unroll
-              for (int q = 0; q < 8; ++q)
-                *reinterpret_cast<uint4*>(tr + (lane & 15) * 128 + ((q ^ (lane & 7)) << 4)) = ch[q];
-            }
-            __syncwarp();
-#pragma unroll
-            for (int st = 0; st < 4; ++st) {
-              const int rr = st * 4 + (lane >> 3);
-              const uint4 val = *reinterpret_cast<const uint4*>(tr + rr * 128 + ((chunk ^ (rr & 7)) << 4));
-              const int orow = m_warp + hf * 16 + rr;
-              if (orow < p.Mw && col < p.Nfix)
-                *reinterpret_cast<uint4*>(p.out + ((long long)t.e * p.Mw + orow) * p.ld_out + col) = val;
-            }
-            __syncwarp();
-          }
-        }
-      } else {
-        // Chunks are numbered so that chunk j of an even tile holds the tile's tokens [32 j, 32 j + 32) and chunk j of an
-        // odd tile its tokens [n - 32 (j + 1), n - 32 j): a chunk is then always inside the 512 columns, and counting j
-        // down from the last chunk starts in the middle columns, the ones the next tile may also use.  This warp's chunks
-        // are j = n_chunks - 1 - half, then every second one down to 0.
-        constexpr bool kSlotRows = (OP == kGemm1Relu || kGated || OP == kDgrad2Mask || kDGated);
-        constexpr int kQueue = 5;                              // (320 / 32) chunks over two warps
-        const int n_chunks = (t.n + 31) >> 5;
-        const bool m_ok = kGated ? unit0 < p.gate_f : m_warp < p.Mw;   // (weight rows come in multiples of 64)
-        const int kept_e = kept_s[t.e];
-        const int row_limit = kSlotRows ? min(p.C, (kept_e + 15) / 16 * 16) : kept_e;
-        const int id_next = id + n_pairs;
-        const int n_next = id_next < n_tiles ? p_decode(p, id_next, kept_s, tile_s).n : 0;
-        const int j_mid = (t.n - max(0, t.n + n_next - kTmemCols)) >> 5;   // chunks j >= j_mid: columns the next tile uses too
-        __nv_bfloat16* out_rows = p.out + ((long long)t.e * p.C + t.row0) * p.ld_out;   // slot-row products: the tile's first row
-        auto chunk_tok0 = [&](int j) { return side ? t.n - 32 * (j + 1) : 32 * j; };
-        auto row_ok = [&](int col) { return col >= 0 && col < t.n && t.row0 + col < row_limit; };
-        // 16-token blocks of 32 hidden units: what GEMM1 saves for dgrad2 is kept per block in fragment order.  block0 is the
-        // block of the tile's first token; 16 tokens further is hid / 32 blocks further.
-        const int words = p.hid >> 5;
-        const long long block0 = ((long long)t.e * p.cb + (t.row0 >> 4)) * words + ((kGated ? unit0 : m_warp) >> 5);
-        auto block_ok = [&](int col) { return m_ok && col >= 0 && col < t.n; };
-        // Everything the epilogue needs from global memory is requested here, before the accumulator is awaited; head of a
-        // queue = next chunk to process.  Lane i of a chunk describes its token column i: the token (scatter products), its
-        // gate, its dropout word.  dgrad2: ReLU mask bits of this thread's fragment, two blocks of 16 tokens.
-        int q_tok[kQueue] = {-1, -1, -1, -1, -1};
-        float q_gate[kQueue] = {1.f, 1.f, 1.f, 1.f, 1.f};
-        uint32_t q_mw[kQueue] = {0u, 0u, 0u, 0u, 0u};
-        if constexpr (!kSlotRows) {
-          const int* tos = p.token_of_slot + (long long)t.e * p.C + t.row0;
-#pragma unroll
-          for (int k = 0; k < kQueue; ++k) {
-            const int j = n_chunks - 1 - half - 2 * k, col = chunk_tok0(j) + lane;
-            q_tok[k] = j >= 0 && row_ok(col) ? tos[col] : -1;
-          }
-          if (OP == kGemm2Combine) {                            // Eq. 2: y = p_i(x) E_i(x)
-#pragma unroll
-            for (int k = 0; k < kQueue; ++k) q_gate[k] = p.gate[max(q_tok[k], 0)];
-          }
-        }
-        if constexpr (DROP && (OP == kGemm1Relu || kGated)) {   // 32 hidden units are one word per row
-          const uint32_t* keep = p.keep_bits + ((long long)t.e * p.C + t.row0) * p.keep_words + ((kGated ? unit0 : m_warp) >> 5);
-#pragma unroll
-          for (int k = 0; k < kQueue; ++k) {
-            const int j = n_chunks - 1 - half - 2 * k, col = chunk_tok0(j) + lane;
-            q_mw[k] = j >= 0 && m_ok && row_ok(col) ? keep[(long long)col * p.keep_words] : 0u;
-          }
-        }
-        if constexpr (OP == kDgrad2Mask) {
-          const uint16_t* hm = p.hmask + block0 * 32 + lane;
-#pragma unroll
-          for (int k = 0; k < kQueue; ++k) {
-            const int j = n_chunks - 1 - half - 2 * k, tok0 = chunk_tok0(j);
-            const uint32_t b0 = j >= 0 && block_ok(tok0) ? hm[(long long)(tok0 >> 4) * p.hid] : 0u;
-            const uint32_t b1 = j >= 0 && block_ok(tok0 + 16) ? hm[(long long)((tok0 >> 4) + 1) * p.hid] : 0u;
-            q_mw[k] = b0 | (b1 << 16);
-          }
-        }
-        // gated dgrad2: the saved factors of this thread's fragment ({GELU(a), b GELU'(a)} as two bfloat16 per element)
-        uint4 gg[kDGated ? 8 : 1];
-        auto fetch_factors = [&](int j) {
-          if constexpr (kDGated) {
-#pragma unroll
-            for (int b = 0; b < 2; ++b) {
-              const int col = chunk_tok0(j) + 16 * b;
-              const bool valid = j >= 0 && block_ok(col);
-              const uint4* src = p.gate_buf + (valid ? (block0 + (long long)(col >> 4) * words) * 128 + lane : 0);
-#pragma unroll
-              for (int q = 0; q < 4; ++q) gg[4 * b + q] = valid ? src[32 * q] : make_uint4(0, 0, 0, 0);
-            }
-          }
-        };
-        fetch_factors(n_chunks - 1 - half);
-        ok = mbar_wait_warp(tfull0 + 8u * side, use & 1u, abort_flag, p.status, 24);
-        if (!ok) break;
-        tc_fence_after();
-        bool released = false, mid_sent = false;
-        uint32_t v[32];                                         // [16 h + 4 g + ..]: weight rows 16 h .., tokens 8 g ..
-        auto load_acc = [&](int j) {
-          const uint32_t at = t_addr + (uint32_t)chunk_tok0(j);  // (-16 in an odd tile's last chunk: the columns before it)
-          tc_ld_16x256b_x4(at, v);
-          tc_ld_16x256b_x4(at + (16u << 16), v + 16);
-        };
-        auto value = [&](int g, int i, int b) { return __uint_as_float(v[16 * (i >> 1) + 4 * g + 2 * (i & 1) + b]); };
-        if (m_ok && n_chunks - 1 - half >= 0) load_acc(n_chunks - 1 - half);
-#pragma unroll 1
-        for (int j = n_chunks - 1 - half; j >= 0 && m_ok; j -= 2) {
-          const int tok0 = chunk_tok0(j);
-          tc_wait_ld_regs(v);
-          if (!mid_sent && j - 2 < j_mid) {                     // this warp's share of the middle columns is read out
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote(tmid0 + 8u * side, 0);
-            mid_sent = true;
-          }
-          if (j - 2 < 0) {                                      // last chunk of this warp: accumulator read out
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_remote(tempty0 + 8u * side, 0);
-            released = true;
-          }
-          if constexpr (kGated) {
-            // GEGLU gating.  Both warps of a pair round their values (a or b of 32 hidden units x 32 tokens); the a warp
-            // gates the chunk's first 16 tokens, the b warp the others: each hands the other its half through its tile,
-            // between two handshakes.
-            uint32_t mine[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {                       // word 4 g + i of this warp's block, and of the other's
-              const int g = k >> 2, i = k & 3;
-              const uint32_t w0 = pack_bf16(value(g, i, 0), value(g, i, 1)), w1 = pack_bf16(value(g + 2, i, 0), value(g + 2, i, 1));
-              mine[k] = role ? w1 : w0;
-              *reinterpret_cast<uint32_t*>(tr + k * 128 + lane * 4) = role ? w0 : w1;
-            }
-            if (j - 2 >= 0) load_acc(j - 2);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(gate_bar);
-            ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 26);     // both tiles are written
-            gate_phase ^= 1u;
-            if (!ok) break;
-            uint32_t other[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) other[k] = *reinterpret_cast<const uint32_t*>(tr_other + k * 128 + lane * 4);
-            __syncwarp();
-            if (lane == 0) mbar_arrive(gate_bar);
-            ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 27);     // both tiles have been read
-            gate_phase ^= 1u;
-            if (!ok) break;
-            const int col0 = tok0 + 16 * role;                  // this warp's block of 16 tokens
-            uint32_t fac[16], hw[8];
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-              const int g = k >> 2, i = k & 3;
-              const uint32_t aw = role ? other[k] : mine[k], bw = role ? mine[k] : other[k];
-              const float2 af = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw));
-              const float2 bf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw));
-              float cdf0, pdf0, cdf1, pdf1;
-              gelu_cdf_pdf(af.x, &cdf0, &pdf0);
-              gelu_cdf_pdf(af.y, &cdf1, &pdf1);
-              float ga0 = af.x * cdf0, ga1 = af.y * cdf1;
-              float gp0 = bf.x * fmaf(af.x, pdf0, cdf0), gp1 = bf.y * fmaf(af.y, pdf1, cdf1);
-              if (DROP) {                                       // expert dropout: the hidden unit's factor on all three
-                const int tk = 16 * role + 8 * g + 2 * (lane & 3), unit = 8 * i + (lane >> 2);
-                const uint32_t kw0 = __shfl_sync(0xffffffffu, q_mw[0], tk), kw1 = __shfl_sync(0xffffffffu, q_mw[0], tk + 1);
-                const float f0 = (kw0 >> unit) & 1u ? p.keep_scale : 0.f, f1 = (kw1 >> unit) & 1u ? p.keep_scale : 0.f;
-                ga0 *= f0; gp0 *= f0; ga1 *= f1; gp1 *= f1;
-              }
-              fac[2 * k] = pack_bf16(ga0, gp0);
-              fac[2 * k + 1] = pack_bf16(ga1, gp1);
-              hw[k] = pack_bf16(ga0 * bf.x, ga1 * bf.y);
-            }
-            if (block_ok(col0)) {
-              uint4* dst = p.gate_buf + (block0 + (long long)(col0 >> 4) * words) * 128 + lane;
-#pragma unroll
-              for (int q = 0; q < 4; ++q) dst[32 * q] = make_uint4(fac[4 * q], fac[4 * q + 1], fac[4 * q + 2], fac[4 * q + 3]);
-            }
-#pragma unroll
-            for (int g = 0; g < 2; ++g) stmatrix_trans(st_addr + 512u * g, hw + 4 * g);
-            __syncwarp();
-#pragma unroll
-            for (int g = 0; g < 2; ++g) {
-              const uint4 val = *reinterpret_cast<const uint4*>(ld_addr + 512 * g);
-              const int col = col0 + 8 * g + (lane >> 2);
-              if (row_ok(col)) *reinterpret_cast<uint4*>(out_rows + (long long)col * p.ld_out + unit0 + (lane & 3) * 8) = val;
-            }
-          } else {
-            constexpr int kSets = kDGated ? 2 : 1;              // gated dgrad2 writes d a and d b from one accumulator
-            uint32_t pk[kSets][16];
-            // dgrad2: a block's bits with the even tokens' in the low half, the odd ones' in the high half
-            const uint32_t mask[2] = {__byte_perm(q_mw[0], 0, 0x4140), __byte_perm(q_mw[0], 0, 0x4342)};
-            if (OP == kGemm2Combine) { gate_s[lane] = q_gate[0]; __syncwarp(); }
-#pragma unroll
-            for (int g = 0; g < 4; ++g) {
-              float2 ga = make_float2(1.f, 1.f);
-              if (OP == kGemm2Combine) ga = *reinterpret_cast<const float2*>(gate_s + 8 * g + 2 * (lane & 3));
-              uint32_t kw0 = 0u, kw1 = 0u;
-              if (DROP && OP == kGemm1Relu) {                   // expert dropout before the rounding and the mask bits
-                kw0 = __shfl_sync(0xffffffffu, q_mw[0], 8 * g + 2 * (lane & 3));
-                kw1 = __shfl_sync(0xffffffffu, q_mw[0], 8 * g + 2 * (lane & 3) + 1);
-              }
-#pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                float x = value(g, i, 0), y = value(g, i, 1);
-                if (OP == kGemm2Combine) { x *= ga.x; y *= ga.y; }
-                if (DROP && OP == kGemm1Relu) {
-                  const int unit = 8 * i + (lane >> 2);
-                  x = (kw0 >> unit) & 1u ? x * p.keep_scale : 0.f;
-                  y = (kw1 >> unit) & 1u ? y * p.keep_scale : 0.f;
-                }
-                if (DROP && OP == kDgrad2Mask) { x *= p.keep_scale; y *= p.keep_scale; }
-                if constexpr (kDGated) {                        // high half: b GELU'(a); low half: GELU(a)
-                  const uint4 f4 = gg[4 * (g >> 1) + 2 * (g & 1) + (i >> 1)];
-                  const uint32_t f0 = i & 1 ? f4.z : f4.x, f1 = i & 1 ? f4.w : f4.y;
-                  pk[0][4 * g + i] = pack_bf16(x * __uint_as_float(f0 & 0xFFFF0000u), y * __uint_as_float(f1 & 0xFFFF0000u));
-                  pk[kSets - 1][4 * g + i] = pack_bf16(x * __uint_as_float(f0 << 16), y * __uint_as_float(f1 << 16));
-                } else {
-                  uint32_t w = pack_bf16(x, y);
-                  if (OP == kGemm1Relu) w = relu_bf16x2(w);
-                  if (OP == kDgrad2Mask)                        // ReLU'(u) = [u > 0]: bits saved by the forward GEMM
-                    w &= ((mask[g >> 1] >> (4 * (g & 1) + i)) & 0x00010001u) * 0xFFFFu;
-                  pk[0][4 * g + i] = w;
-                }
-              }
-            }
-            if (j - 2 >= 0) load_acc(j - 2);                    // in flight while this chunk is stored
-            fetch_factors(j - 2);
-            if (OP == kGemm1Relu) {                             // save [H > 0], one bit per element, in fragment order
-#pragma unroll
-              for (int b = 0; b < 2; ++b) {
-                uint32_t bits = 0;
-#pragma unroll
-                for (int k = 0; k < 8; ++k) bits |= positive_bf16x2(pk[0][8 * b + k]) & (0x00010001u << k);
-                if (block_ok(tok0 + 16 * b))
-                  p.hmask[block0 * 32 + (long long)((tok0 >> 4) + b) * p.hid + lane] = (uint16_t)((bits & 0xFFu) | (bits >> 8));
-              }
-            }
-#pragma unroll
-            for (int set = 0; set < kSets; ++set) {
-              if (set > 0) __syncwarp();                        // the tile's readers of the first set are done
-#pragma unroll
-              for (int g = 0; g < 4; ++g) stmatrix_trans(st_addr + 512u * g, pk[set] + 4 * g);
-              __syncwarp();
-              const int mcol = m_warp + (lane & 3) * 8 + set * p.gate_f;
-#pragma unroll
-              for (int g = 0; g < 4; ++g) {
-                uint4 val = *reinterpret_cast<const uint4*>(ld_addr + 512 * g);
-                if (kSlotRows) {
-                  const int col = tok0 + 8 * g + (lane >> 2);
-                  if (row_ok(col)) *reinterpret_cast<uint4*>(out_rows + (long long)col * p.ld_out + mcol) = val;
-                } else {
-                  const int tok = __shfl_sync(0xffffffffu, q_tok[0], 8 * g + (lane >> 2));
-                  if (tok >= 0) {
-                    const long long off = (long long)tok * p.ld_out + mcol;
-                    if (p.res != nullptr) {
-                      // skip path inside the layer: y = x + g E(x), dx = dy + dH W_in^T (the expert term is already bf16)
-                      if (OP == kGemm2Combine) *reinterpret_cast<uint4*>(p.out2 + off) = val;
-                      const uint4 r = *reinterpret_cast<const uint4*>(p.res + off);
-                      const __nv_bfloat162* rv = reinterpret_cast<const __nv_bfloat162*>(&r);
-                      __nv_bfloat162* vv = reinterpret_cast<__nv_bfloat162*>(&val);
-#pragma unroll
-                      for (int q = 0; q < 4; ++q) {
-                        const float2 a2 = __bfloat1622float2(vv[q]), b2 = __bfloat1622float2(rv[q]);
-                        vv[q] = __floats2bfloat162_rn(a2.x + b2.x, a2.y + b2.y);
-                      }
-                    }
-                    *reinterpret_cast<uint4*>(p.out + off) = val;
-                  }
-                }
-              }
-            }
-          }
-#pragma unroll
-          for (int k = 0; k < kQueue - 1; ++k) {                // advance the queue
-            q_tok[k] = q_tok[k + 1];
-            q_gate[k] = q_gate[k + 1];
-            q_mw[k] = q_mw[k + 1];
-          }
-          __syncwarp();
-        }
-        if (!ok) break;
-        if (!mid_sent) {                                        // this warp had no chunk in this tile
+      for (int j = n_chunks - 1 - half; j >= 0 && m_ok; j -= 2) {
+        const int tok0 = chunk_tok0(j);
+        tc_wait_ld_regs(v);
+        if (!mid_sent && j - 2 < j_mid) {                     // this warp's share of the middle columns is read out
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_remote(tmid0 + 8u * side, 0);
+          mid_sent = true;
         }
-        if (!released) {
+        if (j - 2 < 0) {                                      // last chunk of this warp: accumulator read out
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive_remote(tempty0 + 8u * side, 0);
+          released = true;
         }
+        if constexpr (kGated) {
+          // GEGLU gating.  Both warps of a pair round their values (a or b of 32 hidden units x 32 tokens); the a warp
+          // gates the chunk's first 16 tokens, the b warp the others: each hands the other its half through its tile,
+          // between two handshakes.
+          uint32_t mine[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {                       // word 4 g + i of this warp's block, and of the other's
+            const int g = k >> 2, i = k & 3;
+            const uint32_t w0 = pack_bf16(value(g, i, 0), value(g, i, 1)), w1 = pack_bf16(value(g + 2, i, 0), value(g + 2, i, 1));
+            mine[k] = role ? w1 : w0;
+            *reinterpret_cast<uint32_t*>(tr + k * 128 + lane * 4) = role ? w0 : w1;
+          }
+          if (j - 2 >= 0) load_acc(j - 2);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(gate_bar);
+          ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 26);     // both tiles are written
+          gate_phase ^= 1u;
+          if (!ok) break;
+          uint32_t other[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) other[k] = *reinterpret_cast<const uint32_t*>(tr_other + k * 128 + lane * 4);
+          __syncwarp();
+          if (lane == 0) mbar_arrive(gate_bar);
+          ok = mbar_wait_warp(gate_bar, gate_phase, abort_flag, p.status, 27);     // both tiles have been read
+          gate_phase ^= 1u;
+          if (!ok) break;
+          const int col0 = tok0 + 16 * role;                  // this warp's block of 16 tokens
+          uint32_t fac[16], hw[8];
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int g = k >> 2, i = k & 3;
+            const uint32_t aw = role ? other[k] : mine[k], bw = role ? mine[k] : other[k];
+            const float2 af = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&aw));
+            const float2 bf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&bw));
+            float cdf0, pdf0, cdf1, pdf1;
+            gelu_cdf_pdf(af.x, &cdf0, &pdf0);
+            gelu_cdf_pdf(af.y, &cdf1, &pdf1);
+            float ga0 = af.x * cdf0, ga1 = af.y * cdf1;
+            float gp0 = bf.x * fmaf(af.x, pdf0, cdf0), gp1 = bf.y * fmaf(af.y, pdf1, cdf1);
+            if (DROP) {                                       // expert dropout: the hidden unit's factor on all three
+              const int tk = 16 * role + 8 * g + 2 * (lane & 3), unit = 8 * i + (lane >> 2);
+              const uint32_t kw0 = __shfl_sync(0xffffffffu, q_mw[0], tk), kw1 = __shfl_sync(0xffffffffu, q_mw[0], tk + 1);
+              const float f0 = (kw0 >> unit) & 1u ? p.keep_scale : 0.f, f1 = (kw1 >> unit) & 1u ? p.keep_scale : 0.f;
+              ga0 *= f0; gp0 *= f0; ga1 *= f1; gp1 *= f1;
+            }
+            fac[2 * k] = pack_bf16(ga0, gp0);
+            fac[2 * k + 1] = pack_bf16(ga1, gp1);
+            hw[k] = pack_bf16(ga0 * bf.x, ga1 * bf.y);
+          }
+          if (block_ok(col0)) {
+            uint4* dst = p.gate_buf + (block0 + (long long)(col0 >> 4) * words) * 128 + lane;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dst[32 * q] = make_uint4(fac[4 * q], fac[4 * q + 1], fac[4 * q + 2], fac[4 * q + 3]);
+          }
+#pragma unroll
+          for (int g = 0; g < 2; ++g) stmatrix_trans(st_addr + 512u * g, hw + 4 * g);
+          __syncwarp();
+#pragma unroll
+          for (int g = 0; g < 2; ++g) {
+            const uint4 val = *reinterpret_cast<const uint4*>(ld_addr + 512 * g);
+            const int col = col0 + 8 * g + (lane >> 2);
+            if (row_ok(col)) *reinterpret_cast<uint4*>(out_rows + (long long)col * p.ld_out + unit0 + (lane & 3) * 8) = val;
+          }
+        } else {
+          constexpr int kSets = kDGated ? 2 : 1;              // gated dgrad2 writes d a and d b from one accumulator
+          uint32_t pk[kSets][16];
+          // dgrad2: a block's bits with the even tokens' in the low half, the odd ones' in the high half
+          const uint32_t mask[2] = {__byte_perm(q_mw[0], 0, 0x4140), __byte_perm(q_mw[0], 0, 0x4342)};
+          if (OP == kGemm2Combine) { gate_s[lane] = q_gate[0]; __syncwarp(); }
+#pragma unroll
+          for (int g = 0; g < 4; ++g) {
+            float2 ga = make_float2(1.f, 1.f);
+            if (OP == kGemm2Combine) ga = *reinterpret_cast<const float2*>(gate_s + 8 * g + 2 * (lane & 3));
+            uint32_t kw0 = 0u, kw1 = 0u;
+            if (DROP && OP == kGemm1Relu) {                   // expert dropout before the rounding and the mask bits
+              kw0 = __shfl_sync(0xffffffffu, q_mw[0], 8 * g + 2 * (lane & 3));
+              kw1 = __shfl_sync(0xffffffffu, q_mw[0], 8 * g + 2 * (lane & 3) + 1);
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              float x = value(g, i, 0), y = value(g, i, 1);
+              if (OP == kGemm2Combine) { x *= ga.x; y *= ga.y; }
+              if (DROP && OP == kGemm1Relu) {
+                const int unit = 8 * i + (lane >> 2);
+                x = (kw0 >> unit) & 1u ? x * p.keep_scale : 0.f;
+                y = (kw1 >> unit) & 1u ? y * p.keep_scale : 0.f;
+              }
+              if (DROP && OP == kDgrad2Mask) { x *= p.keep_scale; y *= p.keep_scale; }
+              if constexpr (kDGated) {                        // high half: b GELU'(a); low half: GELU(a)
+                const uint4 f4 = gg[4 * (g >> 1) + 2 * (g & 1) + (i >> 1)];
+                const uint32_t f0 = i & 1 ? f4.z : f4.x, f1 = i & 1 ? f4.w : f4.y;
+                pk[0][4 * g + i] = pack_bf16(x * __uint_as_float(f0 & 0xFFFF0000u), y * __uint_as_float(f1 & 0xFFFF0000u));
+                pk[kSets - 1][4 * g + i] = pack_bf16(x * __uint_as_float(f0 << 16), y * __uint_as_float(f1 << 16));
+              } else {
+                uint32_t w = pack_bf16(x, y);
+                if (OP == kGemm1Relu) w = relu_bf16x2(w);
+                if (OP == kDgrad2Mask)                        // ReLU'(u) = [u > 0]: bits saved by the forward GEMM
+                  w &= ((mask[g >> 1] >> (4 * (g & 1) + i)) & 0x00010001u) * 0xFFFFu;
+                pk[0][4 * g + i] = w;
+              }
+            }
+          }
+          if (j - 2 >= 0) load_acc(j - 2);                    // in flight while this chunk is stored
+          fetch_factors(j - 2);
+          if (OP == kGemm1Relu) {                             // save [H > 0], one bit per element, in fragment order
+#pragma unroll
+            for (int b = 0; b < 2; ++b) {
+              uint32_t bits = 0;
+#pragma unroll
+              for (int k = 0; k < 8; ++k) bits |= positive_bf16x2(pk[0][8 * b + k]) & (0x00010001u << k);
+              if (block_ok(tok0 + 16 * b))
+                p.hmask[block0 * 32 + (long long)((tok0 >> 4) + b) * p.hid + lane] = (uint16_t)((bits & 0xFFu) | (bits >> 8));
+            }
+          }
+#pragma unroll
+          for (int set = 0; set < kSets; ++set) {
+            if (set > 0) __syncwarp();                        // the tile's readers of the first set are done
+#pragma unroll
+            for (int g = 0; g < 4; ++g) stmatrix_trans(st_addr + 512u * g, pk[set] + 4 * g);
+            __syncwarp();
+            const int mcol = m_warp + (lane & 3) * 8 + set * p.gate_f;
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+              uint4 val = *reinterpret_cast<const uint4*>(ld_addr + 512 * g);
+              if (kSlotRows) {
+                const int col = tok0 + 8 * g + (lane >> 2);
+                if (row_ok(col)) *reinterpret_cast<uint4*>(out_rows + (long long)col * p.ld_out + mcol) = val;
+              } else {
+                const int tok = __shfl_sync(0xffffffffu, q_tok[0], 8 * g + (lane >> 2));
+                if (tok >= 0) {
+                  const long long off = (long long)tok * p.ld_out + mcol;
+                  if (p.res != nullptr) {
+                    // skip path inside the layer: y = x + g E(x), dx = dy + dH W_in^T (the expert term is already bf16)
+                    if (OP == kGemm2Combine) *reinterpret_cast<uint4*>(p.out2 + off) = val;
+                    const uint4 r = *reinterpret_cast<const uint4*>(p.res + off);
+                    const __nv_bfloat162* rv = reinterpret_cast<const __nv_bfloat162*>(&r);
+                    __nv_bfloat162* vv = reinterpret_cast<__nv_bfloat162*>(&val);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                      const float2 a2 = __bfloat1622float2(vv[q]), b2 = __bfloat1622float2(rv[q]);
+                      vv[q] = __floats2bfloat162_rn(a2.x + b2.x, a2.y + b2.y);
+                    }
+                  }
+                  *reinterpret_cast<uint4*>(p.out + off) = val;
+                }
+              }
+            }
+          }
+        }
+#pragma unroll
+        for (int k = 0; k < kQueue - 1; ++k) {                // advance the queue
+          q_tok[k] = q_tok[k + 1];
+          q_gate[k] = q_gate[k + 1];
+          q_mw[k] = q_mw[k + 1];
+        }
+        __syncwarp();
+      }
+      if (!ok) break;
+      if (!mid_sent) {                                        // this warp had no chunk in this tile
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote(tmid0 + 8u * side, 0);
+      }
+      if (!released) {
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_remote(tempty0 + 8u * side, 0);
       }
     }
   }
@@ -819,13 +870,42 @@ int pair_grid(Kernel kernel, int* cached_grid, int dev, int sm_count, cudaStream
   return SWITCH_MOE_OK;
 }
 
+uint32_t magic(int d) { return d > 1 ? (uint32_t)((0x100000000ull + (uint64_t)d - 1) / (uint64_t)d) : 0u; }
+
+// Weight gradients: into how many strips a row of `nt` column tiles is cut.  A strip's A operand is loaded once if its
+// k-blocks fit the ring, so longer strips read less (up to 12% of a tile's time at the power limit); but the pairs' shares
+// are whole strips, and experts differ in size, so the last one leaves half a strip idle on average.  Experts that on
+// average do not fit the ring gain nothing and are balanced tile by tile.  Measured for whole training steps under
+// sustained load, tile by tile -> strips: 4096 tokens, 4096 x 10240, 16 experts (strips of 4 and 8) 2408 -> 2279 us; 32768
+// tokens, 768 x 3072, 128 experts (3 and 6) 1316 -> 1279; GEGLU 768 x 2048 (3 and 8) 1437 -> 1402; 20011 tokens, 512 x 1536,
+// 200 experts (two k-blocks per tile: the epilogue bounds it) 579 -> 581.
+int set_strips(PairParams* q, int n_pairs) {
+  const int nt = q->n_ntiles_fixed;
+  const long long rows = (long long)q->E * q->n_mpairs;
+  int best = nt;
+  float best_cost = 0.f;
+  for (int S = q->tokens_per_expert > kPWgradA * kBK ? nt : 1; S <= nt; ++S) {
+    const int L = (nt + S - 1) / S;
+    const float tiles = (float)((rows * S + n_pairs - 1) / n_pairs * L);
+    const float cost = tiles * (1.f + 0.12f * (float)S / (float)nt) + 0.5f * (float)L;
+    if (best_cost == 0.f || cost < best_cost) { best = S; best_cost = cost; }
+  }
+  q->strips = best;
+  const uint64_t per_e = (uint64_t)q->n_mpairs * best;        // the decode is exact while id * divisor < 2^32
+  if ((uint64_t)q->E * per_e * per_e >= 0x100000000ull) return SWITCH_MOE_UNSUPPORTED_SHAPE;
+  q->magic_per_e = magic((int)per_e);
+  q->magic_strips = magic(best);
+  return SWITCH_MOE_OK;
+}
+
 template <int OP, bool DROP = false>
-int launch_pair_op(const CUtensorMap& tmA, const BMapSet& tmB, const PairParams& q, int dev, int sm_count,
+int launch_pair_op(const CUtensorMap& tmA, const BMapSet& tmB, PairParams q, int dev, int sm_count,
                    cudaStream_t st) {
   static int cached_grid[64] = {0};
   int grid = 0;
   const int rc = pair_grid(expert_gemm_pair_kernel<OP, DROP>, cached_grid, dev, sm_count, st, &grid);
   if (rc != SWITCH_MOE_OK) return rc;
+  if (!q.token_op && set_strips(&q, grid / 2) != SWITCH_MOE_OK) return SWITCH_MOE_UNSUPPORTED_SHAPE;
   launch_k(expert_gemm_pair_kernel<OP, DROP>, dim3(grid), dim3(kPThreads), kPSmemBytes, st, tmA, tmB, q);
   return launch_status();
 }
@@ -913,6 +993,7 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
     default: return SWITCH_MOE_INVALID_ARGUMENT;
   }
   if (rc != SWITCH_MOE_OK || rc2 != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
+  q.tokens_per_expert = s.Tv / s.E < s.C ? s.Tv / s.E : s.C;
   q.n_mpairs = (q.Mw + 255) / 256;
   // operand ring of the token products: a stage holds A (16 KB) and this CTA's half of the widest token tile the
   // capacity allows (at most kPairTileTokens / 2 rows of 128 bytes, rounded up to whole 1 KB swizzle atoms)
@@ -921,17 +1002,9 @@ int pair_problem(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, vo
   q.stages = kPRingBytes / q.stage_bytes < kPMaxStages ? kPRingBytes / q.stage_bytes : kPMaxStages;
   q.n_ntiles_fixed = q.token_op ? 0 : (q.Nfix + 255) / 256;
   q.k_blocks_fixed = q.token_op ? K / kBK : 0;
-  auto magic = [](int d) { return d > 1 ? (uint32_t)((0x100000000ull + (uint64_t)d - 1) / (uint64_t)d) : 0u; };
   q.magic_mpairs = magic(q.n_mpairs);
-  q.magic_per_e = magic(q.n_mpairs * (q.n_ntiles_fixed > 0 ? q.n_ntiles_fixed : 1));
-  q.magic_nt = magic(q.n_ntiles_fixed > 0 ? q.n_ntiles_fixed : 1);
-  // the decode's divisions are exact only while id * divisor < 2^32: ids are below E * 16 * n_mpairs * n_ntiles
-  {
-    const uint64_t ids = q.token_op ? (uint64_t)s.max_mtiles * q.n_mpairs
-                                    : (uint64_t)s.E * q.n_mpairs * (q.n_ntiles_fixed > 0 ? q.n_ntiles_fixed : 1);
-    if (ids * (uint64_t)(q.n_mpairs * (q.n_ntiles_fixed > 0 ? q.n_ntiles_fixed : 1)) >= 0x100000000ull)
-      return SWITCH_MOE_UNSUPPORTED_SHAPE;
-  }
+  // (weight gradients: set_strips)
+  if (q.token_op && (uint64_t)s.max_mtiles * q.n_mpairs * q.n_mpairs >= 0x100000000ull) return SWITCH_MOE_UNSUPPORTED_SHAPE;
   *out = q;
   return SWITCH_MOE_OK;
 }
@@ -1000,6 +1073,7 @@ int launch_pair_dgrad1_wgrad1(const Shape& s, const Plan& p, const GemmArgs& a, 
   int split = few_tokens ? (n_pairs * 33 + 37) / 74 : n_pairs / 2;
   if (split < 1) split = 1;
   if (split > n_pairs - 1) split = n_pairs - 1;
+  if (set_strips(&q1, n_pairs - split) != SWITCH_MOE_OK) return SWITCH_MOE_UNSUPPORTED_SHAPE;
   launch_k(kernel, dim3(grid), dim3(kPThreads), kPSmemBytes, st, tmA0, tmB0, q0, tmA1, tmB1, q1, split);
   return launch_status();
 }

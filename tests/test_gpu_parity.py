@@ -427,6 +427,13 @@ def test_layer_at_the_edges_of_the_epilogue_blocks(T, E, cf, kw):
     _check_layer(si.SwitchConfig("epilogue_edges", T, 192, 320, E, cf), sm.GEMM_DEFAULT, TOL_BF16, seed=8, **kw)
 
 
+@pytest.mark.parametrize("E,std", [(148, 0.3), (20, 0.5)])   # whole rows of 3 and 5 tiles per strip; single tiles
+def test_weight_gradients_of_experts_around_the_operand_ring(E, std):
+    # from no token at all over 1 to 6 blocks of 64, which stay in shared memory for a strip of tiles, to more, which do not;
+    # partly filled last tiles on both sides
+    _check_layer(si.SwitchConfig("strips", 40 * E, 640, 1088, E, 11.0, bias_std=std), sm.GEMM_DEFAULT, TOL_BF16, seed=10)
+
+
 def test_capacity_override_is_honoured():
     _check_layer(MID, sm.GEMM_DEFAULT, TOL_BF16, capacity_override=200)
 
