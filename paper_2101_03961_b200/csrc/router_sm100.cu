@@ -32,6 +32,11 @@ namespace {
 // passes, which also leaves no limit on E short of the accumulator's 256 columns.  Stage time, straight-line -> loops:
 // 256 tokens, d_model 768, 128 experts 39 -> 19 us; 32768 tokens 44 -> 36; 20011 tokens, d_model 512, 200 experts (a
 // kernel of its own before, with a pass over the probabilities for the column sums) 260 -> 52.
+//
+// Probabilities and noise cross between memory order and token-per-lane order through shared memory.  With every lane
+// storing its own row, 16 bytes of 32 different rows at a time, the stores alone cost 6 of 25 us (32768 tokens, d_model
+// 768, 128 experts) and 12 of 29 (65536, 256, 128), the noise 10 of 40 (20011, 512, 200); now 22, 23 and 31 in all.  Twice
+// as many epilogue warps, each with half of the experts, gained nothing on top (26, 31, 44 before this).
 struct RouterFwdParams {
   int T, d, E, Epad64, n_blocks, k_blocks, b_atoms, stages, stage_bytes;
   int tiles;                 // 128-token tiles per block: 1 or 2
@@ -48,7 +53,8 @@ constexpr int kRFMaxStages = 6;
 constexpr int kRFRingBytes = 196608;                           // 192 KB of operand stages
 constexpr int kRFOutBytes = 8 * kMaxExperts * 4;               // the epilogue warps' column sums
 constexpr int kRFTailBytes = 256 + kMaxExperts * 4;            // barriers, TMEM pointer, flags; the block's histogram
-constexpr int kRFSmemBytes = 1024 + kRFRingBytes + kRFOutBytes + kRFTailBytes;
+constexpr int kRFTurnBytes = 8 * 32 * 16 * 4;                  // per epilogue warp: 32 tokens x 16 experts
+constexpr int kRFSmemBytes = 1024 + kRFRingBytes + kRFOutBytes + kRFTailBytes + kRFTurnBytes;
 constexpr int kRFThreads = 64 + 2 * 128;                       // TMA warp, MMA warp, 4 epilogue warps per token tile
 
 __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t* r) {
@@ -59,6 +65,14 @@ __device__ __forceinline__ void tc_st32(uint32_t taddr, const uint32_t* r) {
         "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]), "r"(r[17]), "r"(r[18]),
         "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]),
         "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
       : "memory");
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -185,10 +199,36 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
     const bool vec_rows = (p.E & 3) == 0;
     const bool vec_noise = vec_rows && (reinterpret_cast<uintptr_t>(p.noise) & 15u) == 0;   // (the caller's own array)
     float* sums = reinterpret_cast<float*>(smem_gen + kRFRingBytes);
+    // Rows of probabilities and noise move between memory and the lanes that own them through this warp's tile of 32 tokens x
+    // 16 experts (64 bytes per row, 16-byte pieces exchanged by the row): lane l owns row l, and in memory order it handles
+    // piece l % 4 of rows l / 4, l / 4 + 8, ...
+    float* turn = reinterpret_cast<float*>(bar_gen + kRFTailBytes) + (warp - 2) * 512;
+    float4* own = reinterpret_cast<float4*>(turn + lane * 16);
+    const int own_x = (lane >> 1) & 3, row0 = lane >> 2, piece = lane & 3;
+    float4* mem = reinterpret_cast<float4*>(turn + row0 * 16) + (piece ^ ((lane >> 3) & 3));     // row row0 + 8 k: mem[32 k]
     uint32_t acc = 0, acc_phase = 0;
     bool ok = true;
     for (int id = blockIdx.x; id < n_blocks; id += gridDim.x) {
       const int tok = (id * tiles + ti) * kTileM + lg * 32 + lane;       // the token whose logits this lane holds
+      const int tok0 = tok - lane + row0;                     // this lane's first row in memory order
+      float4 z[8];                                            // a chunk of noise, requested one chunk ahead
+      auto load_noise = [&](int c) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const int e = c * 32 + (k >> 2) * 16 + piece * 4, t = tok0 + 8 * (k & 3);
+          const float* src = p.noise + (size_t)t * p.E + e;
+          z[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (t < p.T && vec_noise) {
+            if (e < p.E) z[k] = *reinterpret_cast<const float4*>(src);
+          } else if (t < p.T) {
+            if (e < p.E) z[k].x = src[0];
+            if (e + 1 < p.E) z[k].y = src[1];
+            if (e + 2 < p.E) z[k].z = src[2];
+            if (e + 3 < p.E) z[k].w = src[3];
+          }
+        }
+      };
+      if (p.noise != nullptr) load_noise(0);
       ok = mbar_wait_warp(tfull0 + 8u * acc, acc_phase, abort_flag, p.status, 34);
       // the epilogue warps meet at barriers below: all of them leave together if the bounded wait of any gave up
       if (!ok && lane == 0) *fail_s = 1;
@@ -201,7 +241,6 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       // Pass 1: Eq. 1's maximum and top-1 (first maximum wins) as four interleaved chains, all within this lane.
       float mq[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
       int aq[4] = {0, 1, 2, 3};
-      const float* nrow = p.noise != nullptr && live ? p.noise + (size_t)tok * p.E : nullptr;
 #pragma unroll 1
       for (int c = 0; c < nch; ++c) {
         uint32_t v[32];
@@ -213,23 +252,24 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
             for (int i = 0; i < 32; ++i)
               if (c * 32 + i < p.E) v[i] = __float_as_uint(__uint_as_float(v[i]) + p.bias[c * 32 + i]);
           }
-          if (nrow != nullptr && vec_noise) {                 // 16 bytes of this lane's own row at a time
-            float4 z[8];
+          if (p.noise != nullptr) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
-              if (c * 32 + 4 * i < p.E) z[i] = *reinterpret_cast<const float4*>(nrow + c * 32 + 4 * i);
+            for (int h = 0; h < 2; ++h) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              if (c * 32 + 4 * i >= p.E) continue;
-              v[4 * i] = __float_as_uint(__uint_as_float(v[4 * i]) + z[i].x);
-              v[4 * i + 1] = __float_as_uint(__uint_as_float(v[4 * i + 1]) + z[i].y);
-              v[4 * i + 2] = __float_as_uint(__uint_as_float(v[4 * i + 2]) + z[i].z);
-              v[4 * i + 3] = __float_as_uint(__uint_as_float(v[4 * i + 3]) + z[i].w);
+              for (int k = 0; k < 4; ++k) mem[32 * k] = z[4 * h + k];
+              __syncwarp();
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const float4 n = own[q ^ own_x];
+                const int i = 16 * h + 4 * q;
+                v[i] = __float_as_uint(__uint_as_float(v[i]) + n.x);
+                v[i + 1] = __float_as_uint(__uint_as_float(v[i + 1]) + n.y);
+                v[i + 2] = __float_as_uint(__uint_as_float(v[i + 2]) + n.z);
+                v[i + 3] = __float_as_uint(__uint_as_float(v[i + 3]) + n.w);
+              }
+              __syncwarp();
             }
-          } else if (nrow != nullptr) {
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (c * 32 + i < p.E) v[i] = __float_as_uint(__uint_as_float(v[i]) + nrow[c * 32 + i]);
+            if (c + 1 < nch) load_noise(c + 1);
           }
           tc_st32(t_addr + c * 32, v);
           tc_wait_st();
@@ -275,44 +315,47 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
         p.gate[tok] = inv;
         atomicAdd(&hist_s[am], 1);                            // integer counts: the order does not matter
       }
-      // Pass 3: every thread writes its own token's probabilities, 16 bytes at a time.  Column sums over the warp's 32
-      // tokens (Eq. 6's sum over tokens) by a halving exchange: in each of five steps a lane hands half of its values to
-      // the lane whose index differs in one bit and adds what it receives, so that lane l ends with column 32 c + l
-      // summed over all lanes in a fixed (tree) order.
-      float* prow = p.probs + (size_t)(live ? tok : 0) * p.E;
+      // Pass 3: the probabilities, in memory order, and their column sums over the warp's 32 tokens (Eq. 6's sum over tokens):
+      // over the four rows of a lane, then over the lanes with the same columns, in a fixed order.
+      const float scale = live ? inv : 0.f;                    // rows past the last token add nothing to the sums
 #pragma unroll 1
-      for (int c = 0; c < nch; ++c) {
-        uint32_t v[32];
-        tc_ld32(t_addr + c * 32, v);
+      for (int c = 0; c < p.E; c += 16) {
+        uint32_t v[16];
+        tc_ld16(t_addr + c, v);
         tc_wait_ld();
-        float w[32];
+        __syncwarp();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) w[i] = __uint_as_float(v[i]) * inv;
-        if (live) {
-          if (vec_rows) {
+        for (int q = 0; q < 4; ++q)
+          own[q ^ own_x] = make_float4(__uint_as_float(v[4 * q]) * scale, __uint_as_float(v[4 * q + 1]) * scale,
+                                       __uint_as_float(v[4 * q + 2]) * scale, __uint_as_float(v[4 * q + 3]) * scale);
+        __syncwarp();
+        const int e = c + piece * 4;
+        float4 w[4], sum4;
 #pragma unroll
-            for (int i = 0; i < 32; i += 4)
-              if (c * 32 + i < p.E) *reinterpret_cast<float4*>(prow + c * 32 + i) = make_float4(w[i], w[i + 1], w[i + 2], w[i + 3]);
-          } else {
-#pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (c * 32 + i < p.E) prow[c * 32 + i] = w[i];
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 32; ++i) w[i] = 0.f;             // rows past the last token add nothing to the sums
-        }
-#pragma unroll
-        for (int half = 16; half >= 1; half >>= 1) {
-          const bool upper = (lane & half) != 0;
-#pragma unroll
-          for (int j = 0; j < half; ++j) {
-            const float send = upper ? w[j] : w[j + half];
-            const float keep = upper ? w[j + half] : w[j];
-            w[j] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+        for (int k = 0; k < 4; ++k) {
+          w[k] = mem[32 * k];
+          float* dst = p.probs + (size_t)(tok0 + 8 * k) * p.E + e;
+          if (tok0 + 8 * k < p.T && vec_rows) {
+            if (e < p.E) *reinterpret_cast<float4*>(dst) = w[k];
+          } else if (tok0 + 8 * k < p.T) {
+            if (e < p.E) dst[0] = w[k].x;
+            if (e + 1 < p.E) dst[1] = w[k].y;
+            if (e + 2 < p.E) dst[2] = w[k].z;
+            if (e + 3 < p.E) dst[3] = w[k].w;
           }
         }
-        sums[(warp - 2) * kMaxExperts + c * 32 + lane] = w[0];
+        sum4.x = (w[0].x + w[1].x) + (w[2].x + w[3].x);
+        sum4.y = (w[0].y + w[1].y) + (w[2].y + w[3].y);
+        sum4.z = (w[0].z + w[1].z) + (w[2].z + w[3].z);
+        sum4.w = (w[0].w + w[1].w) + (w[2].w + w[3].w);
+#pragma unroll
+        for (int step = 4; step <= 16; step <<= 1) {
+          sum4.x += __shfl_xor_sync(0xffffffffu, sum4.x, step);
+          sum4.y += __shfl_xor_sync(0xffffffffu, sum4.y, step);
+          sum4.z += __shfl_xor_sync(0xffffffffu, sum4.z, step);
+          sum4.w += __shfl_xor_sync(0xffffffffu, sum4.w, step);
+        }
+        if (row0 == 0) *reinterpret_cast<float4*>(sums + (warp - 2) * kMaxExperts + e) = sum4;
       }
       tc_fence_before();
       __syncwarp();

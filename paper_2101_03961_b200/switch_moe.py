@@ -133,21 +133,19 @@ def _check(status: int, where: str) -> None:
 
 
 def _ptr(t) -> int | None:
-    if t is None:
-        return None
-    if isinstance(t, int):
+    if t is None or isinstance(t, int):
         return t
     return t.data_ptr()
 
 
 # The current stream's handle without a Stream object around it (3 us of host time per call).
-_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_stream, _device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _stream(stream) -> int | None:
     if stream is None:
-        if _raw_stream is not None:
-            return _raw_stream(torch.cuda.current_device())
+        if _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+            return _raw_stream(_device())
         stream = torch.cuda.current_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
