@@ -434,6 +434,14 @@ def test_weight_gradients_of_experts_around_the_operand_ring(E, std):
     _check_layer(si.SwitchConfig("strips", 40 * E, 640, 1088, E, 11.0, bias_std=std), sm.GEMM_DEFAULT, TOL_BF16, seed=10)
 
 
+@pytest.mark.parametrize("d,residual", [(64, False), (64, True), (1088, False), (1088, True)])
+def test_rows_of_dropped_tokens(d, residual):
+    # one slot per expert: the gathers have few warps, so each goes round several times over its dropped tokens; 1088
+    # columns are one 16-byte piece per lane more than four
+    _check_layer(si.SwitchConfig("dropped", 1500, d, 64, 2, 1.0), sm.GEMM_DEFAULT, TOL_BF16, seed=12, capacity_override=1,
+                 residual=residual)
+
+
 def test_capacity_override_is_honoured():
     _check_layer(MID, sm.GEMM_DEFAULT, TOL_BF16, capacity_override=200)
 
