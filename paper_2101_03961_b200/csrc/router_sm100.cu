@@ -286,33 +286,59 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 #pragma unroll
       for (int u = 1; u < 4; ++u)
         if (mq[u] > m || (mq[u] == m && aq[u] < am)) { m = mq[u]; am = aq[u]; }
-      // Pass 2: exponentials (hardware exp2 of a pre-scaled argument: relative error below 1e-6 for |h - m| < 10, inside
-      // the 1e-5 the router is held to), back into tensor memory, and their sum.
-      const float kLog2e = 1.4426950408889634f;
-      const float ms = m * kLog2e;
-      float sq[4] = {0.f, 0.f, 0.f, 0.f};
+      // Pass 2: exponentials, back into tensor memory, and their sum.  Up to 128 experts the hardware's exp2 of an argument
+      // scaled in the same multiply-add: relative error below 1e-6 for h within 10 of m, whatever m is, because the rounding
+      // of m log2(e) is one factor of the whole row and leaves with the sum -- it has to be in the gate's numerator too, so
+      // the gate is formed like the probability it is, from the maximum's own exponential.  Above 128 experts expf of the
+      // difference and one running sum: 2e-7 of the exponential instead of 1e-6, for 7 us (20011 tokens, d_model 512, 200
+      // experts: training step 562 us with the first form, 569 with this one).
+      float sum, top;                                          // top: the maximum's own exponential
+      if (p.E > 128) {
+        sum = 0.f;
+        top = 1.f;
 #pragma unroll 1
-      for (int c = 0; c < nch; ++c) {
-        uint32_t v[32];
-        tc_ld32(t_addr + c * 32, v);
-        tc_wait_ld();
+        for (int c = 0; c < nch; ++c) {
+          uint32_t v[32];
+          tc_ld32(t_addr + c * 32, v);
+          tc_wait_ld();
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          float ex;
-          const float arg = fmaf(__uint_as_float(v[i]), kLog2e, -ms);
-          asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(arg));
-          if (c * 32 + i >= p.E) ex = 0.f;
-          sq[i & 3] += ex;
-          v[i] = __float_as_uint(ex);
+          for (int i = 0; i < 32; ++i) {
+            const float ex = c * 32 + i < p.E ? expf(__uint_as_float(v[i]) - m) : 0.f;
+            sum += ex;
+            v[i] = __float_as_uint(ex);
+          }
+          tc_st32(t_addr + c * 32, v);
         }
-        tc_st32(t_addr + c * 32, v);
+      } else {
+        const float kLog2e = 1.4426950408889634f;
+        const float ms = m * kLog2e;
+        auto exp_minus_m = [&](float h) {
+          float ex;
+          asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(ex) : "f"(fmaf(h, kLog2e, -ms)));
+          return ex;
+        };
+        float sq[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+        for (int c = 0; c < nch; ++c) {
+          uint32_t v[32];
+          tc_ld32(t_addr + c * 32, v);
+          tc_wait_ld();
+#pragma unroll
+          for (int i = 0; i < 32; ++i) {
+            const float ex = c * 32 + i < p.E ? exp_minus_m(__uint_as_float(v[i])) : 0.f;
+            sq[i & 3] += ex;
+            v[i] = __float_as_uint(ex);
+          }
+          tc_st32(t_addr + c * 32, v);
+        }
+        sum = (sq[0] + sq[1]) + (sq[2] + sq[3]);
+        top = exp_minus_m(m);
       }
       tc_wait_st();
-      const float sum = (sq[0] + sq[1]) + (sq[2] + sq[3]);
       const float inv = 1.f / sum;
       if (live) {
         p.expert_index[tok] = am;
-        p.gate[tok] = inv;
+        p.gate[tok] = top * inv;
         atomicAdd(&hist_s[am], 1);                            // integer counts: the order does not matter
       }
       // Pass 3: the probabilities, in memory order, and their column sums over the warp's 32 tokens (Eq. 6's sum over tokens):

@@ -91,6 +91,38 @@ def test_router_ties_go_to_lowest_expert():
     assert np.all(y[C:] == 0.0) and np.isfinite(y).all()
 
 
+@pytest.mark.parametrize("E", [5, 64, 128, 129, 200, 256])
+@pytest.mark.parametrize("offset", [0.0, 300.0, -1000.0])
+def test_gate_is_the_probability_of_the_chosen_expert(E, offset):
+    # a common offset of the logits leaves the softmax alone, and whatever its rounding does to the row it does to both
+    cfg = si.SwitchConfig("offset", 700, 64, 64, E, max(1.25, 1.01 * E / 700))
+    data = si.gen_layer(cfg, seed=13)
+    data["router_bias"] = np.full(E, offset, np.float32)
+    g = GpuLayer(cfg, data)
+    g.fwd()
+    probs = g.view(sm.WS_PROBS).cpu().numpy().reshape(cfg.T, E)
+    np.testing.assert_array_equal(g.view(sm.WS_GATE).cpu().numpy(), probs[np.arange(cfg.T), g.expert_index()])
+    np.testing.assert_allclose(probs.sum(1, dtype=np.float64), 1.0, atol=1e-6)
+
+
+@pytest.mark.parametrize("E,bound", [(128, 2e-6), (129, 2.0 ** -22), (256, 2.0 ** -22)])
+def test_probabilities_of_known_logits(E, bound):
+    # one-hot tokens pick rows of W_r, whose entries are multiples of 1/16 in [-20, 0]: the logits are exact and
+    # p_i / p_max is exp(h_i - h_max).  Above 128 experts: expf (at most 1 ulp) and one rounding of each probability,
+    # 2^-23 + 2 . 2^-24; up to 128 the rounding of an argument of up to 29 (2^-20 ln 2) and exp2's 2^-22 come on top.
+    rng = np.random.default_rng(14)
+    cfg = si.SwitchConfig("known", 640, 64, 64, E, 1.25)
+    data = si.gen_layer(cfg, seed=14)
+    data["x"] = np.eye(64, dtype=np.float32)[np.arange(cfg.T) % 64]
+    data["W_r"] = (-rng.integers(0, 321, (64, E)) / 16.0).astype(np.float32)
+    g = GpuLayer(cfg, data)
+    g.fwd()
+    probs = to_np(g.view(sm.WS_PROBS)).reshape(cfg.T, E)
+    h = np.asarray(data["W_r"], dtype=np.float64)[np.arange(cfg.T) % 64]
+    want = np.exp(h - h.max(axis=1, keepdims=True))
+    np.testing.assert_allclose(probs / probs.max(axis=1, keepdims=True), want, rtol=bound)
+
+
 # ---------------------------------------------------------------------------------------------- dispatch (staged)
 def _plan_case(name, T, E, C, e):
     return name, T, E, C, np.asarray(e, dtype=np.int32)
