@@ -119,7 +119,7 @@ int switch_moe_dispatch_plan(const switch_moe_config* cfg, const int32_t* expert
                              void* workspace, size_t workspace_bytes, void* stream) {
   Ctx c;
   SWMOE_TRY(prepare(cfg, workspace, workspace_bytes, true, &c));
-  return launch_dispatch_plan(c.s, c.p, expert_index, aux_loss, workspace, static_cast<cudaStream_t>(stream));
+  return launch_dispatch_plan(c.s, c.p, expert_index, false, aux_loss, workspace, static_cast<cudaStream_t>(stream));
 }
 
 int switch_moe_fwd(const switch_moe_config* cfg, const void* x, const float* W_r, const float* router_bias,
@@ -135,7 +135,7 @@ int switch_moe_fwd(const switch_moe_config* cfg, const void* x, const float* W_r
   SWMOE_TRY(launch_router_fwd(c.s, c.p, x, W_r, router_bias, cfg->router_noise, true, workspace, st));
   if (c.s.top2) SWMOE_TRY(launch_top2_choice(c.s, c.p, workspace, st));     // assignments T .. 2T - 1
   SWMOE_TRY(mark(cfg, 1, st));
-  SWMOE_TRY(launch_dispatch_plan(c.s, c.p, nullptr, aux_loss, workspace, st));
+  SWMOE_TRY(launch_dispatch_plan(c.s, c.p, nullptr, true, aux_loss, workspace, st));
   SWMOE_TRY(mark(cfg, 2, st));
   // top-2 routing: the experts write one weighted output row per assignment; the two rows of a token are summed last
   void* y_rows = c.s.top2 ? ws_ptr<void>(workspace, c.p.yv) : y;

@@ -730,15 +730,17 @@ int* list128(const Shape& s, const Plan& p, void* ws) {
 }
 }  // namespace
 
-int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, float* aux_loss, void* ws,
-                         cudaStream_t st) {
+int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, bool after_router, float* aux_loss,
+                         void* ws, cudaStream_t st) {
   int* ei = ws_ptr<int>(ws, p.expert_index);
   if (expert_index != nullptr && expert_index != ei) {
     if (cudaMemcpyAsync(ei, expert_index, (size_t)s.Tv * 4, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
       return SWITCH_MOE_CUDA_ERROR;
   }
-  // the tensor-core router's forward kernel leaves the histograms of its own expert choices in the workspace
-  const bool have_hist = expert_index == nullptr && s.router_hist;
+  // The tensor-core router's forward kernel leaves the histograms of its own expert choices in the workspace.  They are
+  // good only right after it: the counting kernel below and every rerouting stage put tables of another layout in their
+  // place, and the expert indices may have been edited since.
+  const bool have_hist = after_router && s.router_hist;
   if (have_hist && s.G == 1) {
     const int token_blocks = (s.T + kFusedTokens - 1) / kFusedTokens;
     launch_k(plan_slots_kernel, dim3(token_blocks), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist), s.router_blocks,

@@ -255,8 +255,10 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 // ---- kernels' host launchers (each returns a switch_moe_status) ----------------------------------------
 int launch_router_fwd(const Shape& s, const Plan& p, const void* x, const float* W_r, const float* bias,
                       const float* noise, bool clear_status, void* ws, cudaStream_t st);
-int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, float* aux_loss, void* ws,
-                         cudaStream_t st);
+// `expert_index` null: the workspace's.  `after_router`: the call follows launch_router_fwd with nothing in between, so that
+// the histograms which that left may be used; otherwise the indices are counted again.
+int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, bool after_router, float* aux_loss,
+                         void* ws, cudaStream_t st);
 int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void* ws, cudaStream_t st);
 // Top-2 routing: second choices (expert and weight) of every token; sums of the two assignments' rows.
 int launch_top2_choice(const Shape& s, const Plan& p, void* ws, cudaStream_t st);

@@ -161,6 +161,39 @@ def test_dispatch_plan_is_bit_exact_given_oracle_routing(case):
     np.testing.assert_array_equal(v(sm.WS_SLOT) >= 0, plan["keep"])
 
 
+@pytest.mark.parametrize("T,E", [(300, 5), (5000, 64), (148 * 128, 128), (148 * 128 + 1, 128), (3000, 200)])
+@pytest.mark.parametrize("stages", [0, 2])
+def test_dispatch_plan_without_an_index_follows_the_workspace(T, E, stages):
+    # whatever filled the workspace's table of counts last: the router, a plan of a caller's indices, a rerouting stage
+    cfg = si.SwitchConfig("plan_again", T, 64, 64, E, max(1.0, 1.01 * E / T), bias_std=0.5)
+    data = si.gen_layer(cfg, seed=15)
+    g = GpuLayer(cfg, data, reroute=stages > 0, reroute_stages=stages)
+
+    def check(e):
+        sm.switch_moe_dispatch_plan(g.cfg, None, g.aux, g.ws)
+        plan = so.dispatch_plan(e, E, g.C)
+        np.testing.assert_array_equal(g.view(sm.WS_COUNT).cpu().numpy(), plan["count"])
+        if stages:
+            alt = g.view(sm.WS_SECOND_CHOICE).cpu().numpy().astype(np.int64).reshape(stages, T)
+            for nxt in alt:
+                assert not (plan["keep"] & (nxt >= 0)).any()
+                plan = so.reroute_overflow(plan, e, nxt, E, g.C)
+        np.testing.assert_array_equal(g.view(sm.WS_KEPT).cpu().numpy(), plan["kept"])
+        np.testing.assert_array_equal(g.view(sm.WS_SLOT).cpu().numpy(), plan["slot"])
+        np.testing.assert_array_equal(g.view(sm.WS_TOKEN_OF_SLOT).cpu().numpy(), plan["token_of_slot"])
+
+    sm.switch_moe_router_fwd(g.cfg, g.x, g.W_r, g.bias, g.ws)
+    routed = g.expert_index()
+    check(routed)
+    check(routed)
+    custom = np.random.default_rng(15).integers(0, E, T)
+    sm.switch_moe_dispatch_plan(g.cfg, torch.from_numpy(custom.astype(np.int32)).cuda(), None, g.ws)
+    check(custom)
+    edited = custom[::-1].copy()
+    g.view(sm.WS_EXPERT_INDEX).copy_(torch.from_numpy(edited.astype(np.int32)))
+    check(edited)
+
+
 def test_dispatch_plan_is_deterministic():
     rng = np.random.default_rng(5)
     e = torch.from_numpy(rng.integers(0, 128, 32768).astype(np.int32)).cuda()
