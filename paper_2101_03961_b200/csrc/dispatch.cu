@@ -261,10 +261,13 @@ plan_assign_kernel(const int* __restrict__ expert_index, const int* __restrict__
 // earlier warps with the same expert) + (earlier lanes with it), in token order, with no atomics deciding a position.
 //
 // Summary (one block): counts, P-sums, the auxiliary loss (Eq. 4-6) and the tile lists.  It runs beside the slots kernel:
-// that kernel lets its successor start only once its own wait on the router is over, hence the summary may read what the
-// router wrote without waiting for anything else.  (As one more block of the slots kernel it did the same work in code and
-// registers that every block had to carry: 96 tokens, d 256, E 8, whole forward pass 29.1 us against 28.4.  Launched
-// after the gather instead, to run beside that, it was no faster and delayed GEMM1 where the gather is short.)
+// that kernel lets its successor start only once its own wait on the router is over, so the router has completed and its
+// tables are in L2 when the summary starts.  It reads them from there (__ldcg), past the L1 lines that an earlier call may
+// have left on its SM: its own wait, which comes last, has not vouched for those yet.  (Waiting first, the plan took 13.3
+// us instead of 9.2 at 256 tokens and 128 experts, 19.5 instead of 13.4 at 20011 and 200.  As one more block of the slots
+// kernel it did the same work in code and registers that every block had to carry: 96 tokens, d 256, E 8, whole forward
+// pass 29.1 us against 28.4.  Launched after the gather instead, to run beside that, it was no faster and delayed GEMM1
+// where the gather is short.)
 constexpr int kFusedTokens = 1024;
 
 // Column sums of the histogram table by the whole block: tot over all rows, pre over rows below row_end, as partial sums
@@ -341,11 +344,11 @@ plan_slots_kernel(const int* __restrict__ expert_index, const int* __restrict__ 
   }
 }
 
-// Launched after plan_slots_kernel.  Reads only what the router wrote, which is complete when it starts; its own wait comes
-// last, so that the next kernel's wait covers everything before this one.
+// Launched after plan_slots_kernel.  Reads only what the router wrote, past L1, and writes what no kernel in flight reads;
+// its own wait comes last, so that the next kernel's wait covers everything before this one.
 __global__ void __launch_bounds__(kFusedTokens)
-plan_summary_kernel(const int* __restrict__ hist, int hist_rows, const float* __restrict__ psum_partial, int T, int E, int Ew,
-                    int C, float alpha, int* __restrict__ count, float* __restrict__ psum, float* __restrict__ aux_loss,
+plan_summary_kernel(const int* hist, int hist_rows, const float* psum_partial, int T, int E, int Ew, int C,
+                    float alpha, int* __restrict__ count, float* __restrict__ psum, float* __restrict__ aux_loss,
                     int* __restrict__ tile_expert, int* __restrict__ tile_row0, int4* __restrict__ ntile,
                     int* __restrict__ count_g, int* __restrict__ group_base) {
   pdl_launch_dependents();
@@ -361,9 +364,9 @@ plan_summary_kernel(const int* __restrict__ hist, int hist_rows, const float* __
       int v[16];
       float f[16];
 #pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = r0 + j * Q < hist_rows ? hist[(size_t)(r0 + j * Q) * E + e] : 0;
+      for (int j = 0; j < 16; ++j) v[j] = r0 + j * Q < hist_rows ? __ldcg(hist + (size_t)(r0 + j * Q) * E + e) : 0;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) f[j] = r0 + j * Q < hist_rows ? psum_partial[(size_t)(r0 + j * Q) * E + e] : 0.f;
+      for (int j = 0; j < 16; ++j) f[j] = r0 + j * Q < hist_rows ? __ldcg(psum_partial + (size_t)(r0 + j * Q) * E + e) : 0.f;
 #pragma unroll
       for (int j = 0; j < 16; ++j) { tot += v[j]; ps += f[j]; }
     }

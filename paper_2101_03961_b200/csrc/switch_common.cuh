@@ -218,7 +218,9 @@ inline T* ws_ptr(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast
 // Every kernel of the layer is launched with programmatic stream serialization: it may be scheduled (and run its
 // prologue: barrier init, tensor-memory allocation) while the previous kernel of the stream is still draining.
 // The contract inside the kernels: call pdl_launch_dependents() first, and pdl_wait() before the first access to
-// global memory; pdl_wait() returns once the previous kernel has completed and its writes are visible.
+// global memory; pdl_wait() returns once the previous kernel has completed and its writes are visible.  One pair departs
+// from it: plan_slots_kernel waits first and triggers after, so that its successor starts only when the kernel before both
+// has completed, and that successor, plan_summary_kernel, reads that kernel's tables from L2 before its own wait.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
