@@ -160,7 +160,8 @@ enum switch_moe_ws_region {
   SWITCH_MOE_WS_H = 10,             /* [E,C,d_ff]    ReLU(x W_in) per slot */
   SWITCH_MOE_WS_DYD = 11,           /* [E,C,d_model] g . dy per slot (backward) */
   SWITCH_MOE_WS_DH = 12,            /* [E,C,d_ff]    gradient of the pre-activation per slot (backward) */
-  SWITCH_MOE_WS_DGATE = 13,         /* float[T]   <dy_t, o_t> for kept tokens (backward) */
+  SWITCH_MOE_WS_DGATE = 13,         /* float[T]   <dy_t, o_t> for kept tokens (backward); 0 where the gate underflowed to 0
+                                       (a second or rerouted choice), since o_t is taken from y_t / g_t */
   SWITCH_MOE_WS_DLOGITS = 14,       /* float[T,E] gradient of the router logits: written by switch_moe_router_bwd, and
                                        by switch_moe_bwd only where the router runs on the FP32 FMA path (the
                                        tensor-core path keeps just the bfloat16 parts it multiplies) */
@@ -201,7 +202,8 @@ int switch_moe_fwd(const switch_moe_config* cfg, const void* x, const float* W_r
  * loss (1.0 when that loss is simply added to the model loss, Section 2.2).  `workspace` must be the one the
  * matching switch_moe_fwd call filled, and x, W_r, W_in, W_out, y the same buffers with unchanged contents.
  *   dx [T,d_model], dW_r [d_model,E] float32, dW_in [E,d_model,d_ff], dW_out [E,d_ff,d_model] (all out).
- * The gate gradient uses o_t = y_t / g_t (g_t >= 1/E > 0).  f carries no gradient (Section 2.2). */
+ * The gate gradient uses o_t = y_t / g_t (g_t >= 1/E > 0 for a first choice; a second or rerouted choice whose g_t
+ * underflowed to 0 contributes nothing, as its gradient is multiplied by the same probability).  f carries no gradient (Section 2.2). */
 int switch_moe_bwd(const switch_moe_config* cfg, const void* dy, float d_aux, const void* x, const float* W_r,
                    const void* W_in, const void* W_out, const void* y, void* workspace, size_t workspace_bytes,
                    void* dx, float* dW_r, void* dW_in, void* dW_out, void* stream);

@@ -711,7 +711,8 @@ gather_dy_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ y, cons
     }
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-    if (lane == 0) dgate[tok] = dot / g;
+    // (a second or rerouted choice may have lost its probability to underflow: its gate's gradient enters dh times that 0)
+    if (lane == 0) dgate[tok] = g != 0.f ? dot / g : 0.f;
   }
   if (dx != nullptr) dropped_rows(slot, T, row_vec, dy, dx, gw, n_warps, lane);
 }

@@ -507,6 +507,27 @@ def test_rows_of_dropped_tokens(d, residual):
                  residual=residual)
 
 
+@pytest.mark.parametrize("kw", [dict(top2=True), dict(top2=True, residual=True), dict(reroute=True),
+                                dict(reroute=True, reroute_stages=3)], ids=lambda k: "_".join(k))
+@pytest.mark.parametrize("path", [sm.GEMM_DEFAULT, sm.GEMM_SIMT])
+def test_gradients_with_gates_that_underflow(kw, path):
+    # one expert has all the probability: second and rerouted choices get a gate of exactly 0 and keep their slots
+    cfg = si.SwitchConfig("zero_gates", 512, 64, 64, 8, 1.25)
+    data = si.gen_layer(cfg, seed=16)
+    data["router_bias"] = np.where(np.arange(cfg.E) == 3, 300.0, 0.0).astype(np.float32)
+    g = GpuLayer(cfg, data, gemm_path=path, **kw)
+    g.fwd()
+    gate, slot = to_np(g.view(sm.WS_GATE)), g.view(sm.WS_SLOT).cpu().numpy()
+    assert ((gate == 0.0) & (slot >= 0)).any()
+    g.bwd()
+    for name in ("y", "dx", "dW_r", "dW_in", "dW_out"):
+        assert torch.isfinite(getattr(g, name).float()).all(), name
+    np.testing.assert_array_equal(to_np(g.view(sm.WS_DGATE))[(gate == 0.0) & (slot >= 0)], 0.0)
+    # p is 1 at one expert and 0 elsewhere: dh = p (G - <p, G>) vanishes up to the rounding of the sum
+    dgate = to_np(g.view(sm.WS_DGATE))[:cfg.T][slot[:cfg.T] >= 0]
+    assert np.abs(to_np(g.dW_r)).max() <= 2.0 ** -20 * cfg.T * (np.abs(dgate).max() + 1.0) * np.abs(data["x"]).max()
+
+
 def test_capacity_override_is_honoured():
     _check_layer(MID, sm.GEMM_DEFAULT, TOL_BF16, capacity_override=200)
 
