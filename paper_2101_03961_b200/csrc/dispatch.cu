@@ -811,6 +811,13 @@ dim3 gather_grid(long long warps, int per_sm) {
   const long long blocks = (warps + 7) / 8, most = (long long)sm_count_or_default() * per_sm;
   return dim3((unsigned)(blocks < most ? blocks : most));
 }
+// Rows to deal out over a gather's warps: the slots', and where it also writes the dropped tokens' rows at least the tokens'
+// (65536 tokens of 1.5 KB, 8 experts of one slot each: x gather
+// 31 us, dy gather with the skip path 37; with warps for the slots alone, a block each, 5.2 and 8.5 ms).
+long long gathered_rows(const Shape& s, bool dropped) {
+  const long long slots = (long long)s.E * s.C;
+  return dropped && s.T > slots ? s.T : slots;
+}
 // Rows past an expert's last token that the GEMMs' tiles may read: the CTA-pair path's tiles end at a multiple of 16.
 int pad_rows(const Shape& s) { return s.gemm_path == 0 ? 16 : kTileM; }
 }  // namespace
@@ -818,7 +825,7 @@ int pad_rows(const Shape& s) { return s.gemm_path == 0 ? 16 : kTileM; }
 int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void* ws, cudaStream_t st) {
   const int row_vec = (int)((size_t)s.d * s.elt / 16);
   // top-2 routing: the output rows of dropped assignments are skipped by the kernel that sums the two choices
-  launch_k(gather_x_kernel, gather_grid(((long long)s.E * s.C + 3) / 4, kGatherBlocksPerSm), dim3(256), 0, st,
+  launch_k(gather_x_kernel, gather_grid((gathered_rows(s, !s.top2) + 3) / 4, kGatherBlocksPerSm), dim3(256), 0, st,
       static_cast<const uint4*>(x), ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.kept),
       ws_ptr<int>(ws, p.slot), s.T, s.E * s.C, s.C, row_vec, pad_rows(s), s.residual, ws_ptr<uint4>(ws, p.xd),
       s.top2 ? nullptr : static_cast<uint4*>(y));
@@ -833,7 +840,7 @@ int launch_gather_dy(const Shape& s, const Plan& p, const void* dy, const void* 
   // with the skip path inside the layer, y holds x + g . E(x): the gate's gradient needs the copy without x
   const void* ysrc = skip ? ws_ptr<char>(ws, p.layer_y) : y;
   auto kernel = s.dtype == SWITCH_MOE_BF16 ? gather_dy_kernel<true> : gather_dy_kernel<false>;
-  launch_k(kernel, gather_grid((long long)s.E * s.C, kGatherDyBlocksPerSm), dim3(256), 0, st, static_cast<const uint4*>(dy),
+  launch_k(kernel, gather_grid(gathered_rows(s, skip), kGatherDyBlocksPerSm), dim3(256), 0, st, static_cast<const uint4*>(dy),
            static_cast<const uint4*>(ysrc), ws_ptr<float>(ws, p.gate), ws_ptr<int>(ws, p.token_of_slot),
            ws_ptr<int>(ws, p.kept), ws_ptr<int>(ws, p.slot), s.T, s.E * s.C, s.C, row_vec, pad_rows(s),
            ws_ptr<uint4>(ws, p.dyd), ws_ptr<float>(ws, p.dgate), skip ? static_cast<uint4*>(dx) : nullptr);

@@ -501,8 +501,7 @@ def test_weight_gradients_of_experts_around_the_operand_ring(E, std):
 
 @pytest.mark.parametrize("d,residual", [(64, False), (64, True), (1088, False), (1088, True)])
 def test_rows_of_dropped_tokens(d, residual):
-    # one slot per expert: the gathers have few warps, so each goes round several times over its dropped tokens; 1088
-    # columns are one 16-byte piece per lane more than four
+    # one slot per expert: nearly every row is a dropped token's; 1088 columns are one 16-byte piece per lane more than four
     _check_layer(si.SwitchConfig("dropped", 1500, d, 64, 2, 1.0), sm.GEMM_DEFAULT, TOL_BF16, seed=12, capacity_override=1,
                  residual=residual)
 
@@ -526,6 +525,35 @@ def test_gradients_with_gates_that_underflow(kw, path):
     # p is 1 at one expert and 0 elsewhere: dh = p (G - <p, G>) vanishes up to the rounding of the sum
     dgate = to_np(g.view(sm.WS_DGATE))[:cfg.T][slot[:cfg.T] >= 0]
     assert np.abs(to_np(g.dW_r)).max() <= 2.0 ** -20 * cfg.T * (np.abs(dgate).max() + 1.0) * np.abs(data["x"]).max()
+
+
+@pytest.mark.parametrize("residual", [False, True])
+def test_many_dropped_tokens_of_a_small_capacity(residual):
+    # more tokens than 32 per warp of either gather; alpha = 0 and no slot: a dropped token's dx is dy, or 0
+    T, d, E = 310_000, 64, 2
+    cfg = sm.make_config(T, d, 64, E, 1.0, 0.0, capacity_override=1, residual=residual)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(17)
+    draw = lambda *shape: torch.randn(*shape, device="cuda", generator=gen).to(torch.bfloat16)
+    x, dy, W_in, W_out = draw(T, d), draw(T, d), draw(E, d, 64), draw(E, 64, d)
+    W_r = torch.randn(d, E, device="cuda", generator=gen)
+    y, dx, dW_in, dW_out, dW_r = (torch.full_like(t, float("nan")) for t in (x, x, W_in, W_out, W_r))
+    aux, ws = torch.empty(1, device="cuda"), sm.allocate_workspace(cfg)
+    ws.fill_(0xFF)
+    events = [torch.cuda.Event(enable_timing=True) for _ in range(sm.STAGE_EVENTS)]
+    for ev in events:
+        ev.record()
+    sm.set_stage_events(cfg, events)
+    for _ in range(2):
+        sm.switch_moe_fwd(cfg, x, W_r, None, W_in, W_out, y, aux, ws)
+        sm.switch_moe_bwd(cfg, dy, 1.0, x, W_r, W_in, W_out, y, ws, dx, dW_r, dW_in, dW_out)
+    sm.switch_moe_check_device_status(cfg, ws)
+    dropped = sm.switch_moe_workspace_view(cfg, ws, sm.WS_SLOT) < 0
+    assert int(dropped.sum()) == T - E
+    assert torch.equal(y[dropped], (x if residual else torch.zeros_like(x))[dropped])
+    assert torch.equal(dx[dropped], (dy if residual else torch.zeros_like(dy))[dropped])
+    # the rows are dealt out over the chip: 40 MB (80 with the skip path) in some 20 us, not the milliseconds of a block or two
+    assert events[2].elapsed_time(events[3]) < 1.0 and events[6].elapsed_time(events[7]) < 1.0
 
 
 def test_capacity_override_is_honoured():
