@@ -77,6 +77,7 @@ __device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t* r) {
 }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+template <bool kWide>                                          // more than 128 experts
 __global__ void __launch_bounds__(kRFThreads, 1)
 router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                      const RouterFwdParams p) {
@@ -293,7 +294,7 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
       // difference and one running sum: 2e-7 of the exponential instead of 1e-6, for 7 us (20011 tokens, d_model 512, 200
       // experts: training step 562 us with the first form, 569 with this one).
       float sum, top;                                          // top: the maximum's own exponential
-      if (p.E > 128) {
+      if constexpr (kWide) {
         sum = 0.f;
         top = 1.f;
 #pragma unroll 1
@@ -735,9 +736,10 @@ int launch_router_tc_fwd(const Shape& s, const Plan& p, const void* x, const flo
   q.gate = ws_ptr<float>(ws, p.gate); q.status = ws_ptr<int>(ws, p.status);
   q.psum_partial = ws_ptr<float>(ws, p.psum_partial); q.hist = ws_ptr<int>(ws, p.hist);
   const int sms = sm_count_or_default(), grid = q.n_blocks < sms ? q.n_blocks : sms;
-  if (cudaFuncSetAttribute(router_fwd_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRFSmemBytes) != cudaSuccess)
+  auto kernel = s.E > 128 ? router_fwd_tc_kernel<true> : router_fwd_tc_kernel<false>;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRFSmemBytes) != cudaSuccess)
     return SWITCH_MOE_CUDA_ERROR;
-  launch_k(router_fwd_tc_kernel, dim3(grid), dim3(64 + 128 * q.tiles), kRFSmemBytes, st, tmA, tmB, q);
+  launch_k(kernel, dim3(grid), dim3(64 + 128 * q.tiles), kRFSmemBytes, st, tmA, tmB, q);
   return launch_status();
 }
 
