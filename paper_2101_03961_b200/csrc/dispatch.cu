@@ -268,7 +268,10 @@ plan_assign_kernel(const int* __restrict__ expert_index, const int* __restrict__
 // kernel it did the same work in code and registers that every block had to carry: 96 tokens, d 256, E 8, whole forward
 // pass 29.1 us against 28.4.  Launched after the gather instead, to run beside that, it was no faster and delayed GEMM1
 // where the gather is short.)
-constexpr int kFusedTokens = 1024;
+// Every block reads the whole table, so the work grows with the square of T, and from some T on one scan kernel and its
+// wait cost less.  Plan, us, these kernels / scan and assignment, at 64, 128, 200 experts: 131072 tokens 13, 17, 28 / 19, 26,
+// 42; 262144 28, 44, 75 / 28, 48, 81; 524288 75, 130, 239 / 50, 85, 153; 1048576 214, 396, 712 / 91, 161, 296.
+constexpr int kFusedTokens = 1024, kFusedMaxTokens = 262144;
 
 // Column sums of the histogram table by the whole block: tot over all rows, pre over rows below row_end, as partial sums
 // per thread (column e = tid % Ew, slice q = tid / Ew of the rows, every Q-th one).
@@ -745,7 +748,7 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
   // good only right after it: the counting kernel below and every rerouting stage put tables of another layout in their
   // place, and the expert indices may have been edited since.
   const bool have_hist = after_router && s.router_hist;
-  if (have_hist && s.G == 1) {
+  if (have_hist && s.G == 1 && s.T <= kFusedMaxTokens) {
     const int token_blocks = (s.T + kFusedTokens - 1) / kFusedTokens;
     launch_k(plan_slots_kernel, dim3(token_blocks), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist), s.router_blocks,
              s.router_block_tokens, s.T, s.E, column_width(s.E), s.Cg, ws_ptr<int>(ws, p.slot),

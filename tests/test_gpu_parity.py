@@ -194,6 +194,44 @@ def test_dispatch_plan_without_an_index_follows_the_workspace(T, E, stages):
     check(edited)
 
 
+def test_plan_of_very_many_tokens():
+    # on both sides of the largest number of tokens that the plan's two side-by-side kernels take; beyond it the plan's time
+    # grows with the tokens, not with their square (four times the tokens: 4 x the time, 9 x with those kernels)
+    E, best = 200, {}
+    for T in (262144, 262145, 1048576):
+        cfg = sm.make_config(T, 64, 64, E, 1.0)
+        gen = torch.Generator(device="cuda")
+        gen.manual_seed(18)
+        draw = lambda *shape: torch.randn(*shape, device="cuda", generator=gen)
+        x, W_in, W_out = (t.to(torch.bfloat16) for t in (draw(T, 64), draw(E, 64, 64), draw(E, 64, 64)))
+        W_r, y, aux, ws = draw(64, E), torch.empty_like(x), torch.empty(1, device="cuda"), sm.allocate_workspace(cfg)
+        ws.fill_(0xFF)
+        events = [torch.cuda.Event(enable_timing=True) for _ in range(sm.STAGE_EVENTS)]
+        for ev in events:
+            ev.record()
+        sm.set_stage_events(cfg, events)
+        best[T] = float("inf")
+        for _ in range(5):
+            sm.switch_moe_fwd(cfg, x, W_r, None, W_in, W_out, y, aux, ws)
+            sm.switch_moe_check_device_status(cfg, ws)
+            best[T] = min(best[T], events[1].elapsed_time(events[2]))
+        view = lambda region: sm.switch_moe_workspace_view(cfg, ws, region)
+        e = view(sm.WS_EXPERT_INDEX).long()
+        order = torch.argsort(e, stable=True)
+        count = torch.bincount(e, minlength=E)
+        pos = torch.empty_like(e)
+        pos[order] = torch.arange(T, device="cuda") - (count.cumsum(0) - count)[e[order]]
+        C = sm.switch_moe_capacity(cfg)
+        slot = torch.where(pos < C, e * C + pos, -1)
+        token_of_slot = torch.full((E * C,), -1, device="cuda", dtype=torch.int64)
+        token_of_slot[slot[slot >= 0]] = torch.nonzero(slot >= 0).flatten()
+        assert torch.equal(view(sm.WS_COUNT).long(), count) and torch.equal(view(sm.WS_KEPT).long(), count.clamp(max=C))
+        assert torch.equal(view(sm.WS_SLOT).long(), slot) and torch.equal(view(sm.WS_TOKEN_OF_SLOT).long(), token_of_slot)
+        psum = view(sm.WS_PROBS).view(T, E).sum(0, dtype=torch.float64)
+        torch.testing.assert_close(view(sm.WS_PSUM).double(), psum, rtol=TOL_ROUTER, atol=0.0)
+    assert best[1048576] < 6.0 * best[262144]
+
+
 def test_dispatch_plan_is_deterministic():
     rng = np.random.default_rng(5)
     e = torch.from_numpy(rng.integers(0, 128, 32768).astype(np.int32)).cuda()
