@@ -303,6 +303,12 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
   const uint32_t tmem_base = *tmem_ptr_s;
   const int n_tiles = kTok ? n_ntiles_listed * p.n_mpairs : p.E * p.n_mpairs * p.strips;
 
+  // Weight gradients: A blocks are released by barriers of their own where a strip has several tiles.  With single tiles
+  // both rings, equally long, move in step, and a stage's release is its A block's too (512 tokens per expert, 768 x 3072, 64
+  // experts: wgrad2 107 us, dgrad1 with wgrad1 214; with the second wait and commit per k-block 111 and 227).
+  static_assert(kPWgradA == kPWgradB, "single tiles: one release per stage");
+  const bool a_ring = !kTok && p.strips < p.n_ntiles_fixed;
+
   // Accumulator columns of this pair's `it`-th tile: even tiles [0, n), odd tiles [512 - n, 512).  Consecutive tiles
   // share the middle columns when n + n_next > 512.
   if (warp == 0) {
@@ -333,7 +339,7 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
         const bool load_a = kTok || j == 0 || !resident;
 #pragma unroll 1
         for (int kb = 0; kb < kbs; ++kb) {
-          if (!kTok && load_a) {
+          if (load_a && a_ring) {
             ok = mbar_wait_warp(aempty0 + 8u * a_slot, a_phase ^ 1u, abort_flag, p.status, 28);
             if (!ok) break;
           }
@@ -434,7 +440,7 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
                     tc_mma_bf16_pair(d_tmem, ad + ks * a_kstep, bd + ks * b_kstep, idesc1, ks > 0 ? 1u : acc0);
               }
               tc_commit_pair(empty0 + 8u * stage);              // frees this stage in both CTAs
-              if (free_a) tc_commit_pair(aempty0 + 8u * a_slot);
+              if (free_a && a_ring) tc_commit_pair(aempty0 + 8u * a_slot);
               if (kb == kbs - 1) tc_commit_pair(tfull0 + 8u * side);   // accumulator complete, in both CTAs
             }
             if (++stage == n_stages) { stage = 0; phase ^= 1u; }

@@ -537,6 +537,12 @@ def test_weight_gradients_of_experts_around_the_operand_ring(E, std):
     _check_layer(si.SwitchConfig("strips", 40 * E, 640, 1088, E, 11.0, bias_std=std), sm.GEMM_DEFAULT, TOL_BF16, seed=10)
 
 
+@pytest.mark.parametrize("T,E,std", [(1800, 3, 0.3), (2600, 5, 1.0)])
+def test_weight_gradients_tile_by_tile(T, E, std):
+    # more than 384 tokens per expert on average: single tiles, up to 36 k-blocks through rings of six, none and few for some
+    _check_layer(si.SwitchConfig("single_tiles", T, 320, 1088, E, 4.0, bias_std=std), sm.GEMM_DEFAULT, TOL_BF16, seed=19)
+
+
 @pytest.mark.parametrize("d,residual", [(64, False), (64, True), (1088, False), (1088, True)])
 def test_rows_of_dropped_tokens(d, residual):
     # one slot per expert: nearly every row is a dropped token's; 1088 columns are one 16-byte piece per lane more than four
