@@ -327,8 +327,7 @@ router_dlogits_kernel(const float* __restrict__ probs, const int* __restrict__ e
             *reinterpret_cast<__nv_bfloat162*>(mid + n) = __floats2bfloat162_rn(G[j][n] - f.x, G[j][n + 1] - f.y);
           }
         } else {
-          hi[0] = __float2bfloat16(G[j][0]);
-          mid[0] = __float2bfloat16(G[j][0] - __bfloat162float(hi[0]));
+          split2(G[j][0], hi, mid);
         }
         const size_t at = (size_t)t * Epad64 + e0;              // NE consecutive experts per lane
         using Vec = typename BfVec<NE>::type;

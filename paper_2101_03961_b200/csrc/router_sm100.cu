@@ -690,9 +690,8 @@ router_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
   }
 }
 
-// wsplit[part][k][e] for e < Epad64 (zero beyond E): W_r = hi + mid + (a remainder below 2^-18 relative that no
-// product uses: the forward logits and the backward dx both stop at hi + mid).  The layer's first kernel: it also clears
-// the status words (`status` may be null).
+// wsplit[part][k][e] for e < Epad64 (zero beyond E): W_r = hi + mid up to 2^-18 relative.  The layer's first kernel: it also
+// clears the status words (`status` may be null).
 __global__ void split_w_kernel(const float* __restrict__ W_r, int d, int E, int Epad64,
                                __nv_bfloat16* __restrict__ wsplit, int* __restrict__ status) {
   pdl_launch_dependents();
@@ -702,9 +701,7 @@ __global__ void split_w_kernel(const float* __restrict__ W_r, int d, int E, int 
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int k = (int)(i / Epad64), e = (int)(i - (size_t)k * Epad64);
-  __nv_bfloat16 h, m, l;
-  split3(e < E ? W_r[(size_t)k * E + e] : 0.f, &h, &m, &l);
-  wsplit[i] = h; wsplit[n + i] = m;
+  split2(e < E ? W_r[(size_t)k * E + e] : 0.f, &wsplit[i], &wsplit[n + i]);
 }
 
 }  // namespace
@@ -719,7 +716,7 @@ int launch_router_tc_fwd(const Shape& s, const Plan& p, const void* x, const flo
            clear_status ? ws_ptr<int>(ws, p.status) : nullptr);
   CUtensorMap tmA, tmB;
   if (make_map(&tmA, x, 1, s.T, s.d, kTileM) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
-  if (make_map(&tmB, wsplit, 3, s.d, s.Epad64, 64) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
+  if (make_map(&tmB, wsplit, 2, s.d, s.Epad64, 64) != SWITCH_MOE_OK) return SWITCH_MOE_CUDA_ERROR;
   RouterFwdParams q{};
   q.T = s.T; q.d = s.d; q.E = s.E; q.Epad64 = s.Epad64;
   q.tiles = s.router_block_tokens / kTileM;
@@ -769,8 +766,8 @@ int launch_router_tc_bwd(const Shape& s, const Plan& p, const void* x, const flo
   q.status = ws_ptr<int>(ws, p.status);
   CUtensorMap tmX, tmH, tmW;
   if (make_map(&tmX, x, 1, s.T, s.d, kTileM) != SWITCH_MOE_OK ||
-      make_map(&tmH, dhsplit, 3, s.T, s.Epad64, kTileM) != SWITCH_MOE_OK ||
-      make_map(&tmW, wsplit, 3, s.d, s.Epad64, kTileM) != SWITCH_MOE_OK)
+      make_map(&tmH, dhsplit, 2, s.T, s.Epad64, kTileM) != SWITCH_MOE_OK ||
+      make_map(&tmW, wsplit, 2, s.d, s.Epad64, kTileM) != SWITCH_MOE_OK)
     return SWITCH_MOE_CUDA_ERROR;
   auto kernel = s.jitter ? router_bwd_tc_kernel<true> : router_bwd_tc_kernel<false>;
   if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kRBSmemBytes) != cudaSuccess)

@@ -187,8 +187,8 @@ inline void make_plan(const Shape& s, Plan* p) {
   p->dh = take(E * C * f * s.elt);
   p->dgate = take(Tv * 4);
   p->dwr_partial = take((size_t)s.dwr_chunks * d * E * 4);
-  p->wsplit = take(3 * d * (size_t)s.Epad64 * 2);
-  p->dhsplit = take(3 * T * (size_t)s.Epad64 * 2);
+  p->wsplit = s.router_tc ? take(2 * d * (size_t)s.Epad64 * 2) : 0;    // bfloat16 parts hi, mid of W_r ..
+  p->dhsplit = s.router_tc ? take(2 * T * (size_t)s.Epad64 * 2) : 0;   // .. and of the logit gradients
   const size_t rows16 = (C + 15) / 16 * 16;                // the tensor-core epilogues save for backward in blocks of 16 rows
   p->hmask = take(E * rows16 * ((f + 31) / 32) * 4);       // one bit per element of H: [H > 0]
   p->layer_y = s.residual ? take(T * d * s.elt) : 0;       // g . E(x) without the skip path (for the gate's gradient)
@@ -202,13 +202,10 @@ inline void make_plan(const Shape& s, Plan* p) {
   p->total = off;
 }
 
-// w = hi + mid + lo with hi, mid, lo bfloat16 (round to nearest); exact to about 2^-24 relative.
-__device__ __forceinline__ void split3(float w, __nv_bfloat16* hi, __nv_bfloat16* mid, __nv_bfloat16* lo) {
-  const __nv_bfloat16 h = __float2bfloat16(w);
-  const float r1 = w - __bfloat162float(h);
-  const __nv_bfloat16 m = __float2bfloat16(r1);
-  const float r2 = r1 - __bfloat162float(m);
-  *hi = h; *mid = m; *lo = __float2bfloat16(r2);
+// w = hi + mid with hi, mid bfloat16 (round to nearest), up to 2^-18 relative.
+__device__ __forceinline__ void split2(float w, __nv_bfloat16* hi, __nv_bfloat16* mid) {
+  *hi = __float2bfloat16(w);
+  *mid = __float2bfloat16(w - __bfloat162float(*hi));
 }
 
 template <typename T>

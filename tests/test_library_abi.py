@@ -49,6 +49,20 @@ def test_workspace_size_is_positive_and_grows(lib):
     assert b >= 2 * slots * (768 + 3072) * 2                   # X_d, H, dY_d, dH in bf16
 
 
+def test_workspace_holds_what_the_kernels_use(lib):
+    T, d, f, E, C = 65536, 256, 512, 128, 640
+    slots = E * C
+    parts = {"slot buffers": 2 * slots * (d + f) * 2, "mask bits": slots * f // 8, "probabilities and logit gradients": 2 * T * E * 4,
+             "bfloat16 parts hi, mid": 2 * (T + d) * E * 2, "dW_r partials": 148 * d * E * 4,
+             "per token and slot": (5 * T + slots) * 4, "tables": 4 * (T // 128) * E * 4, "alignment and small regions": 1 << 17}
+    assert sm.switch_moe_workspace_bytes(sm.make_config(T, d, f, E, 1.25)) <= sum(parts.values())
+    # the float32 router has no bfloat16 parts
+    parts["slot buffers"] *= 2
+    parts["bfloat16 parts hi, mid"] = 0
+    parts["tables"] = 4 * (T // 16) * E * 4
+    assert sm.switch_moe_workspace_bytes(sm.make_config(T, d, f, E, 1.25, dtype=sm.F32)) <= sum(parts.values())
+
+
 @pytest.mark.parametrize("kw,status", [
     (dict(T=0), sm.INVALID_ARGUMENT), (dict(E=0), sm.INVALID_ARGUMENT), (dict(capacity_factor=0.0), sm.INVALID_ARGUMENT),
     (dict(E=257), sm.UNSUPPORTED_SHAPE), (dict(d_model=100), sm.UNSUPPORTED_SHAPE),
