@@ -401,7 +401,7 @@ int launch_tc_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, 
   q.n_ntiles = (q.N + kBN - 1) / kBN;
   q.n_mtiles_fixed = q.token_m ? 0 : (q.M + kTileM - 1) / kTileM;
   q.k_blocks_fixed = q.token_m ? K / kBK : 0;
-  const int grid = sm_count > 0 ? sm_count : 148;
+  const int grid = sm_count > 0 ? sm_count : kChipSms;
   launch_k(grouped_gemm_tc_kernel, dim3(grid), dim3(kThreads), kSmemBytes, st, tmA, tmB, q);
   return launch_status();
 }

@@ -588,7 +588,7 @@ int router_bwd_t(const Shape& s, const Plan& p, const void* x, const float* W_r,
   // the 64-column blocks of d are dealt out over grid.y until there are about four blocks per SM (4096 tokens, d_model
   // 512: 16 us, 80 with one block walking all of d)
   const int tok_blocks = (s.T + 63) / 64, d_blocks = (s.d + 63) / 64;
-  int shares = (4 * 148 + tok_blocks - 1) / tok_blocks;
+  int shares = (4 * kChipSms + tok_blocks - 1) / tok_blocks;
   if (shares > d_blocks) shares = d_blocks;
   const int per_share = (d_blocks + shares - 1) / shares;
   launch_k(router_dx_kernel<XT, NE>, dim3(tok_blocks, (d_blocks + per_share - 1) / per_share), dim3(256), smem, st,
@@ -616,7 +616,7 @@ int launch_router_fwd(const Shape& s, const Plan& p, const void* x, const float*
     if (s.jitter_u == nullptr || !aligned16(s.jitter_u)) return SWITCH_MOE_INVALID_ARGUMENT;
     const size_t n_vec = (size_t)s.T * s.d * s.elt / 16;
     uint4* xr = ws_ptr<uint4>(ws, p.xr);
-    const unsigned blocks = (unsigned)((n_vec + 255) / 256 < 148 * 16 ? (n_vec + 255) / 256 : 148 * 16);
+    const unsigned blocks = (unsigned)((n_vec + 255) / 256 < kChipSms * 16 ? (n_vec + 255) / 256 : kChipSms * 16);
     if (s.dtype == SWITCH_MOE_BF16)
       launch_k(router_jitter_kernel<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, static_cast<const uint4*>(x),
                static_cast<const uint4*>(s.jitter_u), n_vec, xr);

@@ -244,7 +244,7 @@ void launch_op(const SimtProblem& pr, int max_m, int E, cudaStream_t st) {
   // 240, while GEMM1 (1280 blocks) takes 187 and 221.  128 x 128 tiles: 371 and 215 (a third of their rows lie past the
   // experts' last tokens).  GEMM2 of 512 tokens, 64 x 256, 8 experts: 27 us with 64 x 64 tiles and 16 steps per round, 13
   // with 32 x 32 and 64 steps.
-  constexpr long long kEnoughBig = 444, kEnough = 222;
+  constexpr long long kEnoughBig = BigTile::kMinBlocks * kChipSms, kEnough = kChipSms * 3 / 2;
   auto blocks = [&](int bm, int bn) { return (long long)((pr.N + bn - 1) / bn) * ((max_m + bm - 1) / bm) * E; };
   if (blocks(BigTile::BM, BigTile::BN) >= kEnoughBig) launch_tile<ET, OP, BigTile>(pr, max_m, E, st);
   else if (blocks(MidTile::BM, MidTile::BN) >= kEnough) launch_tile<ET, OP, MidTile>(pr, max_m, E, st);

@@ -20,6 +20,8 @@ constexpr int kPairTileTokens = 320;    // widest token tile of the paired-CTA G
 constexpr int kDwrChunkTokens = 512;    // most tokens per split of the dW_r reduction (FP32-FMA router)
 constexpr int kMaxGroups = 64;          // routing groups per call
 constexpr int kStatusWords = 16;        // status words at the start of the workspace
+constexpr int kChipSms = 148;           // SMs of a B200: what block sizes are chosen for (some decide workspace sizes, which
+                                        // are asked for without a device)
 
 struct Shape {
   int T, d, f, E;
@@ -136,20 +138,20 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
   if (s->router_tc) {
     // One 128-token tile per block while there are SMs for all of them, then two tiles that share the staged W_r.
     // (Several routing groups: the plan's kernels count in blocks of 256 tokens.)
-    s->router_block_tokens = G == 1 && cfg->T <= 148 * kTileM ? kTileM : 2 * kTileM;
+    s->router_block_tokens = G == 1 && cfg->T <= kChipSms * kTileM ? kTileM : 2 * kTileM;
     s->router_blocks = (cfg->T + s->router_block_tokens - 1) / s->router_block_tokens;
     // backward: blocks of 128 columns of d_model x splits of the token tiles, one CTA per SM
     const int n_cols = (cfg->d_model + 127) / 128, m_tiles = (cfg->T + kTileM - 1) / kTileM;
-    int splits = n_cols < 148 ? 148 / n_cols : 1;
+    int splits = n_cols < kChipSms ? kChipSms / n_cols : 1;
     if (splits > m_tiles) splits = m_tiles;
     s->dwr_chunks = splits;
   } else {
     // 64 tokens per forward block where that fills the chip, else 16: the kernel is bound by the latency of its k-chunks
-    s->router_block_tokens = cfg->T >= 64 * 148 ? 64 : 16;
+    s->router_block_tokens = cfg->T >= 64 * kChipSms ? 64 : 16;
     s->router_blocks = (cfg->T + s->router_block_tokens - 1) / s->router_block_tokens;
     // x^T dh: blocks of 64 rows of d x splits of the tokens, about four per SM, each with 64 to 512 tokens
     const int k_blocks = (cfg->d_model + 63) / 64;
-    const int want = (4 * 148 + k_blocks - 1) / k_blocks;
+    const int want = (4 * kChipSms + k_blocks - 1) / k_blocks;
     int chunk = ((cfg->T + want - 1) / want + 31) / 32 * 32;
     if (chunk < 64) chunk = 64;
     if (chunk > kDwrChunkTokens) chunk = kDwrChunkTokens;
@@ -244,8 +246,8 @@ inline int launch_status() {
 
 inline int sm_count_or_default() {
   int dev = 0, n = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 148;
-  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 148;
+  if (cudaGetDevice(&dev) != cudaSuccess) return kChipSms;
+  if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return kChipSms;
   return n;
 }
 
