@@ -588,8 +588,8 @@ top2_sum_kernel(const uint4* __restrict__ rows, const uint4* __restrict__ skip, 
 // ---- gathers --------------------------------------------------------------------------------------------------
 // Bound by HBM; a warp per slot row at a time, and no more blocks than are resident at once: a grid of one row per warp
 // spends its time on launching blocks.  The forward gather takes four rows at a time, their loads in flight together
-// (65536 tokens, d_model 256, 128 experts: 27 -> 18 us; 32768 x 768: 24 -> 21); the backward gather, whose rows end in a
-// reduction, is faster with twice the warps and one row each (32768 x 768: 31 us; two rows on half the warps 35).
+// (65536 tokens, d_model 256, 128 experts: 18 us, 27 with one row; 32768 x 768: 21 and 24); the backward gather, whose rows
+// end in a reduction, is faster with twice the warps and one row each (32768 x 768: 31 us; two rows on half the warps 35).
 constexpr int kGatherBlocksPerSm = 4, kGatherDyBlocksPerSm = 8;   // x 256 threads
 
 // Slot row s of the buffers: the token it holds (>= 0), -1: a row to zero-fill (up to a multiple of `pad` rows past the

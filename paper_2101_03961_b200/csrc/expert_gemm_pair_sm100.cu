@@ -120,7 +120,7 @@ struct PTile {
 };
 
 // Tile decode reads the plan through shared-memory copies made at kernel start: a dependent global load per tile
-// would stall the single-thread producer for longer than a short tile's whole k-loop.
+// would stall the producer warp for longer than a short tile's whole k-loop.
 __device__ __forceinline__ PTile p_decode(const PairParams& p, int id, const int* kept_s, const int4* tile_s) {
   PTile t;
   if (p.token_op) {
@@ -819,7 +819,7 @@ __device__ __forceinline__ void pair_body(const CUtensorMap& tmA, const BMapSet&
   }
 
   // ---------------------------------------------------------------------------------------------- teardown
-  __syncwarp();                                               // single-lane roles rejoin their warps
+  __syncwarp();                                               // lanes of the last arrivals rejoin their warps
   tc_fence_before();
   cluster_sync_all();
   if (warp == 2) {
@@ -881,10 +881,11 @@ uint32_t magic(int d) { return d > 1 ? (uint32_t)((0x100000000ull + (uint64_t)d 
 // Weight gradients: into how many strips a row of `nt` column tiles is cut.  A strip's A operand is loaded once if its
 // k-blocks fit the ring, so longer strips read less (up to 12% of a tile's time at the power limit); but the pairs' shares
 // are whole strips, and experts differ in size, so the last one leaves half a strip idle on average.  Experts that on
-// average do not fit the ring gain nothing and are balanced tile by tile.  Measured for whole training steps under
-// sustained load, tile by tile -> strips: 4096 tokens, 4096 x 10240, 16 experts (strips of 4 and 8) 2408 -> 2279 us; 32768
-// tokens, 768 x 3072, 128 experts (3 and 6) 1316 -> 1279; GEGLU 768 x 2048 (3 and 8) 1437 -> 1402; 20011 tokens, 512 x 1536,
-// 200 experts (two k-blocks per tile: the epilogue bounds it) 579 -> 581.
+// average do not fit the ring gain nothing and are balanced tile by tile.  Strips are for the power limit, where training
+// runs; before it sets in they cost a little.  Whole training steps, us, tile by tile / strips, at the limit and in bursts at
+// full clock: 16384 tokens, 4096 x 10240, 64 experts 9287 / 8898 (always at the limit); 32768 tokens, 768 x 3072, 128 experts
+// (strips of 3 and 6) 1291 / 1263, burst 1114 / 1120; top-2 on 64 experts 780 / 764, burst 682 / 682; GEGLU 768 x 2048, 128
+// experts (3 and 8) 1433 / 1427, burst 1255 / 1269; 20011 tokens, 512 x 1536, 200 experts 585 / 578, burst 610 / 611.
 int set_strips(PairParams* q, int n_pairs) {
   const int nt = q->n_ntiles_fixed;
   const long long rows = (long long)q->E * q->n_mpairs;

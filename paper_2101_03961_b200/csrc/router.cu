@@ -249,8 +249,8 @@ __device__ __forceinline__ void load_lane(const float* __restrict__ row, int e0,
 // A warp works on kTok tokens at a time; lane l holds experts NE l .. NE l + NE - 1 of each.  What bounds it is the number
 // of instructions (three quarters of the issue slots with one token per warp, scalar loads and a bound check per expert):
 // rows are loaded as vectors where E allows, experts past E carry p = 0 and need no checks, the loss term stays in
-// registers while the routing group does not change, and the bfloat16 parts are formed in pairs.  32768 tokens, 128 experts
-// 14.2 -> 12.0 us; router backward stage of 65536 tokens, 128 experts 63 -> 59, of top-2 with 64 experts 36 -> 32.
+// registers while the routing group does not change, and the bfloat16 parts are formed in pairs: 12.0 us instead of 14.2
+// (32768 tokens, 128 experts).
 template <int NE, bool kVec>                                   // kVec: E is a multiple of 4
 __global__ void __launch_bounds__(256)
 router_dlogits_kernel(const float* __restrict__ probs, const int* __restrict__ expert_index,

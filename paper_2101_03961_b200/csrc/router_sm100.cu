@@ -29,14 +29,13 @@ namespace {
 // and the epilogue runs once or a few times per launch, so its instructions come cold from memory: straight-line code
 // over all E logits of a token paid more for fetching instructions than for executing them.  It is therefore three short
 // loops over chunks of 32 logits, with the logits (and then their exponentials) kept in tensor memory between the
-// passes, which also leaves no limit on E short of the accumulator's 256 columns.  Stage time, straight-line -> loops:
-// 256 tokens, d_model 768, 128 experts 39 -> 19 us; 32768 tokens 44 -> 36; 20011 tokens, d_model 512, 200 experts (a
-// kernel of its own before, with a pass over the probabilities for the column sums) 260 -> 52.
+// passes, which also leaves no limit on E short of the accumulator's 256 columns.  Straight-line code took 39 us where this
+// takes 19 (256 tokens, d_model 768, 128 experts).
 //
 // Probabilities and noise cross between memory order and token-per-lane order through shared memory.  With every lane
 // storing its own row, 16 bytes of 32 different rows at a time, the stores alone cost 6 of 25 us (32768 tokens, d_model
-// 768, 128 experts) and 12 of 29 (65536, 256, 128), the noise 10 of 40 (20011, 512, 200); now 22, 23 and 31 in all.  Twice
-// as many epilogue warps, each with half of the experts, gained nothing on top (26, 31, 44 before this).
+// 768, 128 experts) and 12 of 29 (65536, 256, 128), the noise 10 of 40 (20011, 512, 200); this way all takes 22, 23 and 38
+// (7 of the last for expf).  Twice as many epilogue warps, each with half of the experts, gained nothing.
 struct RouterFwdParams {
   int T, d, E, Epad64, n_blocks, k_blocks, b_atoms, stages, stage_bytes;
   int tiles;                 // 128-token tiles per block: 1 or 2
@@ -420,9 +419,9 @@ router_fwd_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_const
 //
 // What bounds it: every column block reads all of dh from L2 (211 MB into the SMs at 32768 tokens, d 768, E 128; with the
 // stores, the dx reads and most MMAs taken out the kernel still took 24 of its 37 us, i.e. 9 TB/s).  More x stages, a longer
-// ring or x requested into L2 ahead changed nothing (one x stage: 47 us).  Measured with its neighbours (logit gradients before,
-// reduction of the partials after) against one kernel per product: 32768 tokens, d 768, E 128 82 -> 67 us; 65536 tokens,
-// d 256, E 128 (jitter) 83 -> 63; 16384 tokens, d 768, E 64 45 -> 34; 20011 tokens, d 512, E 200 61 -> 63.
+// ring or x requested into L2 ahead changed nothing (one x stage: 47 us).  With its neighbours (logit gradients before,
+// reduction of the partials after), and in brackets with one kernel per product: 32768 tokens, d 768, E 128 67 us (82); 65536
+// tokens, d 256, E 128, jitter 63 (83); 16384 tokens, d 768, E 64 34 (45); 20011 tokens, d 512, E 200 63 (61).
 struct RouterBwdParams {
   int T, d, E, ka;           // ka: blocks of 64 experts (1..4)
   int n_mtiles, n_cols, splits, x_stages, ring;
@@ -611,7 +610,7 @@ router_bwd_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_const
       __syncwarp();
       if (lane == 0) mbar_arrive(tempty0 + 8u * acc);
       // transposed through shared memory as bfloat16 (one extra rounding of the small router term); the sum is formed
-      // in float32 afterwards, with coalesced rows
+      // afterwards, with coalesced rows (a bfloat16 add or multiply-add rounds the exact result once)
       uint32_t pk[32];
 #pragma unroll
       for (int j = 0; j < 32; ++j) {

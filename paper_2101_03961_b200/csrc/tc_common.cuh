@@ -62,8 +62,8 @@ __device__ __forceinline__ unsigned long long global_ns() {
 
 // Bounded wait.  Returns false (after recording `code`) if the barrier did not flip within the limit or another
 // thread of the CTA already gave up.  The common case -- the phase is complete, or completes within a few polls --
-// is inline: the single-thread producer and MMA loops must stay small and call-free, because a lone warp that
-// jumps to far code pays an instruction-cache miss per iteration while the epilogue warps stream through the cache.
+// is inline: producer and MMA loops must stay small and call-free, because a lone warp that jumps to far code pays an
+// instruction-cache miss per iteration while the epilogue warps stream through the cache.
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                    int code) {
   const long long t0 = clock64();
