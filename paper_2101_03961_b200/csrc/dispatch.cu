@@ -251,9 +251,9 @@ plan_assign_kernel(const int* __restrict__ expert_index, const int* __restrict__
   }
 }
 
-// The plan of one routing group whose block histograms already exist (the tensor-core router's forward kernel leaves
-// hist[r][e] = tokens of its r-th block of `hist_tokens` tokens routed to expert e), in two kernels that both start from
-// that table.
+// The plan of one routing group from block histograms, hist[r][e] = tokens of the r-th block of `hist_tokens` tokens routed to
+// expert e (the tensor-core router's forward kernel leaves them, plan_hist_kernel counts them otherwise), in two kernels that
+// both start from that table.
 //
 // Slots: every block of 1024 tokens adds up the histogram columns itself -- all rows for the totals (kept_i =
 // min(count_i, C), Eq. 3), the rows before its own tokens for its position base -- instead of waiting for a scan kernel:
@@ -350,7 +350,7 @@ plan_slots_kernel(const int* __restrict__ expert_index, const int* __restrict__ 
 // Launched after plan_slots_kernel.  Reads only what the router wrote, past L1, and writes what no kernel in flight reads;
 // its own wait comes last, so that the next kernel's wait covers everything before this one.
 __global__ void __launch_bounds__(kFusedTokens)
-plan_summary_kernel(const int* hist, int hist_rows, const float* psum_partial, int T, int E, int Ew, int C,
+plan_summary_kernel(const int* hist, int hist_rows, const float* psum_partial, int psum_rows, int T, int E, int Ew, int C,
                     float alpha, int* __restrict__ count, float* __restrict__ psum, float* __restrict__ aux_loss,
                     int* __restrict__ tile_expert, int* __restrict__ tile_row0, int4* __restrict__ ntile,
                     int* __restrict__ count_g, int* __restrict__ group_base) {
@@ -363,13 +363,13 @@ plan_summary_kernel(const int* hist, int hist_rows, const float* psum_partial, i
   int tot = 0;
   float ps = 0.f;
   if (e < E) {
-    for (int r0 = q; r0 < hist_rows; r0 += 16 * Q) {            // 16 rows of each table in flight, added in row order
+    for (int r0 = q; r0 < max(hist_rows, psum_rows); r0 += 16 * Q) {   // 16 rows of each table in flight, added in row order
       int v[16];
       float f[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) v[j] = r0 + j * Q < hist_rows ? __ldcg(hist + (size_t)(r0 + j * Q) * E + e) : 0;
 #pragma unroll
-      for (int j = 0; j < 16; ++j) f[j] = r0 + j * Q < hist_rows ? __ldcg(psum_partial + (size_t)(r0 + j * Q) * E + e) : 0.f;
+      for (int j = 0; j < 16; ++j) f[j] = r0 + j * Q < psum_rows ? __ldcg(psum_partial + (size_t)(r0 + j * Q) * E + e) : 0.f;
 #pragma unroll
       for (int j = 0; j < 16; ++j) { tot += v[j]; ps += f[j]; }
     }
@@ -748,19 +748,22 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
   // good only right after it: the counting kernel below and every rerouting stage put tables of another layout in their
   // place, and the expert indices may have been edited since.
   const bool have_hist = after_router && s.router_hist;
-  if (have_hist && s.G == 1 && s.T <= kFusedMaxTokens) {
+  if (!have_hist)
+    launch_k(plan_hist_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, ei, s.Tv, s.E, ws_ptr<int>(ws, p.hist));
+  // (512 tokens, 8 experts, float32, between stage events: counting, slots and summary 13.4 us, counting, scan and assignment
+  // 20.9.)
+  if (s.G == 1 && !s.top2 && s.T <= kFusedMaxTokens) {
     const int token_blocks = (s.T + kFusedTokens - 1) / kFusedTokens;
-    launch_k(plan_slots_kernel, dim3(token_blocks), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist), s.router_blocks,
-             s.router_block_tokens, s.T, s.E, column_width(s.E), s.Cg, ws_ptr<int>(ws, p.slot),
+    const int hist_rows = have_hist ? s.router_blocks : s.plan_blocks;
+    launch_k(plan_slots_kernel, dim3(token_blocks), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist), hist_rows,
+             have_hist ? s.router_block_tokens : kPlanBlockTokens, s.T, s.E, column_width(s.E), s.Cg, ws_ptr<int>(ws, p.slot),
              ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.kept));
-    launch_k(plan_summary_kernel, dim3(1), dim3(kFusedTokens), 0, st, ws_ptr<int>(ws, p.hist), s.router_blocks,
-             ws_ptr<float>(ws, p.psum_partial), s.T, s.E, column_width(s.E), s.Cg, s.alpha, ws_ptr<int>(ws, p.count),
-             ws_ptr<float>(ws, p.psum), aux_loss, list128(s, p, ws), ws_ptr<int>(ws, p.tile_row0),
+    launch_k(plan_summary_kernel, dim3(1), dim3(kFusedTokens), 0, st, ws_ptr<int>(ws, p.hist), hist_rows,
+             ws_ptr<float>(ws, p.psum_partial), s.router_blocks, s.T, s.E, column_width(s.E), s.Cg, s.alpha,
+             ws_ptr<int>(ws, p.count), ws_ptr<float>(ws, p.psum), aux_loss, list128(s, p, ws), ws_ptr<int>(ws, p.tile_row0),
              ws_ptr<int4>(ws, p.ntile), ws_ptr<int>(ws, p.count_g), ws_ptr<int>(ws, p.group_base));
     return launch_reroute(s, p, ws, st);
   }
-  if (!have_hist)
-    launch_k(plan_hist_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, ei, s.Tv, s.E, ws_ptr<int>(ws, p.hist));
   const int Ew = column_width(s.E);
   const int blocks_per_group = s.plan_blocks / s.G;
   int* count_g = ws_ptr<int>(ws, p.count_g);
