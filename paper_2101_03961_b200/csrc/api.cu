@@ -135,11 +135,12 @@ int switch_moe_fwd(const switch_moe_config* cfg, const void* x, const float* W_r
   SWMOE_TRY(launch_router_fwd(c.s, c.p, x, W_r, router_bias, cfg->router_noise, true, workspace, st));
   if (c.s.top2) SWMOE_TRY(launch_top2_choice(c.s, c.p, workspace, st));     // assignments T .. 2T - 1
   SWMOE_TRY(mark(cfg, 1, st));
-  SWMOE_TRY(launch_dispatch_plan(c.s, c.p, nullptr, true, aux_loss, workspace, st));
+  if (!c.s.plan_gather) SWMOE_TRY(launch_dispatch_plan(c.s, c.p, nullptr, true, aux_loss, workspace, st));
   SWMOE_TRY(mark(cfg, 2, st));
   // top-2 routing: the experts write one weighted output row per assignment; the two rows of a token are summed last
   void* y_rows = c.s.top2 ? ws_ptr<void>(workspace, c.p.yv) : y;
-  SWMOE_TRY(launch_gather_x(c.s, c.p, x, y_rows, workspace, st));
+  if (c.s.plan_gather) SWMOE_TRY(launch_plan_gather(c.s, c.p, x, y_rows, aux_loss, workspace, st));
+  else SWMOE_TRY(launch_gather_x(c.s, c.p, x, y_rows, workspace, st));
   GemmArgs a{};
   a.W_in = W_in; a.W_out = W_out; a.y = y_rows; a.x = x;
   SWMOE_TRY(mark(cfg, 3, st));
@@ -327,7 +328,8 @@ int switch_moe_stage_launches(const switch_moe_config* cfg, int32_t* launches_ou
   n[0] = (s.router_tc ? 2 : 1) + (s.jitter ? 1 : 0) + (s.top2 ? 1 : 0);
   // plan: slots and, beside them, the summary when the router left the histograms and there is one routing group; else
   // (histogram,) scan, assign; a stage of rerouting adds four
-  n[1] = (s.router_hist ? 2 : 3) + 4 * s.reroute_stages;
+  // (up to 256 tokens of one group: part of the gather's launch)
+  n[1] = s.plan_gather ? 0 : (s.router_hist ? 2 : 3) + 4 * s.reroute_stages;
   n[2] = 1;                                           // gather
   const int slow = s.gemm_path != 0 ? 1 : 0;   // gating and dropout are element-wise kernels off the CTA-pair path
   n[3] = 1 + (s.geglu ? slow : 0) + (s.dropout ? slow : 0);   // GEMM1 (+ GEGLU gating kernel, + expert dropout kernel)

@@ -13,6 +13,7 @@ namespace swmoe {
 
 constexpr int kMaxExperts = 256;        // router kernels keep ceil(E/32) <= 8 experts per lane
 constexpr int kPlanBlockTokens = 256;   // tokens per dispatch-plan block (one histogram row each)
+constexpr int kSmallTokens = 256;      // up to here the plan and the forward gather are one launch
 constexpr int kTileM = 128;             // token rows per tensor-core tile; tails are zero-filled to this
 constexpr int kPairTileTokens = 320;    // widest token tile of the paired-CTA GEMM (tokens on the MMA's N side, two
                                         // column segments above 256): an expert within the capacity of the paper's
@@ -36,6 +37,7 @@ struct Shape {
   int router_tc;    // 1: router on the tensor cores (bf16 x, bf16 split of fp32 operands); 0: FP32 FMA
   int router_hist;  // 1: the router's forward kernel also writes the dispatch plan's block histograms
   int router_blocks, plan_blocks, max_mtiles, dwr_chunks;
+  int plan_gather;  // 1: dispatch plan and forward gather in one launch
   int router_block_tokens;   // tokens per block of the router's forward kernel: one row of P-sums (tensor cores: and histogram)
   int dwr_chunk_tokens;      // FP32-FMA router: tokens per split of the dW_r sum
   int residual;     // 1: y = x + layer(x), dx = dy + d layer / dx (SWITCH_MOE_FLAG_RESIDUAL)
@@ -134,6 +136,7 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
   s->router_hist = (s->router_tc && !s->top2) ? 1 : 0;
   s->plan_blocks = (s->Tv + kPlanBlockTokens - 1) / kPlanBlockTokens;
   s->max_mtiles = cfg->E * ((s->C + kTileM - 1) / kTileM);
+  s->plan_gather = G == 1 && cfg->T <= kSmallTokens && !s->top2 && !s->reroute ? 1 : 0;
   s->dwr_chunk_tokens = 0;
   if (s->router_tc) {
     // One 128-token tile per block while there are SMs for all of them, then two tiles that share the staged W_r.
@@ -263,6 +266,7 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
 int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void* ws, cudaStream_t st);
 // Top-2 routing: second choices (expert and weight) of every token; sums of the two assignments' rows.
 int launch_top2_choice(const Shape& s, const Plan& p, void* ws, cudaStream_t st);
+int launch_plan_gather(const Shape& s, const Plan& p, const void* x, void* y, float* aux_loss, void* ws, cudaStream_t st);
 // `skip` (may be null): rows added to the sum, the layer's input (forward) or dy (backward) when the layer carries its
 // own residual connection.
 int launch_top2_sum(const Shape& s, const Plan& p, const void* per_assignment, const void* skip, void* out, void* ws,
