@@ -38,7 +38,9 @@ enum switch_moe_dtype { SWITCH_MOE_BF16 = 0, SWITCH_MOE_F32 = 1 };
 
 enum switch_moe_gemm_path {
   SWITCH_MOE_GEMM_DEFAULT = 0, /* bf16: tcgen05 grouped GEMM on CTA pairs (tokens on the MMA N side) and tensor-core
-                                  router; f32: plain FP32 FMA grouped GEMM and router */
+                                  router; f32: products on tcgen05 as sums of exact bfloat16 parts where they are
+                                  large enough (error against float64 no larger than FP32 FMA's), the others and
+                                  the router on FP32 FMA */
   SWITCH_MOE_GEMM_SIMT = 1,    /* validation only: FP32-FMA grouped GEMM and router for either dtype */
   SWITCH_MOE_GEMM_TC_1CTA = 2  /* validation only: single-CTA tcgen05 grouped GEMM with 128-token tiles (bf16) */
 };

@@ -28,6 +28,7 @@ int prepare(const switch_moe_config* cfg, const void* workspace, size_t workspac
 int run_gemm(GemmOp op, const Ctx& c, const GemmArgs& a, void* ws, cudaStream_t st) {
   if (c.s.gemm_path == 0) return launch_pair_gemm(op, c.s, c.p, a, ws, st);
   if (c.s.gemm_path == 2) return launch_tc_gemm(op, c.s, c.p, a, ws, st);
+  if (c.s.f32_tc) return launch_f32_gemm(op, c.s, c.p, a, ws, st);
   return launch_simt_gemm(op, c.s, c.p, a, ws, st);
 }
 

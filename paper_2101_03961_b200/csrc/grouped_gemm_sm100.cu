@@ -344,6 +344,20 @@ int tc::make_map(CUtensorMap* tm, const void* base, long long E, long long rows,
   return r == CUDA_SUCCESS ? SWITCH_MOE_OK : SWITCH_MOE_CUDA_ERROR;
 }
 
+int tc::make_map_f32(CUtensorMap* tm, const void* base, long long E, long long rows, long long cols, int box_cols,
+                     int box_rows) {
+  EncodeTiledFn fn = get_encode_fn();
+  if (fn == nullptr) return SWITCH_MOE_CUDA_ERROR;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)E};
+  cuuint64_t strides[2] = {(cuuint64_t)cols * 4, (cuuint64_t)cols * (cuuint64_t)rows * 4};
+  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, 1};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, estr,
+                  CU_TENSOR_MAP_INTERLEAVE_NONE, box_cols == 32 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                  CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? SWITCH_MOE_OK : SWITCH_MOE_CUDA_ERROR;
+}
+
 
 int launch_tc_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st) {
   int dev = 0, sm_count = 0;

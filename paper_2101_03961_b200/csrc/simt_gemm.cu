@@ -1,8 +1,8 @@
 // Grouped expert GEMMs on the plain FP32 FMA pipes (no tensor cores): the expert FFN h = x W_in, y = ReLU(h) W_out
 // (Section 5, FFN review) and its derivatives, one problem per expert, with the same fused epilogues as the
-// tensor-core path.  This is the arithmetic path of the all-float32 configuration (tensor cores have no exact
-// float32 mode) and a validation path for bfloat16 inputs; accumulation is float32 in both, one fused multiply-add per
-// term in ascending order of the contraction index, whatever the tile.
+// tensor-core path.  These are the small products of the float32 layer (f32_gemm_sm100.cu has the rule and the others) and a
+// validation path for either type; accumulation is float32, one fused multiply-add per term in ascending order of the
+// contraction index, whatever the tile.
 //
 // What bounds it is the FMA pipes: 128 multiply-adds per SM and clock, 74.5 TFLOP/s.  A plain FFMA takes an issue slot
 // per multiply-add and leaves none for the operand loads; the packed form (fma.rn.f32x2, two independent IEEE

@@ -30,14 +30,15 @@ struct Shape {
   int G, Tg, Cg;    // routing groups, tokens per group, capacity of one expert for one group (Eq. 3)
   int dtype;        // switch_moe_dtype
   int gemm_path;    // resolved: 0 = tcgen05 on CTA pairs, 1 = SIMT, 2 = single-CTA tcgen05
+  int f32_tc;       // 1: float32 expert products on the tensor cores (exact bfloat16 parts); 0: FP32 FMA
   float alpha;
   size_t elt;       // bytes per activation / expert-weight element
   int Epad;         // E rounded up to 32 * {1,2,4,8}
   int Epad64;       // E rounded up to a multiple of 64 (tensor-core router operands)
   int router_tc;    // 1: router on the tensor cores (bf16 x, bf16 split of fp32 operands); 0: FP32 FMA
   int router_hist;  // 1: the router's forward kernel also writes the dispatch plan's block histograms
-  int router_blocks, plan_blocks, max_mtiles, dwr_chunks;
   int plan_gather;  // 1: dispatch plan and forward gather in one launch
+  int router_blocks, plan_blocks, max_mtiles, dwr_chunks;
   int router_block_tokens;   // tokens per block of the router's forward kernel: one row of P-sums (tensor cores: and histogram)
   int dwr_chunk_tokens;      // FP32-FMA router: tokens per split of the dW_r sum
   int residual;     // 1: y = x + layer(x), dx = dy + d layer / dx (SWITCH_MOE_FLAG_RESIDUAL)
@@ -100,6 +101,7 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
   s->C = (int)C * G;
   s->elt = cfg->dtype == SWITCH_MOE_BF16 ? 2 : 4;
   s->gemm_path = (cfg->dtype == SWITCH_MOE_F32 || cfg->gemm_path == SWITCH_MOE_GEMM_SIMT) ? 1 : cfg->gemm_path;
+  s->f32_tc = cfg->dtype == SWITCH_MOE_F32 && cfg->gemm_path != SWITCH_MOE_GEMM_SIMT ? 1 : 0;
   if (s->gemm_path != 1 && (cfg->d_model % 64 != 0 || cfg->d_ff % 64 != 0)) return SWITCH_MOE_UNSUPPORTED_SHAPE;
   s->residual = (cfg->flags & SWITCH_MOE_FLAG_RESIDUAL) ? 1 : 0;
   if (s->residual && s->gemm_path == SWITCH_MOE_GEMM_TC_1CTA) return SWITCH_MOE_UNSUPPORTED_SHAPE;
@@ -134,9 +136,9 @@ inline int resolve_shape(const switch_moe_config* cfg, Shape* s) {
   s->Epad64 = (cfg->E + 63) / 64 * 64;
   s->router_tc = s->gemm_path != 1 ? 1 : 0;
   s->router_hist = (s->router_tc && !s->top2) ? 1 : 0;
+  s->plan_gather = G == 1 && cfg->T <= kSmallTokens && !s->top2 && !s->reroute ? 1 : 0;
   s->plan_blocks = (s->Tv + kPlanBlockTokens - 1) / kPlanBlockTokens;
   s->max_mtiles = cfg->E * ((s->C + kTileM - 1) / kTileM);
-  s->plan_gather = G == 1 && cfg->T <= kSmallTokens && !s->top2 && !s->reroute ? 1 : 0;
   s->dwr_chunk_tokens = 0;
   if (s->router_tc) {
     // One 128-token tile per block while there are SMs for all of them, then two tiles that share the staged W_r.
@@ -264,9 +266,9 @@ int launch_router_fwd(const Shape& s, const Plan& p, const void* x, const float*
 int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_index, bool after_router, float* aux_loss,
                          void* ws, cudaStream_t st);
 int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void* ws, cudaStream_t st);
+int launch_plan_gather(const Shape& s, const Plan& p, const void* x, void* y, float* aux_loss, void* ws, cudaStream_t st);
 // Top-2 routing: second choices (expert and weight) of every token; sums of the two assignments' rows.
 int launch_top2_choice(const Shape& s, const Plan& p, void* ws, cudaStream_t st);
-int launch_plan_gather(const Shape& s, const Plan& p, const void* x, void* y, float* aux_loss, void* ws, cudaStream_t st);
 // `skip` (may be null): rows added to the sum, the layer's input (forward) or dy (backward) when the layer carries its
 // own residual connection.
 int launch_top2_sum(const Shape& s, const Plan& p, const void* per_assignment, const void* skip, void* out, void* ws,
@@ -322,6 +324,7 @@ struct GemmArgs {
   const void* x; const void* dy;         // skip-path sources (residual configuration only): y += x, dx += dy
 };
 int launch_simt_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
+int launch_f32_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
 int launch_tc_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
 int launch_pair_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
 int launch_pair_dgrad1_wgrad1(const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);

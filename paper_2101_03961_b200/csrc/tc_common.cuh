@@ -183,6 +183,8 @@ __device__ __forceinline__ uint64_t make_smem_desc(uint32_t addr, uint32_t lbo_b
 
 // bf16 tensor [E][rows][cols] (cols contiguous), box {64 cols, box_rows rows, 1}, 128-byte swizzle, zero OOB fill.
 int make_map(CUtensorMap* tm, const void* base, long long E, long long rows, long long cols, int box_rows);
+// float32 tensor [E][rows][cols], box {box_cols, box_rows, 1}, zero OOB fill; 128-byte swizzle where a box row is 128 bytes.
+int make_map_f32(CUtensorMap* tm, const void* base, long long E, long long rows, long long cols, int box_cols, int box_rows);
 
 }  // namespace tc
 }  // namespace swmoe

@@ -1,0 +1,112 @@
+"""The float32 layer's expert products on the tensor cores, each against float64 products of the operands that the call left
+in its workspace, at the edges of the kernel's tiles and chunks; and values that bfloat16 parts cannot hold."""
+import math
+
+import pytest
+import torch
+
+from paper_2101_03961_b200 import switch_moe as sm
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(T, d, f, E, cf, path, residual=False, seed=1, spoil=None):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+
+    def normal(*shape):
+        return torch.empty(shape, device="cuda").normal_(generator=g)
+
+    t = {"x": normal(T, d), "dy": normal(T, d), "W_in": normal(E, d, f) * (0.1 / d) ** 0.5,
+         "W_out": normal(E, f, d) * (0.1 / f) ** 0.5, "W_r": torch.zeros(d, E, device="cuda"), "noise": 2.0 * normal(T, E)}
+    if spoil is not None:
+        spoil(t)
+    cfg = sm.make_config(T, d, f, E, cf, dtype=sm.F32, residual=residual, gemm_path=path)
+    cfg.router_noise = t["noise"].data_ptr()                   # W_r = 0: the noise decides the routing, dx has no router term
+    ws = sm.allocate_workspace(cfg)
+    ws.fill_(0xFF)                                             # stale rows read as NaN
+    for k in ("y", "dx"):
+        t[k] = torch.empty_like(t["x"])
+    for k in ("W_r", "W_in", "W_out"):
+        t["d" + k] = torch.empty_like(t[k])
+    aux = torch.empty(1, device="cuda")
+    sm.switch_moe_fwd(cfg, t["x"], t["W_r"], None, t["W_in"], t["W_out"], t["y"], aux, ws)
+    sm.switch_moe_bwd(cfg, t["dy"], 1.0, t["x"], t["W_r"], t["W_in"], t["W_out"], t["y"], ws, t["dx"], t["dW_r"], t["dW_in"],
+                      t["dW_out"])
+    sm.switch_moe_check_device_status(cfg, ws)
+    C = sm.switch_moe_capacity(cfg)
+    view = lambda region: sm.switch_moe_workspace_view(cfg, ws, region)  # noqa: E731
+    for name, region, cols in (("X", sm.WS_XD, d), ("H", sm.WS_H, f), ("dY", sm.WS_DYD, d), ("dH", sm.WS_DH, f)):
+        t[name] = view(region).view(torch.float32).view(E, C, cols)
+    t["kept"] = view(sm.WS_KEPT).tolist()
+    t["tokens"] = view(sm.WS_TOKEN_OF_SLOT).view(E, C).long()
+    t["gate"] = view(sm.WS_GATE)
+    return t
+
+
+def _errors(t, residual):
+    """Relative Frobenius error of each product, and the contraction lengths of the weight gradients."""
+    num, den = {}, {}
+
+    def add(name, got, want):
+        num[name] = num.get(name, 0.0) + float(((got.double() - want) ** 2).sum())
+        den[name] = den.get(name, 0.0) + float((want ** 2).sum())
+
+    for e, n in enumerate(t["kept"]):
+        x, h, dy, dh = (t[k][e, :n].double() for k in ("X", "H", "dY", "dH"))
+        w_in, w_out, tok = t["W_in"][e].double(), t["W_out"][e].double(), t["tokens"][e, :n]
+        add("gemm1", t["H"][e, :n], (x @ w_in).clamp(min=0))
+        skip_y, skip_dx = (t["x"][tok].double(), t["dy"][tok].double()) if residual else (0.0, 0.0)
+        add("gemm2", t["y"][tok], (h @ w_out) * t["gate"][tok].double()[:, None] + skip_y)
+        add("dgrad2", t["dH"][e, :n], (dy @ w_out.T) * (h > 0))
+        add("dgrad1", t["dx"][tok], dh @ w_in.T + skip_dx)
+        add("wgrad2", t["dW_out"][e], h.T @ dy)
+        add("wgrad1", t["dW_in"][e], x.T @ dh)
+    return {k: math.sqrt(num[k] / den[k]) for k in num}
+
+
+SHAPES = [
+    (1024, 128, 512, 4, 1.25, False),      # whole tiles of m, two tiles of tokens
+    (4100, 72, 1000, 16, 1.25, True),      # remainders of m, of a chunk and of 16 tokens; the skip path
+    (5000, 8, 3000, 8, 2.0, False),        # contractions of one MMA step and of many chunks
+    (3000, 520, 24, 60, 2.0, True),        # about 50 tokens per expert
+    (4096, 512, 2048, 16, 1.0, False),     # a full capacity of 256
+    (1500, 264, 1032, 50, 1.25, False),    # about 30 tokens per expert: a chunk, less and more
+]
+
+
+@pytest.mark.parametrize("T,d,f,E,cf,residual", SHAPES)
+def test_products_of_exact_parts(T, d, f, E, cf, residual):
+    """Bound: of n = ceil(K / 32) chunks each truncates two sums at the size of the chunk (2^-23 each; chunks are independent,
+    together 4 2^-24 of the result), and the float32 sum over the chunks rounds n times at the size of a running sum of random
+    terms (2^-24 sqrt(n / 2)); one more rounding for the gate and the skip path each."""
+    t = _layer(T, d, f, E, cf, sm.GEMM_DEFAULT, residual)
+    errs = _errors(t, residual)
+    fma = _errors(_layer(T, d, f, E, cf, sm.GEMM_SIMT, residual), residual)
+    tokens = max(t["kept"])
+    for name, K in (("gemm1", d), ("gemm2", f), ("dgrad2", d), ("dgrad1", f), ("wgrad2", tokens), ("wgrad1", tokens)):
+        assert errs[name] <= 2.0 ** -24 * (6.0 + math.sqrt(math.ceil(K / 32) / 2.0)), (name, errs)
+        assert errs[name] <= 1.05 * fma[name], (name, errs, fma)     # no less precise than a chain of fused multiply-adds
+    again = _layer(T, d, f, E, cf, sm.GEMM_DEFAULT, residual)
+    for k in ("y", "dx", "dW_in", "dW_out"):
+        assert torch.equal(t[k], again[k])
+
+
+def test_values_that_the_parts_cannot_hold():
+    """Infinities, NaN and the largest floats come out as they do from fused multiply-adds, and stay where they belong."""
+    def spoil(t):
+        t["W_in"][0, 3, 5] = math.inf
+        t["W_in"][1, 4, 6] = math.nan
+        t["W_out"][2, 7, 9] = -math.inf
+        t["W_out"][0, 100, 2] = 3.4028234e38
+        t["W_in"][3, 10, 7] = 3.4e38
+        t["dy"][17, 11] = math.inf
+        t["dy"][18, 12] = math.nan
+
+    a, b = (_layer(2048, 128, 512, 4, 1.25, path, residual=True, spoil=spoil) for path in (sm.GEMM_DEFAULT, sm.GEMM_SIMT))
+    for k in ("y", "dx", "dW_in", "dW_out"):
+        ra, rb = a[k], b[k]
+        assert torch.equal(torch.isnan(ra), torch.isnan(rb)), k
+        assert torch.equal(torch.isposinf(ra), torch.isposinf(rb)) and torch.equal(torch.isneginf(ra), torch.isneginf(rb)), k
+        fin = torch.isfinite(rb) & (rb.abs() < 1e30)
+        assert float((ra[fin] - rb[fin]).norm()) <= 1e-5 * float(rb[fin].norm()), k
