@@ -664,6 +664,7 @@ gather_x_kernel(const uint4* __restrict__ x, const int* __restrict__ token_of_sl
 // takes one.  Every block ranks all tokens itself (a token per thread, in token order as in plan_slots_kernel, no atomics) and
 // then moves its share of the rows; block 0 also leaves what the summary leaves.  96 tokens, d 256, E 8, whole forward pass
 // 26.7 us before, 24.2 with this; 256 tokens, d 768, E 128 187.5 and 184.4.
+__host__ __device__ inline int small_plan_parts(int C, int pad) { return ((C < pad ? C : pad) + 15) / 16; }
 __global__ void __launch_bounds__(kSmallTokens)
 plan_gather_small_kernel(const int* __restrict__ expert_index, const float* __restrict__ psum_partial, int psum_rows, int T,
                          int E, int C, float alpha, int row_vec, int pad, int residual, const uint4* __restrict__ x,
@@ -736,11 +737,15 @@ plan_gather_small_kernel(const int* __restrict__ expert_index, const float* __re
     }
   }
   // empty slots, and the zero rows that a tile may read past an expert's last token (see slot_source)
-  for (int ex = gw; ex < E; ex += n_warps) {
-    const int k = kept_s[ex], zero_end = min(C, (k + pad - 1) / pad * pad);
-    for (int pos = k + lane; pos < C; pos += 32) token_of_slot[ex * C + pos] = -1;
+  // 16 of them per warp at a time
+  const int parts = small_plan_parts(C, pad);
+  for (int i = gw; i < E * parts; i += n_warps) {
+    const int ex = i / parts, part = i - ex * parts, k = kept_s[ex], r0 = k + 16 * part;
+    const int r1 = min(min(C, (k + pad - 1) / pad * pad), r0 + 16);
+    if (part == 0)
+      for (int pos = k + lane; pos < C; pos += 32) token_of_slot[ex * C + pos] = -1;
     uint4* rows = xd + (size_t)ex * C * row_vec;
-    for (int v = k * row_vec + lane; v < zero_end * row_vec; v += 32) rows[v] = make_uint4(0, 0, 0, 0);
+    for (int v = r0 * row_vec + lane; v < r1 * row_vec; v += 32) rows[v] = make_uint4(0, 0, 0, 0);
   }
   if (blockIdx.x == 0)
     write_tile_lists(term, kept_s, E, alpha * (float)E, aux_loss, tile_expert, tile_row0, ntile);
@@ -928,8 +933,9 @@ int launch_gather_x(const Shape& s, const Plan& p, const void* x, void* y, void*
 // launch_dispatch_plan and launch_gather_x in one launch, where `s.plan_gather` says so.
 int launch_plan_gather(const Shape& s, const Plan& p, const void* x, void* y, float* aux_loss, void* ws, cudaStream_t st) {
   const int row_vec = (int)((size_t)s.d * s.elt / 16);
-  const int rows = s.T > s.E ? s.T : s.E, warps = kSmallTokens / 32;
-  launch_k(plan_gather_small_kernel, dim3((unsigned)((rows + warps - 1) / warps)), dim3(kSmallTokens), 0, st,
+  const int zero_parts = s.E * small_plan_parts(s.C, pad_rows(s)), rows = s.T > zero_parts ? s.T : zero_parts;
+  const int warps = kSmallTokens / 32, blocks = (rows + warps - 1) / warps;
+  launch_k(plan_gather_small_kernel, dim3((unsigned)(blocks < kChipSms ? blocks : kChipSms)), dim3(kSmallTokens), 0, st,
            ws_ptr<int>(ws, p.expert_index), ws_ptr<float>(ws, p.psum_partial), s.router_blocks, s.T, s.E, s.C, s.alpha, row_vec,
            pad_rows(s), s.residual, static_cast<const uint4*>(x), ws_ptr<uint4>(ws, p.xd), static_cast<uint4*>(y),
            ws_ptr<int>(ws, p.slot), ws_ptr<int>(ws, p.token_of_slot), ws_ptr<int>(ws, p.count), ws_ptr<int>(ws, p.kept),

@@ -13,7 +13,7 @@ from tests.test_gpu_parity import _check_layer
     (1, 64, 1, 1.0, {}), (31, 64, 3, 1.0, dict(residual=True)), (33, 192, 5, 2.0, {}), (96, 256, 8, 2.0, dict(residual=True)),
     (129, 128, 64, 2.0, {}), (255, 64, 65, 1.25, dict(jitter_eps=0.2)), (256, 320, 128, 2.0, dict(noise_eps=0.3)),
     (256, 128, 129, 2.0, {}), (256, 64, 256, 1.0, dict(residual=True)), (200, 64, 126, 4.0, dict(geglu=True)),
-    (256, 64, 2, 0.5, dict(residual=True)), (257, 128, 128, 2.0, {}), (256, 64, 8, 1.0, dict(reroute=True)),
+    (256, 64, 2, 0.5, dict(residual=True)), (250, 64, 3, 4.0, {}), (257, 128, 128, 2.0, {}), (256, 64, 8, 1.0, dict(reroute=True)),
 ])
 @pytest.mark.parametrize("dtype", [si.DTYPE_BF16, si.DTYPE_F32])
 def test_small_calls_match_oracle(T, d, E, cf, kw, dtype):
