@@ -618,15 +618,16 @@ int launch_op(const CUtensorMap& tmA, const CUtensorMap& tmB, const F32Problem& 
 }  // namespace
 
 // Which float32 products run here, by what they multiply (2 rows d f) and, for weight gradients, by the tokens per expert.  A
-// launch has about 4 us more to set up than an FMA kernel (tensor memory, barriers, cold code): 8 us against 5 at 17 MFLOP, as
-// fast at about 70 to 100 (1024 tokens, 128 x 256, 8 experts: GEMM1 13.0 us here, 11.7 there; 600 tokens, 128 x 1024, 16: 13.0
-// and 15.2), then ahead (4096 tokens, 512 x 2048, 16: see above).  A weight gradient of few tokens is bound by writing its
-// output, and a tile's one or two stages hide none of that (64 experts of 768 x 3072: 191 us here and 173 there with 16 tokens
-// each, 184 and 204 with 24).  GEMM1 and dgrad2 multiply the same, so the mask that one leaves is the one that the other reads.
+// launch has about 3 us more to set up than an FMA kernel (tensor memory, barriers, cold code).  Between stage events, here /
+// FMA kernels, us, GEMM1, GEMM2, wgrad2: 17 MFLOP (512 tokens, 64 x 256, 8 experts) 10.9 / 8.4, 14.2 / 14.1, 12.7 / 9.6; 67 (1024
+// tokens, 128 x 256, 8) 12.7 / 12.1, 14.6 / 14.7, 14.4 / 12.1; 79 (300 tokens, 256 x 512, 4) 14.1 / 13.8, 17.9 / 20.2, 12.3 / 12.3;
+// 157 (600 tokens, 128 x 1024, 16) 13.6 / 14.6, 25.0 / 32.7, 12.3 / 12.3.  A weight gradient of few tokens is bound by writing its
+// output, and a tile's one or two stages hide none of that (64 experts of 768 x 3072: 8 tokens each 209 / 141, 16 tokens 193 /
+// 173, 24 tokens 174 / 204).  GEMM1 and dgrad2 multiply the same, so the mask that one leaves is the one that the other reads.
 bool f32_on_tensor_cores(GemmOp op, const Shape& s) {
-  const double rows = s.Tv < (double)s.E * s.C ? s.Tv : (double)s.E * s.C;
-  if (2.0 * rows * s.d * s.f < 1.2e8) return false;
-  return (op != kWgrad2 && op != kWgrad1) || rows >= 20.0 * s.E;
+  const double rows = s.Tv < (double)s.E * s.C ? s.Tv : (double)s.E * s.C, flops = 2.0 * rows * s.d * s.f;
+  if (op == kWgrad2 || op == kWgrad1) return flops >= 1.2e8 && rows >= 20.0 * s.E;
+  return flops >= 7e7;
 }
 
 int launch_f32_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st) {

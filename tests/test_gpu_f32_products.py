@@ -66,7 +66,7 @@ def _errors(t, residual):
 
 
 SHAPES = [
-    (1024, 128, 512, 4, 1.25, False),      # whole tiles of m, two tiles of tokens
+    (1024, 128, 512, 4, 1.25, False),      # whole tiles of m, several tiles of tokens
     (4100, 72, 1000, 16, 1.25, True),      # remainders of m, of a chunk and of 16 tokens; the skip path
     (5000, 8, 3000, 8, 2.0, False),        # contractions of one MMA step and of many chunks
     (3000, 520, 24, 60, 2.0, True),        # about 50 tokens per expert
