@@ -2,16 +2,18 @@
 // FFN h = x W_in, y = ReLU(h) W_out (Section 5, FFN review) and its derivatives, float32 in, float32 out, with the fused
 // epilogues of the FMA kernels in simt_gemm.cu.
 //
-// Arithmetic.  A float32 is the exact sum of three bfloat16 parts, x = h + m + l (8 + 8 + 8 significand bits, each rounded
-// to nearest), and a product of two bfloat16 is exact in float32.  Of the nine cross products six are formed (h.h, h.m, m.h,
-// m.m, h.l, l.h); the other three are below 2^-25 of the product.  The tensor pipe adds into its float32 accumulator with
+// Arithmetic.  A float32 times 2^24 is the exact sum of three bfloat16 parts, h + m + l (8 + 8 + 8 significand bits, each
+// rounded to nearest), from the smallest subnormal up to 2^104 (unscaled, l of an operand below 2^-110 would reach under
+// bfloat16's smallest subnormal: 2^-118 came out exact to 1e-5 only), and a product of two bfloat16 is exact in float32; the
+// sums are scaled back by 2^-48.  Of the nine cross products six are formed (h.h, h.m, m.h, m.m, h.l, l.h); the other three
+// are below 2^-25 of the product.  The tensor pipe adds into its float32 accumulator with
 // truncation, so a long sum left there would drift: here an accumulator lives for kK = 32 steps of the contraction only.
 // Within such a chunk the five correction products (at most 2^-8 of the sum) go first and h.h last, then the chunk is read
 // out of tensor memory and added to a float32 sum in registers, round to nearest.  A chain of one fused multiply-add per step
 // rounds at the size of the running sum K times, this one K / 32 times (and twice inside a chunk): the error against
 // float64 is smaller than the FMA kernels' at every contraction length (tests/test_gpu_f32_products.py holds it to that).
-// Values a bfloat16 cannot hold (infinities, NaN, |x| at the end of the range) turn up as a non-finite result; that
-// element is then formed again by a plain chain of fused multiply-adds from the float32 operands.
+// Values that the parts cannot hold (infinities, NaN, |x| from 2^104 on) and sums from 2^80 on turn up as a non-finite result;
+// that element is then formed again by a plain chain of fused multiply-adds from the float32 operands.
 //
 // Layout.  All six products are written out[n][m], m contiguous: m = weight columns or rows on the MMA's M side (tiles of
 // 128, TMEM lanes), n = an expert's tokens, or the other index of a weight gradient, on the N side, at most 128 wide (64 sums
@@ -56,6 +58,8 @@ constexpr int kTabBytes = kEpiWarps * kHalf * 8;     // output row and scale per
 constexpr int kCumBytes = (2 * kMaxExperts + 1 + 2 * 10) * 4;
 constexpr int kF32Smem = 1024 + kLoadStages * kLoadBytes + kPartStages * kPartStage + kTabBytes + 256 + kCumBytes;
 constexpr int kWidths = kNMax / 16;                  // candidate tile widths: 16, 32 .. kNMax
+
+constexpr float kUp = 16777216.f, kDown = 1.f / (kUp * kUp);    // scale of the operands, of the sums
 
 struct F32Problem {
   const float* A; long long a_es, a_ms, a_ks;        // A(e, m, k) element strides (the loads go through the tensor maps)
@@ -124,6 +128,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 // x minus the packed bfloat16 pair h (exact: h is x rounded to bfloat16).
 __device__ __forceinline__ float2 minus_pair(float2 x, uint32_t h) {
   uint64_t r;
@@ -135,9 +144,9 @@ __device__ __forceinline__ uint32_t bf16_pair(float2 v) {
   const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
   return *reinterpret_cast<const uint32_t*>(&b);
 }
-// Two consecutive floats of the contraction -> packed bfloat16 pairs of their three parts.
+// Two consecutive floats of the contraction -> packed bfloat16 pairs of the three parts of x 2^24.
 __device__ __forceinline__ void split3(float x0, float x1, uint32_t* h, uint32_t* m, uint32_t* l) {
-  float2 x = make_float2(x0, x1);
+  float2 x = unpack2(mul2(pack2(x0, x1), pack2(kUp, kUp)));
   *h = bf16_pair(x);
   x = minus_pair(x, *h);
   *m = bf16_pair(x);
@@ -556,7 +565,7 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
         float v[8];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float2 a = unpack2(sum[4 * g + j]);
+          const float2 a = unpack2(mul2(sum[4 * g + j], pack2(kDown, kDown)));
           v[2 * j] = a.x; v[2 * j + 1] = a.y;
         }
         const int left = mine - 8 * g;

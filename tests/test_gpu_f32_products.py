@@ -92,6 +92,25 @@ def test_products_of_exact_parts(T, d, f, E, cf, residual):
         assert torch.equal(t[k], again[k])
 
 
+@pytest.mark.parametrize("scale", [
+    dict(x=-118, W_in=74, W_out=46, dy=-46), dict(dy=-118, W_out=74), dict(W_out=-118, W_in=33, dy=33),
+    dict(W_in=-118, x=60, W_out=60, dy=-50), dict(x=-59, W_in=-59, W_out=60), dict(dy=-59, W_out=-59, W_in=60)],
+    ids=["x", "dy", "W_out", "W_in", "H", "dH"])
+def test_products_of_small_operands(scale):
+    """Operands around 2^-118, subnormal ones among them, in every product that has such an operand: a power of two changes no
+    rounding, so the bound of ordinary operands holds."""
+    def spoil(t):
+        for name, e in scale.items():
+            t[name] *= 2.0 ** e
+
+    shape = (2048, 128, 512, 4, 1.25)
+    t = _layer(*shape, sm.GEMM_DEFAULT, spoil=spoil)
+    errs, fma, tokens = _errors(t, False), _errors(_layer(*shape, sm.GEMM_SIMT, spoil=spoil), False), max(t["kept"])
+    for name, K in (("gemm1", 128), ("gemm2", 512), ("dgrad2", 128), ("dgrad1", 512), ("wgrad2", tokens), ("wgrad1", tokens)):
+        assert errs[name] <= 2.0 ** -24 * (6.0 + math.sqrt(math.ceil(K / 32) / 2.0)), (name, errs)
+        assert errs[name] <= fma[name], (name, errs, fma)
+
+
 def test_values_that_the_parts_cannot_hold():
     """Infinities, NaN and the largest floats come out as they do from fused multiply-adds, and stay where they belong."""
     def spoil(t):
