@@ -13,7 +13,7 @@
 // rounds at the size of the running sum K times, this one K / 32 times (and twice inside a chunk): the error against
 // float64 is smaller than the FMA kernels' at every contraction length (tests/test_gpu_f32_products.py holds it to that).
 // Values that the parts cannot hold (infinities, NaN, |x| from 2^104 on) and sums from 2^80 on turn up as a non-finite result;
-// that element is then formed again by a plain chain of fused multiply-adds from the float32 operands.
+// that element, and no other, is then formed again by a plain chain of fused multiply-adds from the float32 operands (redo).
 //
 // Layout.  All six products are written out[n][m], m contiguous: m = weight columns or rows on the MMA's M side (tiles of
 // 128, TMEM lanes), n = an expert's tokens, or the other index of a weight gradient, on the N side, at most 128 wide (64 sums
@@ -30,6 +30,8 @@
 // instruction caches.  Taking out any one of conversion of A, of B, the correction MMAs, or the adding up shortened a product by
 // 6 to 14%.  4096 tokens, 512 x 2048, 16 experts, between stage events, FMA kernels / here: GEMM1 190 / 79 us, GEMM2 236 / 86,
 // dgrad2 215 / 78, wgrad2 171 / 69, dgrad1 243 / 84, wgrad1 171 / 68 (109 to 126 TFLOP/s; the FMA pipes' peak is 74.5).
+#include <cfloat>
+
 #include "tc_common.cuh"
 
 namespace swmoe {
@@ -154,31 +156,80 @@ __device__ __forceinline__ void split3(float x0, float x1, uint32_t* h, uint32_t
 }
 
 // The element-wise end of a product for one output.  `live`: ReLU'(u) of this output (dgrad2); `skip`: the row added on the
-// skip path (combine, scatter).
+// skip path (combine, scatter).  What is not finite is left so in the output, for redo to find, unless it is `final`.
 template <int OP>
-__device__ __forceinline__ void finish(const F32Problem& p, long long at, float scale, float v, bool live, float skip) {
+__device__ __forceinline__ void finish(const F32Problem& p, long long at, float scale, float v, bool live, float skip,
+                                       bool final = false) {
   if (OP == kGemm2Combine) v *= scale;
-  if (OP == kGemm1Relu && !p.plain) v = fmaxf(v, 0.f);
+  if (OP == kGemm1Relu && !p.plain && (final || v >= -FLT_MAX)) v = fmaxf(v, 0.f);
   if (OP == kDgrad2Mask && !p.plain) v = live ? v : 0.f;
   if (OP == kGemm2Combine && p.out2 != nullptr) p.out2[at] = v;
   if ((OP == kGemm2Combine || OP == kDgrad1Scatter) && p.res != nullptr) v += skip;
   p.out[at] = v;
 }
 
-// The results of one m over a warp's columns again, by chains of fused multiply-adds.
+// The results of one m over a warp's columns that are not finite in the output, by a chain of fused multiply-adds each, in
+// ascending order of the contraction.  Four columns share the loads of A, four steps of them are in flight, 16 bytes at a time
+// along whichever axis is contiguous; eight columns at a time were up to a quarter faster, but spilled registers of the kernel.  A
+// step of 8192 tokens, 256 x 1024, 4 experts, every element of dy, W_in or W_out NaN: 8.8, 2.8, 7.2 ms, on the FMA kernels 0.84.
+// `progress` changes as it goes: the other warps of the block wait for this one under a limit, and start that anew whenever it
+// has, so that the limit holds for a contraction of any length.
 template <int OP>
-__device__ __noinline__ void redo(const F32Problem& p, int e, int n0, int K, int m, int mine, const int2* tab) {
-  for (int c = 0; c < mine; ++c) {
-    const float* a = p.A + e * p.a_es + m * p.a_ms;
-    const float* b = p.B + e * p.b_es + (n0 + c) * p.b_ns;
-    float s = 0.f;
-    for (int k = 0; k < K; ++k) s = fmaf(a[k * p.a_ks], b[k * p.b_ks], s);
-    const long long at = (long long)tab[c].x * p.ld_out + m;
-    uint8_t* byte = p.hmask + ((long long)e * p.hrows + (n0 + c) / 8) * p.hcols + m;
-    const bool live = OP == kDgrad2Mask && !p.plain && (*byte >> (c & 7) & 1);
-    if (OP == kGemm1Relu && !p.plain) *byte = (uint8_t)((c & 7 ? *byte & ~(1 << (c & 7)) : 0) | (s > 0.f ? 1 << (c & 7) : 0));
-    const bool skip = (OP == kGemm2Combine || OP == kDgrad1Scatter) && p.res != nullptr;
-    finish<OP>(p, at, __int_as_float(tab[c].y), s, live, skip ? p.res[at] : 0.f);
+__device__ __noinline__ void redo(const F32Problem& p, int e, int n0, int K, int m, int mine, const int2* tab,
+                                  volatile int* progress) {
+  constexpr bool kToken = OP != kWgrad2 && OP != kWgrad1;              // B contiguous along the contraction, else along n
+  constexpr bool kAKMajor = OP == kDgrad2Mask || OP == kDgrad1Scatter; // A contiguous along the contraction, else along m
+  const float* a = p.A + e * p.a_es + m * p.a_ms;
+  for (int c0 = 0; c0 < mine; c0 += 4) {
+    uint32_t cols = 0;
+    for (int c = 0; c < min(4, mine - c0); ++c)
+      cols |= fabsf(p.out[(long long)tab[c0 + c].x * p.ld_out + m]) <= FLT_MAX ? 0u : 1u << c;
+    if (cols == 0) continue;
+    const float* b[4];                                        // token products: a row per column, rows of good ones not touched
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      b[c] = p.B + e * p.b_es + (n0 + c0 + (kToken ? (cols >> c & 1u ? c : __ffs(cols) - 1) : 0)) * p.b_ns;
+    float s[4] = {};
+    for (int k = 0; k < K; k += 4) {
+      float av[4], bv[4][4];
+      if (kAKMajor) {
+        *reinterpret_cast<float4*>(av) = *reinterpret_cast<const float4*>(a + k);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) av[j] = k + j < K ? a[(k + j) * p.a_ks] : 0.f;
+      }
+      if (kToken) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<float4*>(bv[c]) = *reinterpret_cast<const float4*>(b[c] + k);
+      } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 row = *reinterpret_cast<const float4*>(b[0] + min(k + j, K - 1) * p.b_ks);
+          bv[0][j] = row.x; bv[1][j] = row.y; bv[2][j] = row.z; bv[3][j] = row.w;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        if (kToken || k + j < K) {                            // (token products: K is a multiple of 8)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) s[c] = fmaf(av[j], bv[c][j], s[c]);
+        }
+      }
+      if ((k & 1023) == 0) *progress = (int)clock64();
+    }
+    uint8_t* byte = p.hmask + ((long long)e * p.hrows + (n0 + c0) / 8) * p.hcols + m;
+    const uint32_t sh = c0 & 4, old = (OP == kDgrad2Mask || OP == kGemm1Relu) && !p.plain ? *byte : 0u, live = old >> sh;
+    uint32_t bits = old & ~(cols << sh);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      if ((cols >> c & 1u) == 0) continue;
+      const int2 r = tab[c0 + c];
+      const long long at = (long long)r.x * p.ld_out + m;
+      const bool skip = (OP == kGemm2Combine || OP == kDgrad1Scatter) && p.res != nullptr;
+      finish<OP>(p, at, __int_as_float(r.y), s[c], live >> c & 1u, skip ? p.res[at] : 0.f, true);
+      bits |= s[c] > 0.f ? 1u << (c + sh) : 0u;
+    }
+    if (OP == kGemm1Relu && !p.plain) *byte = (uint8_t)bits;
   }
 }
 
@@ -204,9 +255,9 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   auto dfull = [&](int s) { return bars + 8u * (2 * (kLoadStages + kPartBars) + s); };
   auto dempty = [&](int s) { return bars + 8u * (2 * (kLoadStages + kPartBars) + 2 + s); };
   constexpr int kBars = 2 * (kLoadStages + kPartBars) + 4;
-  static_assert(8 * kBars + 8 <= 256, "barrier block");
+  static_assert(8 * kBars + 12 <= 256, "barrier block");
   volatile uint32_t* tmem_ptr_s = reinterpret_cast<volatile uint32_t*>(bar_gen + 8 * kBars);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 8 * kBars + 4);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(bar_gen + 8 * kBars + 4);     // and, behind it, redo's progress
   int* kept_s = reinterpret_cast<int*>(bar_gen + 256);       // tokens per expert
   int* cum_s = kept_s + kMaxExperts;                         // [E + 1] token tiles of earlier experts
   float* cost_s = reinterpret_cast<float*>(cum_s + kMaxExperts + 1);
@@ -220,7 +271,7 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
     for (int s = 0; s < kLoadStages; ++s) { mbar_init(lfull(s), 1); mbar_init(lempty(s), 4); }
     for (int s = 0; s < kPartBars; ++s) { mbar_init(pfull(s), 4); mbar_init(pempty(s), 1); }
     for (int s = 0; s < 2; ++s) { mbar_init(dfull(s), 1); mbar_init(dempty(s), kEpiWarps); }
-    *abort_flag = 0;
+    abort_flag[0] = abort_flag[1] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -322,7 +373,7 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const int boxes = (t.n_mma + kBoxRows - 1) / kBoxRows;
       const uint32_t bytes = kALoad + (kToken ? boxes * kBoxRows : kNFix) * kK * 4;
       for (int k0 = 0; k0 < t.K; k0 += kK) {
-        ok = mbar_wait_warp(lempty(stage), phase ^ 1u, abort_flag, p.status, 51);
+        ok = mbar_wait_warp<true>(lempty(stage), phase ^ 1u, abort_flag, p.status, 51);
         if (!ok) break;
         if (elect_one()) {
           const uint32_t a_dst = base + stage * kLoadBytes, b_dst = a_dst + kALoad;
@@ -362,8 +413,8 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 #pragma unroll 1
       for (int k0 = 0; k0 < t.K; k0 += kK, turn ^= 1) {
         if (turn == w) {                                      // this warp's accumulator is number w
-          ok = mbar_wait_warp(dempty(w), dphase ^ 1u, abort_flag, p.status, 52) &&
-               mbar_wait_warp(pfull(pbar), pphase, abort_flag, p.status, 53);
+          ok = mbar_wait_warp<true>(dempty(w), dphase ^ 1u, abort_flag, p.status, 52) &&
+               mbar_wait_warp<true>(pfull(pbar), pphase, abort_flag, p.status, 53);
           if (!ok) break;
           tc_fence_after();
           const int ps = pbar < kPartStages ? pbar : pbar - kPartStages;
@@ -391,7 +442,7 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
             }
             __syncwarp();
             dphase ^= 1u;
-            ok = mbar_wait_warp(dempty(w), dphase ^ 1u, abort_flag, p.status, 52);
+            ok = mbar_wait_warp<true>(dempty(w), dphase ^ 1u, abort_flag, p.status, 52);
             if (!ok) break;
             tc_fence_after();
             if (elect_one()) {
@@ -418,10 +469,10 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const F32Tile t = decode(id);
       for (int k0 = 0; k0 < t.K; k0 += kK, turn ^= 1) {
         if (turn == group) {
-          ok = mbar_wait_warp(lfull(ls), lphase, abort_flag, p.status, 54) &&
+          ok = mbar_wait_warp<true>(lfull(ls), lphase, abort_flag, p.status, 54) &&
                (pbar < kPartStages                            // the buffer's previous stage was three stages ago
-                    ? mbar_wait_warp(pempty(pbar + kPartStages), pphase ^ 1u, abort_flag, p.status, 55)
-                    : mbar_wait_warp(pempty(pbar - kPartStages), pphase, abort_flag, p.status, 55));
+                    ? mbar_wait_warp<true>(pempty(pbar + kPartStages), pphase ^ 1u, abort_flag, p.status, 55)
+                    : mbar_wait_warp<true>(pempty(pbar - kPartStages), pphase, abort_flag, p.status, 55));
           if (!ok) break;
           tc_fence_after();
           const int ps = pbar < kPartStages ? pbar : pbar - kPartStages;
@@ -532,7 +583,7 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       const bool twice = t.apart() && t.K > 0;                // two chunks, both in the same accumulator
       const int chunks = twice ? 2 : (t.K + kK - 1) / kK;
       for (int c = 0; c < chunks; ++c) {
-        ok = mbar_wait_warp(dfull(d), d ? dphase1 : dphase0, abort_flag, p.status, 56);
+        ok = mbar_wait_warp<true>(dfull(d), d ? dphase1 : dphase0, abort_flag, p.status, 56);
         if (!ok) break;
         tc_fence_after();
         const uint32_t ta = tmem_base + ((uint32_t)(lg * 32) << 16) + (uint32_t)(d * kNMax + c0);
@@ -602,7 +653,7 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
       };
       static_assert(kHalf == 64, "eight groups of 8 columns");
       (void)(group(0) && group(1) && group(2) && group(3) && group(4) && group(5) && group(6) && group(7));
-      if (check != check) redo<OP>(p, t.e, t.n0 + c0, t.K, m, mine, tab);
+      if (check != check) redo<OP>(p, t.e, t.n0 + c0, t.K, m, mine, tab, abort_flag + 1);
       __syncwarp();
     }
   }

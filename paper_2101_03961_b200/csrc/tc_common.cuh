@@ -64,13 +64,20 @@ __device__ __forceinline__ unsigned long long global_ns() {
 // thread of the CTA already gave up.  The common case -- the phase is complete, or completes within a few polls --
 // is inline: producer and MMA loops must stay small and call-free, because a lone warp that jumps to far code pays an
 // instruction-cache miss per iteration while the epilogue warps stream through the cache.
+// kProgress: the limit starts anew whenever the word behind the abort flag has changed (long finite work elsewhere in the block).
+template <bool kProgress = false>
 static __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                    int code) {
-  const long long t0 = clock64();
+  long long t0 = clock64();
+  int seen = kProgress ? abort_flag[1] : 0;
   for (uint32_t spin = 1;; ++spin) {
     if (mbar_try_wait(bar, parity)) return true;
     if ((spin & 255u) == 0) {
       if (*abort_flag != 0) return false;
+      if (kProgress && abort_flag[1] != seen) {
+        seen = abort_flag[1];
+        t0 = clock64();
+      }
       if (clock64() - t0 > kWaitLimitCycles) {
         *abort_flag = 1;
         if (atomicCAS(status, 0, code) == 0) {
@@ -99,6 +106,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 // about 1000 cycles per 64-deep k-block of the expert products whatever the loads and the tensor pipe did (GEMM1 at
 // 32768 tokens, 768 x 3072, 128 experts: 189 us with single-lane loops, 162 us with these).  The polls sit in one asm
 // block so that no divergent branch separates the lanes.
+template <bool kProgress = false>
 __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status,
                                                int code) {
   uint32_t ok;
@@ -117,7 +125,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
       : "r"(bar), "r"(parity)
       : "memory");
   if (__all_sync(0xffffffffu, ok != 0)) return true;
-  return __all_sync(0xffffffffu, mbar_wait_slow(bar, parity, abort_flag, status, code));
+  return __all_sync(0xffffffffu, mbar_wait_slow<kProgress>(bar, parity, abort_flag, status, code));
 }
 // True in one lane of a converged warp, always the same one (tcgen05.commit covers the MMAs of its own thread).
 __device__ __forceinline__ bool elect_one() {

@@ -10,7 +10,7 @@ from paper_2101_03961_b200 import switch_moe as sm
 pytestmark = pytest.mark.gpu
 
 
-def _layer(T, d, f, E, cf, path, residual=False, seed=1, spoil=None):
+def _layer(T, d, f, E, cf, path, residual=False, seed=1, spoil=None, events=None):
     g = torch.Generator(device="cuda")
     g.manual_seed(seed)
 
@@ -30,9 +30,13 @@ def _layer(T, d, f, E, cf, path, residual=False, seed=1, spoil=None):
     for k in ("W_r", "W_in", "W_out"):
         t["d" + k] = torch.empty_like(t[k])
     aux = torch.empty(1, device="cuda")
+    if events:
+        events[0].record()
     sm.switch_moe_fwd(cfg, t["x"], t["W_r"], None, t["W_in"], t["W_out"], t["y"], aux, ws)
     sm.switch_moe_bwd(cfg, t["dy"], 1.0, t["x"], t["W_r"], t["W_in"], t["W_out"], t["y"], ws, t["dx"], t["dW_r"], t["dW_in"],
                       t["dW_out"])
+    if events:
+        events[1].record()
     sm.switch_moe_check_device_status(cfg, ws)
     C = sm.switch_moe_capacity(cfg)
     view = lambda region: sm.switch_moe_workspace_view(cfg, ws, region)  # noqa: E731
@@ -129,3 +133,49 @@ def test_values_that_the_parts_cannot_hold():
         assert torch.equal(torch.isposinf(ra), torch.isposinf(rb)) and torch.equal(torch.isneginf(ra), torch.isneginf(rb)), k
         fin = torch.isfinite(rb) & (rb.abs() < 1e30)
         assert float((ra[fin] - rb[fin]).norm()) <= 1e-5 * float(rb[fin].norm()), k
+
+
+def test_a_value_that_is_not_finite_changes_no_other_result():
+    """Tokens that share a tile with a bad one, and rows of a weight gradient beside a bad one, keep their bits."""
+    def spoil(t):
+        t["dy"][17, 11] = math.inf
+        t["dy"][18, 12] = math.nan
+        t["W_in"][2, 5, 40] = math.inf
+
+    shape = (2048, 128, 512, 4, 1.25, sm.GEMM_DEFAULT)
+    clean, bad = _layer(*shape), _layer(*shape, spoil=spoil)
+    assert clean["kept"] == bad["kept"] and torch.equal(clean["tokens"], bad["tokens"])
+    for k in ("H", "dH"):                                      # rows of the other tokens, and the other hidden units
+        for e, n in enumerate(clean["kept"]):
+            a, b = clean[k][e, :n], bad[k][e, :n]
+            other = (clean["tokens"][e, :n] != 17) & (clean["tokens"][e, :n] != 18)
+            units = torch.arange(a.shape[1], device="cuda") != (40 if e == 2 else -1)
+            assert torch.equal(a[other][:, units], b[other][:, units]), (k, e)
+    tokens = torch.ones(2048, dtype=torch.bool, device="cuda")
+    tokens[17] = tokens[18] = False
+    tokens[clean["tokens"][2, :clean["kept"][2]]] = False      # every token of the expert with the bad weight
+    for k in ("y", "dx"):
+        assert torch.equal(clean[k][tokens], bad[k][tokens]), k
+    for k in ("dW_in", "dW_out"):
+        for e in (0, 1, 3):
+            fin = torch.isfinite(bad[k][e])
+            assert fin.float().mean() > 0.4 and torch.equal(clean[k][e][fin], bad[k][e][fin]), (k, e)
+
+
+@pytest.mark.parametrize("spoiled", ["dy", "W_in", "W_out"])
+def test_time_of_results_that_are_not_finite(spoiled):
+    """Every element of an operand NaN: all of up to four products are formed again, which takes a bounded multiple of the fused
+    multiply-add kernels' time (measured: 3 to 10.5 for a whole step)."""
+    def spoil(t):
+        t[spoiled].fill_(math.nan)
+
+    best = {}
+    for path in (sm.GEMM_DEFAULT, sm.GEMM_SIMT):
+        start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        times = []
+        for _ in range(3):
+            torch.cuda.synchronize()
+            t = _layer(8192, 256, 1024, 4, 1.25, path, spoil=spoil, events=(start, end))
+            times.append(start.elapsed_time(end))
+        best[path] = min(times)
+    assert best[sm.GEMM_DEFAULT] <= 20.0 * best[sm.GEMM_SIMT], best
