@@ -6,7 +6,7 @@
 // rounded to nearest), from the smallest subnormal up to 2^104 (unscaled, l of an operand below 2^-110 would reach under
 // bfloat16's smallest subnormal: 2^-118 came out exact to 1e-5 only), and a product of two bfloat16 is exact in float32; the
 // sums are scaled back by 2^-48.  Of the nine cross products six are formed (h.h, h.m, m.h, m.m, h.l, l.h); the other three
-// are below 2^-25 of the product.  The tensor pipe adds into its float32 accumulator with
+// are below 2^-25 of the product (contractions of at most 16 steps form them too).  The tensor pipe adds into its float32 accumulator with
 // truncation, so a long sum left there would drift: here an accumulator lives for kK = 32 steps of the contraction only.
 // Within such a chunk the five correction products (at most 2^-8 of the sum) go first and h.h last, then the chunk is read
 // out of tensor memory and added to a float32 sum in registers, round to nearest.  A chain of one fused multiply-add per step
@@ -80,7 +80,8 @@ struct F32Problem {
 struct F32Tile {
   int e, m0, n0, n_valid, n_mma, K;
   // A contraction of one step of the MMA is two chunks, the corrections and the high parts: what the pipe truncates there
-  // is all the error there is, and the products of the high parts alone rarely reach past the accumulator's last bit.
+  // is all the error there is, and the products of the high parts alone rarely reach past the accumulator's last bit.  All
+  // eight corrections then: a single product comes out rounded once, like an FMA's (without the three smallest 2% less exact).
   __device__ __forceinline__ bool apart() const { return K <= kUmmaK; }
 };
 
@@ -420,23 +421,24 @@ f32_expert_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
           const int ps = pbar < kPartStages ? pbar : pbar - kPartStages;
           const uint32_t dt = tmem_base + (uint32_t)w * kNMax, at = a_tmem + (uint32_t)ps * kAStageCols;
           const uint64_t bd = b_desc0 + (uint64_t)(ps * (kPartStage >> 4));
-          // part pairs (A, B), 0 = high, 1 = middle, 2 = low: the corrections from the smallest up, then high . high
-          constexpr int pa[6] = {2, 0, 1, 1, 0, 0}, pb[6] = {0, 2, 1, 0, 1, 0};
+          // part pairs (A, B), 0 = high, 1 = middle, 2 = low: the corrections from the smallest up, then high . high; the first
+          // three in contractions of one step only
+          constexpr int pa[9] = {2, 1, 2, 2, 0, 1, 1, 0, 0}, pb[9] = {2, 2, 1, 0, 2, 1, 0, 1, 0};
           if (!apart) {
             if (elect_one()) {
 #pragma unroll
-              for (int q = 0; q < 6; ++q)
+              for (int q = 3; q < 9; ++q)
 #pragma unroll
                 for (int ks = 0; ks < kK / kUmmaK; ++ks)
                   tc_mma_bf16_ts(dt, at + pa[q] * kAPartCols + ks * (kUmmaK / 2), bd + pb[q] * kPartStep + ks * kStep, idesc,
-                                 q + ks > 0 ? 1u : 0u);
+                                 q + ks > 3 ? 1u : 0u);
               tc_commit(pempty(pbar));                          // frees the parts once these MMAs have read them
               tc_commit(dfull(w));
             }
           } else {                                            // one step in two chunks, see F32Tile::apart
             if (elect_one()) {
 #pragma unroll
-              for (int q = 0; q < 5; ++q)
+              for (int q = 0; q < 8; ++q)
                 tc_mma_bf16_ts(dt, at + pa[q] * kAPartCols, bd + pb[q] * kPartStep, idesc, q > 0 ? 1u : 0u);
               tc_commit(dfull(w));
             }
