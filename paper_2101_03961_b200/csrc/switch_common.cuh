@@ -221,7 +221,7 @@ inline T* ws_ptr(void* ws, size_t off) { return reinterpret_cast<T*>(static_cast
 // ---- programmatic dependent launch --------------------------------------------------------------------------
 // Every kernel of the layer is launched with programmatic stream serialization: it may be scheduled (and run its
 // prologue: barrier init, tensor-memory allocation) while the previous kernel of the stream is still draining.
-// The contract inside the kernels: call pdl_launch_dependents() first, and pdl_wait() before the first access to
+// The contract inside the kernels: call pdl_launch_dependents() first (f32_expert_gemm_kernel: last), and pdl_wait() before the first access to
 // global memory; pdl_wait() returns once the previous kernel has completed and its writes are visible.  One pair departs
 // from it: plan_slots_kernel waits first and triggers after, so that its successor starts only when the kernel before both
 // has completed, and that successor, plan_summary_kernel, reads that kernel's tables from L2 before its own wait.
@@ -232,14 +232,14 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 inline bool& launch_failed_flag() { static thread_local bool failed = false; return failed; }
 
-template <typename Kern, typename... Args>
+template <bool kEarly = true, typename Kern, typename... Args>
 inline void launch_k(Kern kernel, dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr; cfg.numAttrs = 1;
+  cfg.attrs = attr; cfg.numAttrs = kEarly ? 1 : 0;
   if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) launch_failed_flag() = true;
 }
 
@@ -324,6 +324,7 @@ struct GemmArgs {
   const void* x; const void* dy;         // skip-path sources (residual configuration only): y += x, dx += dy
 };
 int launch_simt_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
+bool f32_on_tensor_cores(GemmOp op, const Shape& s);
 int launch_f32_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
 int launch_tc_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);
 int launch_pair_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st);

@@ -203,3 +203,44 @@ def test_time_of_results_that_are_not_finite(spoiled):
             times.append(start.elapsed_time(end))
         best[path] = min(times)
     assert best[sm.GEMM_DEFAULT] <= 20.0 * best[sm.GEMM_SIMT], best
+
+
+def _stage_times(T, d, f, E, cf, path, geglu=False, n=9):
+    """Median time (us) of each product's stage, element-wise kernels included."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(1)
+
+    def normal(*shape):
+        return torch.empty(shape, device="cuda").normal_(generator=g)
+
+    x, dy, W_r = normal(T, d), normal(T, d), normal(d, E) * (0.1 / d) ** 0.5
+    W_in, W_out = normal(E, d, 2 * f if geglu else f) * (0.1 / d) ** 0.5, normal(E, f, d) * (0.1 / f) ** 0.5
+    cfg = sm.make_config(T, d, f, E, cf, dtype=sm.F32, gemm_path=path, geglu=geglu)
+    ws, aux = sm.allocate_workspace(cfg), torch.empty(1, device="cuda")
+    y, dx, dW_r, dW_in, dW_out = (torch.empty_like(t) for t in (x, x, W_r, W_in, W_out))
+    events = [torch.cuda.Event(enable_timing=True) for _ in range(sm.STAGE_EVENTS)]
+    for ev in events:
+        ev.record()
+    sm.set_stage_events(cfg, events)
+    stages = {name: i for i, name in enumerate(sm.STAGE_NAMES)
+              if name in ("gemm1_relu", "gemm2_combine", "dgrad2_mask", "wgrad2", "dgrad1_scatter", "wgrad1")}
+    times = {name: [] for name in stages}
+    for i in range(n + 2):
+        sm.switch_moe_fwd(cfg, x, W_r, None, W_in, W_out, y, aux, ws)
+        sm.switch_moe_bwd(cfg, dy, 1.0, x, W_r, W_in, W_out, y, ws, dx, dW_r, dW_in, dW_out)
+        torch.cuda.synchronize()
+        for name, k in stages.items():
+            if i >= 2:
+                times[name].append(1e3 * events[k].elapsed_time(events[k + 1]))
+    sm.switch_moe_check_device_status(cfg, ws)
+    return {name: sorted(v)[n // 2] for name, v in times.items()}
+
+
+@pytest.mark.parametrize("T,d,f,E,geglu", [
+    (160, 120, 3744, 3, True),             # few long rows to gate behind the products
+])
+def test_products_are_no_slower_than_fused_multiply_adds(T, d, f, E, geglu):
+    """Shapes at which the tensor cores have little to win: no stage may take longer than the FMA kernels' by more than 15%
+    and the events' resolution (where they were chosen wrongly it was 1.3 to 2.3 times)."""
+    a, b = (_stage_times(T, d, f, E, 1.25, path, geglu) for path in (sm.GEMM_DEFAULT, sm.GEMM_SIMT))
+    assert all(a[k] <= 1.15 * b[k] + 2.0 for k in a), (a, b)
