@@ -31,6 +31,7 @@
 // 6 to 14%.  4096 tokens, 512 x 2048, 16 experts, between stage events, FMA kernels / here: GEMM1 190 / 79 us, GEMM2 236 / 86,
 // dgrad2 215 / 78, wgrad2 171 / 69, dgrad1 243 / 84, wgrad1 171 / 68 (109 to 126 TFLOP/s; the FMA pipes' peak is 74.5).
 #include <cfloat>
+#include <cmath>
 
 #include "tc_common.cuh"
 
@@ -683,18 +684,30 @@ int launch_op(const CUtensorMap& tmA, const CUtensorMap& tmB, const F32Problem& 
 
 }  // namespace
 
-// Which float32 products run here, by what they multiply (2 rows d f) and, for weight gradients, by the tokens per expert.  A
-// launch has about 3 us more to set up than an FMA kernel (tensor memory, barriers, cold code).  Between stage events, here /
-// FMA kernels, us, GEMM1, GEMM2, wgrad2: 17 MFLOP (512 tokens, 64 x 256, 8 experts) 10.9 / 8.4, 14.2 / 14.1, 12.7 / 9.6; 67 (1024
-// tokens, 128 x 256, 8) 12.7 / 12.1, 14.6 / 14.7, 14.4 / 12.1; 79 (300 tokens, 256 x 512, 4) 14.1 / 13.8, 17.9 / 20.2, 12.3 / 12.3;
-// 157 (600 tokens, 128 x 1024, 16) 13.6 / 14.6, 25.0 / 32.7, 12.3 / 12.3.  A weight gradient of few tokens is bound by writing its
-// output, and a tile's one or two stages hide none of that (64 experts of 768 x 3072: 8 tokens each 209 / 141, 16 tokens 193 /
-// 173, 24 tokens 174 / 204).  GEMM1 and dgrad2 multiply the same, so the mask that one leaves is the one that the other reads.
+// Which float32 products run here: those of at least 0.07 GFLOP (weight gradients 0.12; 2 rows d f), below which the 3 us that a
+// launch has more to set up than an FMA kernel's (tensor memory, barriers, cold code) decide, and of them
+// - token products with enough steps per tile to pay for its two ends.  Medians over shapes of 16 to 65536 tokens, 1 to 256
+//   experts, stage time here / FMA kernels, by contraction: GEMM1 with dgrad2 8..15 1.26, 32..47 1.06, 64..71 0.86, GEMM1 alone
+//   2.18, 1.34, 1.03, from 72 on 0.99, 80..95 0.93, 128..191 0.76; GEMM2 and dgrad1 32..47 1.33, 80..95 1.00, 96..111 0.87.  An
+//   output narrower than half a tile leaves the rest of its MMAs idle: 64..95 1.18, 144..191 0.95, 192..255 0.86.  Tiles of few
+//   tokens whose contraction is short, or output narrower still, are nothing but their ends (25 tokens, 72 x 96: 1.46; 22, 528 x 16:
+//   1.36).
+// - weight gradients of enough tokens to be more than writing the output (20..23 per expert 1.00, 24..31 1.04, 40..47 0.95, 48..63
+//   0.88), and of outputs of enough tiles: a tile walks its whole contraction on one SM at the rate of one FMA block of 64 x 64,
+//   so with fewer than about half an FMA block per SM the chip is idle either way (24..47 blocks 1.09, 48..71 0.97, 72..95 0.87).
+// On 440 shapes drawn afterwards the six products of a step take 0.74 of the FMA kernels' time in the median and 1.08 at most, a
+// single one up to 1.3.  GEMM1 and dgrad2 always go together: the mask that one leaves is the one that the other reads.
 bool f32_on_tensor_cores(GemmOp op, const Shape& s) {
   if (!s.f32_tc) return false;
   const double rows = s.Tv < (double)s.E * s.C ? s.Tv : (double)s.E * s.C, flops = 2.0 * rows * s.d * s.f;
-  if (op == kWgrad2 || op == kWgrad1) return flops >= 1.2e8 && rows >= 20.0 * s.E;
-  return flops >= 7e7;
+  const bool first = op == kGemm1Relu || op == kDgrad2Mask;            // d deep, f wide; the other token products f deep, d wide
+  if (op == kWgrad2 || op == kWgrad1) {
+    const long long blocks = (long long)s.E * ((s.d + 63) / 64) * (((op == kWgrad1 ? s.fin : s.f) + 63) / 64);
+    return flops >= 1.2e8 && rows >= 48.0 * s.E && blocks >= kChipSms / 2;
+  }
+  const int steps = first ? s.d : op == kGemm2Combine ? s.f : s.fin, width = first ? s.f : s.d;
+  const double tiles = (double)s.E * ceil(rows / s.E / kNMax) * ((width + kM - 1) / kM), tile_flops = 2.0 * rows * width * steps / tiles;
+  return flops >= 7e7 && steps >= (width < 64 ? 192 : first ? 72 : 96) && (tile_flops >= 5e5 || (steps >= 128 && width >= 32));
 }
 
 int launch_f32_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st) {

@@ -69,28 +69,37 @@ def _errors(t, residual):
     return {k: math.sqrt(num[k] / den[k]) for k in num}
 
 
-SHAPES = [
-    (1024, 128, 512, 4, 1.25, False),      # whole tiles of m, several tiles of tokens
-    (4100, 72, 1000, 16, 1.25, True),      # remainders of m, of a chunk and of 16 tokens; the skip path
-    (5000, 8, 3000, 8, 2.0, False),        # contractions of one MMA step and of many chunks
-    (3000, 520, 24, 60, 2.0, True),        # about 50 tokens per expert
-    (4096, 512, 2048, 16, 1.0, False),     # a full capacity of 256
-    (1500, 264, 1032, 50, 1.25, False),    # about 30 tokens per expert: a chunk, less and more
+FIRST, SECOND, WEIGHTS = ("gemm1", "dgrad2"), ("gemm2", "dgrad1"), ("wgrad2", "wgrad1")
+SHAPES = [                                 # and the products that are large enough for the tensor cores
+    (1024, 128, 512, 4, 1.25, False, FIRST + SECOND),                # whole tiles of m, several tiles of tokens
+    (4100, 72, 1000, 16, 1.25, True, FIRST + SECOND + WEIGHTS),      # remainders of m, of a chunk and of 16 tokens; the skip path
+    (5000, 8, 3000, 8, 2.0, False, SECOND + WEIGHTS),                # eight rows of a tile, many chunks
+    (3000, 520, 24, 60, 2.0, True, FIRST),                           # 24 rows of a tile, about 50 tokens per expert
+    (4096, 512, 2048, 16, 1.0, False, FIRST + SECOND + WEIGHTS),     # a full capacity of 256
+    (1500, 264, 1032, 50, 1.25, False, FIRST + SECOND),              # about 30 tokens per expert: a chunk, less and more
+    (3000, 264, 1032, 50, 1.25, False, FIRST + SECOND + WEIGHTS),    # about 60: two chunks, less and more
 ]
 
 
-@pytest.mark.parametrize("T,d,f,E,cf,residual", SHAPES)
-def test_products_of_exact_parts(T, d, f, E, cf, residual):
+@pytest.mark.parametrize("T,d,f,E,cf,residual,parts", SHAPES)
+def test_products_of_exact_parts(T, d, f, E, cf, residual, parts):
     """Bound: of n = ceil(K / 32) chunks each truncates two sums at the size of the chunk (2^-23 each; chunks are independent,
     together 4 2^-24 of the result), and the float32 sum over the chunks rounds n times at the size of a running sum of random
-    terms (2^-24 sqrt(n / 2)); one more rounding for the gate and the skip path each."""
+    terms (2^-24 sqrt(n / 2)); one more rounding for the gate and the skip path each.  Fused multiply-adds round K times, each
+    by up to 2^-24 (2^-24 / sqrt(3) in the mean) of a running sum, together 0.41 sqrt(K) 2^-24.  The error also says which kernel
+    a product went to: the same on both paths, or well below the chain's (from 60 steps on by more than a quarter; with the skip
+    path the sum's own rounding is most of either)."""
     t = _layer(T, d, f, E, cf, sm.GEMM_DEFAULT, residual)
     errs = _errors(t, residual)
     fma = _errors(_layer(T, d, f, E, cf, sm.GEMM_SIMT, residual), residual)
     tokens = max(t["kept"])
     for name, K in (("gemm1", d), ("gemm2", f), ("dgrad2", d), ("dgrad1", f), ("wgrad2", tokens), ("wgrad1", tokens)):
-        assert errs[name] <= 2.0 ** -24 * (6.0 + math.sqrt(math.ceil(K / 32) / 2.0)), (name, errs)
-        assert errs[name] <= 1.05 * fma[name], (name, errs, fma)     # no less precise than a chain of fused multiply-adds
+        assert fma[name] <= 2.0 ** -24 * (2.0 + 0.5 * math.sqrt(K)), (name, fma)
+        if name in parts:
+            assert errs[name] <= 2.0 ** -24 * (6.0 + math.sqrt(math.ceil(K / 32) / 2.0)), (name, errs)
+            assert errs[name] <= (0.95 if residual else 0.85) * fma[name], (name, errs, fma)
+        else:
+            assert abs(errs[name] - fma[name]) <= 0.02 * fma[name], (name, errs, fma)
     again = _layer(T, d, f, E, cf, sm.GEMM_DEFAULT, residual)
     for k in ("y", "dx", "dW_in", "dW_out"):
         assert torch.equal(t[k], again[k])
@@ -131,7 +140,7 @@ def test_products_of_small_operands(scale):
         for name, e in scale.items():
             t[name] *= 2.0 ** e
 
-    shape = (2048, 128, 512, 4, 1.25)
+    shape = (2048, 128, 512, 8, 1.25)
     t = _layer(*shape, sm.GEMM_DEFAULT, spoil=spoil)
     errs, fma, tokens = _errors(t, False), _errors(_layer(*shape, sm.GEMM_SIMT, spoil=spoil), False), max(t["kept"])
     for name, K in (("gemm1", 128), ("gemm2", 512), ("dgrad2", 128), ("dgrad1", 512), ("wgrad2", tokens), ("wgrad1", tokens)):
@@ -150,7 +159,7 @@ def test_values_that_the_parts_cannot_hold():
         t["dy"][17, 11] = math.inf
         t["dy"][18, 12] = math.nan
 
-    a, b = (_layer(2048, 128, 512, 4, 1.25, path, residual=True, spoil=spoil) for path in (sm.GEMM_DEFAULT, sm.GEMM_SIMT))
+    a, b = (_layer(2048, 128, 512, 8, 1.25, path, residual=True, spoil=spoil) for path in (sm.GEMM_DEFAULT, sm.GEMM_SIMT))
     for k in ("y", "dx", "dW_in", "dW_out"):
         ra, rb = a[k], b[k]
         assert torch.equal(torch.isnan(ra), torch.isnan(rb)), k
@@ -166,7 +175,7 @@ def test_a_value_that_is_not_finite_changes_no_other_result():
         t["dy"][18, 12] = math.nan
         t["W_in"][2, 5, 40] = math.inf
 
-    shape = (2048, 128, 512, 4, 1.25, sm.GEMM_DEFAULT)
+    shape = (2048, 128, 512, 8, 1.25, sm.GEMM_DEFAULT)
     clean, bad = _layer(*shape), _layer(*shape, spoil=spoil)
     assert clean["kept"] == bad["kept"] and torch.equal(clean["tokens"], bad["tokens"])
     for k in ("H", "dH"):                                      # rows of the other tokens, and the other hidden units
@@ -238,6 +247,12 @@ def _stage_times(T, d, f, E, cf, path, geglu=False, n=9):
 
 @pytest.mark.parametrize("T,d,f,E,geglu", [
     (160, 120, 3744, 3, True),             # few long rows to gate behind the products
+    (9651, 24, 2120, 5, False),            # short contractions: GEMM1
+    (23182, 1144, 8, 35, False),           # and GEMM2, dgrad1
+    (22440, 120, 32, 44, False),           # narrow outputs
+    (5650, 72, 96, 226, False),            # 25 tokens per expert
+    (14008, 32, 376, 3, False),            # weight gradients of few tiles
+    (5148, 232, 160, 240, False),          # and of few tokens
 ])
 def test_products_are_no_slower_than_fused_multiply_adds(T, d, f, E, geglu):
     """Shapes at which the tensor cores have little to win: no stage may take longer than the FMA kernels' by more than 15%
