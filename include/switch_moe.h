@@ -38,9 +38,10 @@ enum switch_moe_dtype { SWITCH_MOE_BF16 = 0, SWITCH_MOE_F32 = 1 };
 
 enum switch_moe_gemm_path {
   SWITCH_MOE_GEMM_DEFAULT = 0, /* bf16: tcgen05 grouped GEMM on CTA pairs (tokens on the MMA N side) and tensor-core
-                                  router; f32: products on tcgen05 as sums of exact bfloat16 parts where they are
-                                  large enough (error against float64 no larger than FP32 FMA's), the others and
-                                  the router on FP32 FMA */
+                                  router; f32: products on tcgen05 as sums of exact bfloat16 parts where their
+                                  shape makes that the faster way (error against float64 no larger than FP32 FMA's;
+                                  results that are not finite, or from 2^80 on, are formed by FP32 FMA), the others
+                                  and the router on FP32 FMA */
   SWITCH_MOE_GEMM_SIMT = 1,    /* validation only: FP32-FMA grouped GEMM and router for either dtype */
   SWITCH_MOE_GEMM_TC_1CTA = 2  /* validation only: single-CTA tcgen05 grouped GEMM with 128-token tiles (bf16) */
 };
@@ -128,6 +129,8 @@ typedef struct switch_moe_config {
                                 records events 6..11 before (6 gather dy, 7 dgrad2, 8 wgrad2, 9 dgrad1, 10 wgrad1,
                                 11 router backward) and event 12 after.  With gemm_path 0 dgrad1 and wgrad1 are one
                                 launch: event 10 follows it, so stage 9 spans both products and stage 10 is empty.
+                                Up to 256 tokens of one group, without TOP2 and REROUTE, the dispatch plan is part
+                                of the gather's launch: stage 1 is empty and stage 2 spans both.
                                 For per-kernel timing only. */
   const float* router_noise; /* DEVICE float[T, E] added to the router logits before the softmax, or NULL (default).
                                 The router pseudo-code of the appendix adds uniform(1 - eps, 1 + eps) noise to the

@@ -327,9 +327,9 @@ int switch_moe_stage_launches(const switch_moe_config* cfg, int32_t* launches_ou
   // forward.  Router: the kernel itself and, on the tensor cores, the bf16 split of W_r; input jitter adds the
   // element-wise product, top-2 routing the second-choice kernel.
   n[0] = (s.router_tc ? 2 : 1) + (s.jitter ? 1 : 0) + (s.top2 ? 1 : 0);
-  // plan: slots and, beside them, the summary when the router left the histograms and there is one routing group; else
-  // (histogram,) scan, assign; a stage of rerouting adds four
-  // (up to 256 tokens of one group: part of the gather's launch)
+  // plan: (histograms, where the router left none,) then slots and summary side by side, or scan and assignment for several
+  // groups, top-2 routing and above 262144 tokens; a stage of rerouting adds four.  Up to 256 tokens of one group, without
+  // rerouting: part of the gather's launch
   n[1] = s.plan_gather ? 0 : (s.router_hist ? 2 : 3) + 4 * s.reroute_stages;
   n[2] = 1;                                           // gather
   const int slow = s.gemm_path != 0 ? 1 : 0;   // gating and dropout are element-wise kernels off the CTA-pair path

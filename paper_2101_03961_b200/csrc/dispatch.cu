@@ -347,8 +347,9 @@ plan_slots_kernel(const int* __restrict__ expert_index, const int* __restrict__ 
   }
 }
 
-// Launched after plan_slots_kernel.  Reads only what the router wrote, past L1, and writes what no kernel in flight reads;
-// its own wait comes last, so that the next kernel's wait covers everything before this one.
+// Launched after plan_slots_kernel.  Reads only what the kernels before that one wrote (the router its P-sums and, on the
+// tensor cores, the histograms; plan_hist_kernel those of the other calls), past L1, and writes what no kernel in flight reads;
+// plan_slots_kernel has waited for all of them before it lets this one start.  Its own wait comes last, so that the next kernel's wait covers everything before this one.
 __global__ void __launch_bounds__(kFusedTokens)
 plan_summary_kernel(const int* hist, int hist_rows, const float* psum_partial, int psum_rows, int T, int E, int Ew, int C,
                     float alpha, int* __restrict__ count, float* __restrict__ psum, float* __restrict__ aux_loss,
@@ -676,6 +677,7 @@ plan_gather_small_kernel(const int* __restrict__ expert_index, const float* __re
   pdl_launch_dependents();
   pdl_wait();
   constexpr int kWarps = kSmallTokens / 32;
+  static_assert(kSmallTokens >= kMaxExperts, "a thread per token and per expert");
   __shared__ int warp_cnt[kWarps][kMaxExperts];
   __shared__ int kept_s[kMaxExperts], slot_s[kSmallTokens];
   __shared__ float term[kMaxExperts];

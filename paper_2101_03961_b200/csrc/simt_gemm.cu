@@ -9,7 +9,7 @@
 // multiply-adds) halves the slots.  In the large tile a thread keeps 8 x 8 outputs (two groups of 4 rows x two groups of
 // 4 columns), so four 16-byte shared-memory loads feed 64 multiply-adds, and the next k-chunk travels from global memory
 // to registers while the current one is multiplied; three blocks of four warps per SM leave it 168 registers.  Warps whose rows lie past an expert's last token multiply nothing.
-// Measured at 4096 tokens, 512 x 2048, 16 experts: weight gradients 168 us each (51 TFLOP/s) where 64 x 64 tiles with plain
+// Measured at 4096 tokens, 512 x 2048, 16 experts (on this path; by default that layer runs on the tensor cores): weight gradients 168 us each (51 TFLOP/s) where 64 x 64 tiles with plain
 // FFMA and no prefetch took 330; GEMM1 187 (377), dgrad2 214 (385).
 #include "switch_common.cuh"
 
@@ -240,7 +240,7 @@ template <typename ET, int OP>
 void launch_op(const SimtProblem& pr, int max_m, int E, cudaStream_t st) {
   // The largest tile that still occupies the chip: below that a launch waits for the few blocks there are, each walking
   // its whole contraction, and smaller tiles spread the outputs over more SMs.  64 x 128 tiles (three blocks per SM) want
-  // as many blocks as are resident: at 4096 tokens, 512 x 2048, 16 experts GEMM2's 320 blocks took 299 us, 64 x 64 tiles
+  // as many blocks as are resident: at 4096 tokens, 512 x 2048, 16 experts (SWITCH_MOE_GEMM_SIMT) GEMM2's 320 blocks took 299 us, 64 x 64 tiles
   // 240, while GEMM1 (1280 blocks) takes 187 and 221.  128 x 128 tiles: 371 and 215 (a third of their rows lie past the
   // experts' last tokens).  GEMM2 of 512 tokens, 64 x 256, 8 experts: 27 us with 64 x 64 tiles and 16 steps per round, 13
   // with 32 x 32 and 64 steps.

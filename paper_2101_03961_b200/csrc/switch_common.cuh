@@ -13,7 +13,11 @@ namespace swmoe {
 
 constexpr int kMaxExperts = 256;        // router kernels keep ceil(E/32) <= 8 experts per lane
 constexpr int kPlanBlockTokens = 256;   // tokens per dispatch-plan block (one histogram row each)
-constexpr int kSmallTokens = 256;      // up to here the plan and the forward gather are one launch
+constexpr int kSmallTokens = 256;      // up to here the plan and the forward gather are one launch, a token per thread.  Forward
+                                       // passes with one launch / three, us: 96 tokens, d 256, 8 experts 24.5 / 27.8; 256, d 256, 8
+                                       // 24.5 / 27.9; 256, d 768, 128 181.5 / 185.6.  Blocks of 512 threads: 300 and 512 tokens, d 256,
+                                       // 8 gain (25.5 / 27.8, 25.7 / 28.7), the three above lose 0.6, 0.7, 1.2, float32 training of
+                                       // 512 tokens 2.3
 constexpr int kTileM = 128;             // token rows per tensor-core tile; tails are zero-filled to this
 constexpr int kPairTileTokens = 320;    // widest token tile of the paired-CTA GEMM (tokens on the MMA's N side, two
                                         // column segments above 256): an expert within the capacity of the paper's

@@ -5,7 +5,10 @@ import math
 import pytest
 import torch
 
+from paper_2101_03961_b200 import inputs as si
 from paper_2101_03961_b200 import switch_moe as sm
+from tests.gpu_helpers import TOL_F32
+from tests.test_gpu_parity import _check_layer, _check_top2
 
 pytestmark = pytest.mark.gpu
 
@@ -259,3 +262,19 @@ def test_products_are_no_slower_than_fused_multiply_adds(T, d, f, E, geglu):
     and the events' resolution (where they were chosen wrongly it was 1.3 to 2.3 times)."""
     a, b = (_stage_times(T, d, f, E, 1.25, path, geglu) for path in (sm.GEMM_DEFAULT, sm.GEMM_SIMT))
     assert all(a[k] <= 1.15 * b[k] + 2.0 for k in a), (a, b)
+
+
+@pytest.mark.parametrize("kw", [
+    dict(geglu=True), dict(geglu=True, dropout=0.3, residual=True), dict(dropout=0.3), dict(dropout=0.3, noise_eps=0.3),
+    dict(reroute=True), dict(reroute=True, reroute_stages=3, geglu=True), dict(groups=2, residual=True), dict(jitter_eps=0.2)],
+    ids=lambda kw: "-".join(kw))
+def test_options_on_tensor_core_products_match_oracle(kw):
+    """Every product on the tensor cores (256 tokens per expert, f not a multiple of a tile), checked like every other layer."""
+    _check_layer(si.SwitchConfig("f32_options", 2048, 128, 352, 8, 1.0, bias_std=0.5, dtype=si.DTYPE_F32), sm.GEMM_DEFAULT,
+                 TOL_F32, d_aux=0.7, **kw)
+
+
+@pytest.mark.parametrize("residual", [False, True])
+def test_top2_on_tensor_core_products_matches_oracle(residual):
+    _check_top2(si.SwitchConfig("f32_top2", 2048, 128, 352, 8, 1.0, bias_std=0.5, dtype=si.DTYPE_F32), sm.GEMM_DEFAULT, TOL_F32,
+                residual=residual, expect_mix=False)

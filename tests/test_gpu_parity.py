@@ -344,8 +344,10 @@ def test_tiny_fp32_layer_matches_oracle():
     (1111, 264, 520, 7),        # medium tiles with remainders
     (2050, 136, 2056, 16),      # large tiles for d_ff outputs, medium ones for d_model outputs
     (9600, 40, 72, 5)])         # 64 router tokens per block, the longest x^T dh splits
-def test_float32_layer_on_every_tile_size_matches_oracle(T, d, f, E):
-    _check_layer(si.SwitchConfig("f32_tiles", T, d, f, E, 1.25, dtype=si.DTYPE_F32), sm.GEMM_DEFAULT, TOL_F32)
+@pytest.mark.parametrize("path", [sm.GEMM_DEFAULT, sm.GEMM_SIMT], ids=["default", "fma"])
+def test_float32_layer_on_every_tile_size_matches_oracle(T, d, f, E, path):
+    """The tile sizes are the FMA kernels'; on the default path the third and fourth shape run on the tensor cores."""
+    _check_layer(si.SwitchConfig("f32_tiles", T, d, f, E, 1.25, dtype=si.DTYPE_F32), path, TOL_F32)
 
 
 @pytest.mark.parametrize("cfg", [MID, RAGGED, MANY], ids=lambda c: c.name)

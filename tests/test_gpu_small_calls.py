@@ -21,6 +21,12 @@ def test_small_calls_match_oracle(T, d, E, cf, kw, dtype):
     _check_layer(cfg, sm.GEMM_DEFAULT, TOL_F32 if dtype == si.DTYPE_F32 else TOL_BF16, **kw)
 
 
+@pytest.mark.gpu
+def test_small_float32_call_with_tensor_core_products_matches_oracle():
+    cfg = si.SwitchConfig("small_tc", 250, 320, 576, 3, 1.25, bias_std=0.3, dtype=si.DTYPE_F32)
+    _check_layer(cfg, sm.GEMM_DEFAULT, TOL_F32, residual=True)
+
+
 def test_small_calls_have_fewer_launches():
     small, large = (sm.switch_moe_stage_launches(sm.make_config(T, 256, 512, 64, 2.0)) for T in (256, 257))
     assert (small["dispatch_plan"], small["gather_x"]) == (0, 1) and (large["dispatch_plan"], large["gather_x"]) == (2, 1)
