@@ -328,7 +328,7 @@ int switch_moe_stage_launches(const switch_moe_config* cfg, int32_t* launches_ou
   // element-wise product, top-2 routing the second-choice kernel.
   n[0] = (s.router_tc ? 2 : 1) + (s.jitter ? 1 : 0) + (s.top2 ? 1 : 0);
   // plan: (histograms, where the router left none,) then slots and summary side by side, or scan and assignment for several
-  // groups, top-2 routing and above 262144 tokens; a stage of rerouting adds four.  Up to 256 tokens of one group, without
+  // groups, top-2 routing and larger tables (launch_dispatch_plan has the line); a stage of rerouting adds four.  Up to 256 tokens of one group, without
   // rerouting: part of the gather's launch
   n[1] = s.plan_gather ? 0 : (s.router_hist ? 2 : 3) + 4 * s.reroute_stages;
   n[2] = 1;                                           // gather

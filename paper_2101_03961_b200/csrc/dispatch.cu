@@ -844,9 +844,13 @@ int launch_dispatch_plan(const Shape& s, const Plan& p, const int32_t* expert_in
   const bool have_hist = after_router && s.router_hist;
   if (!have_hist)
     launch_k(plan_hist_kernel, dim3(s.plan_blocks), dim3(kPlanBlockTokens), 0, st, ei, s.Tv, s.E, ws_ptr<int>(ws, p.hist));
-  // (512 tokens, 8 experts, float32, between stage events: counting, slots and summary 13.4 us, counting, scan and assignment
-  // 20.9.)
-  if (s.G == 1 && !s.top2 && s.T <= kFusedMaxTokens) {
+  // Slots and summary each read whole tables (every block the counts, one block those and the router's P-sums), the scan reads
+  // them once and serially.  Where the router has left the counts that is the faster form up to kFusedMaxTokens; where they are
+  // counted first, up to 2^21 cells of tokens x experts and 2^15 of P-sums (of at most 1024 rows).  Staged plan, us, so / by scan: bf16
+  // 32768 tokens, 64 experts 13.1 / 13.6; 49152, 128 18.9 / 16.9; 32768, 256 19.4 / 17.5; float32 4096, 128 13.0 / 14.9; 4096, 256
+  // 17.2 / 17.0; 65536, 8 13.5 / 15.1; 131072, 8 19.3 / 17.5; 262144, 256 155 / 111.
+  const bool counted_small = (long long)s.T * s.E <= 1 << 21 && s.router_blocks <= 1024 && s.router_blocks * s.E <= 1 << 15;
+  if (s.G == 1 && !s.top2 && s.T <= kFusedMaxTokens && (have_hist || counted_small)) {
     const int token_blocks = (s.T + kFusedTokens - 1) / kFusedTokens;
     const int hist_rows = have_hist ? s.router_blocks : s.plan_blocks;
     launch_k(plan_slots_kernel, dim3(token_blocks), dim3(kFusedTokens), 0, st, ei, ws_ptr<int>(ws, p.hist), hist_rows,

@@ -216,20 +216,69 @@ def test_plan_of_very_many_tokens():
             sm.switch_moe_check_device_status(cfg, ws)
             best[T] = min(best[T], events[1].elapsed_time(events[2]))
         view = lambda region: sm.switch_moe_workspace_view(cfg, ws, region)
-        e = view(sm.WS_EXPERT_INDEX).long()
-        order = torch.argsort(e, stable=True)
-        count = torch.bincount(e, minlength=E)
-        pos = torch.empty_like(e)
-        pos[order] = torch.arange(T, device="cuda") - (count.cumsum(0) - count)[e[order]]
         C = sm.switch_moe_capacity(cfg)
-        slot = torch.where(pos < C, e * C + pos, -1)
-        token_of_slot = torch.full((E * C,), -1, device="cuda", dtype=torch.int64)
-        token_of_slot[slot[slot >= 0]] = torch.nonzero(slot >= 0).flatten()
+        count, slot, token_of_slot = _plan_of(view(sm.WS_EXPERT_INDEX).long(), E, C)
         assert torch.equal(view(sm.WS_COUNT).long(), count) and torch.equal(view(sm.WS_KEPT).long(), count.clamp(max=C))
         assert torch.equal(view(sm.WS_SLOT).long(), slot) and torch.equal(view(sm.WS_TOKEN_OF_SLOT).long(), token_of_slot)
         psum = view(sm.WS_PROBS).view(T, E).sum(0, dtype=torch.float64)
         torch.testing.assert_close(view(sm.WS_PSUM).double(), psum, rtol=TOL_ROUTER, atol=0.0)
     assert best[1048576] < 6.0 * best[262144]
+
+
+def _plan_of(e, E, C):
+    """The dispatch plan of expert indices `e` (a device tensor): count, slot, token_of_slot."""
+    order = torch.argsort(e, stable=True)
+    count = torch.bincount(e, minlength=E)
+    pos = torch.empty_like(e)
+    pos[order] = torch.arange(len(e), device="cuda") - (count.cumsum(0) - count)[e[order]]
+    slot = torch.where(pos < C, e * C + pos, -1)
+    token_of_slot = torch.full((E * C,), -1, device="cuda", dtype=torch.int64)
+    token_of_slot[slot[slot >= 0]] = torch.nonzero(slot >= 0).flatten()
+    return count, slot, token_of_slot
+
+
+@pytest.mark.parametrize("T,E,dtype", [
+    (8192, 256, sm.BF16), (8193, 256, sm.BF16),                # 2^21 cells of tokens x experts
+    (8192, 64, sm.F32), (8193, 64, sm.F32),                    # 2^15 cells of P-sums
+    (65536, 8, sm.F32), (65537, 8, sm.F32)])                   # 1024 rows of P-sums
+def test_plan_on_both_sides_of_the_largest_counted_tables(T, E, dtype):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(19)
+    cfg = sm.make_config(T, 64, 64, E, 1.0, dtype=dtype)
+    x = torch.randn(T, 64, device="cuda", generator=gen).to(torch.bfloat16 if dtype == sm.BF16 else torch.float32)
+    W_r, aux, ws = torch.randn(64, E, device="cuda", generator=gen), torch.empty(1, device="cuda"), sm.allocate_workspace(cfg)
+    ws.fill_(0xFF)
+    sm.switch_moe_router_fwd(cfg, x, W_r, None, ws)
+    sm.switch_moe_dispatch_plan(cfg, None, aux, ws)
+    torch.cuda.synchronize()
+    view = lambda region: sm.switch_moe_workspace_view(cfg, ws, region)
+    C = sm.switch_moe_capacity(cfg)
+    count, slot, token_of_slot = _plan_of(view(sm.WS_EXPERT_INDEX).long(), E, C)
+    assert torch.equal(view(sm.WS_COUNT).long(), count) and torch.equal(view(sm.WS_KEPT).long(), count.clamp(max=C))
+    assert torch.equal(view(sm.WS_SLOT).long(), slot) and torch.equal(view(sm.WS_TOKEN_OF_SLOT).long(), token_of_slot)
+    psum = view(sm.WS_PROBS).view(T, E).sum(0, dtype=torch.float64)
+    torch.testing.assert_close(view(sm.WS_PSUM).double(), psum, rtol=TOL_ROUTER, atol=0.0)
+    loss = cfg.alpha * E * float((count.double() / T * psum / T).sum())
+    assert abs(float(aux) - loss) <= TOL_ROUTER * loss
+
+
+def test_counted_plan_of_many_cells_goes_by_scan():
+    # one token more than the other form ever takes must not be the faster call (it was, 111 us against 155)
+    E, times = 256, {}
+    for T in (262144, 262145):
+        cfg = sm.make_config(T, 64, 64, E, 1.0, dtype=sm.F32)
+        ws, e = sm.allocate_workspace(cfg), torch.randint(0, E, (T,), dtype=torch.int32, device="cuda")
+        ws.zero_()
+        times[T] = []
+        for _ in range(5):
+            start, end = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+            start.record()
+            for _ in range(10):
+                sm.switch_moe_dispatch_plan(cfg, e, None, ws)
+            end.record()
+            torch.cuda.synchronize()
+            times[T].append(start.elapsed_time(end))
+    assert min(times[262144]) <= 1.15 * min(times[262145]), times
 
 
 def test_dispatch_plan_is_deterministic():
