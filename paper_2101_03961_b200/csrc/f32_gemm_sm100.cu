@@ -684,27 +684,25 @@ int launch_op(const CUtensorMap& tmA, const CUtensorMap& tmB, const F32Problem& 
 
 }  // namespace
 
-// Which float32 products run here: those of at least 0.07 GFLOP (weight gradients 0.12; 2 rows d f), below which the 3 us that a
+// Which float32 products run here: those of at least 0.07 GFLOP (weight gradients 0.09; 2 rows d f), below which the 3 us that a
 // launch has more to set up than an FMA kernel's (tensor memory, barriers, cold code) decide, and of them
-// - token products with enough steps per tile to pay for its two ends.  Medians over shapes of 16 to 65536 tokens, 1 to 256
-//   experts, stage time here / FMA kernels, by contraction: GEMM1 with dgrad2 8..15 1.26, 32..47 1.06, 64..71 0.86, GEMM1 alone
-//   2.18, 1.34, 1.03, from 72 on 0.99, 80..95 0.93, 128..191 0.76; GEMM2 and dgrad1 32..47 1.33, 80..95 1.00, 96..111 0.87.  An
-//   output narrower than half a tile leaves the rest of its MMAs idle: 64..95 1.18, 144..191 0.95, 192..255 0.86.  Tiles of few
-//   tokens whose contraction is short, or output narrower still, are nothing but their ends (25 tokens, 72 x 96: 1.46; 22, 528 x 16:
-//   1.36).
-// - weight gradients of enough tokens to be more than writing the output (20..23 per expert 1.00, 24..31 1.04, 40..47 0.95, 48..63
-//   0.88), and of outputs of enough tiles: a tile walks its whole contraction on one SM at the rate of one FMA block of 64 x 64,
-//   so with fewer than about half an FMA block per SM the chip is idle either way (24..47 blocks 1.09, 48..71 0.97, 72..95 0.87).
-// On 440 shapes drawn afterwards the six products of a step take 0.74 of the FMA kernels' time in the median and 1.08 at most, a
-// single one up to 1.3.  GEMM1 and dgrad2 always go together: the mask that one leaves is the one that the other reads.
+// - token products with enough steps per tile to pay for its two ends.  Whole forward passes with the product here / on FMA,
+//   medians over shapes of 16 to 65536 tokens, 1 to 256 experts, by contraction: GEMM1 8..15 1.21, 32..47 1.08, 64..71 1.03, 72..79
+//   0.99, 96..127 0.94; GEMM2 8..15 1.16, 32..47 1.06, 80..95 0.97 (steps: up to 1.07), 96..111 0.97 (1.00), 128..191 0.90.  An output
+//   narrower than half a tile leaves the rest of its MMAs idle: 64..95 1.06, 144..191 0.99 (up to 1.11), 192..255 0.94.  Tiles of
+//   few tokens whose contraction is short, or output narrower still, are nothing but their ends: GEMM1 of 25 tokens per expert, 72 x
+//   96, 226 experts 18.4 / 12.6 us; 22, 528 x 16, 194 30.7 / 22.5.
+// - weight gradients of enough tokens to be more than writing the output: whole steps, tokens per expert 4..7 1.12, 12..15 1.07,
+//   20..31 1.01, 32..47 0.99, 64..127 0.96, more 0.82.  (A tile walks its contraction on one SM at the rate of one FMA block of
+//   64 x 64.  Where outputs have few tiles the FMA kernels are up to a fifth faster by themselves, but in a row of launches their
+//   few blocks crowd onto the first free SMs: 13764 tokens, 16 x 472, 2 GEGLU experts, a step 463 us here, 836 there.)
+// On 660 shapes no call is slower by more than 2% than with all products on FMA; forward passes take 0.73, steps 0.70 of its time
+// in the mean.  GEMM1 and dgrad2 always go together: the mask that one leaves is the one that the other reads.
 bool f32_on_tensor_cores(GemmOp op, const Shape& s) {
   if (!s.f32_tc) return false;
   const double rows = s.Tv < (double)s.E * s.C ? s.Tv : (double)s.E * s.C, flops = 2.0 * rows * s.d * s.f;
+  if (op == kWgrad2 || op == kWgrad1) return flops >= 9e7 && rows >= 24.0 * s.E;
   const bool first = op == kGemm1Relu || op == kDgrad2Mask;            // d deep, f wide; the other token products f deep, d wide
-  if (op == kWgrad2 || op == kWgrad1) {
-    const long long blocks = (long long)s.E * ((s.d + 63) / 64) * (((op == kWgrad1 ? s.fin : s.f) + 63) / 64);
-    return flops >= 1.2e8 && rows >= 48.0 * s.E && blocks >= kChipSms / 2;
-  }
   const int steps = first ? s.d : op == kGemm2Combine ? s.f : s.fin, width = first ? s.f : s.d;
   const double tiles = (double)s.E * ceil(rows / s.E / kNMax) * ((width + kM - 1) / kM), tile_flops = 2.0 * rows * width * steps / tiles;
   return flops >= 7e7 && steps >= (width < 64 ? 192 : first ? 72 : 96) && (tile_flops >= 5e5 || (steps >= 128 && width >= 32));
