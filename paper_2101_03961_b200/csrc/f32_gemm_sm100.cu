@@ -689,7 +689,7 @@ int launch_op(const CUtensorMap& tmA, const CUtensorMap& tmB, const F32Problem& 
 // - token products with enough steps per tile to pay for its two ends.  Whole forward passes with the product here / on FMA,
 //   medians over shapes of 16 to 65536 tokens, 1 to 256 experts, by contraction: GEMM1 8..15 1.21, 32..47 1.08, 64..71 1.03, 72..79
 //   0.99, 96..127 0.94; GEMM2 8..15 1.16, 32..47 1.06, 80..95 0.97 (steps: up to 1.07), 96..111 0.97 (1.00), 128..191 0.90.  An output
-//   narrower than half a tile leaves the rest of its MMAs idle: 64..95 1.06, 144..191 0.99 (up to 1.11), 192..255 0.94.  Tiles of
+//   no wider than half a tile leaves the rest of its MMAs idle: 64..95 1.06, 144..191 0.99 (up to 1.11), 192..255 0.94.  Tiles of
 //   few tokens whose contraction is short, or output narrower still, are nothing but their ends: GEMM1 of 25 tokens per expert, 72 x
 //   96, 226 experts 18.4 / 12.6 us; 22, 528 x 16, 194 30.7 / 22.5.
 // - weight gradients of enough tokens to be more than writing the output: whole steps, tokens per expert 4..7 1.12, 12..15 1.07,
@@ -705,7 +705,7 @@ bool f32_on_tensor_cores(GemmOp op, const Shape& s) {
   const bool first = op == kGemm1Relu || op == kDgrad2Mask;            // d deep, f wide; the other token products f deep, d wide
   const int steps = first ? s.d : op == kGemm2Combine ? s.f : s.fin, width = first ? s.f : s.d;
   const double tiles = (double)s.E * ceil(rows / s.E / kNMax) * ((width + kM - 1) / kM), tile_flops = 2.0 * rows * width * steps / tiles;
-  return flops >= 7e7 && steps >= (width < 64 ? 192 : first ? 72 : 96) && (tile_flops >= 5e5 || (steps >= 128 && width >= 32));
+  return flops >= 7e7 && steps >= (width <= 64 ? 192 : first ? 72 : 96) && (tile_flops >= 5e5 || (steps >= 128 && width >= 32));
 }
 
 int launch_f32_gemm(GemmOp op, const Shape& s, const Plan& p, const GemmArgs& a, void* ws, cudaStream_t st) {

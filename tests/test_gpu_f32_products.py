@@ -261,6 +261,7 @@ def _call_times(T, d, f, E, geglu):
     (9651, 8, 2120, 5, False),             # short contractions: GEMM1
     (23182, 1144, 8, 35, False),           # and GEMM2, dgrad1
     (22440, 120, 32, 44, False),           # narrow outputs
+    (27995, 64, 104, 55, False),           # half a tile wide
     (5650, 72, 96, 226, False),            # 25 tokens per expert and little else
     (13764, 16, 472, 2, True),             # weight gradients of few tiles
     (600, 232, 1160, 150, False),          # and of few tokens
