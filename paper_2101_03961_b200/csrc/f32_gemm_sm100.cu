@@ -29,7 +29,7 @@
 // adding up and the waits between the roles issue in 60% of all slots, and the code of all roles together streams through the
 // instruction caches.  Taking out any one of conversion of A, of B, the correction MMAs, or the adding up shortened a product by
 // 6 to 14%.  4096 tokens, 512 x 2048, 16 experts, between stage events, FMA kernels / here: GEMM1 187 / 80 us, GEMM2 233 / 86,
-// dgrad2 213 / 78, wgrad2 170 / 69, dgrad1 242 / 84, wgrad1 170 / 69 (108 to 126 TFLOP/s; the FMA pipes' peak is 74.5).
+// dgrad2 213 / 78, wgrad2 170 / 69, dgrad1 242 / 84, wgrad1 170 / 69 (100 to 125 TFLOP/s; the FMA pipes' peak is 74.5).
 #include <cfloat>
 #include <cmath>
 
